@@ -14,7 +14,8 @@
 // coincident (remainder at its R -> 0 limit, no gradient term).
 //
 // Stage 1: one thread per (block, test triangle, source triangle) computes
-//          the 3x3 slot integrals of both operators into a scratch buffer.
+//          the 3x3 slot integrals of both operators into a scratch buffer
+//          from the 3x3 barycentric moments of G and of its gradient factor.
 // Stage 2: one thread per (block, test RWG, source RWG) sums the 2 x 2
 //          triangle combinations of the two RWGs with their amplitudes.
 // Blocks are processed in chunks so the scratch stays below 256 MB.
@@ -37,6 +38,8 @@ struct TriGeo {
     double area;
     double n[3];     // unit normal (v1-v0) x (v2-v0)
     double scale;    // max(|v1-v0|, |v2-v0|)
+    double lh[9];    // unit vector of edge i, v_i -> v_{i+1}
+    double u[9];     // its in-plane outward normal lh x n
 };
 
 struct RwgSlots {    // the two (triangle, slot) pairs of an RWG with amplitude sgn*len/(2A)
@@ -45,7 +48,14 @@ struct RwgSlots {    // the two (triangle, slot) pairs of an RWG with amplitude 
     double c[2];
 };
 
-__constant__ double c_w[7];
+__constant__ double c_wl[21];   // w_q lambda_u(q) of the rule at [3 q + u]
+
+// the 7-point rule: the centroid, then two orbits of three points with one
+// barycentric coordinate b and two a
+constexpr double kS15 = 3.8729833462074168852;
+constexpr double kRa1 = (6.0 - kS15) / 21.0, kRb1 = (9.0 + 2.0 * kS15) / 21.0;
+constexpr double kRa2 = (6.0 + kS15) / 21.0, kRb2 = (9.0 - 2.0 * kS15) / 21.0;
+constexpr double kRw0 = 9.0 / 40.0, kRw1 = (155.0 - kS15) / 1200.0, kRw2 = (155.0 + kS15) / 1200.0;
 
 struct Vec3 {
     double x, y, z;
@@ -60,98 +70,99 @@ __device__ __forceinline__ Vec3 cross(Vec3 a, Vec3 b) {
 }
 __device__ __forceinline__ double norm3(Vec3 a) { return sqrt(dot(a, a)); }
 
-// G and grad_r G = (r - r') * gfac, far form
-__device__ __forceinline__ void green_far(double R, double k, double2& G, double2& gfac) {
+// 4 pi G and 4 pi times the factor of grad_r G = (r - r') gfac, far form, from
+// R2 = |r - r'|^2.  The phase is taken as kR / pi for sincospi, whose range
+// reduction is exact.
+__device__ __forceinline__ void green_far(double R2, double k, double kpi, double2& G, double2& gfac) {
+    const double ri = rsqrt(R2), R1 = R2 * ri, R = fma(0.5 * ri, fma(-R1, R1, R2), R1);
     double s, c;
-    sincos(k * R, &s, &c);
-    const double2 e = make_double2(c, -s);                       // e^{-jkR}
-    G = make_double2(e.x / (kFourPi * R), e.y / (kFourPi * R));
-    const double2 a = make_double2(1.0, k * R);                  // 1 + jkR
-    const double2 ae = cmul(a, e);
-    const double d = -1.0 / (kFourPi * R * R * R);
-    gfac = make_double2(ae.x * d, ae.y * d);
+    sincospi(kpi * R, &s, &c);
+    G = make_double2(c * ri, -s * ri);                           // e^{-jkR} / R
+    const double kR = k * R, m = -ri * ri;
+    // -(1 + jkR) e^{-jkR} / R^3
+    gfac = make_double2(m * fma(-kR, G.y, G.x), m * fma(kR, G.x, G.y));
 }
 
-// remainder after removing 1/(4 pi R): series for kR < 0.1, closed form otherwise
-__device__ __forceinline__ void green_smooth(double R, double k, double2& Gs, double2& gfac) {
-    const double kR = k * R;
-    if (kR < 0.1) {
-        // (e^{-jkR}-1)/R = sum_{n>=1} c_n R^{n-1},  d/dR = sum_{n>=2} c_n (n-1) R^{n-2},
-        // c_n = (-jk)^n / n!
-        double2 c = make_double2(1.0, 0.0);
-        double2 g = make_double2(0.0, 0.0), h = make_double2(0.0, 0.0);
-        double Rp_n1 = 1.0;    // R^{n-1}
-        double Rp_n2 = 0.0;    // R^{n-2}
-        for (int n = 1; n < 12; ++n) {
-            c = cmul(c, make_double2(0.0, -k / (double)n));
-            g.x += c.x * Rp_n1;
-            g.y += c.y * Rp_n1;
-            if (n >= 2) {
-                h.x += c.x * (double)(n - 1) * Rp_n2;
-                h.y += c.y * (double)(n - 1) * Rp_n2;
-            }
-            Rp_n2 = Rp_n1;
-            Rp_n1 *= R;
-        }
-        Gs = make_double2(g.x / kFourPi, g.y / kFourPi);
-        if (R > 0.0) gfac = make_double2(h.x / (kFourPi * R), h.y / (kFourPi * R));
-        else gfac = make_double2(0.0, 0.0);
+// remainder after removing 1/R (times 4 pi): power series for kR < 0.5 (no
+// cancellation), closed form otherwise
+__device__ __forceinline__ void green_smooth(double R, double k, double kpi, double2& Gs, double2& gfac) {
+    const double z = k * R;
+    if (z < 0.5) {
+        // (e^{-jz} - 1) / R and (1 - (1 + jz) e^{-jz}) / R^3 with e^{-jz} = cos z - j sin z:
+        // real and imaginary parts are even/odd series in w = z^2
+        const double w = z * z;
+        constexpr double f3 = 1.0 / 6, f5 = f3 / 20, f7 = f5 / 42, f9 = f7 / 72, f11 = f9 / 110, f13 = f11 / 156, f15 = f13 / 210;
+        constexpr double f2 = 0.5, f4 = f2 / 12, f6 = f4 / 30, f8 = f6 / 56, f10 = f8 / 90, f12 = f10 / 132, f14 = f12 / 182, f16 = f14 / 240;
+        // (1 - cos z) / w, sin z / z
+        const double pc = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, f14, -f12), f10), -f8), f6), -f4), f2);
+        const double ps = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, f15, -f13), f11), -f9), f7), -f5), f3);
+        // sin z / z = 1 - w (f3 - w f5 + w^2 f7 - ...)
+        Gs = make_double2(-k * z * pc, -k * fma(-w, ps, 1.0));
+        // (1 - cos z - z sin z) / w = sum (-1)^m (2m - 1) / (2m)! w^(m-1)
+        const double qr = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, 15 * f16, -13 * f14), 11 * f12), -9 * f10), 7 * f8), -5 * f6), 3 * f4), -f2);
+        // (sin z - z cos z) / z^3 = sum (-1)^(m+1) 2m / (2m + 1)! w^(m-1)
+        const double qi = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, 14 * f15, -12 * f13), 10 * f11), -8 * f9), 6 * f7), -4 * f5), 2 * f3);
+        const double ri = R > 0.0 ? 1.0 / R : 0.0;
+        const double k2 = k * k;
+        gfac = make_double2(k2 * ri * qr, R > 0.0 ? k2 * k * qi : 0.0);
         return;
     }
-    double s, cc;
-    sincos(kR, &s, &cc);
-    const double2 e = make_double2(cc, -s);
-    Gs = make_double2((e.x - 1.0) / (kFourPi * R), e.y / (kFourPi * R));
-    const double2 ae = cmul(make_double2(1.0, kR), e);           // (1 + jkR) e
-    const double R2 = R * R;
-    const double2 hh = make_double2((1.0 - ae.x) / R2, -ae.y / R2);
-    gfac = make_double2(hh.x / (kFourPi * R), hh.y / (kFourPi * R));
+    const double ri = 1.0 / R;
+    double s, c;
+    sincospi(kpi * R, &s, &c);
+    Gs = make_double2((c - 1.0) * ri, -s * ri);
+    const double ri3 = ri * ri * ri;
+    gfac = make_double2(ri3 * (1.0 - fma(z, s, c)), ri3 * fma(-z, c, s));
 }
 
 // Lossy region (Sec. II-B, k_v = w sqrt(mu0 eps_v) with complex eps_v): the
 // same two functions for k = kr + j ki, e^{-jkR} = e^{ki R} e^{-j kr R}.
-__device__ __forceinline__ double2 exp_mjkR(double R, double kr, double ki) {
+__device__ __forceinline__ double2 exp_mjkR(double R, double kpi, double ki) {
     double s, c;
-    sincos(kr * R, &s, &c);
+    sincospi(kpi * R, &s, &c);
     const double m = exp(ki * R);
     return make_double2(m * c, -m * s);
 }
 
-__device__ __forceinline__ void green_far_cx(double R, double kr, double ki, double2& G, double2& gfac) {
-    const double2 e = exp_mjkR(R, kr, ki);
-    G = make_double2(e.x / (kFourPi * R), e.y / (kFourPi * R));
-    const double2 ae = cmul(make_double2(1.0 - ki * R, kr * R), e);     // (1 + jkR) e
-    const double d = -1.0 / (kFourPi * R * R * R);
+__device__ __forceinline__ void green_far_cx(double R2, double kr, double kpi, double ki, double2& G, double2& gfac) {
+    const double ri = rsqrt(R2), R1 = R2 * ri, R = fma(0.5 * ri, fma(-R1, R1, R2), R1);
+    const double2 e = exp_mjkR(R, kpi, ki);
+    G = make_double2(e.x * ri, e.y * ri);
+    const double2 ae = cmul(make_double2(1.0 - ki * R, kr * R), G);     // (1 + jkR) e^{-jkR} / R
+    const double d = -ri * ri;
     gfac = make_double2(ae.x * d, ae.y * d);
 }
 
-__device__ __forceinline__ void green_smooth_cx(double R, double kr, double ki, double2& Gs, double2& gfac) {
-    if (hypot(kr, ki) * R < 0.1) {
-        double2 c = make_double2(1.0, 0.0);
+__device__ __forceinline__ void green_smooth_cx(double R, double kr, double kpi, double ki, double2& Gs,
+                                                double2& gfac) {
+    const double2 z = make_double2(ki * R, -kr * R);                    // -jkR
+    const double2 jk = make_double2(ki, -kr);                           // -jk
+    if (z.x * z.x + z.y * z.y < 0.25) {
+        // (e^z - 1) / z = sum z^m / (m + 1)!, (1 - (1 - z) e^z) / z^2 = sum z^m (m + 1) / (m + 2)!
         double2 g = make_double2(0.0, 0.0), h = make_double2(0.0, 0.0);
-        double Rp_n1 = 1.0, Rp_n2 = 0.0;
-        for (int n = 1; n < 12; ++n) {
-            c = cmul(c, make_double2(ki / (double)n, -kr / (double)n));   // (-jk)^n / n!
-            g.x += c.x * Rp_n1;
-            g.y += c.y * Rp_n1;
-            if (n >= 2) {
-                h.x += c.x * (double)(n - 1) * Rp_n2;
-                h.y += c.y * (double)(n - 1) * Rp_n2;
-            }
-            Rp_n2 = Rp_n1;
-            Rp_n1 *= R;
+#pragma unroll
+        for (int m = 14; m >= 0; --m) {
+            double f = 1.0;
+#pragma unroll
+            for (int i = 2; i <= m + 1; ++i) f /= i;                    // 1 / (m + 1)!
+            g = cmul(g, z);
+            g.x += f;
+            h = cmul(h, z);
+            h.x += f * (m + 1) / (m + 2);
         }
-        Gs = make_double2(g.x / kFourPi, g.y / kFourPi);
-        if (R > 0.0) gfac = make_double2(h.x / (kFourPi * R), h.y / (kFourPi * R));
-        else gfac = make_double2(0.0, 0.0);
+        Gs = cmul(jk, g);
+        const double ri = R > 0.0 ? 1.0 / R : 0.0;
+        const double2 k2 = cmul(jk, jk);
+        const double2 hh = cmul(k2, h);
+        gfac = make_double2(hh.x * ri, hh.y * ri);
         return;
     }
-    const double2 e = exp_mjkR(R, kr, ki);
-    Gs = make_double2((e.x - 1.0) / (kFourPi * R), e.y / (kFourPi * R));
+    const double ri = 1.0 / R;
+    const double2 e = exp_mjkR(R, kpi, ki);
+    Gs = make_double2((e.x - 1.0) * ri, e.y * ri);
     const double2 ae = cmul(make_double2(1.0 - ki * R, kr * R), e);
-    const double R2 = R * R;
-    const double2 hh = make_double2((1.0 - ae.x) / R2, -ae.y / R2);
-    gfac = make_double2(hh.x / (kFourPi * R), hh.y / (kFourPi * R));
+    const double ri3 = ri * ri * ri;
+    gfac = make_double2((1.0 - ae.x) * ri3, -ae.y * ri3);
 }
 
 __device__ __forceinline__ double edge_log(double lp, double lm, double Rp, double Rm, double R02) {
@@ -162,7 +173,7 @@ __device__ __forceinline__ double edge_log(double lp, double lm, double Rp, doub
 
 // closed-form int 1/R, int (rho'-rho)/R, int grad_r(1/R) over source triangle;
 // also returns rho (projection of r on the plane, after the in-plane snap)
-__device__ void potentials(Vec3 r, const TriGeo& T, double& I0, Vec3& I1, Vec3& Ig, Vec3& rho) {
+__device__ __forceinline__ void potentials(Vec3 r, const TriGeo& T, double& I0, Vec3& I1, Vec3& Ig, Vec3& rho) {
     const Vec3 v0 = v3(T.v), n = v3(T.n);
     double d = dot(n, r - v0);
     if (fabs(d) <= 1e-9 * T.scale) d = 0.0;
@@ -175,130 +186,210 @@ __device__ void potentials(Vec3 r, const TriGeo& T, double& I0, Vec3& I1, Vec3& 
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const Vec3 a = v3(T.v + 3 * i), b = v3(T.v + 3 * ((i + 1) % 3));
-        const Vec3 ba = b - a;
-        const double le = norm3(ba);
-        const Vec3 lh = (1.0 / le) * ba;
-        const Vec3 u = cross(lh, n);
+        const Vec3 lh = v3(T.lh + 3 * i), u = v3(T.u + 3 * i);
         const double lp = dot(b - rho, lh), lm = dot(a - rho, lh);
         const double t = dot(a - rho, u);
         const double R02 = t * t + d * d;
         const double Rp = sqrt(R02 + lp * lp), Rm = sqrt(R02 + lm * lm);
         const double f = edge_log(lp, lm, Rp, Rm, R02);
-        const double beta = atan2(t * lp, R02 + ad * Rp) - atan2(t * lm, R02 + ad * Rm);
-        I0 += t * f - ad * beta;
+        I0 += t * f;
         I1 = I1 + (0.5 * (R02 * f + lp * Rp - lm * Rm)) * u;
         fu = fu + f * u;
-        bsum += beta;
+        if (ad > 0.0) {
+            // difference of the two angles atan2(t l, R02 + |d| R), both inside (-pi/2, pi/2)
+            const double xp = R02 + ad * Rp, xm = R02 + ad * Rm, yp = t * lp, ym = t * lm;
+            bsum += atan2(yp * xm - xp * ym, xp * xm + yp * ym);
+        }
     }
+    I0 -= ad * bsum;
     const double sg = (d > 0.0) - (d < 0.0);
     Ig = (-sg * bsum) * n - fu;
 }
 
 // out[((b*Tt + t)*Ts + s)*18 + {0..8: L(i,j), 9..17: K(i,j)}]; CX: complex
-// wavenumber k + j ki (lossy region), else ki is ignored
-template <bool CX>
+// wavenumber k + j ki (lossy region), else ki is ignored; SING: closed-form
+// 1/R parts.
+//
+// On a triangle r - v_i = sum_u lambda_u (v_u - v_i), so every slot integral
+// is a combination of the 3 x 3 barycentric moments M[u][v] = sum_qp w_q w_p
+// lambda_u(q) lambda_v(p) f(r_q, r'_p) of f = G and f = gfac:
+//   L(i, j) = sum_{u != i, v != j} MG[u][v] (v_u - v_i).(s_v - s_j) - 4/k^2 sum MG
+// and, with r - r' = a + c - b (a = r - v_i, b = r' - s_j, c = v_i - s_j),
+// a.((r - r') x b) = c.(b x a):
+//   K(i, j) = sum_{u != i, v != j} Mg[u][v] c.((s_v - s_j) x (v_u - v_i)),
+// where the triple product depends, up to sign, on the two edges only (9
+// values).  The kernel is bound by the FP64 rate (2 FMA per clock and SM):
+// distance, rsqrt, sincospi and 7 operations for the moments are left per
+// point pair, 0.135 ns on average over 25 blocks of 192 x 192 triangles
+// (6.1 ms), against 0.37 ns (16.6 ms) when each point pair updated the 9 + 9
+// slot integrals.
+template <bool CX, bool SING>
 __global__ void __launch_bounds__(128)
 tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict__ sg, int Ts,
-                 const double* __restrict__ shifts, const int8_t* __restrict__ sing, int b0,
-                 double k, double ki, double2* __restrict__ out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int t = blockIdx.y;
-    const int bl = blockIdx.z;
-    if (s >= Ts) return;
-    const int b = b0 + bl;
+                 const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out) {
+    const int pair = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pair >= Tt * Ts) return;
+    const int t = pair / Ts, s = pair - t * Ts;
+    const int bl = blockIdx.y;
     const TriGeo& A = tg[t];
     const TriGeo& S = sg[s];
-    const Vec3 sh = v3(shifts + 3 * b);
-    const bool singular = sing[b] != 0;
-    double2 ik2c;                                   // 4 / k^2
-    if constexpr (CX) {
-        const double2 k2 = make_double2(k * k - ki * ki, 2.0 * k * ki);
-        const double d = 4.0 / (k2.x * k2.x + k2.y * k2.y);
-        ik2c = make_double2(k2.x * d, -k2.y * d);
-    } else {
-        ik2c = make_double2(4.0 / (k * k), 0.0);
-    }
-    const double ik2 = ik2c.x;
-    double2 CL[9], CK[9];
+    const Vec3 sh = v3(shifts + 3 * (b0 + bl));
+    const double kpi = k * 0.31830988618379067154;
+    // [G.x, G.y, g.x, g.y] of the moments
+    double M[3][3][4];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) CL[q] = CK[q] = make_double2(0.0, 0.0);
-    const Vec3 tv[3] = {v3(A.v) + sh, v3(A.v + 3) + sh, v3(A.v + 6) + sh};
-    const Vec3 sv[3] = {v3(S.v), v3(S.v + 3), v3(S.v + 6)};
-    double2 sumWG = make_double2(0.0, 0.0);
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+        for (int v = 0; v < 3; ++v)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) M[u][v][c] = 0.0;
+    // closed-form parts: sums over q of w_q lambda_u times I1 + I0 (rho - s_0), I0, Ig
+    Vec3 PA[3], PC[3];
+    double PB[3];
+    if constexpr (SING) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            PA[u] = PC[u] = {0.0, 0.0, 0.0};
+            PB[u] = 0.0;
+        }
+    }
+#pragma unroll 1
     for (int q = 0; q < 7; ++q) {
         const Vec3 r = v3(A.q + 3 * q) + sh;
-        const double wq = c_w[q] * A.area;
-        const Vec3 a[3] = {r - tv[0], r - tv[1], r - tv[2]};
+        double N[3][4], base[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) N[0][c] = N[1][c] = N[2][c] = base[c] = 0.0;
+#pragma unroll
         for (int p = 0; p < 7; ++p) {
-            const Vec3 rp = v3(S.q + 3 * p);
-            const double W = wq * c_w[p] * S.area;
-            const Vec3 diff = r - rp;
-            double R = norm3(diff);
-            double2 G, gf;
-            // coincident points (up to rounding) take the R -> 0 limit of the
-            // remainder: -jk/(4 pi) and no gradient term
-            if (singular && R <= 1e-9 * S.scale) R = 0.0;
-            if constexpr (CX) {
-                if (singular) green_smooth_cx(R, k, ki, G, gf);
-                else green_far_cx(R, k, ki, G, gf);
+            const Vec3 diff = r - v3(S.q + 3 * p);
+            const double R2 = dot(diff, diff);
+            double2 G, g;
+            if constexpr (SING) {
+                // coincident points (up to rounding) take the R -> 0 limit of the
+                // remainder: -jk/(4 pi) and no gradient term
+                double R = sqrt(R2);
+                if (R <= 1e-9 * S.scale) R = 0.0;
+                if constexpr (CX) green_smooth_cx(R, k, kpi, ki, G, g);
+                else green_smooth(R, k, kpi, G, g);
             } else {
-                if (singular) green_smooth(R, k, G, gf);
-                else green_far(R, k, G, gf);
+                if constexpr (CX) green_far_cx(R2, k, kpi, ki, G, g);
+                else green_far(R2, k, kpi, G, g);
             }
-            const double2 WG = make_double2(W * G.x, W * G.y);
-            sumWG.x += WG.x;
-            sumWG.y += WG.y;
-            const double2 Wg = make_double2(W * gf.x, W * gf.y);
-            const Vec3 bj[3] = {rp - sv[0], rp - sv[1], rp - sv[2]};
+            const double f[4] = {G.x, G.y, g.x, g.y};
+            const double wb = p == 0 ? kRw0 / 3.0 : p < 4 ? kRw1 * kRa1 : kRw2 * kRa2;
+            const double wv = p < 4 ? kRw1 * (kRb1 - kRa1) : kRw2 * (kRb2 - kRa2);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const Vec3 dxb = cross(diff, bj[j]);     // (r-r') x b_j
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const double ab = dot(a[i], bj[j]);
-                    CL[3 * i + j].x += WG.x * ab;
-                    CL[3 * i + j].y += WG.y * ab;
-                    const double trip = dot(a[i], dxb);    // a . ((r-r') x b)
-                    CK[3 * i + j].x += Wg.x * trip;
-                    CK[3 * i + j].y += Wg.y * trip;
-                }
+            for (int c = 0; c < 4; ++c) {
+                base[c] = fma(wb, f[c], base[c]);
+                if (p > 0) N[(p - 1) % 3][c] = fma(wv, f[c], N[(p - 1) % 3][c]);
             }
         }
-        if (singular) {
+        const double wl[3] = {c_wl[3 * q], c_wl[3 * q + 1], c_wl[3 * q + 2]};
+#pragma unroll
+        for (int v = 0; v < 3; ++v)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double f = N[v][c] + base[c];
+#pragma unroll
+                for (int u = 0; u < 3; ++u) M[u][v][c] = fma(wl[u], f, M[u][v][c]);
+            }
+        if constexpr (SING) {
             double I0;
             Vec3 I1, Ig, rho;
             potentials(r, S, I0, I1, Ig, rho);
-            const double f = wq / kFourPi;
+            const Vec3 PL = I1 + I0 * (rho - v3(S.v));
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const Vec3 vecL = I1 + I0 * (rho - sv[j]);
-                const Vec3 cr = cross(Ig, r - sv[j]);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    CL[3 * i + j].x += f * (dot(a[i], vecL) - ik2 * I0);
-                    if constexpr (CX) CL[3 * i + j].y -= f * ik2c.y * I0;
-                    CK[3 * i + j].x += f * dot(a[i], cr);
-                }
+            for (int u = 0; u < 3; ++u) {
+                PA[u] = PA[u] + wl[u] * PL;
+                PB[u] = fma(wl[u], I0, PB[u]);
+                PC[u] = PC[u] + wl[u] * Ig;
             }
         }
     }
-    double2* o = out + (((size_t)bl * Tt + t) * Ts + s) * 18;
+    const Vec3 tv[3] = {v3(A.v) + sh, v3(A.v + 3) + sh, v3(A.v + 6) + sh};
+    const Vec3 sv[3] = {v3(S.v), v3(S.v + 3), v3(S.v + 6)};
+    // edge w of a triangle runs from vertex w + 1 to w + 2: dot products and
+    // triple products of every edge pair
+    double D[3][3], V[3][3];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        if constexpr (CX) {
-            const double2 t = cmul(ik2c, sumWG);
-            o[q] = make_double2(CL[q].x - t.x, CL[q].y - t.y);
-        } else {
-            o[q] = make_double2(CL[q].x - ik2 * sumWG.x, CL[q].y - ik2 * sumWG.y);
+    for (int w = 0; w < 3; ++w) {
+        const Vec3 te = v3(A.v + 3 * ((w + 2) % 3)) - v3(A.v + 3 * ((w + 1) % 3));
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            const Vec3 se = sv[(x + 2) % 3] - sv[(x + 1) % 3];
+            D[w][x] = dot(te, se);
+            V[w][x] = dot(tv[(w + 1) % 3] - sv[(x + 1) % 3], cross(se, te));
         }
-        o[9 + q] = CK[q];
     }
+    double2 ik2;                                    // 4 / k^2
+    if constexpr (CX) {
+        const double2 k2 = make_double2(k * k - ki * ki, 2.0 * k * ki);
+        const double d = 4.0 / (k2.x * k2.x + k2.y * k2.y);
+        ik2 = make_double2(k2.x * d, -k2.y * d);
+    } else {
+        ik2 = make_double2(4.0 / (k * k), 0.0);
+    }
+    const double fr = A.area * S.area / kFourPi;    // regular part
+    const double fs = A.area / kFourPi;             // closed-form part
+    double2 sum = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            sum.x += M[u][v][0];
+            sum.y += M[u][v][1];
+        }
+    double2 div = make_double2(fr * sum.x, fr * sum.y);
+    if constexpr (SING) div.x += fs * (PB[0] + PB[1] + PB[2]);
+    if constexpr (CX) div = cmul(ik2, div);
+    else div = make_double2(ik2.x * div.x, ik2.x * div.y);
+    double2* o = out + ((size_t)bl * Tt * Ts + pair) * 18;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            double l[2] = {0.0, 0.0}, kk[2] = {0.0, 0.0};
+#pragma unroll
+            for (int du = 1; du < 3; ++du)
+#pragma unroll
+                for (int dv = 1; dv < 3; ++dv) {
+                    // vertex i + du and the edge between i and it: w = i + 2 (du = 1, i -> i + 1 runs
+                    // along edge w) or w = i + 1 (du = 2, against it)
+                    const int u = (i + du) % 3, v = (j + dv) % 3;
+                    const int w = (i + 3 - du) % 3, x = (j + 3 - dv) % 3;
+                    const double sgn = (du == dv) ? 1.0 : -1.0;
+                    const double dd = sgn * D[w][x], vv = sgn * V[w][x];
+                    l[0] = fma(dd, M[u][v][0], l[0]);
+                    l[1] = fma(dd, M[u][v][1], l[1]);
+                    kk[0] = fma(vv, M[u][v][2], kk[0]);
+                    kk[1] = fma(vv, M[u][v][3], kk[1]);
+                }
+            double2 L = make_double2(fr * l[0] - div.x, fr * l[1] - div.y);
+            double2 K = make_double2(fr * kk[0], fr * kk[1]);
+            if constexpr (SING) {
+                const Vec3 sj = sv[j] - sv[0], c = tv[i] - sv[j];
+                double ls = 0.0, ks = 0.0;
+#pragma unroll
+                for (int du = 1; du < 3; ++du) {
+                    const int u = (i + du) % 3;
+                    const Vec3 te = v3(A.v + 3 * u) - v3(A.v + 3 * i);
+                    ls += dot(te, PA[u] - PB[u] * sj);
+                    ks += dot(PC[u], cross(c, te));
+                }
+                L.x += fs * ls;
+                K.x += fs * ks;
+            }
+            o[3 * i + j] = L;
+            o[9 + 3 * i + j] = K;
+        }
 }
 
-// L[b][m][n], K[b][m][n] from the slot integrals of one chunk
+// L[o][m][n], K[o][m][n], o = slot[b] (b without a slot list), from the slot
+// integrals of one chunk
 __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots* __restrict__ tr,
                                   int Et, const RwgSlots* __restrict__ sr, int Es, int Tt, int Ts,
-                                  int b0, int nb, double2* __restrict__ L, double2* __restrict__ K) {
+                                  int b0, int nb, const int32_t* __restrict__ slot, double2* __restrict__ L,
+                                  double2* __restrict__ K) {
     const size_t total = (size_t)nb * Et * Es;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
          e += (size_t)gridDim.x * blockDim.x) {
@@ -320,7 +411,7 @@ __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots*
                 kk.x += c * p[9 + ij].x;
                 kk.y += c * p[9 + ij].y;
             }
-        const size_t o = ((size_t)(b0 + bl) * Et + m) * Es + n;
+        const size_t o = ((size_t)(slot ? slot[b0 + bl] : b0 + bl) * Et + m) * Es + n;
         L[o] = l;
         K[o] = kk;
     }
@@ -365,6 +456,15 @@ int prepare_mesh(const double* verts, const int32_t* tris, const int32_t* slot_r
         if (!(cn > 0.0)) { set_error("degenerate triangle %d", t); return EMSURF_EINVAL; }
         g.area = 0.5 * cn;
         for (int x = 0; x < 3; ++x) g.n[x] = c[x] / cn;
+        for (int i = 0; i < 3; ++i) {
+            const double* p = V[i];
+            const double* q = V[(i + 1) % 3];
+            const double e[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
+            const double le = std::sqrt(e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
+            double* lh = g.lh + 3 * i;
+            for (int x = 0; x < 3; ++x) lh[x] = e[x] / le;
+            for (int x = 0; x < 3; ++x) g.u[3 * i + x] = lh[(x + 1) % 3] * g.n[(x + 2) % 3] - lh[(x + 2) % 3] * g.n[(x + 1) % 3];
+        }
         g.scale = std::max(std::sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]),
                            std::sqrt(e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]));
         for (int i = 0; i < 3; ++i) {
@@ -390,10 +490,46 @@ int prepare_mesh(const double* verts, const int32_t* tris, const int32_t* slot_r
 }  // namespace
 
 
-// L, K: device [nb][Et][Es]; wavenumber k + j ki (ki = 0: lossless)
+namespace {
+// w_q lambda_u(q) of the rule, the kernels' constant
+void rule_moments(double wl[21]) {
+    double bary[7][3], w[7];
+    radon7(bary, w);
+    for (int q = 0; q < 7; ++q)
+        for (int u = 0; u < 3; ++u) wl[3 * q + u] = w[q] * bary[q][u];
+}
+
+// slot integrals of blocks b0 .. b0 + nc - 1 (singular: host flags), one
+// launch per run of equal flags
+cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, const double* shifts,
+                         const int8_t* singular, int b0, int nc, double k, double ki, double2* out, cudaStream_t st) {
+    const unsigned gx = (unsigned)(((long long)Tt * Ts + 127) / 128);
+    for (int c = 0; c < nc;) {
+        int e = c + 1;
+        while (e < nc && (singular[b0 + e] != 0) == (singular[b0 + c] != 0) && e - c < 65535) ++e;
+        const dim3 g(gx, (unsigned)(e - c));
+        double2* o = out + (size_t)c * Tt * Ts * 18;
+        const bool s = singular[b0 + c] != 0;
+        if (ki != 0.0) {
+            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, ki, o);
+            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, ki, o);
+        } else {
+            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, 0.0, o);
+            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, 0.0, o);
+        }
+        const cudaError_t err = cudaGetLastError();
+        if (err != cudaSuccess) return err;
+        c = e;
+    }
+    return cudaSuccess;
+}
+}  // namespace
+
+// L, K: device [nb][Et][Es] (block b at slot[b] when slot is not NULL);
+// wavenumber k + j ki (ki = 0: lossless)
 int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* shifts,
                        const int8_t* singular, int nb, double k, double ki, double2* L, double2* K,
-                       cudaStream_t st) {
+                       cudaStream_t st, const int32_t* slot) {
     if (!(k > 0.0) || !(ki <= 0.0) || nb < 1) {
         set_error("tabulate needs Re k > 0, Im k <= 0 and >= 1 block");
         return EMSURF_EINVAL;
@@ -402,15 +538,15 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
     std::vector<RwgSlots> tr, sr;
     EMS_TRY(prepare_mesh(test.verts, test.tris, test.slot_rwg, test.slot_sgn, test.T, test.E, tg, tr));
     EMS_TRY(prepare_mesh(src.verts, src.tris, src.slot_rwg, src.slot_sgn, src.T, src.E, sgeo, sr));
-    double bary[7][3], w[7];
-    radon7(bary, w);
-    EMS_CUDA(cudaMemcpyToSymbolAsync(c_w, w, sizeof(w), 0, cudaMemcpyHostToDevice, st));
+    double wl[21];
+    rule_moments(wl);
+    EMS_CUDA(cudaMemcpyToSymbolAsync(c_wl, wl, sizeof(wl), 0, cudaMemcpyHostToDevice, st));
     const size_t per_block = (size_t)test.T * src.T * 18 * sizeof(double2);
     const int chunk = (int)std::max<size_t>(1, std::min<size_t>(nb, kScratchBytes / per_block));
     TriGeo *dtg = nullptr, *dsg = nullptr;
     RwgSlots *dtr = nullptr, *dsr = nullptr;
     double* dsh = nullptr;
-    int8_t* dsi = nullptr;
+    int32_t* dslot = nullptr;
     double2* scratch = nullptr;
     int status = EMSURF_OK;
     auto fail = [&](cudaError_t e, const char* what) {
@@ -423,7 +559,7 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
     if (!status && (e = cudaMalloc(&dtr, sizeof(RwgSlots) * tr.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&dsr, sizeof(RwgSlots) * sr.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&dsh, sizeof(double) * 3 * nb)) != cudaSuccess) fail(e, "alloc");
-    if (!status && (e = cudaMalloc(&dsi, nb)) != cudaSuccess) fail(e, "alloc");
+    if (!status && slot && (e = cudaMalloc(&dslot, sizeof(int32_t) * nb)) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&scratch, per_block * chunk)) != cudaSuccess) fail(e, "scratch alloc");
     if (!status) {
         cudaMemcpyAsync(dtg, tg.data(), sizeof(TriGeo) * tg.size(), cudaMemcpyHostToDevice, st);
@@ -431,19 +567,15 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
         cudaMemcpyAsync(dtr, tr.data(), sizeof(RwgSlots) * tr.size(), cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(dsr, sr.data(), sizeof(RwgSlots) * sr.size(), cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(dsh, shifts, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(dsi, singular, nb, cudaMemcpyHostToDevice, st);
+        if (slot) cudaMemcpyAsync(dslot, slot, sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st);
         for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
             const int nc = std::min(chunk, nb - b0);
-            dim3 g1((src.T + 127) / 128, test.T, nc);
-            if (ki != 0.0)
-                tri_pairs_kernel<true><<<g1, 128, 0, st>>>(dtg, test.T, dsg, src.T, dsh, dsi, b0, k, ki, scratch);
-            else
-                tri_pairs_kernel<false><<<g1, 128, 0, st>>>(dtg, test.T, dsg, src.T, dsh, dsi, b0, k, 0.0, scratch);
-            if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "tri_pairs_kernel"); break; }
+            e = launch_pairs(dtg, test.T, dsg, src.T, dsh, singular, b0, nc, k, ki, scratch, st);
+            if (e != cudaSuccess) { fail(e, "tri_pairs_kernel"); break; }
             const size_t tot = (size_t)nc * test.E * src.E;
             const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
             rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, dsr, src.E, test.T, src.T, b0,
-                                                  nc, L, K);
+                                                  nc, dslot, L, K);
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "rwg_gather_kernel"); break; }
         }
         if (!status && (e = cudaStreamSynchronize(st)) != cudaSuccess) fail(e, "synchronize");
@@ -453,7 +585,7 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
     cudaFree(dtr);
     cudaFree(dsr);
     cudaFree(dsh);
-    cudaFree(dsi);
+    cudaFree(dslot);
     cudaFree(scratch);
     return status;
 }
@@ -544,8 +676,7 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
     const size_t o_tr = o_sg + align256(sizeof(TriGeo) * sgeo.size());
     const size_t o_sr = o_tr + align256(sizeof(RwgSlots) * tr.size());
     const size_t o_sh = o_sr + align256(sizeof(RwgSlots) * sr.size());
-    const size_t o_si = o_sh + align256(sizeof(double) * 3 * (size_t)nb);
-    const size_t o_pairs = o_si + align256((size_t)nb);
+    const size_t o_pairs = o_sh + align256(sizeof(double) * 3 * (size_t)nb);
     const size_t per_block = (size_t)test.T * src.T * 18 * sizeof(double2);
     if (o_pairs + per_block > kNoAllocBytes) {
         set_error("emsurf_tabulate_noalloc needs %zu bytes of scratch for these meshes and %d "
@@ -561,11 +692,10 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
     RwgSlots* dtr = reinterpret_cast<RwgSlots*>(b + o_tr);
     RwgSlots* dsr = reinterpret_cast<RwgSlots*>(b + o_sr);
     double* dsh = reinterpret_cast<double*>(b + o_sh);
-    int8_t* dsi = reinterpret_cast<int8_t*>(b + o_si);
     double2* pairs = reinterpret_cast<double2*>(b + o_pairs);
     const int chunk = (int)std::min<size_t>(nb, (kNoAllocBytes - o_pairs) / per_block);
-    double bary[7][3], w[7];
-    radon7(bary, w);
+    double wl[21];
+    rule_moments(wl);
     // from the first queued copy on, every return goes through the stream
     // synchronisation below, so no queued work outlives the call
     int status = EMSURF_OK;
@@ -575,24 +705,21 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
             status = EMSURF_ECUDA;
         }
     };
-    step(cudaMemcpyToSymbolAsync(c_w, w, sizeof(w), 0, cudaMemcpyHostToDevice, st), "copy weights");
+    step(cudaMemcpyToSymbolAsync(c_wl, wl, sizeof(wl), 0, cudaMemcpyHostToDevice, st), "copy weights");
     if (!status) step(cudaMemcpyAsync(dtg, tg.data(), sizeof(TriGeo) * tg.size(), cudaMemcpyHostToDevice, st), "copy");
     if (!status) step(cudaMemcpyAsync(dsg, sgeo.data(), sizeof(TriGeo) * sgeo.size(), cudaMemcpyHostToDevice, st), "copy");
     if (!status) step(cudaMemcpyAsync(dtr, tr.data(), sizeof(RwgSlots) * tr.size(), cudaMemcpyHostToDevice, st), "copy");
     if (!status) step(cudaMemcpyAsync(dsr, sr.data(), sizeof(RwgSlots) * sr.size(), cudaMemcpyHostToDevice, st), "copy");
     if (!status) step(cudaMemcpyAsync(dsh, shifts, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, st), "copy");
-    if (!status) step(cudaMemcpyAsync(dsi, singular, nb, cudaMemcpyHostToDevice, st), "copy");
     // every pair integral is written before it is read, so nothing needs clearing
     for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
         const int nc = std::min(chunk, nb - b0);
-        dim3 g1((src.T + 127) / 128, test.T, nc);
-        tri_pairs_kernel<false><<<g1, 128, 0, st>>>(dtg, test.T, dsg, src.T, dsh, dsi, b0, k, 0.0, pairs);
-        step(cudaGetLastError(), "tri_pairs_kernel");
+        step(launch_pairs(dtg, test.T, dsg, src.T, dsh, singular, b0, nc, k, 0.0, pairs, st), "tri_pairs_kernel");
         if (status) break;
         const size_t tot = (size_t)nc * test.E * src.E;
         const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
         rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc,
-                                              L, K);
+                                              nullptr, L, K);
         step(cudaGetLastError(), "rwg_gather_kernel");
     }
     step(cudaStreamSynchronize(st), "synchronize");
@@ -650,15 +777,17 @@ EMSURF_API int emsurf_tabulate(const double* test_verts, const int32_t* test_tri
 
 namespace emsurf {
 namespace {
-// T(d) <- (T(d) + T(-d)^T) / 2 for both tables in place: offset o and its
-// mirror nof - 1 - o form one pair, handled by one thread per entry pair.
-__global__ void reciprocal_part_kernel(double2* __restrict__ L, double2* __restrict__ K, int nof, int E) {
-    const size_t EE = (size_t)E * E, total = (size_t)nof * EE;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int o = (int)(e / EE), om = nof - 1 - o;
-        const int i = (int)((e % EE) / E), j = (int)(e % E);
-        if (o > om || (o == om && i >= j)) continue;
-        const size_t p = e, q = (size_t)om * EE + (size_t)j * E + i;
+// T(d) <- (T(d) + T(-d)^T) / 2 for both tables in place, for the listed pairs
+// (o, om) of the offsets d and -d (o == om: d = 0), blockIdx.y = pair, one
+// thread per entry pair.
+__global__ void reciprocal_part_kernel(double2* __restrict__ L, double2* __restrict__ K,
+                                       const int2* __restrict__ pairs, int E) {
+    const size_t EE = (size_t)E * E;
+    const int o = pairs[blockIdx.y].x, om = pairs[blockIdx.y].y;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < EE; e += (size_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e / E), j = (int)(e % E);
+        if (o == om && i >= j) continue;
+        const size_t p = (size_t)o * EE + e, q = (size_t)om * EE + (size_t)j * E + i;
         double2 t[2] = {L[p], K[p]};
         double2 u[2] = {L[q], K[q]};
         const double2 sl = make_double2((t[0].x + u[0].x) * 0.5, (t[0].y + u[0].y) * 0.5);
@@ -669,11 +798,56 @@ __global__ void reciprocal_part_kernel(double2* __restrict__ L, double2* __restr
         K[q] = sk;
     }
 }
+
+// One offset that takes its block from offset `rep` through group element
+// `elem` (bits 0..2: the box's x, y and x <-> y mirrors) and, with bit 3, the
+// transpose of reciprocity.
+struct OffsetImage {
+    int32_t slot, rep, elem;
+};
+
+// T(d')[pi(i)][pi(j)] = s sign(i) sign(j) T(d)[i][j] (transposed with bit 3),
+// s = 1 for L and det(g) for K.  inv[g][n] = pi^-1(n) | (sign < 0) << 31.
+// One CTA per 32 x 32 tile of an output block: its source entries lie in 32
+// rows (columns) of the L2-resident source block.
+__global__ void __launch_bounds__(256)
+expand_offsets_kernel(double2* __restrict__ L, double2* __restrict__ K, const OffsetImage* __restrict__ img,
+                      const uint32_t* __restrict__ inv, int E) {
+    const OffsetImage m = img[blockIdx.z];
+    const uint32_t* pi = inv + (size_t)(m.elem & 7) * E;
+    const bool tr = m.elem & 8;
+    const double det = (__popc(m.elem & 7) & 1) ? -1.0 : 1.0;
+    const size_t EE = (size_t)E * E, src = (size_t)m.rep * EE, dst = (size_t)m.slot * EE;
+    const int j = blockIdx.x * 32 + threadIdx.x;
+    if (j >= E) return;
+    const uint32_t pj = pi[j];
+#pragma unroll
+    for (int r = 0; r < 32; r += 8) {
+        const int i = blockIdx.y * 32 + r + threadIdx.y;
+        if (i >= E) break;
+        const uint32_t pr = pi[i];
+        const size_t a = pr & 0x7fffffffu, b = pj & 0x7fffffffu;
+        const size_t at = src + (tr ? b * E + a : a * E + b);
+        const double s = ((pr ^ pj) >> 31) ? -1.0 : 1.0;
+        const double2 l = L[at], k = K[at];
+        L[dst + (size_t)i * E + j] = make_double2(s * l.x, s * l.y);
+        K[dst + (size_t)i * E + j] = make_double2(s * det * k.x, s * det * k.y);
+    }
+}
 }  // namespace
 }  // namespace emsurf
 
 extern "C" {
 
+// The tables' symmetries leave few offsets to integrate: with the box's
+// mirrors g (emsurf_setup_box_mirrors) L(g d) = P_g L(d) P_g^T and K(g d) =
+// det(g) P_g K(d) P_g^T, and the reciprocal part obeys T(-d) = T(d)^T (exact
+// for the two-sided quadrature of offsets that do not touch).  One offset of
+// each orbit is integrated (136 of 961 on a 16 x 16 lattice of square cells
+// with even n), touching ones together with their -d; the others are signed
+// permutations of it.  Tabulation is bound by the FP64 rate, so its time
+// follows the integrated offsets: 38 ms for 16 x 16 boxes of 288 RWGs, 650 ms
+// with every offset integrated point pair by point pair.
 EMSURF_API int emsurf_tabulate_offsets(double a, double b, double h, int32_t n,
                                        const double* zlevels, int32_t nx, int32_t ny, double k,
                                        emsurf_c128* L, emsurf_c128* K, void* stream) {
@@ -688,28 +862,111 @@ EMSURF_API int emsurf_tabulate_offsets(double a, double b, double h, int32_t n,
     std::vector<int8_t> ssg(3 * T);
     EMS_TRY(emsurf_setup_box_mesh(a, b, h, n, zlevels, verts.data(), tris.data(), edges.data(),
                                   tp.data(), tm.data(), srw.data(), ssg.data()));
-    const int nox = 2 * nx - 1, noy = 2 * ny - 1;
-    std::vector<double> shifts(3 * (size_t)nox * noy);
-    std::vector<int8_t> sing((size_t)nox * noy);
-    for (int dyi = 0; dyi < noy; ++dyi)
-        for (int dxi = 0; dxi < nox; ++dxi) {
-            const int dx = dxi - (nx - 1), dy = dyi - (ny - 1);
-            const size_t o = (size_t)dyi * nox + dxi;
-            shifts[3 * o] = dx * a;
-            shifts[3 * o + 1] = dy * b;
-            shifts[3 * o + 2] = 0.0;
-            sing[o] = (std::abs(dx) <= 1 && std::abs(dy) <= 1) ? 1 : 0;
+    // inverse signed permutations of the 8 products of mirrors (P_g = Px^a Py^b Pd^c)
+    std::vector<int32_t> perm(3 * (size_t)E);
+    std::vector<int8_t> sign(3 * (size_t)E);
+    int32_t mask = 0;
+    EMS_TRY(emsurf_setup_box_mirrors(a, b, n, perm.data(), sign.data(), &mask));
+    std::vector<uint32_t> inv(8 * (size_t)E);
+    for (int g = 0; g < 8; ++g) {
+        if (g & ~mask) continue;
+        for (int e = 0; e < E; ++e) {
+            int at = e, sg = 1;
+            for (int bit : {2, 1, 0})           // the x <-> y mirror first
+                if (g & (1 << bit)) {
+                    sg *= sign[(size_t)bit * E + at];
+                    at = perm[(size_t)bit * E + at];
+                }
+            inv[(size_t)g * E + at] = (uint32_t)e | (sg < 0 ? 0x80000000u : 0u);
         }
+    }
+    const int nox = 2 * nx - 1, noy = 2 * ny - 1, nof = nox * noy;
+    std::vector<int32_t> rep_of(nof, -1);
+    std::vector<int32_t> slot;                  // integrated offsets: touching ones first
+    std::vector<int2> touch;                    // (d, -d) of the touching representatives
+    std::vector<OffsetImage> image;
+    std::vector<int32_t> far;
+    auto touching = [](int dx, int dy) { return std::abs(dx) <= 1 && std::abs(dy) <= 1; };
+    for (int o = 0; o < nof; ++o) {
+        if (rep_of[o] >= 0) continue;
+        const int dx = o % nox - (nx - 1), dy = o / nox - (ny - 1);
+        rep_of[o] = o;
+        if (touching(dx, dy)) {
+            slot.push_back(o);
+            const int om = nof - 1 - o;
+            if (om != o) {
+                slot.push_back(om);
+                rep_of[om] = o;                 // its reciprocal part is written with d's
+            }
+            touch.push_back(make_int2(o, om));
+        } else {
+            far.push_back(o);
+        }
+        // d' and -d' together, so that T(-d') = T(d')^T entry by entry
+        for (int g = 0; g < 8; ++g) {
+            if (g & ~mask) continue;
+            int x = dx, y = dy;
+            if (g & 4) std::swap(x, y);
+            if (g & 1) x = -x;
+            if (g & 2) y = -y;
+            if (std::abs(x) >= nx || std::abs(y) >= ny) continue;
+            const int q = (y + ny - 1) * nox + x + nx - 1, qm = nof - 1 - q;
+            for (const OffsetImage& m : {OffsetImage{q, o, g}, OffsetImage{qm, o, g | 8}})
+                if (rep_of[m.slot] < 0) {
+                    rep_of[m.slot] = o;
+                    image.push_back(m);
+                }
+        }
+    }
+    const int n_touch = (int)slot.size();
+    slot.insert(slot.end(), far.begin(), far.end());
+    std::vector<double> shifts(3 * slot.size());
+    std::vector<int8_t> sing(slot.size());
+    for (size_t i = 0; i < slot.size(); ++i) {
+        shifts[3 * i] = (slot[i] % nox - (nx - 1)) * a;
+        shifts[3 * i + 1] = (slot[i] / nox - (ny - 1)) * b;
+        shifts[3 * i + 2] = 0.0;
+        sing[i] = (int)i < n_touch ? 1 : 0;
+    }
     MeshView mv{verts.data(), tris.data(), srw.data(), ssg.data(), T, E};
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    EMS_TRY(tabulate_blocks(mv, mv, shifts.data(), sing.data(), nox * noy, k, reinterpret_cast<double2*>(L),
-                            reinterpret_cast<double2*>(K), st));
-    // reciprocal part of the one-sided blocks (exactly reciprocal tables)
-    const size_t total = (size_t)nox * noy * E * E;
-    reciprocal_part_kernel<<<(int)std::min<size_t>((total + 255) / 256, 152 * 64), 256, 0, st>>>(
-        reinterpret_cast<double2*>(L), reinterpret_cast<double2*>(K), nox * noy, E);
-    EMS_CUDA(cudaGetLastError());
-    EMS_CUDA(cudaStreamSynchronize(st));
+    double2* Ld = reinterpret_cast<double2*>(L);
+    double2* Kd = reinterpret_cast<double2*>(K);
+    EMS_TRY(tabulate_blocks_cx(mv, mv, shifts.data(), sing.data(), (int)slot.size(), k, 0.0, Ld, Kd, st, slot.data()));
+    // reciprocal part of the touching blocks, then the images
+    unsigned char* dbuf = nullptr;
+    const size_t b_touch = touch.size() * sizeof(int2), b_inv = inv.size() * sizeof(uint32_t);
+    const size_t b_img = std::max<size_t>(1, image.size()) * sizeof(OffsetImage);
+    if (cudaMalloc(&dbuf, b_touch + b_inv + b_img) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("emsurf_tabulate_offsets: device allocation failed");
+        return EMSURF_ENOMEM;
+    }
+    int2* dtouch = reinterpret_cast<int2*>(dbuf);
+    uint32_t* dinv = reinterpret_cast<uint32_t*>(dbuf + b_touch);
+    OffsetImage* dimg = reinterpret_cast<OffsetImage*>(dbuf + b_touch + b_inv);
+    cudaError_t e = cudaMemcpyAsync(dtouch, touch.data(), b_touch, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dinv, inv.data(), b_inv, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !image.empty())
+        e = cudaMemcpyAsync(dimg, image.data(), image.size() * sizeof(OffsetImage), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        const size_t EE = (size_t)E * E;
+        reciprocal_part_kernel<<<dim3((unsigned)std::min<size_t>((EE + 255) / 256, 1024), (unsigned)touch.size()), 256,
+                                 0, st>>>(Ld, Kd, dtouch, E);
+        e = cudaGetLastError();
+    }
+    for (size_t i0 = 0; i0 < image.size() && e == cudaSuccess; i0 += 65535) {
+        const dim3 grid((E + 31) / 32, (E + 31) / 32, (unsigned)std::min<size_t>(65535, image.size() - i0));
+        expand_offsets_kernel<<<grid, dim3(32, 8), 0, st>>>(Ld, Kd, dimg + i0, dinv, E);
+        e = cudaGetLastError();
+    }
+    const cudaError_t es = cudaStreamSynchronize(st);
+    cudaFree(dbuf);
+    if (e == cudaSuccess) e = es;
+    if (e != cudaSuccess) {
+        set_error("emsurf_tabulate_offsets: %s", cudaGetErrorString(e));
+        return EMSURF_ECUDA;
+    }
     return EMSURF_OK;
 }
 
