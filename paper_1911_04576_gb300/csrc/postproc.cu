@@ -12,6 +12,7 @@
 // x = U_o Y~.  Bistatic RCS sigma = 4 pi |F|^2 / |E_inc|^2.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "common.cuh"
@@ -32,6 +33,12 @@ struct RwgQuad {
 __device__ __forceinline__ double2 cexpj(double phase) {   // e^{j phase}
     double s, c;
     sincos(phase, &s, &c);
+    return make_double2(c, s);
+}
+
+__device__ __forceinline__ double2 cexpjpi(double phase) {   // e^{j pi phase}
+    double s, c;
+    sincospi(phase, &s, &c);
     return make_double2(c, s);
 }
 
@@ -88,29 +95,6 @@ __global__ void excitation_scatter_kernel(const double2* __restrict__ V0, const 
     }
 }
 
-// Rv[d][e][3] = int Lam_e e^{jk rhat_d . r'}
-__global__ void radiation_kernel(const RwgQuad* __restrict__ q, int E, const double* __restrict__ rhat,
-                                 int D, double k, double2* __restrict__ Rv) {
-    const size_t total = (size_t)D * E;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total;
-         x += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(x % E);
-        const int d = (int)(x / E);
-        const double* rh = rhat + 3 * d;
-        const RwgQuad& Q = q[e];
-        double2 acc[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-        for (int i = 0; i < 14; ++i) {
-            const double2 ph = cexpj(k * (rh[0] * Q.r[i][0] + rh[1] * Q.r[i][1] + rh[2] * Q.r[i][2]));
-            for (int c = 0; c < 3; ++c) {
-                const double a = Q.w[i] * (Q.r[i][c] - Q.p[i][c]);
-                acc[c].x += a * ph.x;
-                acc[c].y += a * ph.y;
-            }
-        }
-        for (int c = 0; c < 3; ++c) Rv[x * 3 + c] = acc[c];
-    }
-}
-
 // X1[m][r K + k] = sign * Y[r][idx[m K + k]]: every cell's box currents
 template <typename C>
 __global__ void gather_cells_kernel(const double2* __restrict__ Y, const int32_t* __restrict__ idx,
@@ -131,134 +115,321 @@ __global__ void gather_cells_kernel(const double2* __restrict__ Y, const int32_t
 }
 
 // The array factor of every column: S[d][n] = sum_m e^{jk rhat_d . c_m}
-// X1[m][n], c_m = (ix a, iy b, 0).  A block computes kLsD directions x kLsN
-// columns; the phase of cell m factors into per-direction tables
-// e^{jk rx a ix} e^{jk ry b iy} (one sincos per direction and row or column of
-// the lattice instead of one per term), X1 is staged kLsM cells at a time.
-// Each thread holds 2 directions x 4 columns (columns tn + 16 c, so a
-// warp's shared-memory reads are consecutive).  T: arithmetic type (double
-// for FP64 handles; float, with float accumulation over the cells, for
-// FP32 / MIXED handles).
-constexpr int kLsD = 32, kLsN = 64, kLsM = 16, kLsThreads = 256;
+// X1[m][n], c_m = (ix a, iy b, 0).  A block computes 32 directions x 96
+// columns, 16 cells at a time: X1 and the cells' phases are staged in shared
+// memory, the phases as products of the direction's e^{jk rx a ix} and
+// e^{jk ry b iy} (from phase_table_kernel; TAB false: one sincos per direction
+// and cell, for lattices whose tables do not fit).  A warp holds 4
+// directions, each lane 3 columns, so a phase is one broadcast read for the
+// warp.  T: arithmetic type (double for FP64 handles; float, with float
+// accumulation over the cells, for FP32 / MIXED handles).  Bound by the FMA
+// rate.  16 x 16 cells, 576 columns, 65,160 directions (1.1 ms at the FP32 FMA
+// rate): 1.9 ms and 0.14 ms for the tables; 3.5 ms with 2 x 4 sums per thread, the tables formed by
+// every block, and the phase product and the cell's index division redone by
+// every thread.  64 directions per block (8 per warp) left one block per SM
+// and took a quarter longer.
+constexpr int kLsM = 16, kLsThreads = 256, kLsCpt = 3, kLsDpt = 4;
 
+
+// tab[d][i] = e^{jk rx a i} for i < nx, e^{jk ry b (i - nx)} for the ny above
 template <typename T, typename C>
+__global__ void phase_table_kernel(const double* __restrict__ rhat, int nd, int nx, int ny, double a, double b,
+                                   double k, C* __restrict__ tab) {
+    const int n = nx + ny;
+    const long long total = (long long)nd * n;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const int d = (int)(e / n), i = (int)(e - (long long)d * n);
+        double sn, cs;
+        sincos(i < nx ? k * a * rhat[3 * d] * i : k * b * rhat[3 * d + 1] * (i - nx), &sn, &cs);
+        tab[e].x = (T)cs;
+        tab[e].y = (T)sn;
+    }
+}
+
+template <typename T, typename C, bool TAB>
 __global__ void __launch_bounds__(kLsThreads)
-lattice_sum_tiled_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, double a, double b,
-                         const double* __restrict__ rhat, int nd, double k, C* __restrict__ S) {
+lattice_sum_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, double a, double b,
+                   const double* __restrict__ rhat, const C* __restrict__ tab, int nd, double k, C* __restrict__ S) {
+    constexpr int DPT = kLsDpt, ND = 8 * DPT, NC = 32 * kLsCpt;
+    constexpr int kXPer = kLsM * NC / kLsThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* px = reinterpret_cast<C*>(smem_raw);            // [kLsD][nx]
-    C* py = px + kLsD * nx;                            // [kLsD][ny]
-    C* xs = py + kLsD * ny;                            // [kLsM][kLsN]
-    const int d0 = blockIdx.y * kLsD, n0 = blockIdx.x * kLsN;
-    for (int e = threadIdx.x; e < kLsD * nx; e += blockDim.x) {
-        const int dd = e / nx, ix = e - dd * nx, d = d0 + dd;
-        double sn = 0.0, cs = 1.0;
-        if (d < nd) sincos(k * a * rhat[3 * d] * ix, &sn, &cs);
-        px[e].x = (T)cs;
-        px[e].y = (T)sn;
+    C* xs = reinterpret_cast<C*>(smem_raw);            // [kLsM][NC]
+    C* ps = xs + kLsM * NC;                            // [kLsM][ND]
+    C* px = ps + kLsM * ND;                            // [nx][ND]
+    C* py = px + (TAB ? nx * ND : 0);                  // [ny][ND]
+    const int d0 = blockIdx.y * ND, n0 = blockIdx.x * NC;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (TAB) {
+        for (int e = threadIdx.x; e < ND * (nx + ny); e += blockDim.x) {
+            const int i = e / ND, dd = e - i * ND, d = d0 + dd;
+            C v;
+            v.x = (T)1;
+            v.y = (T)0;
+            if (d < nd) v = tab[(size_t)d * (nx + ny) + i];
+            px[e] = v;
+        }
     }
-    for (int e = threadIdx.x; e < kLsD * ny; e += blockDim.x) {
-        const int dd = e / ny, iy = e - dd * ny, d = d0 + dd;
-        double sn = 0.0, cs = 1.0;
-        if (d < nd) sincos(k * b * rhat[3 * d + 1] * iy, &sn, &cs);
-        py[e].x = (T)cs;
-        py[e].y = (T)sn;
-    }
-    const int tn = threadIdx.x & 15, td = threadIdx.x >> 4;     // 16 column groups x 16 direction pairs
-    C acc[2][4];
+    C acc[DPT][kLsCpt];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < DPT; ++i)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[i][c].x = acc[i][c].y = (T)0;
-    const C* pxa = px + (2 * td) * nx;
-    const C* pxb = pxa + nx;
-    const C* pya = py + (2 * td) * ny;
-    const C* pyb = pya + ny;
+        for (int c = 0; c < kLsCpt; ++c) acc[i][c].x = acc[i][c].y = (T)0;
+    // one stage's cells are summed on their own and then added: fewer roundings
+    // at the size of the whole sum
+    C part[DPT][kLsCpt];
+    C xr[kXPer];
+    auto load = [&](int m0) {
+#pragma unroll
+        for (int q = 0; q < kXPer; ++q) {
+            const int e = threadIdx.x + q * kLsThreads, mm = e / NC, c = e - mm * NC;
+            xr[q].x = xr[q].y = (T)0;
+            if (m0 + mm < M && n0 + c < N) xr[q] = X1[(size_t)(m0 + mm) * N + n0 + c];
+        }
+    };
+    load(0);
     for (int m0 = 0; m0 < M; m0 += kLsM) {
         __syncthreads();
-        for (int e = threadIdx.x; e < kLsM * kLsN; e += blockDim.x) {
-            const int mm = e / kLsN, c = e - mm * kLsN;
-            C v;
-            v.x = v.y = (T)0;
-            if (m0 + mm < M && n0 + c < N) v = X1[(size_t)(m0 + mm) * N + n0 + c];
-            xs[e] = v;
-        }
-        __syncthreads();
-        const int mend = min(kLsM, M - m0);
-        for (int mm = 0; mm < mend; ++mm) {
-            const int m = m0 + mm, iy = m / nx, ix = m - iy * nx;
-            C pa, pb;
-            pa.x = pxa[ix].x * pya[iy].x - pxa[ix].y * pya[iy].y;
-            pa.y = pxa[ix].x * pya[iy].y + pxa[ix].y * pya[iy].x;
-            pb.x = pxb[ix].x * pyb[iy].x - pxb[ix].y * pyb[iy].y;
-            pb.y = pxb[ix].x * pyb[iy].y + pxb[ix].y * pyb[iy].x;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const C x = xs[mm * kLsN + tn + 16 * c];
-                acc[0][c].x += pa.x * x.x - pa.y * x.y;
-                acc[0][c].y += pa.x * x.y + pa.y * x.x;
-                acc[1][c].x += pb.x * x.x - pb.y * x.y;
-                acc[1][c].y += pb.x * x.y + pb.y * x.x;
+        for (int q = 0; q < kXPer; ++q) xs[threadIdx.x + q * kLsThreads] = xr[q];
+        for (int e = threadIdx.x; e < kLsM * ND; e += kLsThreads) {
+            const int mm = e / ND, dd = e - mm * ND, m = min(m0 + mm, M - 1), iy = m / nx, ix = m - iy * nx;
+            C v;
+            if constexpr (TAB) {
+                const C u = px[ix * ND + dd], w = py[iy * ND + dd];
+                v.x = u.x * w.x - u.y * w.y;
+                v.y = u.x * w.y + u.y * w.x;
+            } else {
+                const int d = min(d0 + dd, nd - 1);
+                double sn, cs;
+                sincos(k * (a * rhat[3 * d] * ix + b * rhat[3 * d + 1] * iy), &sn, &cs);
+                v.x = (T)cs;
+                v.y = (T)sn;
+            }
+            ps[e] = v;
+        }
+        if (m0 + kLsM < M) load(m0 + kLsM);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < DPT; ++i)
+#pragma unroll
+            for (int c = 0; c < kLsCpt; ++c) part[i][c].x = part[i][c].y = (T)0;
+        // cells past M: X1 is zero there
+#pragma unroll 4
+        for (int mm = 0; mm < kLsM; ++mm) {
+            C x[kLsCpt];
+#pragma unroll
+            for (int c = 0; c < kLsCpt; ++c) x[c] = xs[mm * NC + lane + 32 * c];
+            const C* pw = ps + mm * ND + warp * DPT;
+#pragma unroll
+            for (int i = 0; i < DPT; i += 2) {
+                // two directions' phases (16 or 32 bytes, the same for the whole warp)
+                const C pa = pw[i], pb = pw[i + 1];
+#pragma unroll
+                for (int c = 0; c < kLsCpt; ++c) {
+                    part[i][c].x += pa.x * x[c].x;
+                    part[i][c].x -= pa.y * x[c].y;
+                    part[i][c].y += pa.x * x[c].y;
+                    part[i][c].y += pa.y * x[c].x;
+                    part[i + 1][c].x += pb.x * x[c].x;
+                    part[i + 1][c].x -= pb.y * x[c].y;
+                    part[i + 1][c].y += pb.x * x[c].y;
+                    part[i + 1][c].y += pb.y * x[c].x;
+                }
             }
         }
+#pragma unroll
+        for (int i = 0; i < DPT; ++i)
+#pragma unroll
+            for (int c = 0; c < kLsCpt; ++c) {
+                acc[i][c].x += part[i][c].x;
+                acc[i][c].y += part[i][c].y;
+            }
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int d = d0 + 2 * td + i;
+    for (int i = 0; i < DPT; ++i) {
+        const int d = d0 + warp * DPT + i;
         if (d >= nd) continue;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int n = n0 + tn + 16 * c;
+        for (int c = 0; c < kLsCpt; ++c) {
+            const int n = n0 + lane + 32 * c;
             if (n < N) S[(size_t)d * N + n] = acc[i][c];
         }
     }
 }
 
+// The box as translates of a few triangle shapes: with t = shape c moved by
+// its first vertex (X[ix], Y[iy], Z[iz]) the radiation integral of slot i of t
+// is  sgn e^{jk rhat . v0_t} U_{c,i}(rhat),
+// U_{c,i} = len_i / (2A) int_c (r' - v_i) e^{jk rhat . r'}.  A shape's slot i has
+// the same len_i / (2A) on every member, so
+//   N = sum_{c,i} U_{c,i} sum_{t in c} sgn e^{jk rhat . v0_t} S[rwg(t, i)]:
+// the phases need one sincos per distinct coordinate and the U ones 7 per
+// shape (about 155 per direction for 288 RWGs, 20 shapes) instead of 14 per
+// RWG (4032).
+struct BoxShape {
+    double r[21];       // quadrature points relative to v_0
+    double f[63];       // [i][q][x] w_q A len_i / (2A) (r_q - v_i)
+    double v[9];        // vertices relative to v_0
+};
+struct BoxTri {
+    int16_t ix, iy, iz, shape;
+};
+struct BoxMember {
+    int32_t tri, rwg;   // rwg | (sgn < 0) << 31
+};
+struct BoxShapes {
+    std::vector<BoxShape> shape;
+    std::vector<BoxTri> tri;
+    std::vector<double> coord;          // X, Y, Z one after the other
+    int nc[3] = {0, 0, 0};
+    std::vector<int32_t> slot;          // 3 shape + i, most members first
+    std::vector<int32_t> ptr;           // members of slot[s]: ptr[s] .. ptr[s + 1]
+    std::vector<BoxMember> mem;
+};
+struct BoxDev {
+    const BoxShape* shape;
+    const BoxTri* tri;
+    const double* coord;
+    const int32_t *slot, *ptr;
+    const BoxMember* mem;
+    int nshape, ntri, nx, ny, nz, nslot;
+};
+
 // F[r][d] = -(jk/4pi) [N_perp - rhat x L_M] of the column sums S[d][r K + e]
-template <typename C>
-__global__ void far_field_kernel(const C* __restrict__ S, const double2* __restrict__ Rv,
-                                 const double* __restrict__ rhat, int D, int E, int R, double k,
-                                 double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
-    const size_t total = (size_t)R * D;
+// (S_J in e < E, S_M in e >= E), one warp per direction; lanes share the
+// coordinate phases, the shapes' points and the (shape, slot) sums through the
+// warp's shared memory.  PH: the triangles' phases are kept there too (else
+// they are formed per member, for meshes whose phases do not fit).  All FP64,
+// and bound by its rate.  16 x 16 boxes of 288 RWGs, 65,160 directions: 2.9 ms;
+// with the radiation vectors of every (direction, RWG) written out first this
+// and the kernel before it took 20.6 ms.
+constexpr int kFfWarps = 4;     // directions per block (fewer where their shared memory does not fit)
+
+template <typename C, bool PH>
+__global__ void __launch_bounds__(32 * kFfWarps)
+far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ rhat, int nd, int E, int R, double k,
+                 double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ncoord = g.nx + g.ny + g.nz;
+    const int per = ncoord + 7 * g.nshape + 3 * g.nslot + (PH ? g.ntri : 0);
+    double2* cp = reinterpret_cast<double2*>(smem_raw) + (size_t)warp * per;   // coordinate phases
+    double2* eq = cp + ncoord;                                                 // point phases [shape][7]
+    double2* U = eq + 7 * g.nshape;                                            // [slot][3]
+    double2* tp = U + 3 * g.nslot;                                             // triangle phases
     const int K = 2 * E;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total;
-         x += (size_t)gridDim.x * blockDim.x) {
-        const int d = (int)(x % D), r = (int)(x / D);
-        const double* rh = rhat + 3 * d;
-        const C* s = S + (size_t)d * R * K + (size_t)r * K;
-        const double2* rv = Rv + (size_t)d * E * 3;
-        double2 N[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-        double2 L[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-        for (int e = 0; e < E; ++e) {
-            const double2 sj = make_double2((double)s[e].x, (double)s[e].y);
-            const double2 sm = make_double2((double)s[E + e].x, (double)s[E + e].y);
-            for (int c = 0; c < 3; ++c) {
-                cfma(N[c], sj, rv[3 * e + c]);
-                cfma(L[c], sm, rv[3 * e + c]);
+    const int nw = blockDim.x >> 5;
+    const double kpi = k * 0.31830988618379067154, k4 = k / kFourPi;
+    for (int d = blockIdx.x * nw + warp; d < nd; d += gridDim.x * nw) {
+        const double rh[3] = {rhat[3 * d], rhat[3 * d + 1], rhat[3 * d + 2]};
+        __syncwarp();
+        for (int e = lane; e < ncoord; e += 32)
+            cp[e] = cexpjpi(kpi * (e < g.nx ? rh[0] : e < g.nx + g.ny ? rh[1] : rh[2]) * g.coord[e]);
+        for (int e = lane; e < 7 * g.nshape; e += 32) {
+            const int c = e / 7, q = e - 7 * c;
+            const double* r = g.shape[c].r + 3 * q;
+            eq[e] = cexpjpi(kpi * (rh[0] * r[0] + rh[1] * r[1] + rh[2] * r[2]));
+        }
+        __syncwarp();
+        auto tri_phase = [&](const BoxTri t) {
+            return cmul(cmul(cp[t.ix], cp[g.nx + t.iy]), cp[g.nx + g.ny + t.iz]);
+        };
+        if constexpr (PH)
+            for (int t = lane; t < g.ntri; t += 32) tp[t] = tri_phase(g.tri[t]);
+        for (int s = lane; s < g.nslot; s += 32) {
+            const int c = g.slot[s] / 3, i = g.slot[s] - 3 * c;
+            const double* H = g.shape[c].f + 21 * i;
+            double2 u[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
+            for (int q = 0; q < 7; ++q) {
+                const double2 p = eq[7 * c + q];
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                    const double f = H[3 * q + x];
+                    u[x].x = fma(f, p.x, u[x].x);
+                    u[x].y = fma(f, p.y, u[x].y);
+                }
             }
+#pragma unroll
+            for (int x = 0; x < 3; ++x) U[3 * s + x] = u[x];
         }
-        double2 rn = make_double2(0, 0);
-        for (int c = 0; c < 3; ++c) {
-            rn.x += rh[c] * N[c].x;
-            rn.y += rh[c] * N[c].y;
+        __syncwarp();
+        for (int r = 0; r < R; ++r) {
+            const C* sr = S + (size_t)d * R * K + (size_t)r * K;
+            double2 NL[6];
+#pragma unroll
+            for (int x = 0; x < 6; ++x) NL[x] = make_double2(0, 0);
+            for (int s = lane; s < g.nslot; s += 32) {
+                double2 aj = make_double2(0, 0), am = make_double2(0, 0);
+                for (int q = g.ptr[s]; q < g.ptr[s + 1]; ++q) {
+                    const BoxMember b = g.mem[q];
+                    const int e = b.rwg & 0x7fffffff;
+                    C sj = sr[e], sm = sr[E + e];
+                    if (b.rwg < 0) {
+                        sj.x = -sj.x;
+                        sj.y = -sj.y;
+                        sm.x = -sm.x;
+                        sm.y = -sm.y;
+                    }
+                    double2 ph;
+                    if constexpr (PH) ph = tp[b.tri];
+                    else ph = tri_phase(g.tri[b.tri]);
+                    cfma(aj, ph, make_double2((double)sj.x, (double)sj.y));
+                    cfma(am, ph, make_double2((double)sm.x, (double)sm.y));
+                }
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                    const double2 u = U[3 * s + x];
+                    cfma(NL[x], aj, u);
+                    cfma(NL[3 + x], am, u);
+                }
+            }
+            // reduce-scatter of the 12 sums (padded to 16) over the warp: lanes 2 v
+            // and 2 v + 1 end with value v, which is then shared out
+            double v[16];
+#pragma unroll
+            for (int x = 0; x < 6; ++x) {
+                v[2 * x] = NL[x].x;
+                v[2 * x + 1] = NL[x].y;
+            }
+            v[12] = v[13] = v[14] = v[15] = 0.0;
+#pragma unroll
+            for (int n = 16, D = 16; n > 1; n >>= 1, D >>= 1) {
+                const bool up = lane & D;
+#pragma unroll
+                for (int c = 0; c < n / 2; ++c) {
+                    const double send = up ? v[c] : v[c + n / 2];
+                    const double keep = up ? v[c + n / 2] : v[c];
+                    v[c] = keep + __shfl_xor_sync(0xffffffffu, send, D);
+                }
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+#pragma unroll
+            for (int x = 0; x < 6; ++x) {
+                NL[x].x = __shfl_sync(0xffffffffu, v[0], 4 * x);
+                NL[x].y = __shfl_sync(0xffffffffu, v[0], 4 * x + 2);
+            }
+            const double2 *N = NL, *L = NL + 3;
+            double2 rn = make_double2(0, 0);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                rn.x += rh[c] * N[c].x;
+                rn.y += rh[c] * N[c].y;
+            }
+            double mag = 0.0;
+            double2* f = F + ((size_t)r * ndir_all + d) * 3;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+                // N_perp - rhat x L, times -(jk / 4pi)
+                const double2 rxl = make_double2(rh[c1] * L[c2].x - rh[c2] * L[c1].x,
+                                                 rh[c1] * L[c2].y - rh[c2] * L[c1].y);
+                const double2 w = make_double2(N[c].x - rn.x * rh[c] - rxl.x, N[c].y - rn.y * rh[c] - rxl.y);
+                const double2 fc = make_double2(k4 * w.y, -k4 * w.x);
+                if (lane == c) f[c] = fc;
+                mag += fc.x * fc.x + fc.y * fc.y;
+            }
+            if (rcs && lane == 0) rcs[(size_t)r * ndir_all + d] = kFourPi * mag;
         }
-        double2 v[3];
-        for (int c = 0; c < 3; ++c) {
-            const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-            // N_perp - rhat x L
-            const double2 rxl = make_double2(rh[c1] * L[c2].x - rh[c2] * L[c1].x,
-                                             rh[c1] * L[c2].y - rh[c2] * L[c1].y);
-            v[c] = make_double2(N[c].x - rn.x * rh[c] - rxl.x, N[c].y - rn.y * rh[c] - rxl.y);
-        }
-        double mag = 0.0;
-        double2* f = F + ((size_t)r * ndir_all + d) * 3;
-        for (int c = 0; c < 3; ++c) {
-            // -(jk / 4pi) v
-            const double2 fc = make_double2(k * v[c].y / kFourPi, -k * v[c].x / kFourPi);
-            f[c] = fc;
-            mag += fc.x * fc.x + fc.y * fc.y;
-        }
-        if (rcs) rcs[(size_t)r * ndir_all + d] = kFourPi * mag;
     }
 }
 
@@ -313,6 +484,96 @@ int box_quadrature(double a, double b, double h, int n, const double* zlevels, i
     return EMSURF_OK;
 }
 
+// index of x in v (appended when no entry lies within tol)
+int coord_index(std::vector<double>& v, double x, double tol) {
+    for (size_t i = 0; i < v.size(); ++i)
+        if (std::fabs(v[i] - x) <= tol) return (int)i;
+    v.push_back(x);
+    return (int)v.size() - 1;
+}
+
+int box_shapes(double a, double b, double h, int n, const double* zlevels, int E_expected, BoxShapes& out) {
+    int32_t V, T, E;
+    EMS_TRY(emsurf_setup_box_counts(n, &V, &T, &E));
+    if (E != E_expected) {
+        set_error("box mesh n=%d has %d RWGs, the handle has %d", n, E, E_expected);
+        return EMSURF_EINVAL;
+    }
+    std::vector<double> verts(3 * V);
+    std::vector<int32_t> tris(3 * T), edges(2 * E), tp(E), tm(E), srw(3 * T);
+    std::vector<int8_t> ssg(3 * T);
+    EMS_TRY(emsurf_setup_box_mesh(a, b, h, n, zlevels, verts.data(), tris.data(), edges.data(),
+                                  tp.data(), tm.data(), srw.data(), ssg.data()));
+    const double s15 = std::sqrt(15.0);
+    const double a1 = (6.0 - s15) / 21.0, b1 = (9.0 + 2.0 * s15) / 21.0;
+    const double a2 = (6.0 + s15) / 21.0, b2 = (9.0 - 2.0 * s15) / 21.0;
+    const double w1 = (155.0 - s15) / 1200.0, w2 = (155.0 + s15) / 1200.0;
+    const double B[7][3] = {{1.0 / 3, 1.0 / 3, 1.0 / 3}, {b1, a1, a1}, {a1, b1, a1}, {a1, a1, b1},
+                            {b2, a2, a2}, {a2, b2, a2}, {a2, a2, b2}};
+    const double W[7] = {9.0 / 40.0, w1, w1, w1, w2, w2, w2};
+    // translates agree to rounding; distinct ones differ by parts of an edge
+    const double tol = 1e-12 * std::max(std::max(std::fabs(a), std::fabs(b)), std::fabs(h));
+    std::vector<double> coord[3];
+    out.tri.resize(T);
+    for (int t = 0; t < T; ++t) {
+        double P[3][3], e[9];
+        for (int v = 0; v < 3; ++v)
+            for (int x = 0; x < 3; ++x) P[v][x] = verts[3 * tris[3 * t + v] + x];
+        for (int v = 0; v < 3; ++v)
+            for (int x = 0; x < 3; ++x) e[3 * v + x] = P[v][x] - P[0][x];
+        size_t c = 0;
+        for (; c < out.shape.size(); ++c) {
+            double dmax = 0.0;
+            for (int q = 0; q < 9; ++q) dmax = std::max(dmax, std::fabs(out.shape[c].v[q] - e[q]));
+            if (dmax <= tol) break;
+        }
+        if (c == out.shape.size()) {
+            BoxShape s;
+            for (int q = 0; q < 9; ++q) s.v[q] = e[q];
+            const double cr[3] = {e[4] * e[8] - e[5] * e[7], e[5] * e[6] - e[3] * e[8], e[3] * e[7] - e[4] * e[6]};
+            const double A = 0.5 * std::sqrt(cr[0] * cr[0] + cr[1] * cr[1] + cr[2] * cr[2]);
+            for (int q = 0; q < 7; ++q)
+                for (int x = 0; x < 3; ++x) s.r[3 * q + x] = B[q][1] * e[3 + x] + B[q][2] * e[6 + x];
+            for (int i = 0; i < 3; ++i) {
+                const double *p = e + 3 * ((i + 1) % 3), *q = e + 3 * ((i + 2) % 3);
+                const double len = std::sqrt((p[0] - q[0]) * (p[0] - q[0]) + (p[1] - q[1]) * (p[1] - q[1]) +
+                                             (p[2] - q[2]) * (p[2] - q[2]));
+                for (int g = 0; g < 7; ++g)
+                    for (int x = 0; x < 3; ++x)
+                        s.f[21 * i + 3 * g + x] = W[g] * A * (len / (2.0 * A)) * (s.r[3 * g + x] - e[3 * i + x]);
+            }
+            out.shape.push_back(s);
+        }
+        BoxTri& bt = out.tri[t];
+        bt.shape = (int16_t)c;
+        bt.ix = (int16_t)coord_index(coord[0], P[0][0], tol);
+        bt.iy = (int16_t)coord_index(coord[1], P[0][1], tol);
+        bt.iz = (int16_t)coord_index(coord[2], P[0][2], tol);
+    }
+    for (int x = 0; x < 3; ++x) {
+        out.nc[x] = (int)coord[x].size();
+        out.coord.insert(out.coord.end(), coord[x].begin(), coord[x].end());
+    }
+    std::vector<std::vector<BoxMember>> mem(3 * out.shape.size());
+    for (int t = 0; t < T; ++t)
+        for (int i = 0; i < 3; ++i) {
+            const int m = srw[3 * t + i];
+            if (m < 0) continue;
+            mem[3 * (size_t)out.tri[t].shape + i].push_back(
+                BoxMember{t, ssg[3 * t + i] < 0 ? (int32_t)((uint32_t)m | 0x80000000u) : m});
+        }
+    out.slot.resize(mem.size());
+    for (size_t s = 0; s < mem.size(); ++s) out.slot[s] = (int32_t)s;
+    std::stable_sort(out.slot.begin(), out.slot.end(),
+                     [&](int x, int y) { return mem[x].size() > mem[y].size(); });
+    out.ptr.assign(1, 0);
+    for (int s : out.slot) {
+        out.mem.insert(out.mem.end(), mem[s].begin(), mem[s].end());
+        out.ptr.push_back((int32_t)out.mem.size());
+    }
+    return EMSURF_OK;
+}
+
 template <typename T>
 int to_device(T** d, const T* h, size_t n, cudaStream_t st) {
     EMS_CUDA(cudaMalloc(d, sizeof(T) * std::max<size_t>(n, 1)));
@@ -327,52 +588,105 @@ struct Scoped {
     }
 };
 
+template <typename T, typename C, bool TAB>
+int launch_lattice_sum(emsurf_handle* h, const C* X1, int N, double a, double b, const double* dr, const C* tab, int nd,
+                       double k, C* S, size_t smem, cudaStream_t st) {
+    constexpr int ND = 8 * kLsDpt, kMaxDirs = 65535 * ND;      // directions in grid rows
+    EMS_TRY(set_smem_once(lattice_sum_kernel<T, C, TAB>, smem));
+    for (int d0 = 0; d0 < nd; d0 += kMaxDirs) {
+        const int n = std::min(nd - d0, kMaxDirs);
+        const dim3 g((unsigned)((N + 32 * kLsCpt - 1) / (32 * kLsCpt)), (unsigned)((n + ND - 1) / ND));
+        lattice_sum_kernel<T, C, TAB><<<g, kLsThreads, smem, st>>>(
+            X1, h->M, N, h->nx, h->ny, a, b, dr + 3 * (size_t)d0, TAB ? tab + (size_t)d0 * (h->nx + h->ny) : nullptr, n, k,
+            S + (size_t)d0 * N);
+        EMS_CUDA(cudaGetLastError());
+    }
+    return EMSURF_OK;
+}
+
 template <typename T, typename C>
-int far_field_run(emsurf_handle* h, const std::vector<RwgQuad>& q, double a, double b, double k,
-                  const emsurf_c128* Y, int nrhs, int ndir, const double* rhat, emsurf_c128* F, double* rcs,
-                  cudaStream_t st) {
+int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, double k, const emsurf_c128* Y,
+                  int nrhs, int ndir, const double* rhat, emsurf_c128* F, double* rcs, cudaStream_t st) {
     const int E = h->E, K = h->K, M = h->M, N = nrhs * K;
-    // directions in chunks so the per-chunk arrays stay under ~512 MB
-    const size_t per_dir = (size_t)E * 3 * sizeof(double2) + (size_t)N * sizeof(C);
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(ndir, (512ull << 20) / per_dir));
-    Scoped sc;
-    RwgQuad* dq;
-    double* dr;
-    double2* Rv;
-    C *S, *X1;
-    EMS_TRY(to_device(&dq, q.data(), q.size(), st));
-    sc.p.push_back(dq);
-    EMS_TRY(to_device(&dr, rhat, 3 * (size_t)ndir, st));
-    sc.p.push_back(dr);
-    EMS_CUDA(cudaMalloc(&Rv, sizeof(double2) * (size_t)chunk * E * 3));
-    sc.p.push_back(Rv);
-    EMS_CUDA(cudaMalloc(&S, sizeof(C) * (size_t)chunk * N));
-    sc.p.push_back(S);
-    EMS_CUDA(cudaMalloc(&X1, sizeof(C) * (size_t)M * N));
-    sc.p.push_back(X1);
-    gather_cells_kernel<C><<<(int)std::min<size_t>(((size_t)M * N + 255) / 256, 152 * 32), 256, 0, st>>>(
-        reinterpret_cast<const double2*>(Y), h->d_uo_index, h->d_uo_sign, M, K, nrhs, h->n_unique, X1);
-    EMS_CUDA(cudaGetLastError());
-    const size_t lsm = ((size_t)kLsD * (h->nx + h->ny) + (size_t)kLsM * kLsN) * sizeof(C);
-    if (lsm > 227 * 1024) {
+    if ((32 * (size_t)(h->nx + h->ny) + 16 * 64) * sizeof(C) > 227 * 1024) {
         set_error("emsurf_far_field: lattice %d x %d too large for the phase tables", h->nx, h->ny);
         return EMSURF_EINVAL;
     }
-    EMS_TRY(set_smem_once(lattice_sum_tiled_kernel<T, C>, lsm));
+    // directions in chunks whose column sums stay in L2 between the two kernels
+    // (at least enough directions to fill the device)
+    const int chunk = (int)std::min<size_t>(
+        ndir, std::max<size_t>(4096, (48ull << 20) / ((size_t)N * sizeof(C))));
+    // one device buffer: currents, column sums, directions and the box tables
+    size_t bytes = 0;
+    auto part = [&](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_x = part(sizeof(C) * (size_t)M * N), o_s = part(sizeof(C) * (size_t)chunk * N);
+    // phase tables, while a block's part fits in shared memory
+    const size_t lsm0 = ((size_t)kLsM * 32 * kLsCpt + (size_t)kLsM * 8 * kLsDpt) * sizeof(C);
+    const size_t lsm = lsm0 + (size_t)8 * kLsDpt * (h->nx + h->ny) * sizeof(C);
+    const bool tabs = lsm <= 227 * 1024;
+    const size_t o_p = part(tabs ? sizeof(C) * (size_t)chunk * (h->nx + h->ny) : 0);
+    const size_t o_r = part(sizeof(double) * 3 * (size_t)ndir);
+    const size_t o_tab = bytes;
+    const size_t o_shape = part(box.shape.size() * sizeof(BoxShape)), o_tri = part(box.tri.size() * sizeof(BoxTri));
+    const size_t o_coord = part(box.coord.size() * sizeof(double)), o_slot = part(box.slot.size() * sizeof(int32_t));
+    const size_t o_ptr = part(box.ptr.size() * sizeof(int32_t)), o_mem = part(box.mem.size() * sizeof(BoxMember));
+    Scoped sc;
+    unsigned char* buf = nullptr;
+    EMS_CUDA(cudaMalloc(&buf, bytes));
+    sc.p.push_back(buf);
+    std::vector<unsigned char> tab(bytes - o_tab);
+    auto fill = [&](size_t at, const auto& v) { std::memcpy(tab.data() + at - o_tab, v.data(), v.size() * sizeof(v[0])); };
+    fill(o_shape, box.shape);
+    fill(o_tri, box.tri);
+    fill(o_coord, box.coord);
+    fill(o_slot, box.slot);
+    fill(o_ptr, box.ptr);
+    fill(o_mem, box.mem);
+    EMS_CUDA(cudaMemcpyAsync(buf + o_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
+    EMS_CUDA(cudaMemcpyAsync(buf + o_r, rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
+    C *X1 = reinterpret_cast<C*>(buf + o_x), *S = reinterpret_cast<C*>(buf + o_s);
+    const double* dr = reinterpret_cast<const double*>(buf + o_r);
+    const BoxDev g{reinterpret_cast<const BoxShape*>(buf + o_shape), reinterpret_cast<const BoxTri*>(buf + o_tri),
+                   reinterpret_cast<const double*>(buf + o_coord), reinterpret_cast<const int32_t*>(buf + o_slot),
+                   reinterpret_cast<const int32_t*>(buf + o_ptr), reinterpret_cast<const BoxMember*>(buf + o_mem),
+                   (int)box.shape.size(), (int)box.tri.size(), box.nc[0], box.nc[1], box.nc[2], (int)box.slot.size()};
+    gather_cells_kernel<C><<<(int)std::min<size_t>(((size_t)M * N + 255) / 256, 152 * 32), 256, 0, st>>>(
+        reinterpret_cast<const double2*>(Y), h->d_uo_index, h->d_uo_sign, M, K, nrhs, h->n_unique, X1);
+    EMS_CUDA(cudaGetLastError());
+    // far field: triangle phases in shared memory while one warp's fit
+    const size_t per = (box.coord.size() + 7 * box.shape.size() + 3 * box.slot.size()) * sizeof(double2);
+    const size_t per_ph = per + box.tri.size() * sizeof(double2);
+    const bool ph = per_ph <= 200 * 1024;
+    int warps = kFfWarps;
+    while (warps > 1 && (ph ? per_ph : per) * warps > 200 * 1024) warps /= 2;
+    const size_t fsm = (ph ? per_ph : per) * warps;
+    if (ph) EMS_TRY(set_smem_once(far_field_kernel<C, true>, fsm));
+    else EMS_TRY(set_smem_once(far_field_kernel<C, false>, fsm));
     double2* Fo = reinterpret_cast<double2*>(F);
     for (int d0 = 0; d0 < ndir; d0 += chunk) {
         const int nd = std::min(chunk, ndir - d0);
-        const size_t t1 = (size_t)nd * E;
-        radiation_kernel<<<(int)std::min<size_t>((t1 + 127) / 128, 152 * 32), 128, 0, st>>>(
-            dq, E, dr + 3 * (size_t)d0, nd, k, Rv);
-        EMS_CUDA(cudaGetLastError());
-        const dim3 g2((unsigned)((N + kLsN - 1) / kLsN), (unsigned)((nd + kLsD - 1) / kLsD));
-        lattice_sum_tiled_kernel<T, C><<<g2, kLsThreads, lsm, st>>>(X1, M, N, h->nx, h->ny, a, b,
-                                                                     dr + 3 * (size_t)d0, nd, k, S);
-        EMS_CUDA(cudaGetLastError());
-        const size_t t3 = (size_t)nrhs * nd;
-        far_field_kernel<C><<<(int)std::min<size_t>((t3 + 127) / 128, 152 * 32), 128, 0, st>>>(
-            S, Rv, dr + 3 * (size_t)d0, nd, E, nrhs, k, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
+        const double* drc = dr + 3 * (size_t)d0;
+        if (tabs) {
+            C* tab = reinterpret_cast<C*>(buf + o_p);
+            const size_t tn = (size_t)nd * (h->nx + h->ny);
+            phase_table_kernel<T, C><<<(int)std::min<size_t>((tn + 127) / 128, 152 * 32), 128, 0, st>>>(
+                drc, nd, h->nx, h->ny, a, b, k, tab);
+            EMS_CUDA(cudaGetLastError());
+            EMS_TRY((launch_lattice_sum<T, C, true>(h, X1, N, a, b, drc, tab, nd, k, S, lsm, st)));
+        } else {
+            EMS_TRY((launch_lattice_sum<T, C, false>(h, X1, N, a, b, drc, nullptr, nd, k, S, lsm0, st)));
+        }
+        const int blocks = std::min((nd + warps - 1) / warps, h->num_sms * 32);
+        if (ph)
+            far_field_kernel<C, true><<<blocks, 32 * warps, fsm, st>>>(S, g, drc, nd, E, nrhs, k, Fo + (size_t)d0 * 3,
+                                                                           rcs ? rcs + d0 : nullptr, ndir);
+        else
+            far_field_kernel<C, false><<<blocks, 32 * warps, fsm, st>>>(S, g, drc, nd, E, nrhs, k, Fo + (size_t)d0 * 3,
+                                                                         rcs ? rcs + d0 : nullptr, ndir);
         EMS_CUDA(cudaGetLastError());
     }
     EMS_CUDA(cudaStreamSynchronize(st));
@@ -428,10 +742,10 @@ EMSURF_API int emsurf_far_field(emsurf_handle* h, double a, double b, double hgt
         return EMSURF_EINVAL;
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    std::vector<RwgQuad> q;
-    EMS_TRY(box_quadrature(a, b, hgt, n, zlevels, h->E, q));
-    if (h->precision == EMSURF_FP64) return far_field_run<double, double2>(h, q, a, b, k, Y, nrhs, ndir, rhat, F, rcs, st);
-    return far_field_run<float, float2>(h, q, a, b, k, Y, nrhs, ndir, rhat, F, rcs, st);
+    BoxShapes box;
+    EMS_TRY(box_shapes(a, b, hgt, n, zlevels, h->E, box));
+    if (h->precision == EMSURF_FP64) return far_field_run<double, double2>(h, box, a, b, k, Y, nrhs, ndir, rhat, F, rcs, st);
+    return far_field_run<float, float2>(h, box, a, b, k, Y, nrhs, ndir, rhat, F, rcs, st);
 }
 
 }  // extern "C"
