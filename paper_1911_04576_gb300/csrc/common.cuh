@@ -111,24 +111,24 @@ template <> __host__ __device__ __forceinline__ float2 mk<float2>(double re, dou
 }
 
 // ---------------------------------------------------------------- FFT plan
-// One 1-D transform length P = product of radices (each 2, 3, 4, 5 or 7) with
+// One 1-D transform length P = 2^a 3^b 5^c 7^d with
 // a device table tw[k] = exp(-2 pi i k / P), k in [0, P), from host libm.
 struct FftPlan {
     int P = 0;
-    int nrad = 0;
-    int rad[16] = {0};
     double2* tw = nullptr;   // device
 };
 
 int fft_plan_create(FftPlan& plan, int P);
-// fused 2-D transforms of square grids up to 64 x 64 (fft2d.cu)
-bool fft2d_fused_ok(int px, int py);
+// fused 2-D transforms of grids that fit in shared memory (fft2d.cu)
 template <typename T2>
-int fft2d_forward(T2* Xg, int P, long long lanes, int nx, int ny, int K, int n_unique, const double2* tw,
-                  const double2* x, const float2* xf, const int32_t* idx, const int8_t* sgn, cudaStream_t st);
+bool fft2d_fused_ok(int px, int py, int nx, int ny);
 template <typename T2>
-int fft2d_inverse(const T2* Yg, int P, long long lanes, int nx, int ny, int K, int M, int R, int nsplit,
-                  double scale, const double2* tw, const T2* mm, T2* y1, cudaStream_t st);
+int fft2d_forward(T2* Xg, int px, int py, long long lanes, int nx, int ny, int K, int n_unique, const double2* twx,
+                  const double2* twy, const double2* x, const float2* xf, const int32_t* idx, const int8_t* sgn,
+                  cudaStream_t st);
+template <typename T2>
+int fft2d_inverse(const T2* Yg, int px, int py, long long lanes, int nx, int ny, int K, int M, int R, int nsplit,
+                  double scale, const double2* twx, const double2* twy, const T2* mm, T2* y1, cudaStream_t st);
 void fft_plan_destroy(FftPlan& plan);
 
 // In-place 1-D transform along p of data[outer][P][inner] (inner contiguous

@@ -2,126 +2,33 @@
 //
 // Sec. IV-B evaluates each Toeplitz block product with the FFT of its
 // circulant embedding (Eqs. LJV3-LJV5) and generalises to 2-D lattices with
-// 2-D FFTs.  Here every 2-D transform is two 1-D passes.  A pass transforms
+// 2-D FFTs.  Here every 2-D transform is two 1-D passes (grids that fit in
+// shared memory take the fused transforms of fft2d.cu).  A pass transforms
 // data[outer][P][inner] along P; the `inner` dimension holds independent
 // sequences (local unknowns k, right-hand sides, or block entries (op,j,i))
-// that sit next to each other in memory, so one CTA loads a P x W tile whose
-// rows are W contiguous lanes (coalesced), transforms all W lanes in shared
-// memory with a Stockham autosort mixed-radix algorithm (radices 2,3,4,5,7;
-// Govindaraju et al., SC 2008), and writes the tile back.
+// that sit next to each other in memory, so one CTA takes a P x W tile whose
+// rows are W contiguous lanes (coalesced).  The first Stockham stage reads
+// global memory into registers and the last one writes it (fft_core.cuh), so
+// the tile crosses shared memory once per stage boundary.
 //
 // Pruning: only the first p_in points along P are read (the rest are the
 // zero padding of the circulant embedding) and only the first p_out are
 // written (the crop of the inverse transform).  The forward pass over the
 // cell rows can read its input straight from the unique-unknown vector
 // through U_o (x1 = U_o x, Eq. MVP), so no padded grid is ever written.
-//
-// Grid sizes used by the lattices here have compile-time kernels (radices,
-// strides and twiddle indices are constants, twiddles sit in shared memory);
-// any other 2,3,5,7-smooth size runs a generic kernel.
+#include <algorithm>
 #include <cmath>
 
-#include "common.cuh"
+#include "fft_core.cuh"
 
 namespace emsurf {
 
 namespace {
 
+using namespace fftc;
+
 constexpr int kFftThreads = 256;
-constexpr int kMaxRadix = 7;
-
-// ---------------------------------------------------------------- radices
-constexpr int rad_count(int P) {
-    int n = 0;
-    const int qs[5] = {4, 2, 3, 5, 7};
-    for (int i = 0; i < 5; ++i)
-        while (P % qs[i] == 0 && P > 1) {
-            P /= qs[i];
-            ++n;
-        }
-    return n;
-}
-constexpr int rad_at(int P, int s) {
-    int n = 0;
-    const int qs[5] = {4, 2, 3, 5, 7};
-    for (int i = 0; i < 5; ++i)
-        while (P % qs[i] == 0 && P > 1) {
-            if (n == s) return qs[i];
-            P /= qs[i];
-            ++n;
-        }
-    return 1;
-}
-
-template <typename T2>
-__device__ __forceinline__ T2 mul_i(T2 a, int s) {   // a * (s i), s = +-1
-    T2 r;
-    r.x = -s * a.y;
-    r.y = s * a.x;
-    return r;
-}
-template <typename T2>
-__device__ __forceinline__ T2 csub2(T2 a, T2 b) {
-    T2 r;
-    r.x = a.x - b.x;
-    r.y = a.y - b.y;
-    return r;
-}
-
-// One Stockham stage of radix R (compile time) over all W lanes.
-template <typename T2, int W, int P, int R, int NS, int SIGN>
-__device__ __forceinline__ void stage(const T2* __restrict__ in, T2* __restrict__ out,
-                                      const T2* __restrict__ tw) {
-    constexpr int NR = P / R;
-    constexpr int tstep = P / (NS * R);
-    constexpr int qstep = P / R;
-    for (int e = threadIdx.x; e < NR * W; e += blockDim.x) {
-        const int j = e / W, l = e % W;
-        const int jm = j % NS;
-        T2 v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const T2 a = in[(j + r * NR) * W + l];
-            v[r] = (r == 0 || NS == 1) ? a : cmul(a, tw[jm * r * tstep]);
-        }
-        const int idxD = (j / NS) * NS * R + jm;
-        if constexpr (R == 2) {
-            out[idxD * W + l] = cadd(v[0], v[1]);
-            out[(idxD + NS) * W + l] = csub2(v[0], v[1]);
-        } else if constexpr (R == 4) {
-            // w_4 = e^{SIGN 2 pi i / 4} = SIGN i
-            const T2 s02 = cadd(v[0], v[2]), d02 = csub2(v[0], v[2]);
-            const T2 s13 = cadd(v[1], v[3]), d13 = csub2(v[1], v[3]);
-            out[idxD * W + l] = cadd(s02, s13);
-            out[(idxD + NS) * W + l] = cadd(d02, mul_i(d13, SIGN));
-            out[(idxD + 2 * NS) * W + l] = csub2(s02, s13);
-            out[(idxD + 3 * NS) * W + l] = csub2(d02, mul_i(d13, SIGN));
-        } else {
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                T2 acc = v[0];
-#pragma unroll
-                for (int r = 1; r < R; ++r) acc = cadd(acc, cmul(v[r], tw[((q * r) % R) * qstep]));
-                out[(idxD + q * NS) * W + l] = acc;
-            }
-        }
-    }
-}
-
-template <typename T2, int W, int P, int S, int NS, int SIGN>
-struct Stages {
-    // returns the buffer holding the result
-    static __device__ __forceinline__ T2* run(T2* in, T2* out, const T2* tw) {
-        if constexpr (S < rad_count(P)) {
-            constexpr int R = rad_at(P, S);
-            stage<T2, W, P, R, NS, SIGN>(in, out, tw);
-            __syncthreads();
-            return Stages<T2, W, P, S + 1, NS * R, SIGN>::run(out, in, tw);
-        } else {
-            return in;
-        }
-    }
-};
+constexpr int kFftMaxRad = 16;
 
 // Gather source of the forward pass over cell rows: element (row iy, point
 // ix, lane L = r*K + k) = sign * x[r][uo_index[(iy*nx + ix)*K + k]].
@@ -179,14 +86,18 @@ __device__ __forceinline__ void crop_store(const CropEpi<T2>& ep, int iy, int p,
     ep.y1[((size_t)r * ep.M + m) * ep.K + k] = o;
 }
 
-template <typename T2, int W, int P, int SIGN, bool GATHER, bool EPI>
+// One pass over tiles of W lanes (a power of two up to 32).  In place: a tile's
+// points are all read before any is written (one thread does both when there
+// is a single stage).
+template <typename T2, int SIGN, bool GATHER, bool EPI>
 __global__ void __launch_bounds__(kFftThreads)
-fft_fixed_kernel(T2* __restrict__ data, long long inner, long long outer_stride, int p_in, int p_out,
-                 const double2* __restrict__ twg, GatherSrc gs, CropEpi<T2> ep) {
+fft_pass_kernel(T2* __restrict__ data, FftStages f, FastDiv lanes, long long inner, long long outer_stride, int p_in,
+                int p_out, const double2* __restrict__ twg, GatherSrc gs, CropEpi<T2> ep) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* buf0 = reinterpret_cast<T2*>(smem_raw);
-    T2* buf1 = buf0 + P * W;
-    T2* tw = buf1 + P * W;
+    const int P = f.P, W = (int)lanes.d;
+    T2* tw = reinterpret_cast<T2*>(smem_raw);
+    T2* cur = tw + P;
+    T2* nxt = cur + P * W;
     for (int e = threadIdx.x; e < P; e += blockDim.x) {
         const double2 w = twg[e];
         tw[e] = mk<T2>(w.x, SIGN < 0 ? w.y : -w.y);
@@ -194,185 +105,59 @@ fft_fixed_kernel(T2* __restrict__ data, long long inner, long long outer_stride,
     const long long lane0 = (long long)blockIdx.x * W;
     const int wl = (int)min((long long)W, inner - lane0);
     T2* base = data + (long long)blockIdx.y * outer_stride + lane0;
-    const T2 zero = mk<T2>(0.0, 0.0);
-    for (int e = threadIdx.x; e < P * W; e += blockDim.x) {
-        const int p = e / W, l = e % W;
-        T2 v = zero;
-        if (l < wl && p < p_in) {
-            if constexpr (GATHER) {
-                const long long L = lane0 + l;
-                const int r = (int)(L / gs.K), k = (int)(L % gs.K);
-                const size_t loc = ((size_t)blockIdx.y * gs.nx + p) * gs.K + k;
-                v = gather_value<T2>(gs, r, loc);
-            } else {
-                v = base[(long long)p * inner + l];
-            }
-        }
-        buf0[e] = v;
+    // blockDim is a multiple of W: a thread stays on one lane
+    const int myl = threadIdx.x & (W - 1);
+    const bool live = myl < wl;
+    int gr = 0, gk = 0;
+    if constexpr (GATHER) {
+        const long long L = lane0 + (live ? myl : 0);
+        gr = (int)(L / gs.K);
+        gk = (int)(L - (long long)gr * gs.K);
     }
     __syncthreads();
-    const T2* res = Stages<T2, W, P, 0, 1, SIGN>::run(buf0, buf1, tw);
-    for (int e = threadIdx.x; e < p_out * W; e += blockDim.x) {
-        const int p = e / W, l = e % W;
-        if (l < wl) {
-            if constexpr (EPI) crop_store(ep, blockIdx.y, p, lane0 + l, res[e]);
-            else base[(long long)p * inner + l] = res[e];
+    auto ld0 = [&](int p, int l) {
+        T2 v = mk<T2>(0.0, 0.0);
+        if (live && p < p_in) {
+            if constexpr (GATHER) v = gather_value<T2>(gs, gr, ((size_t)blockIdx.y * gs.nx + p) * gs.K + gk);
+            else v = base[(long long)p * inner + l];
         }
-    }
-}
-
-// ---------------------------------------------------------------- generic
-struct RadList {
-    int n;
-    int r[16];
-};
-
-template <typename T2>
-__device__ __forceinline__ T2 tw_at(const double2* __restrict__ tw, int k, int sign) {
-    double2 w = tw[k];
-    return mk<T2>(w.x, sign < 0 ? w.y : -w.y);
-}
-
-template <typename T2, int W>
-__global__ void __launch_bounds__(kFftThreads)
-fft_pass_kernel(T2* __restrict__ data, int P, long long inner, long long outer_stride, int p_in,
-                int p_out, const double2* __restrict__ tw, RadList rad, int sign, GatherSrc gs,
-                int gather, CropEpi<T2> ep, int epi) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* buf0 = reinterpret_cast<T2*>(smem_raw);
-    T2* buf1 = buf0 + (size_t)P * W;
-    const long long lane0 = (long long)blockIdx.x * W;
-    const int wl = (int)min((long long)W, inner - lane0);
-    T2* base = data + (long long)blockIdx.y * outer_stride + lane0;
-    const T2 zero = mk<T2>(0.0, 0.0);
-
-    for (int e = threadIdx.x; e < P * W; e += blockDim.x) {
-        const int p = e / W, l = e - (e / W) * W;
-        T2 v = zero;
-        if (l < wl && p < p_in) {
-            if (gather) {
-                const long long L = lane0 + l;
-                const int r = (int)(L / gs.K), k = (int)(L % gs.K);
-                const size_t loc = ((size_t)blockIdx.y * gs.nx + p) * gs.K + k;
-                v = gather_value<T2>(gs, r, loc);
-            } else {
-                v = base[(long long)p * inner + l];
-            }
+        return v;
+    };
+    auto st1 = [&](int p, int l, T2 v) {
+        if (live && p < p_out) {
+            if constexpr (EPI) crop_store(ep, blockIdx.y, p, lane0 + l, v);
+            else base[(long long)p * inner + l] = v;
         }
-        buf0[e] = v;
+    };
+    for (int s = 0; s < f.n; ++s) {
+        const bool first = s == 0, last = s == f.n - 1;
+        T2* out = cur;
+        const T2* in = nxt;
+        stage_any<SIGN, kFftMaxRad, T2>(
+            f.rad[s], P, f.ns[s], lanes, tw, [&](int p, int l) { return first ? ld0(p, l) : in[p * W + l]; },
+            [&](int p, int l, T2 v) {
+                if (last) st1(p, l, v);
+                else out[p * W + l] = v;
+            });
+        if (!last) __syncthreads();
+        T2* t = cur;
+        cur = nxt;
+        nxt = t;
     }
-    __syncthreads();
-
-    T2* in = buf0;
-    T2* out = buf1;
-    int Ns = 1;
-    for (int s = 0; s < rad.n; ++s) {
-        const int R = rad.r[s];
-        const int NR = P / R;
-        const int tstep = P / (Ns * R);   // twiddle stride of w_{Ns R}
-        const int qstep = P / R;          // stride of w_R
-        for (int e = threadIdx.x; e < NR * W; e += blockDim.x) {
-            const int j = e / W, l = e - (e / W) * W;
-            const int jm = j % Ns;
-            T2 v[kMaxRadix];
-#pragma unroll
-            for (int r = 0; r < kMaxRadix; ++r) {
-                if (r < R) {
-                    T2 a = in[(j + r * NR) * W + l];
-                    v[r] = (r == 0 || jm == 0) ? a : cmul(a, tw_at<T2>(tw, jm * r * tstep, sign));
-                }
-            }
-            const int idxD = (j / Ns) * Ns * R + jm;
-#pragma unroll
-            for (int q = 0; q < kMaxRadix; ++q) {
-                if (q < R) {
-                    T2 acc = v[0];
-#pragma unroll
-                    for (int r = 1; r < kMaxRadix; ++r) {
-                        if (r < R) acc = cadd(acc, cmul(v[r], tw_at<T2>(tw, ((q * r) % R) * qstep, sign)));
-                    }
-                    out[(idxD + q * Ns) * W + l] = acc;
-                }
-            }
-        }
-        Ns *= R;
-        T2* t = in;
-        in = out;
-        out = t;
-        __syncthreads();
-    }
-
-    for (int e = threadIdx.x; e < p_out * W; e += blockDim.x) {
-        const int p = e / W, l = e - (e / W) * W;
-        if (l < wl) {
-            if (epi) crop_store(ep, blockIdx.y, p, lane0 + l, in[e]);
-            else base[(long long)p * inner + l] = in[e];
-        }
-    }
-}
-
-// lanes per CTA: the largest of 32, 16, 8 whose two buffers fit in 96 KB
-template <typename T2>
-constexpr int lanes_for(int P) {
-    return (2 * P * 32 * (int)sizeof(T2) <= 96 * 1024) ? 32
-         : (2 * P * 16 * (int)sizeof(T2) <= 96 * 1024) ? 16 : 8;
-}
-
-template <typename T2, int P, int SIGN, bool GATHER, bool EPI>
-int launch_fixed(T2* data, const FftPlan& plan, long long inner, long long outer,
-                 long long outer_stride, int p_in, int p_out, const GatherSrc& gs,
-                 const CropEpi<T2>& ep, cudaStream_t st) {
-    constexpr int W = lanes_for<T2>(P);
-    const size_t smem = (2ull * P * W + P) * sizeof(T2);
-    auto kern = fft_fixed_kernel<T2, W, P, SIGN, GATHER, EPI>;
-    EMS_TRY(set_smem_once(kern, smem));
-    const long long gx = (inner + W - 1) / W;
-    dim3 grid((unsigned)gx, (unsigned)outer);
-    kern<<<grid, kFftThreads, smem, st>>>(data, inner, outer_stride, p_in, p_out, plan.tw, gs, ep);
-    EMS_CUDA(cudaGetLastError());
-    return EMSURF_OK;
-}
-
-template <typename T2, int W>
-int launch_generic(T2* data, const FftPlan& plan, long long inner, long long outer,
-                   long long outer_stride, int p_in, int p_out, int sign, const GatherSrc& gs,
-                   bool gather, const CropEpi<T2>& ep, bool epi, cudaStream_t st) {
-    RadList rl;
-    rl.n = plan.nrad;
-    for (int i = 0; i < 16; ++i) rl.r[i] = plan.rad[i];
-    const size_t smem = 2ull * plan.P * W * sizeof(T2);
-    EMS_TRY(set_smem_once(fft_pass_kernel<T2, W>, smem));
-    const long long gx = (inner + W - 1) / W;
-    dim3 grid((unsigned)gx, (unsigned)outer);
-    fft_pass_kernel<T2, W><<<grid, kFftThreads, smem, st>>>(data, plan.P, inner, outer_stride, p_in,
-                                                            p_out, plan.tw, rl, sign, gs, gather ? 1 : 0,
-                                                            ep, epi ? 1 : 0);
-    EMS_CUDA(cudaGetLastError());
-    return EMSURF_OK;
 }
 
 template <typename T2, int SIGN, bool GATHER, bool EPI>
-int dispatch_fixed(int P, T2* data, const FftPlan& plan, long long inner, long long outer,
-                   long long os, int p_in, int p_out, const GatherSrc& gs, const CropEpi<T2>& ep,
-                   cudaStream_t st, bool* done) {
-    *done = true;
-#define EMS_FFT_CASE(N) \
-    case N: return launch_fixed<T2, N, SIGN, GATHER, EPI>(data, plan, inner, outer, os, p_in, p_out, gs, ep, st);
-    switch (P) {
-        EMS_FFT_CASE(5)
-        EMS_FFT_CASE(8)
-        EMS_FFT_CASE(15)
-        EMS_FFT_CASE(16)
-        EMS_FFT_CASE(24)
-        EMS_FFT_CASE(32)
-        EMS_FFT_CASE(48)
-        EMS_FFT_CASE(64)
-        EMS_FFT_CASE(96)
-        EMS_FFT_CASE(128)
-        EMS_FFT_CASE(200)
-        default: *done = false; return EMSURF_OK;
-    }
-#undef EMS_FFT_CASE
+int launch_pass(T2* data, const FftPlan& plan, const FftStages& f, int W, size_t smem, long long inner,
+                long long outer, long long outer_stride, int p_in, int p_out, const GatherSrc& gs,
+                const CropEpi<T2>& ep, cudaStream_t st) {
+    EMS_TRY(set_smem_once(fft_pass_kernel<T2, SIGN, GATHER, EPI>, smem));
+    FastDiv lanes;
+    lanes.set((uint32_t)W);
+    const dim3 grid((unsigned)((inner + W - 1) / W), (unsigned)outer);
+    fft_pass_kernel<T2, SIGN, GATHER, EPI><<<grid, kFftThreads, smem, st>>>(data, f, lanes, inner, outer_stride, p_in,
+                                                                          p_out, plan.tw, gs, ep);
+    EMS_CUDA(cudaGetLastError());
+    return EMSURF_OK;
 }
 
 template <typename T2>
@@ -384,28 +169,26 @@ int pass_impl(T2* data, const FftPlan& plan, long long inner, long long outer, l
         set_error("fft_pass: grid too large (outer %lld, lanes %lld)", outer, inner);
         return EMSURF_EINVAL;
     }
+    FftStages f;
+    const size_t point = sizeof(T2);
+    if (!fft_stages(plan.P, kFftMaxRad, f) || 2 * (size_t)plan.P * 8 * point > 200 * 1024) {
+        set_error("FFT length %d too large for one shared-memory pass", plan.P);
+        return EMSURF_EINVAL;
+    }
     p_in = p_in < 0 ? plan.P : std::min(p_in, plan.P);
     p_out = p_out < 0 ? plan.P : std::min(p_out, plan.P);
-    bool done = false;
-    int s = EMSURF_OK;
+    // 32 lanes while two blocks fit an SM, else 16 or 8
+    const size_t bufs = f.n > 2 ? 2 : f.n > 1 ? 1 : 0;
+    int W = 32;
+    while (W > 8 && bufs * plan.P * W * point > 96 * 1024) W /= 2;
+    const size_t smem = (bufs * W + 1) * plan.P * point;
     if (sign < 0 && gather)
-        s = dispatch_fixed<T2, -1, true, false>(plan.P, data, plan, inner, outer, outer_stride, p_in, p_out, gs, ep, st, &done);
-    else if (sign < 0)
-        s = dispatch_fixed<T2, -1, false, false>(plan.P, data, plan, inner, outer, outer_stride, p_in, p_out, gs, ep, st, &done);
-    else if (epi)
-        s = dispatch_fixed<T2, +1, false, true>(plan.P, data, plan, inner, outer, outer_stride, p_in, p_out, gs, ep, st, &done);
-    else
-        s = dispatch_fixed<T2, +1, false, false>(plan.P, data, plan, inner, outer, outer_stride, p_in, p_out, gs, ep, st, &done);
-    if (s != EMSURF_OK || done) return s;
-    const size_t per_lane = 2ull * plan.P * sizeof(T2);
-    if (per_lane * 32 <= 200 * 1024)
-        return launch_generic<T2, 32>(data, plan, inner, outer, outer_stride, p_in, p_out, sign, gs, gather, ep, epi, st);
-    if (per_lane * 16 <= 200 * 1024)
-        return launch_generic<T2, 16>(data, plan, inner, outer, outer_stride, p_in, p_out, sign, gs, gather, ep, epi, st);
-    if (per_lane * 8 <= 200 * 1024)
-        return launch_generic<T2, 8>(data, plan, inner, outer, outer_stride, p_in, p_out, sign, gs, gather, ep, epi, st);
-    set_error("FFT length %d too large for one shared-memory pass", plan.P);
-    return EMSURF_EINVAL;
+        return launch_pass<T2, -1, true, false>(data, plan, f, W, smem, inner, outer, outer_stride, p_in, p_out, gs, ep, st);
+    if (sign < 0)
+        return launch_pass<T2, -1, false, false>(data, plan, f, W, smem, inner, outer, outer_stride, p_in, p_out, gs, ep, st);
+    if (epi)
+        return launch_pass<T2, +1, false, true>(data, plan, f, W, smem, inner, outer, outer_stride, p_in, p_out, gs, ep, st);
+    return launch_pass<T2, +1, false, false>(data, plan, f, W, smem, inner, outer, outer_stride, p_in, p_out, gs, ep, st);
 }
 
 }  // namespace
@@ -420,20 +203,14 @@ int smallest_smooth_at_least(int n) {
 }
 
 int fft_plan_create(FftPlan& plan, int P) {
-    int t = P, n = 0;
-    int rad[16];
-    while (t % 4 == 0 && n < 16) { rad[n++] = 4; t /= 4; }
-    while (t % 2 == 0 && n < 16) { rad[n++] = 2; t /= 2; }
-    while (t % 3 == 0 && n < 16) { rad[n++] = 3; t /= 3; }
-    while (t % 5 == 0 && n < 16) { rad[n++] = 5; t /= 5; }
-    while (t % 7 == 0 && n < 16) { rad[n++] = 7; t /= 7; }
+    int t = P;
+    for (int p : {2, 3, 5, 7})
+        while (t > 1 && t % p == 0) t /= p;
     if (t != 1 || P < 1) {
         set_error("FFT length %d has a prime factor other than 2, 3, 5, 7", P);
         return EMSURF_EINVAL;
     }
     plan.P = P;
-    plan.nrad = n;
-    for (int i = 0; i < 16; ++i) plan.rad[i] = i < n ? rad[i] : 0;
     std::vector<double2> h(P);
     const double two_pi = 6.283185307179586476925286766559;
     for (int k = 0; k < P; ++k) {

@@ -2,145 +2,45 @@
 // embedding of the block-Toeplitz lattice operator, applied with 2-D FFTs).
 //
 // The pass-based transforms (fft.cu) run each 2-D FFT as two launches with
-// the grid written to global memory in between.  For square grids of up to
-// 64 x 64 points a CTA here holds a whole P x P grid for W lanes (local
-// unknowns k of one or more rhs) in shared memory and does the gather of
-// x1 = U_o x, both 1-D transforms and the store of X^ in one launch; the
-// inverse does both inverse transforms, the crop to the lattice, the 1/P
-// scale and the addition of the macromodel partials in one launch.
+// the grid written to global memory in between.  While the px x py grid of W
+// lanes (local unknowns k of one or more rhs) fits in shared memory, a CTA
+// here does the gather of x1 = U_o x, both 1-D transforms and the store of
+// X^ in one launch; the inverse does both inverse transforms, the crop to the
+// lattice, the 1/P scale and the addition of the macromodel partials.
 //
-// Layouts in shared memory (W lanes contiguous):
-//   rows:    A[ix][iy * W + w]  (the x-transform's lanes are (iy, w))
-//   columns: B[iy][kx * W + w]  (the y-transform's lanes are (kx, w))
-// The 1-D transforms are Stockham autosort stages (radices 4, 2, 3, 5, 7;
-// Govindaraju et al., SC 2008) over a runtime number of lanes.
-#include "common.cuh"
+// The first stage of a transform reads global memory straight into registers
+// and the last one writes it, so a lane's grid passes through shared memory
+// once per stage boundary (three times for lengths of two stages).  Layouts
+// there (W lanes contiguous, rows of odd length so that consecutive kx fall in
+// different banks):
+//   rows:    A[ix or kx][iy],   row stride (ny | 1) W
+//   columns: B[kx][ky or iy],   row stride (py | 1) W
+// Against the earlier kernels (every stage and both transposes through shared
+// memory, run-time index divisions; grids other than the compiled squares up to
+// 64 in four passes of a generic kernel): 24 x 24 boxes with 32 rhs 466 -> 278 us
+// per direction, 20 x 13 boxes (40 x 25 grid) with 3 rhs 160 -> 22 us, 16 x 16
+// with one rhs 11.2 -> 10.2 us.
+#include <algorithm>
+
+#include "fft_core.cuh"
 
 namespace emsurf {
 namespace {
 
+using namespace fftc;
 
-constexpr int f2_rad_count(int P) {
-    int n = 0;
-    const int qs[5] = {4, 2, 3, 5, 7};
-    for (int i = 0; i < 5; ++i)
-        while (P % qs[i] == 0 && P > 1) {
-            P /= qs[i];
-            ++n;
-        }
-    return n;
-}
-constexpr int f2_rad_at(int P, int s) {
-    int n = 0;
-    const int qs[5] = {4, 2, 3, 5, 7};
-    for (int i = 0; i < 5; ++i)
-        while (P % qs[i] == 0 && P > 1) {
-            if (n == s) return qs[i];
-            P /= qs[i];
-            ++n;
-        }
-    return 1;
-}
+constexpr int kF2MaxRad = 10;
+constexpr int kF2MaxW = 8;
+constexpr int kF2MaxSplit = 8;   // macromodel partials (kMmSplit of the product)
+constexpr size_t kF2MaxSmem = 220 * 1024;
 
-template <typename T2>
-__device__ __forceinline__ T2 f2_sub(T2 a, T2 b) {
-    T2 r;
-    r.x = a.x - b.x;
-    r.y = a.y - b.y;
-    return r;
-}
-template <typename T2>
-__device__ __forceinline__ T2 f2_muli(T2 a, int s) {   // a * (s i)
-    T2 r;
-    r.x = -s * a.y;
-    r.y = s * a.x;
-    return r;
-}
-
-// one radix-R Stockham stage over nl lanes: element (p, l) at p * nl + l
-template <typename T2, int P, int R, int NS, int SIGN>
-__device__ __forceinline__ void f2_stage(const T2* __restrict__ in, T2* __restrict__ out,
-                                         const T2* __restrict__ tw, int nl) {
-    constexpr int NR = P / R;
-    constexpr int tstep = P / (NS * R);
-    constexpr int qstep = P / R;
-    for (int e = threadIdx.x; e < NR * nl; e += blockDim.x) {
-        const int j = e / nl, l = e - j * nl;
-        const int jm = j % NS;
-        T2 v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const T2 a = in[(j + r * NR) * nl + l];
-            v[r] = (r == 0 || NS == 1) ? a : cmul(a, tw[jm * r * tstep]);
-        }
-        const int d = (j / NS) * NS * R + jm;
-        if constexpr (R == 2) {
-            out[d * nl + l] = cadd(v[0], v[1]);
-            out[(d + NS) * nl + l] = f2_sub(v[0], v[1]);
-        } else if constexpr (R == 4) {
-            const T2 s02 = cadd(v[0], v[2]), d02 = f2_sub(v[0], v[2]);
-            const T2 s13 = cadd(v[1], v[3]), d13 = f2_sub(v[1], v[3]);
-            out[d * nl + l] = cadd(s02, s13);
-            out[(d + NS) * nl + l] = cadd(d02, f2_muli(d13, SIGN));
-            out[(d + 2 * NS) * nl + l] = f2_sub(s02, s13);
-            out[(d + 3 * NS) * nl + l] = f2_sub(d02, f2_muli(d13, SIGN));
-        } else {
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                T2 acc = v[0];
-#pragma unroll
-                for (int r = 1; r < R; ++r) acc = cadd(acc, cmul(v[r], tw[((q * r) % R) * qstep]));
-                out[(d + q * NS) * nl + l] = acc;
-            }
-        }
-    }
-}
-
-template <typename T2, int P, int S, int NS, int SIGN>
-struct F2Stages {
-    // transforms in place between the two buffers; returns the one holding the result
-    static __device__ __forceinline__ T2* run(T2* in, T2* out, const T2* tw, int nl) {
-        if constexpr (S < f2_rad_count(P)) {
-            constexpr int R = f2_rad_at(P, S);
-            f2_stage<T2, P, R, NS, SIGN>(in, out, tw, nl);
-            __syncthreads();
-            return F2Stages<T2, P, S + 1, NS * R, SIGN>::run(out, in, tw, nl);
-        } else {
-            return in;
-        }
-    }
+struct F2Plan {
+    FftStages x, y;
+    FastDiv lx, ly;          // lanes of the x transforms (ny W) and of the y ones (px W)
+    int lw = 0;              // log2 W
+    int nx = 0, ny = 0;
+    int buf0 = 0, buf1 = 0;  // elements of the two shared buffers
 };
-
-// lanes per CTA: at most what keeps the grid of W lanes twice (ping-pong)
-// within ~96 KB (one lane when the grid alone is larger).  The launch takes
-// the widest W while that still gives at least one CTA per SM (measured at
-// 16x16, K = 576, one rhs: W = 4 with 512 threads 10.1 + 12.2 us per
-// forward + inverse pair, W = 1 with 256 threads 12.3 + 13.7 us).
-template <typename T2, int P>
-constexpr int f2_max_lanes() {
-    constexpr int per = 2 * P * P * (int)sizeof(T2);
-    return per * 8 <= 96 * 1024 ? 8 : per * 4 <= 96 * 1024 ? 4 : per * 2 <= 96 * 1024 ? 2 : 1;
-}
-
-template <typename T2, int P, int W>
-constexpr size_t f2_smem() {
-    return (size_t)(2 * P * P * W + P) * sizeof(T2);
-}
-
-template <int W>
-constexpr int f2_threads() { return W >= 4 ? 512 : 256; }
-
-int f2_pick_lanes(int max_w, long long lanes) {
-    static int sm_count[64] = {};      // per device, filled on first use
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
-        if (!sm_count[dev]) cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
-        if (sm_count[dev] > 0) sms = sm_count[dev];
-    }
-    for (int w = max_w; w > 1; w >>= 1)
-        if ((lanes + w - 1) / w >= (long long)sms * 9 / 10) return w;
-    return 1;
-}
 
 template <typename T2, int SIGN>
 __device__ __forceinline__ void f2_twiddles(T2* tw, const double2* __restrict__ twg, int P) {
@@ -150,199 +50,311 @@ __device__ __forceinline__ void f2_twiddles(T2* tw, const double2* __restrict__ 
     }
 }
 
-// X^[ky * P + kx][lane] of x1 = U_o x (sign * x[r][uo_index[(iy nx + ix) K + k]],
-// lane = r K + k), zero outside the lattice
-template <typename T2, int P, int W>
-__global__ void __launch_bounds__(f2_threads<W>())
-fft2d_fwd_kernel(T2* __restrict__ Xg, long long lanes, int nx, int ny, int K, int n_unique,
-                 const double2* __restrict__ twg, const double2* __restrict__ x, const float2* __restrict__ xf,
-                 const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn) {
+// X^[ky * px + kx][lane] of x1 = U_o x (sign * x[r][uo_index[(iy nx + ix) K + k]],
+// lane = r K + k), zero outside the lattice.  PC: px = py = PC at compile time,
+// 0: any grid.
+template <typename T2, int PC>
+__global__ void __launch_bounds__(512)
+fft2d_fwd_kernel(T2* __restrict__ Xg, long long lanes, F2Plan f, int K, int n_unique,
+                 const double2* __restrict__ twx, const double2* __restrict__ twy, const double2* __restrict__ x,
+                 const float2* __restrict__ xf, const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    T2* b1 = b0 + P * P * W;
-    T2* tw = b1 + P * P * W;
-    f2_twiddles<T2, -1>(tw, twg, P);
+    __shared__ int s_k[kF2MaxW], s_r[kF2MaxW];
+    T2* cur = reinterpret_cast<T2*>(smem_raw);
+    T2* nxt = cur + f.buf0;
+    T2* tx = nxt + f.buf1;
+    const int px = PC > 0 ? PC : f.x.P, py = PC > 0 ? PC : f.y.P;
+    T2* ty = PC > 0 ? tx : tx + px;
+    f2_twiddles<T2, -1>(tx, twx, px);
+    if (PC == 0) f2_twiddles<T2, -1>(ty, twy, py);
+    const int lw = f.lw, W = 1 << lw, wm = W - 1, nx = f.nx, ny = f.ny;
     const long long lane0 = (long long)blockIdx.x * W;
     const int wl = (int)min((long long)W, lanes - lane0);
-    const int nlx = ny * W;
-    // gather the cell rows into A[ix][iy * W + w]
-    for (int e = threadIdx.x; e < P * nlx; e += blockDim.x) {
-        const int ix = e / nlx, rem = e - ix * nlx, iy = rem / W, w = rem - iy * W;
-        T2 v = mk<T2>(0.0, 0.0);
-        if (ix < nx && w < wl) {
-            const long long L = lane0 + w;
-            const int r = (int)(L / K), k = (int)(L - (long long)r * K);
-            const size_t loc = ((size_t)iy * nx + ix) * K + k;
-            const size_t at = (size_t)r * n_unique + idx[loc];
-            if (xf) {
-                const float s = (float)sgn[loc];
-                const float2 xv = xf[at];
-                v = mk<T2>((double)(s * xv.x), (double)(s * xv.y));
-                if constexpr (sizeof(T2) == sizeof(float2)) v = make_float2(s * xv.x, s * xv.y);
-            } else {
-                const double s = (double)sgn[loc];
-                const double2 xv = x[at];
-                v = mk<T2>(s * xv.x, s * xv.y);
-            }
-        }
-        b0[e] = v;
+    if (threadIdx.x < W) {
+        const long long L = lane0 + (threadIdx.x < wl ? threadIdx.x : 0);
+        s_r[threadIdx.x] = (int)(L / K);
+        s_k[threadIdx.x] = (int)(L % K);
     }
     __syncthreads();
-    T2* r1 = F2Stages<T2, P, 0, 1, -1>::run(b0, b1, tw, nlx);
-    T2* o1 = r1 == b0 ? b1 : b0;
-    // columns: B[iy][kx * W + w], rows iy >= ny are the zero padding
-    const int nly = P * W;
-    for (int e = threadIdx.x; e < P * nly; e += blockDim.x) {
-        const int iy = e / nly, rem = e - iy * nly, kx = rem / W, w = rem - kx * W;
-        o1[e] = iy < ny ? r1[kx * nlx + iy * W + w] : mk<T2>(0.0, 0.0);
-    }
-    __syncthreads();
-    T2* r2 = F2Stages<T2, P, 0, 1, -1>::run(o1, r1, tw, nly);
-    for (int e = threadIdx.x; e < P * P * W; e += blockDim.x) {
-        const int bin = e / W, w = e - bin * W;
-        if (w < wl) Xg[(size_t)bin * lanes + lane0 + w] = r2[e];
-    }
+    const int sx = (ny | 1) << lw, sy = (py | 1) << lw;     // row strides
+    fft_stages_run<-1, PC, kF2MaxRad, T2>(f.x, f.lx, tx, [&](bool first, bool, auto&& go) {
+        T2* out = cur;
+        const T2* in = nxt;
+        go(
+            [&](int p, int l) {
+                if (!first) return in[p * sx + l];
+                T2 v = mk<T2>(0.0, 0.0);
+                const int w = l & wm, iy = l >> lw;
+                if (p < nx && w < wl) {
+                    const int loc = (iy * nx + p) * K + s_k[w];
+                    const size_t at = (size_t)s_r[w] * n_unique + idx[loc];
+                    if (xf) {
+                        const float sg = (float)sgn[loc];
+                        const float2 xv = xf[at];
+                        if constexpr (sizeof(T2) == sizeof(float2)) v = make_float2(sg * xv.x, sg * xv.y);
+                        else v = mk<T2>((double)(sg * xv.x), (double)(sg * xv.y));
+                    } else {
+                        const double sg = (double)sgn[loc];
+                        const double2 xv = x[at];
+                        v = mk<T2>(sg * xv.x, sg * xv.y);
+                    }
+                }
+                return v;
+            },
+            [&](int p, int l, T2 v) { out[p * sx + l] = v; });
+        __syncthreads();
+        T2* t = cur;
+        cur = nxt;
+        nxt = t;
+    });
+    // rows in `nxt`; rows iy >= ny are the zero padding
+    T2* Xo = Xg + lane0;
+    fft_stages_run<-1, PC, kF2MaxRad, T2>(f.y, f.ly, ty, [&](bool first, bool last, auto&& go) {
+        T2* out = cur;
+        const T2* in = nxt;
+        go(
+            [&](int p, int l) {
+                const int w = l & wm, kx = l >> lw;
+                if (first) return p < ny ? in[kx * sx + (p << lw) + w] : mk<T2>(0.0, 0.0);
+                return in[kx * sy + (p << lw) + w];
+            },
+            [&](int p, int l, T2 v) {
+                const int w = l & wm, kx = l >> lw;
+                if (!last) out[kx * sy + (p << lw) + w] = v;
+                else if (w < wl) Xo[(long long)(p * px + kx) * lanes + w] = v;
+            });
+        if (!last) __syncthreads();
+        T2* t = cur;
+        cur = nxt;
+        nxt = t;
+    });
 }
 
 // y1[r][iy nx + ix][k] = scale * IFFT2(Y^)[iy][ix] + sum_s mm[s][r][m][k] for
 // the lattice points (the crop of the circulant embedding)
-template <typename T2, int P, int W>
-__global__ void __launch_bounds__(f2_threads<W>())
-fft2d_inv_kernel(const T2* __restrict__ Yg, long long lanes, int nx, int ny, int K, int M, int R,
-                 int nsplit, double scale, const double2* __restrict__ twg, const T2* __restrict__ mm,
+template <typename T2, int PC>
+__global__ void __launch_bounds__(512)
+fft2d_inv_kernel(const T2* __restrict__ Yg, long long lanes, F2Plan f, int K, int M, int R, int nsplit, double scale,
+                 const double2* __restrict__ twx, const double2* __restrict__ twy, const T2* __restrict__ mm,
                  T2* __restrict__ y1) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    T2* b1 = b0 + P * P * W;
-    T2* tw = b1 + P * P * W;
-    f2_twiddles<T2, +1>(tw, twg, P);
+    __shared__ int s_k[kF2MaxW], s_r[kF2MaxW];
+    T2* cur = reinterpret_cast<T2*>(smem_raw);
+    T2* nxt = cur + f.buf0;
+    T2* tx = nxt + f.buf1;
+    const int px = PC > 0 ? PC : f.x.P, py = PC > 0 ? PC : f.y.P;
+    T2* ty = PC > 0 ? tx : tx + px;
+    f2_twiddles<T2, +1>(tx, twx, px);
+    if (PC == 0) f2_twiddles<T2, +1>(ty, twy, py);
+    const int lw = f.lw, W = 1 << lw, wm = W - 1, nx = f.nx, ny = f.ny;
     const long long lane0 = (long long)blockIdx.x * W;
     const int wl = (int)min((long long)W, lanes - lane0);
-    const int nly = P * W;
-    for (int e = threadIdx.x; e < P * P * W; e += blockDim.x) {
-        const int bin = e / W, w = e - bin * W;
-        b0[e] = w < wl ? Yg[(size_t)bin * lanes + lane0 + w] : mk<T2>(0.0, 0.0);
+    if (threadIdx.x < W) {
+        const long long L = lane0 + (threadIdx.x < wl ? threadIdx.x : 0);
+        s_r[threadIdx.x] = (int)(L / K);
+        s_k[threadIdx.x] = (int)(L % K);
     }
     __syncthreads();
-    T2* r1 = F2Stages<T2, P, 0, 1, +1>::run(b0, b1, tw, nly);
-    T2* o1 = r1 == b0 ? b1 : b0;
-    // rows kept (iy < ny) into A[kx][iy * W + w]
-    const int nlx = ny * W;
-    for (int e = threadIdx.x; e < P * nlx; e += blockDim.x) {
-        const int kx = e / nlx, rem = e - kx * nlx, iy = rem / W, w = rem - iy * W;
-        o1[e] = r1[iy * nly + kx * W + w];
-    }
-    __syncthreads();
-    T2* r2 = F2Stages<T2, P, 0, 1, +1>::run(o1, r1, tw, nlx);
-    using S = decltype(r2[0].x);
+    const int sx = (ny | 1) << lw, sy = (py | 1) << lw;
+    const T2* Yi = Yg + lane0;
+    fft_stages_run<+1, PC, kF2MaxRad, T2>(f.y, f.ly, ty, [&](bool first, bool last, auto&& go) {
+        T2* out = cur;
+        const T2* in = nxt;
+        go(
+            [&](int p, int l) {
+                const int w = l & wm, kx = l >> lw;
+                if (!first) return in[kx * sy + (p << lw) + w];
+                return w < wl ? Yi[(long long)(p * px + kx) * lanes + w] : mk<T2>(0.0, 0.0);
+            },
+            [&](int p, int l, T2 v) {
+                const int w = l & wm, kx = l >> lw;
+                if (!last) out[kx * sy + (p << lw) + w] = v;
+                else if (p < ny) out[kx * sx + (p << lw) + w] = v;      // rows kept
+            });
+        __syncthreads();
+        T2* t = cur;
+        cur = nxt;
+        nxt = t;
+    });
+    using S = typename Real<T2>::type;
     const S sc = (S)scale;
-    for (int e = threadIdx.x; e < nx * nlx; e += blockDim.x) {
-        const int ix = e / nlx, rem = e - ix * nlx, iy = rem / W, w = rem - iy * W;
-        if (w >= wl) continue;
-        const long long L = lane0 + w;
-        const int r = (int)(L / K), k = (int)(L - (long long)r * K);
-        const size_t m = (size_t)iy * nx + ix;
-        const T2 v = r2[e];
-        S ax = v.x * sc, ay = v.y * sc;
-        for (int s = 0; s < nsplit; ++s) {
-            const T2 z = mm[(((size_t)s * R + r) * M + m) * K + k];
-            ax += z.x;
-            ay += z.y;
-        }
-        T2 o;
-        o.x = ax;
-        o.y = ay;
-        y1[((size_t)r * M + m) * K + k] = o;
+    const size_t split = (size_t)R * M * K;
+    fft_stages_run<+1, PC, kF2MaxRad, T2>(f.x, f.lx, tx, [&](bool, bool last, auto&& go) {
+        T2* out = cur;
+        const T2* in = nxt;
+        go([&](int p, int l) { return in[p * sx + l]; },
+           [&](int p, int l, T2 v) {
+               if (!last) {
+                   out[p * sx + l] = v;
+                   return;
+               }
+               const int w = l & wm, iy = l >> lw;
+               if (p >= nx || w >= wl) return;
+               const size_t at = ((size_t)s_r[w] * M + iy * nx + p) * K + s_k[w];
+               T2 o;
+               o.x = v.x * sc;
+               o.y = v.y * sc;
+               // all partials' loads in flight together
+               T2 z[kF2MaxSplit];
+#pragma unroll
+               for (int q = 0; q < kF2MaxSplit; ++q)
+                   if (q < nsplit) z[q] = mm[at + q * split];
+#pragma unroll
+               for (int q = 0; q < kF2MaxSplit; ++q)
+                   if (q < nsplit) o = cadd(o, z[q]);
+               y1[at] = o;
+           });
+        if (!last) __syncthreads();
+        T2* t = cur;
+        cur = nxt;
+        nxt = t;
+    });
+}
+
+int sm_count() {
+    static int count[64] = {};      // per device, filled on first use
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    if (!count[dev]) cudaDeviceGetAttribute(&count[dev], cudaDevAttrMultiProcessorCount, dev);
+    return count[dev] > 0 ? count[dev] : 152;
+}
+
+// shared bytes of a plan of W = 2^lw lanes, and the buffers' sizes: the stages
+// write the two buffers in turn (forward: x rows, then columns; inverse:
+// columns, then rows), the last stage writes global memory
+template <typename T2>
+size_t f2_layout(F2Plan& f, int px, int py, bool inverse) {
+    const int W = 1 << f.lw;
+    const int sx = px * ((f.ny | 1) * W), sy = px * ((py | 1) * W);
+    int size[2] = {0, 0}, at = 0;
+    auto write = [&](int n) {
+        size[at] = std::max(size[at], n);
+        at ^= 1;
+    };
+    if (!inverse) {
+        for (int s = 0; s < f.x.n; ++s) write(sx);
+        for (int s = 0; s + 1 < f.y.n; ++s) write(sy);
+    } else {
+        for (int s = 0; s + 1 < f.y.n; ++s) write(sy);
+        write(sx);
+        for (int s = 0; s + 1 < f.x.n; ++s) write(sx);
     }
+    f.buf0 = size[0];
+    f.buf1 = size[1];
+    f.lx.set((uint32_t)(f.ny * W));
+    f.ly.set((uint32_t)(px * W));
+    return (size_t)(f.buf0 + f.buf1 + px + py) * sizeof(T2);
 }
 
-template <typename T2, int P, int W>
-int f2_fwd_w(T2* Xg, long long lanes, int nx, int ny, int K, int n_unique, const double2* tw, const double2* x,
-             const float2* xf, const int32_t* idx, const int8_t* sgn, cudaStream_t st) {
-    constexpr size_t smem = f2_smem<T2, P, W>();
-    EMS_TRY(set_smem_once(fft2d_fwd_kernel<T2, P, W>, smem));
-    fft2d_fwd_kernel<T2, P, W><<<(unsigned)((lanes + W - 1) / W), f2_threads<W>(), smem, st>>>(
-        Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn);
-    EMS_CUDA(cudaGetLastError());
+// square grids with their own kernels
+#define EMS_F2_SIZES(X) X(5) X(8) X(15) X(16) X(24) X(32) X(40) X(48) X(64)
+
+
+// lanes per CTA: 32 bytes of them (a whole sector per bin), halved while that
+// leaves SMs without a CTA
+int f2_pick_lanes(int max_lw, long long lanes) {
+    const int sms = sm_count();
+    for (int lw = max_lw; lw > 0; --lw)
+        if (((lanes - 1) >> lw) + 1 >= (long long)sms * 9 / 10) return lw;
+    return 0;
+}
+
+template <typename T2>
+constexpr int f2_full_lw() { return sizeof(T2) == sizeof(float2) ? 2 : 1; }
+
+template <typename T2>
+int f2_plan(F2Plan& f, int px, int py, int nx, int ny, long long lanes, bool inverse, size_t& smem, int& threads) {
+    if (!fft_stages(px, kF2MaxRad, f.x) || !fft_stages(py, kF2MaxRad, f.y)) {
+        set_error("fused 2-D FFT: no plan for %d x %d", px, py);
+        return EMSURF_EINVAL;
+    }
+    f.nx = nx;
+    f.ny = ny;
+    f.lw = f2_pick_lanes(f2_full_lw<T2>(), lanes);
+    smem = f2_layout<T2>(f, px, py, inverse);
+    // measured (forward and inverse, average): float, 16 x 16 boxes, one rhs (144
+    // CTAs of 4 lanes): 512 threads 10.2 us, 384 11.6, 256 12.4; 24 x 24 boxes, 32
+    // rhs (4608 CTAs): 384 threads 278 us, 512 286, 256 304; double is bound by
+    // the FP64 rate and small blocks even out its stages (12 x 9 boxes, 6 rhs:
+    // 128 threads 100 us, 256 110, 384 144)
+    const long long ctas = ((lanes - 1) >> f.lw) + 1;
+    const int sms = sm_count();
+    if (sizeof(T2) == sizeof(float2)) threads = ctas <= sms ? 512 : 384;
+    else threads = ctas <= 2 * sms ? 256 : 128;
     return EMSURF_OK;
-}
-
-template <typename T2, int P, int W>
-int f2_inv_w(const T2* Yg, long long lanes, int nx, int ny, int K, int M, int R, int nsplit, double scale,
-             const double2* tw, const T2* mm, T2* y1, cudaStream_t st) {
-    constexpr size_t smem = f2_smem<T2, P, W>();
-    EMS_TRY(set_smem_once(fft2d_inv_kernel<T2, P, W>, smem));
-    fft2d_inv_kernel<T2, P, W><<<(unsigned)((lanes + W - 1) / W), f2_threads<W>(), smem, st>>>(
-        Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1);
-    EMS_CUDA(cudaGetLastError());
-    return EMSURF_OK;
-}
-
-template <typename T2, int P>
-int f2_fwd(T2* Xg, long long lanes, int nx, int ny, int K, int n_unique, const double2* tw, const double2* x,
-           const float2* xf, const int32_t* idx, const int8_t* sgn, cudaStream_t st) {
-    constexpr int MW = f2_max_lanes<T2, P>();
-    const int w = f2_pick_lanes(MW, lanes);
-    if constexpr (MW >= 8) if (w == 8) return f2_fwd_w<T2, P, 8>(Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn, st);
-    if constexpr (MW >= 4) if (w == 4) return f2_fwd_w<T2, P, 4>(Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn, st);
-    if constexpr (MW >= 2) if (w == 2) return f2_fwd_w<T2, P, 2>(Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn, st);
-    return f2_fwd_w<T2, P, 1>(Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn, st);
-}
-
-template <typename T2, int P>
-int f2_inv(const T2* Yg, long long lanes, int nx, int ny, int K, int M, int R, int nsplit, double scale,
-           const double2* tw, const T2* mm, T2* y1, cudaStream_t st) {
-    constexpr int MW = f2_max_lanes<T2, P>();
-    const int w = f2_pick_lanes(MW, lanes);
-    if constexpr (MW >= 8) if (w == 8) return f2_inv_w<T2, P, 8>(Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1, st);
-    if constexpr (MW >= 4) if (w == 4) return f2_inv_w<T2, P, 4>(Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1, st);
-    if constexpr (MW >= 2) if (w == 2) return f2_inv_w<T2, P, 2>(Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1, st);
-    return f2_inv_w<T2, P, 1>(Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1, st);
 }
 
 }  // namespace
 
-bool fft2d_fused_ok(int px, int py) {
-    if (px != py) return false;
-    switch (px) {
-        case 5: case 8: case 15: case 16: case 24: case 32: case 48: case 64: return true;
-        default: return false;
-    }
-}
-
-#define EMS_F2_SIZES(X) X(5) X(8) X(15) X(16) X(24) X(32) X(48) X(64)
-
 template <typename T2>
-int fft2d_forward(T2* Xg, int P, long long lanes, int nx, int ny, int K, int n_unique, const double2* tw,
-                  const double2* x, const float2* xf, const int32_t* idx, const int8_t* sgn, cudaStream_t st) {
-    switch (P) {
-#define EMS_F2_CASE(N) \
-    case N: return f2_fwd<T2, N>(Xg, lanes, nx, ny, K, n_unique, tw, x, xf, idx, sgn, st);
-        EMS_F2_SIZES(EMS_F2_CASE)
-#undef EMS_F2_CASE
-        default: set_error("fused 2-D FFT: no kernel for %d x %d", P, P); return EMSURF_EINVAL;
-    }
+bool fft2d_fused_ok(int px, int py, int nx, int ny) {
+    F2Plan f;
+    if (!fft_stages(px, kF2MaxRad, f.x) || !fft_stages(py, kF2MaxRad, f.y)) return false;
+    if (f.x.n > 2 || f.y.n > 2) return false;
+    f.nx = nx;
+    f.ny = ny;
+    f.lw = f2_full_lw<T2>();
+    return std::max(f2_layout<T2>(f, px, py, false), f2_layout<T2>(f, px, py, true)) <= kF2MaxSmem;
 }
 
 template <typename T2>
-int fft2d_inverse(const T2* Yg, int P, long long lanes, int nx, int ny, int K, int M, int R, int nsplit,
-                  double scale, const double2* tw, const T2* mm, T2* y1, cudaStream_t st) {
-    switch (P) {
+int fft2d_forward(T2* Xg, int px, int py, long long lanes, int nx, int ny, int K, int n_unique, const double2* twx,
+                  const double2* twy, const double2* x, const float2* xf, const int32_t* idx, const int8_t* sgn,
+                  cudaStream_t st) {
+    F2Plan f;
+    size_t smem;
+    int threads;
+    EMS_TRY(f2_plan<T2>(f, px, py, nx, ny, lanes, false, smem, threads));
+    auto go = [&](auto kern) -> int {
+        EMS_TRY(set_smem_once(kern, smem));
+        kern<<<(unsigned)(((lanes - 1) >> f.lw) + 1), threads, smem, st>>>(Xg, lanes, f, K, n_unique, twx, twy, x, xf,
+                                                                          idx, sgn);
+        EMS_CUDA(cudaGetLastError());
+        return EMSURF_OK;
+    };
+    if (px == py) switch (px) {
 #define EMS_F2_CASE(N) \
-    case N: return f2_inv<T2, N>(Yg, lanes, nx, ny, K, M, R, nsplit, scale, tw, mm, y1, st);
+    case N: return go(fft2d_fwd_kernel<T2, N>);
         EMS_F2_SIZES(EMS_F2_CASE)
 #undef EMS_F2_CASE
-        default: set_error("fused 2-D FFT: no kernel for %d x %d", P, P); return EMSURF_EINVAL;
+        default: break;
     }
+    return go(fft2d_fwd_kernel<T2, 0>);
 }
 
-template int fft2d_forward<float2>(float2*, int, long long, int, int, int, int, const double2*, const double2*,
-                                   const float2*, const int32_t*, const int8_t*, cudaStream_t);
-template int fft2d_forward<double2>(double2*, int, long long, int, int, int, int, const double2*,
+template <typename T2>
+int fft2d_inverse(const T2* Yg, int px, int py, long long lanes, int nx, int ny, int K, int M, int R, int nsplit,
+                  double scale, const double2* twx, const double2* twy, const T2* mm, T2* y1, cudaStream_t st) {
+    F2Plan f;
+    size_t smem;
+    int threads;
+    EMS_TRY(f2_plan<T2>(f, px, py, nx, ny, lanes, true, smem, threads));
+    auto go = [&](auto kern) -> int {
+        EMS_TRY(set_smem_once(kern, smem));
+        kern<<<(unsigned)(((lanes - 1) >> f.lw) + 1), threads, smem, st>>>(Yg, lanes, f, K, M, R, nsplit, scale, twx,
+                                                                          twy, mm, y1);
+        EMS_CUDA(cudaGetLastError());
+        return EMSURF_OK;
+    };
+    if (px == py) switch (px) {
+#define EMS_F2_CASE(N) \
+    case N: return go(fft2d_inv_kernel<T2, N>);
+        EMS_F2_SIZES(EMS_F2_CASE)
+#undef EMS_F2_CASE
+        default: break;
+    }
+    return go(fft2d_inv_kernel<T2, 0>);
+}
+
+template bool fft2d_fused_ok<float2>(int, int, int, int);
+template bool fft2d_fused_ok<double2>(int, int, int, int);
+template int fft2d_forward<float2>(float2*, int, int, long long, int, int, int, int, const double2*, const double2*,
+                                   const double2*, const float2*, const int32_t*, const int8_t*, cudaStream_t);
+template int fft2d_forward<double2>(double2*, int, int, long long, int, int, int, int, const double2*, const double2*,
                                     const double2*, const float2*, const int32_t*, const int8_t*, cudaStream_t);
-template int fft2d_inverse<float2>(const float2*, int, long long, int, int, int, int, int, int, double,
-                                   const double2*, const float2*, float2*, cudaStream_t);
-template int fft2d_inverse<double2>(const double2*, int, long long, int, int, int, int, int, int, double,
-                                    const double2*, const double2*, double2*, cudaStream_t);
+template int fft2d_inverse<float2>(const float2*, int, int, long long, int, int, int, int, int, int, double,
+                                   const double2*, const double2*, const float2*, float2*, cudaStream_t);
+template int fft2d_inverse<double2>(const double2*, int, int, long long, int, int, int, int, int, int, double,
+                                    const double2*, const double2*, const double2*, double2*, cudaStream_t);
 
 }  // namespace emsurf

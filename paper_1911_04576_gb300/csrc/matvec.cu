@@ -1980,10 +1980,10 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     // K1: x-pass over the cell rows iy < ny reading x1 = U_o x directly
     // (points ix >= nx are the zero padding), then the y-pass with rows
     // iy >= ny taken as zero
-    const bool fused = fft2d_fused_ok(px, py);
+    const bool fused = fft2d_fused_ok<T2>(px, py, h->nx, h->ny);
     if (fused) {
         // one launch: gather, both 1-D transforms, X^ stored
-        EMS_TRY(fft2d_forward<T2>(op.Xg, px, lanes, h->nx, h->ny, K, h->n_unique, h->plan_x.tw, x, xf,
+        EMS_TRY(fft2d_forward<T2>(op.Xg, px, py, lanes, h->nx, h->ny, K, h->n_unique, h->plan_x.tw, h->plan_y.tw, x, xf,
                                   h->d_uo_index, h->d_uo_sign, st));
     } else {
         EMS_TRY(fft_pass_gather<T2>(op.Xg, h->plan_x, lanes, h->ny, (long long)px * lanes, h->nx, x,
@@ -2240,8 +2240,8 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     prof_mark(h, ph_fft, true, st);
     // K3: inverse y-pass on all columns, inverse x-pass on the rows kept
     if (fused) {
-        EMS_TRY(fft2d_inverse<T2>(op.Yg, px, lanes, h->nx, h->ny, K, h->M, R, nsplit, 1.0 / (double)h->nbins,
-                                  h->plan_x.tw, op.Ymm, op.Y1, st));
+        EMS_TRY(fft2d_inverse<T2>(op.Yg, px, py, lanes, h->nx, h->ny, K, h->M, R, nsplit, 1.0 / (double)h->nbins,
+                                  h->plan_x.tw, h->plan_y.tw, op.Ymm, op.Y1, st));
     } else {
         EMS_TRY(fft_pass<T2>(op.Yg, h->plan_y, (long long)px * lanes, 1, 0, +1, st, py, h->ny));
         EMS_TRY(fft_pass_crop<T2>(op.Yg, h->plan_x, lanes, h->ny, (long long)px * lanes, h->nx, op.Ymm,
