@@ -939,9 +939,9 @@ def main():
                   "n_matvec": last["n_matvec"], "rel_residual": last["rel_residual"],
                   "converged": last["converged"]},
         "operator_arithmetic": {"fp32": "complex64 operator, FP32 arithmetic (inner GMRES)",
-                                "fp64_accuracy": "single-rhs FP64-operator products in double-single "
-                                                 "FP32 arithmetic (~48-bit products, scaled hi/lo "
-                                                 "planes); FP64 FFTs, residuals, orthogonalisation"},
+                                "fp64_accuracy": "FP64-operator products from exact base-256 digits "
+                                                 "of 55-bit integers on the tensor cores (FP64 "
+                                                 "accuracy); FP64 FFTs, residuals, orthogonalisation"},
         "fp64_preconditioned": {"solve_ms": round(t64p, 3), "iters": info64p[0]["iters"],
                                 "n_matvec": info64p[0]["n_matvec"],
                                 "converged": info64p[0]["converged"],

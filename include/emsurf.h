@@ -71,15 +71,14 @@ typedef struct emsurf_handle emsurf_handle;
  *  grid_px/py   FFT grid; 0 = smallest 2,3,5-smooth >= 2N-1; else >= 2N-1
  *               with no prime factor above 7 (EINVAL otherwise)
  *  max_rhs      largest nrhs later passed to matvec/solve (>= 1).  Handles
- *               holding the FP64 operator also keep its spectrum and the
- *               macromodels as FP32 hi/lo planes (same bytes) for the
- *               double-single FP64-accuracy kernels, when device_mem_budget
- *               leaves room.  Their operands are scaled by powers of two
- *               (the spectrum and the macromodels at create, each rhs of a
- *               product by its largest component) and the FP64 results
- *               scaled back, so FP32's exponent range limits only parts
- *               more than ~2^100 below the largest of their array (relative
- *               error per term a few 2^-48 of that largest).  The FP32
+ *               holding the FP64 operator keep its spectrum and the
+ *               macromodels as planes of base-256 digits (7 bytes per real
+ *               number) for the FP64-accuracy kernels, when
+ *               device_mem_budget leaves room.  The digits hold 55 bits
+ *               below the largest component of each matrix row and of each
+ *               vector (of a bin or a cell), products and sums of digits are
+ *               exact, and terms below 2^-50 of row times vector maximum are
+ *               left out.  The FP32
  *               operator (EMSURF_FP32, MIXED) stores complex64 values and
  *               needs table and macromodel entries inside FP32's range.
  *  tables_on_device  0: offset_L/K and macromodels are host pointers;
@@ -180,7 +179,7 @@ EMSURF_API int emsurf_create(const emsurf_problem* problem, emsurf_handle** out)
 
 /* emsurf_create for a lattice whose Fourier-domain blocks another handle
  * already holds (no counterpart in the paper; used by the serving cache):
- * the new handle reads `share`'s spectra (FP64 or its double-single planes,
+ * the new handle reads `share`'s spectra (FP64 or its digit planes,
  * FP32, tensor-core planes) instead of building its own, and builds only
  * what depends on the problem's macromodels and type map (macromodel
  * copies, work space, preconditioner).  offset_L/offset_K are not read

@@ -238,7 +238,10 @@ int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* 
         EMS_TRY(derive_fp32_operator(h, p, share));
         h->have32 = true;
     }
-    if (h->have64) EMS_TRY(build_ds_planes(h, share));
+    if (h->have64) {
+        EMS_TRY(slices_build(h, share));
+        EMS_TRY(operator_work<double2>(h, h->op64, h->sl_Z ? 1 : kMmSplit));
+    }
     if (p->tensor_cores && h->have32 && h->E >= 64) EMS_TRY(tc_build(h, share));
     if (share) {
         h->near_L = share->near_L;
@@ -254,12 +257,13 @@ int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* 
         EMS_TRY(pc_build(h, p));
     }
     EMS_CUDA(cudaStreamSynchronize(h->setup_stream));
-    // with the double-single planes every FP64-accuracy bin multiply reads
-    // them (one rhs and several), so the complex128 spectrum is not needed
-    // after create: its bytes (those of the planes) are given back
-    if (h->have64 && h->ds_planes && h->op64.Bhat) {
-        dev_free(h, h->op64.Bhat, (size_t)h->nbins * 2 * (size_t)h->E * h->E * sizeof(double2));
+    // with the digit planes no FP64-accuracy product reads the complex128
+    // spectrum: it is given back, and the vectors' digits take their work space
+    if (h->sl_A) {
+        if (h->op64.Bhat && !share)
+            dev_free(h, h->op64.Bhat, (size_t)h->nbins * 2 * (size_t)h->E * h->E * sizeof(double2));
         h->op64.Bhat = nullptr;
+        EMS_TRY(slices_work(h));
     }
     return EMSURF_OK;
 }
@@ -309,8 +313,6 @@ int clear_wait_error(emsurf_handle* h) {
     EMS_CUDA(cudaDeviceSynchronize());
     EMS_CUDA(cudaMemset(h->d_err, 0, sizeof(int)));
     if (h->d_pair_cnt) EMS_CUDA(cudaMemset(h->d_pair_cnt, 0, h->pair_cnt_bytes));
-    if (h->d_ds_max) EMS_CUDA(cudaMemset(h->d_ds_max, 0, sizeof(unsigned long long) * std::max(1, h->max_rhs)));
-    if (h->d_ds_cnt) EMS_CUDA(cudaMemset(h->d_ds_cnt, 0, sizeof(unsigned) * std::max(1, h->max_rhs)));
     if (h->d_grid_bar) EMS_CUDA(cudaMemset(h->d_grid_bar, 0, 2 * sizeof(unsigned)));
     return EMSURF_OK;
 }

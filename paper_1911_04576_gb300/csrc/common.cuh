@@ -12,6 +12,7 @@
 namespace emsurf {
 
 constexpr int kMmGroup = 4;   // cells of one type per macromodel CTA
+constexpr int kMmSplit = 8;   // k' chunks of the SIMT macromodel products
 
 // ---------------------------------------------------------------- errors
 void set_error(const char* fmt, ...);
@@ -167,7 +168,7 @@ struct Operator {
     T2* Zt = nullptr;
     T2* Xg = nullptr;      // work grid [bins][R][2E] (forward)
     T2* Yg = nullptr;      // work grid [bins][R][2E] (inverse)
-    T2* Ymm = nullptr;     // macromodel partial outputs [split][R][M][2E]
+    T2* Ymm = nullptr;     // macromodel partial outputs [split][R][M][2E] (one split with digit planes)
     T2* Y1 = nullptr;      // local-space product [R][M][2E]
     T2 coef[4];
 };
@@ -218,19 +219,18 @@ struct emsurf_handle {
     int32_t* d_orb_bin = nullptr;     // [nst][orb_G] bin of each slot (-1: none)
     int32_t* d_orb_elem = nullptr;    // [nst][orb_G] its group element
     uint32_t* d_orb_perm = nullptr;   // [orb_G][2E] signed index of T_e
-    // FP64-accuracy single-rhs bin multiply from FP32 hi/lo pairs: spectrum
-    // planes [bin][hi, lo][op][j][i] and the split X^ [bin][hi, lo][2E]
-    float2* ds_planes = nullptr;
-    float2* ds_x = nullptr;
-    float2* ds_zt = nullptr;          // the macromodels as hi/lo planes [t][hi, lo][k'][k]
-    // powers of two that keep the double-single operands inside FP32's
-    // exponent range: [0] spectrum planes, [1] macromodel planes (both were
-    // split from the FP64 values times these), [2 + r] rhs r of the current
-    // product (from max |x_r|); the kernels divide their FP64 outputs back
-    double* d_ds_scale = nullptr;
-    double h_ds_scale0 = 1.0;         // the spectrum planes' scale (host copy)
-    unsigned long long* d_ds_max = nullptr;   // per-rhs running maxima of the scale kernel (kept at 0)
-    unsigned* d_ds_cnt = nullptr;             // its per-rhs block arrival counters (kept at 0)
+    // FP64-accuracy products from exact integer digits (slices.cu): digit planes
+    // and row scales of the spectrum and the macromodels, work space of the
+    // vectors' digits, macromodel entries (type, first column) per rhs count
+    unsigned char* sl_A = nullptr;
+    double* sl_rs = nullptr;
+    unsigned char* sl_Z = nullptr;
+    double* sl_zrs = nullptr;
+    unsigned char *sl_X = nullptr, *sl_Xc = nullptr;
+    double *sl_xs = nullptr, *sl_xcs = nullptr;
+    int sl_bins = 0;                  // bins whose vectors' digits are held at a time
+    std::vector<void*> sl_ent;
+    std::vector<int> sl_nent;
     int pair_grid = 0;                // CTAs of the pair kernel (equal slab ranges)
     float2* d_pair_part = nullptr;    // partial row sums of straddling bins [cta][2][2E]
     int* d_pair_cnt = nullptr;        // arrival counters [stored bin][row warp]
@@ -352,6 +352,9 @@ int tabulate_blocks(const MeshView& test, const MeshView& src, const double* shi
 template <typename T2>
 int build_operator(emsurf_handle* h, Operator<T2>& op, const emsurf_problem* pr,
                    const Operator<T2>* share = nullptr);
+// work grids and macromodel partials of an operator
+template <typename T2>
+int operator_work(emsurf_handle* h, Operator<T2>& op, int mm_split);
 // share: a handle of the same lattice whose Fourier-domain blocks are reused
 int derive_fp32_operator(emsurf_handle* h, const emsurf_problem* pr, const emsurf_handle* share = nullptr);
 // mirror orbits of the spectrum's bins (setup.cpp): the bin of group element
@@ -366,7 +369,13 @@ void mirror_orbits(int px, int py, int G, std::vector<int32_t>& rep, std::vector
                    std::vector<int32_t>& oelem);
 int adopt_fp32_form(emsurf_handle* h, const emsurf_handle* share);
 int clear_wait_error(emsurf_handle* h);
-int build_ds_planes(emsurf_handle* h, const emsurf_handle* share = nullptr);
+// exact-digit products (slices.cu)
+size_t slice_plane_bytes(size_t mats, int rows, int n);
+int slices_build(emsurf_handle* h, const emsurf_handle* share = nullptr);
+int slices_work(emsurf_handle* h);
+int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st);
+int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
+                    cudaStream_t st);
 int grid_barrier_selftest(emsurf_handle* h, long long limit, cudaStream_t st);
 template <typename T2>
 int apply_operator(emsurf_handle* h, Operator<T2>& op, const double2* x, double2* y, int nrhs,

@@ -22,8 +22,6 @@ namespace emsurf {
 
 namespace {
 
-constexpr int kMmSplit = 8;   // k' chunks of the macromodel product
-
 // ------------------------------------------------ placement of the tables
 // Bhat[bin(d)][op][j][i] = table_op(d)[i][j] for one chunk of offsets;
 // stage holds [nchunk][2][E][E] complex128 (row-major i, j).
@@ -366,294 +364,6 @@ __global__ void binmul_tma_kernel(const float2* __restrict__ Bhat, const float2*
 size_t binmul_tma_smem(int E) {
     return (size_t)kBmStages * 2 * kBmJB * E * sizeof(float2) + 4ull * E * sizeof(float2) +
            2ull * kBmStages * sizeof(uint64_t);
-}
-
-// ------------------------------------------------ K2, FP64 accuracy from FP32 arithmetic, one rhs
-// The FP64 bin multiply is bound by this part's FP64 rate (~1/60 of FP32).
-// Here every FP64 value v is held as a pair of floats, hi = rn(v) and
-// lo = rn(v - hi) (|v - hi - lo| <= 2^-48 |v|), and each complex product is
-// accumulated in double-single arithmetic: the rounding error of hi*hi is
-// recovered exactly with an FMA, the cross terms hi*lo + lo*hi are added to
-// it, and the partial sums are pairs (s, c) updated with Knuth's TwoSum, so
-// each product term carries a relative error of a few 2^-48 (the lo*lo term,
-// ~2^-48, is dropped).  The row sums are turned into FP64 at the end.  The
-// spectrum planes hold the same bytes as the FP64 spectrum; one thread per
-// test row as in binmul_tma_kernel, kDsJB-column slabs (hi and lo of L^ and
-// K^) in a kDsStages-deep ring fed by bulk copies.
-constexpr int kDsJB = 6;
-constexpr int kDsStages = 3;
-
-// (hi, lo) += (ah + al)(bh + bl); no operation is contracted or reassociated
-__device__ __forceinline__ void ds_mac(float& hi, float& lo, float ah, float al, float bh, float bl) {
-    const float p = __fmul_rn(ah, bh);
-    float e = __fmaf_rn(ah, bh, -p);           // ah bh - p, exactly
-    e = __fmaf_rn(ah, bl, e);
-    e = __fmaf_rn(al, bh, e);
-    const float s = __fadd_rn(hi, p);          // TwoSum(hi, p) = s + t exactly
-    const float bb = __fsub_rn(s, hi);
-    const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    lo = __fadd_rn(lo, __fadd_rn(t, e));
-    hi = s;
-}
-
-struct DsC {   // complex double-single accumulator
-    float rh, rl, ih, il;
-};
-__device__ __forceinline__ void ds_cmac(DsC& a, float2 xh, float2 xl, float2 bh, float2 bl) {
-    ds_mac(a.rh, a.rl, xh.x, xl.x, bh.x, bl.x);
-    ds_mac(a.rh, a.rl, -xh.y, -xl.y, bh.y, bl.y);
-    ds_mac(a.ih, a.il, xh.x, xl.x, bh.y, bl.y);
-    ds_mac(a.ih, a.il, xh.y, xl.y, bh.x, bl.x);
-}
-__device__ __forceinline__ double2 ds_value(const DsC& a) {
-    return make_double2((double)a.rh + (double)a.rl, (double)a.ih + (double)a.il);
-}
-
-// out[b][0][r] = rn(s v), out[b][1][r] = rn(s v - out[b][0][r]) for v = in[b][r],
-// blocks b of `chunk` complex values; s = *scale (a power of two, exact), or 1
-__global__ void split_hilo_kernel(float2* __restrict__ out, const double2* __restrict__ in, size_t chunk,
-                                  size_t total, const double* __restrict__ scale) {
-    const double sc = scale ? *scale : 1.0;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = e / chunk, r = e - b * chunk;
-        const double2 v = make_double2(sc * in[e].x, sc * in[e].y);
-        const float2 hi = make_float2((float)v.x, (float)v.y);
-        const float2 lo = make_float2((float)(v.x - (double)hi.x), (float)(v.y - (double)hi.y));
-        out[b * 2 * chunk + r] = hi;
-        out[b * 2 * chunk + chunk + r] = lo;
-    }
-}
-
-// scale[r] = 2^-e with 2^(e-1) <= max over the r-th vector of |re|, |im| < 2^e
-// (1 when the vector is zero or not finite): after it the vector's largest
-// component lies in [0.5, 1), far from FP32 overflow, and FP32 subnormals only
-// touch parts below 2^-100 of the largest.  Grid (blocks, R): every block
-// folds its maximum into maxbits[r] (the bit patterns of non-negative doubles
-// order like the values); the last block of rhs r to arrive (arrival counter)
-// writes the scale and resets maxbits[r] and count[r] for the next product.
-__global__ void __launch_bounds__(256) pow2_scale_kernel(const double2* __restrict__ v, size_t len,
-                                                         unsigned long long* __restrict__ maxbits,
-                                                         unsigned* __restrict__ count, double* __restrict__ scale) {
-    __shared__ double s_m[256];
-    __shared__ bool s_last;
-    const int r = blockIdx.y;
-    const double2* b = v + (size_t)r * len;
-    double m = 0.0;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < len; e += (size_t)gridDim.x * blockDim.x)
-        m = fmax(m, fmax(fabs(b[e].x), fabs(b[e].y)));
-    s_m[threadIdx.x] = m;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) s_m[threadIdx.x] = fmax(s_m[threadIdx.x], s_m[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        atomicMax(&maxbits[r], (unsigned long long)__double_as_longlong(s_m[0]));
-        __threadfence();
-        s_last = atomicAdd(&count[r], 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last && threadIdx.x == 0) {
-        __threadfence();
-        const double mx = __longlong_as_double((long long)atomicExch(&maxbits[r], 0ull));
-        count[r] = 0u;
-        scale[r] = (mx > 0.0 && mx <= 1.7e308) ? ldexp(1.0, -(ilogb(mx) + 1)) : 1.0;
-    }
-}
-
-// grid-wide variant for one large array: per-CTA maxima in part[], then one CTA
-__global__ void __launch_bounds__(256) absmax_part_kernel(const double2* __restrict__ v, size_t n,
-                                                          double* __restrict__ part) {
-    __shared__ double s_m[256];
-    double m = 0.0;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-        m = fmax(m, fmax(fabs(v[e].x), fabs(v[e].y)));
-    s_m[threadIdx.x] = m;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) s_m[threadIdx.x] = fmax(s_m[threadIdx.x], s_m[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = s_m[0];
-}
-
-// planes: [bin][hi, lo][op][j][i] float2; xs: [bin][hi, lo][2E]; Yh: [bin][2E] FP64
-__global__ void binmul_ds_kernel(const float2* __restrict__ planes, const float2* __restrict__ xs,
-                                 double2* __restrict__ Yh, int E, int nbins, double2 ca, double2 cb,
-                                 double2 cg, double2 cd, int* __restrict__ err,
-                                 const double* __restrict__ scale) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int stage_elems = 4 * kDsJB * E;      // [hi, lo][L, K][kDsJB][E]
-    float2* sbuf = reinterpret_cast<float2*>(smem_raw);
-    float2* xbuf = sbuf + (size_t)kDsStages * stage_elems;      // [2 buffers][hi, lo][2E]
-    uint64_t* full = reinterpret_cast<uint64_t*>(xbuf + 8 * E);
-    uint64_t* empty = full + kDsStages;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ncw = (E + 31) / 32;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kDsStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], ncw);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    const int nloc = (nbins - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int nj = (E + kDsJB - 1) / kDsJB;
-    const long long total = (long long)nloc * nj;
-    const size_t EE = (size_t)E * E;
-    if (warp == 0) {
-        if (lane != 0) return;
-        const uint64_t pol = l2_evict_first();
-        const uint32_t bytes_x = (uint32_t)(4 * E * sizeof(float2));
-        int s = 0, jb = 0, t = 0;
-        uint32_t ph = 0;
-        long long issued = 0;
-        bool ok = true;
-        for (long long q = 0; q < total; ++q) {
-            if (q >= kDsStages && !mbar_wait(&empty[s], ph ^ 1u)) {
-                ok = false;
-                break;
-            }
-            const int bin = (int)blockIdx.x + t * (int)gridDim.x;
-            const int j0 = jb * kDsJB, jn = min(kDsJB, E - j0);
-            const uint32_t bytes_op = (uint32_t)(jn * E * sizeof(float2));
-            mbar_expect_tx(&full[s], 4 * bytes_op + (jb == 0 ? bytes_x : 0u));
-            float2* dst = sbuf + (size_t)s * stage_elems;
-            for (int pl = 0; pl < 2; ++pl)
-                for (int o = 0; o < 2; ++o)
-                    bulk_g2s_hint(dst + (pl * 2 + o) * kDsJB * E,
-                                  planes + (((size_t)bin * 2 + pl) * 2 + o) * EE + (size_t)j0 * E, bytes_op,
-                                  &full[s], pol);
-            if (jb == 0) bulk_g2s(xbuf + (t & 1) * 4 * E, xs + (size_t)bin * 4 * E, bytes_x, &full[s]);
-            issued = q + 1;
-            if (++s == kDsStages) { s = 0; ph ^= 1u; }
-            if (++jb == nj) { jb = 0; ++t; }
-        }
-        if (!ok) {
-            atomicExch(err, 1);
-            for (long long u = (issued > kDsStages ? issued - kDsStages : 0); u < issued; ++u)
-                mbar_wait(&full[u % kDsStages], (uint32_t)((u / kDsStages) & 1));
-        }
-        return;
-    }
-    const int i = (warp - 1) * 32 + lane;
-    DsC lj{0.f, 0.f, 0.f, 0.f}, lm = lj, kj = lj, km = lj;
-    int s = 0, jb = 0, t = 0;
-    uint32_t ph = 0;
-    for (long long q = 0; q < total; ++q) {
-        if (!mbar_wait(&full[s], ph)) {
-            atomicExch(err, 1);
-            return;
-        }
-        const float2* S = sbuf + (size_t)s * stage_elems;
-        const float2* X = xbuf + (t & 1) * 4 * E;       // [hi, lo][2E]
-        const int j0 = jb * kDsJB, jn = min(kDsJB, E - j0);
-        if (i < E) {
-#pragma unroll
-            for (int jj = 0; jj < kDsJB; ++jj) {
-                if (jj < jn) {
-                    const float2 lh = S[(0 * kDsJB + jj) * E + i], kh = S[(1 * kDsJB + jj) * E + i];
-                    const float2 ll = S[(2 * kDsJB + jj) * E + i], kl = S[(3 * kDsJB + jj) * E + i];
-                    const float2 xjh = X[j0 + jj], xmh = X[E + j0 + jj];
-                    const float2 xjl = X[2 * E + j0 + jj], xml = X[3 * E + j0 + jj];
-                    ds_cmac(lj, xjh, xjl, lh, ll);
-                    ds_cmac(lm, xmh, xml, lh, ll);
-                    ds_cmac(kj, xjh, xjl, kh, kl);
-                    ds_cmac(km, xmh, xml, kh, kl);
-                }
-            }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);
-        if (jb == nj - 1) {
-            if (i < E) {
-                const int bin = (int)blockIdx.x + t * (int)gridDim.x;
-                double2* Y = Yh + (size_t)bin * 2 * E;
-                const double u = 1.0 / (scale[0] * scale[2]);       // exact: powers of two
-                const double2 yj = cadd(cmul(ca, ds_value(lj)), cmul(cb, ds_value(km)));
-                const double2 ym = cadd(cmul(cg, ds_value(kj)), cmul(cd, ds_value(lm)));
-                Y[i] = make_double2(u * yj.x, u * yj.y);
-                Y[E + i] = make_double2(u * ym.x, u * ym.y);
-            }
-            lj = lm = kj = km = DsC{0.f, 0.f, 0.f, 0.f};
-        }
-        if (++s == kDsStages) { s = 0; ph ^= 1u; }
-        if (++jb == nj) { jb = 0; ++t; }
-    }
-}
-
-// Several rhs: RB of them per pass share each load of the hi/lo planes (the
-// register-blocked form of binmul_kernel); X^ is split into hi/lo while it is
-// staged in shared memory.  Compute-bound (about 60 FP32 operations per
-// complex multiply-add), so the planes are streamed once per RB rhs.
-template <int RB>
-__global__ void binmul_ds_multi_kernel(const float2* __restrict__ planes, const double2* __restrict__ Xh,
-                                       double2* __restrict__ Yh, int E, int nbins, int R, int r0,
-                                       double2 ca, double2 cb, double2 cg, double2 cd,
-                                       const double* __restrict__ scale) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* xh = reinterpret_cast<float2*>(smem_raw);   // [RB][2E] hi
-    float2* xl = xh + (size_t)RB * 2 * E;               // [RB][2E] lo
-    const int K = 2 * E;
-    const size_t EE = (size_t)E * E;
-    for (int bin = blockIdx.x; bin < nbins; bin += gridDim.x) {
-        __syncthreads();
-        const double2* X = Xh + (size_t)bin * R * K;
-        for (int e = threadIdx.x; e < RB * K; e += blockDim.x) {
-            const int r = e / K, k = e - r * K;
-            double2 v = make_double2(0.0, 0.0);
-            if (r0 + r < R) {
-                const double sc = scale[2 + r0 + r];
-                v = X[(size_t)(r0 + r) * K + k];
-                v = make_double2(sc * v.x, sc * v.y);
-            }
-            const float2 hi = make_float2((float)v.x, (float)v.y);
-            xh[e] = hi;
-            xl[e] = make_float2((float)(v.x - (double)hi.x), (float)(v.y - (double)hi.y));
-        }
-        __syncthreads();
-        const float2* Lh = planes + (size_t)bin * 4 * EE;
-        const float2* Kh = Lh + EE;
-        const float2* Ll = Lh + 2 * EE;
-        const float2* Kl = Lh + 3 * EE;
-        for (int i = threadIdx.x; i < E; i += blockDim.x) {
-            DsC lj[RB], lm[RB], kj[RB], km[RB];
-#pragma unroll
-            for (int r = 0; r < RB; ++r) lj[r] = lm[r] = kj[r] = km[r] = DsC{0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-            for (int j = 0; j < E; ++j) {
-                const size_t o = (size_t)j * E + i;
-                const float2 lh = __ldg(Lh + o), kh = __ldg(Kh + o), ll = __ldg(Ll + o), kl = __ldg(Kl + o);
-#pragma unroll
-                for (int r = 0; r < RB; ++r) {
-                    const float2 xjh = xh[r * K + j], xmh = xh[r * K + E + j];
-                    const float2 xjl = xl[r * K + j], xml = xl[r * K + E + j];
-                    ds_cmac(lj[r], xjh, xjl, lh, ll);
-                    ds_cmac(lm[r], xmh, xml, lh, ll);
-                    ds_cmac(kj[r], xjh, xjl, kh, kl);
-                    ds_cmac(km[r], xmh, xml, kh, kl);
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < RB; ++r) {
-                if (r0 + r < R) {
-                    double2* Y = Yh + ((size_t)bin * R + r0 + r) * K;
-                    const double u = 1.0 / (scale[0] * scale[2 + r0 + r]);
-                    const double2 yj = cadd(cmul(ca, ds_value(lj[r])), cmul(cb, ds_value(km[r])));
-                    const double2 ym = cadd(cmul(cg, ds_value(kj[r])), cmul(cd, ds_value(lm[r])));
-                    Y[i] = make_double2(u * yj.x, u * yj.y);
-                    Y[E + i] = make_double2(u * ym.x, u * ym.y);
-                }
-            }
-        }
-    }
-}
-
-size_t binmul_ds_smem(int E) {
-    return (size_t)kDsStages * 4 * kDsJB * E * sizeof(float2) + 8ull * E * sizeof(float2) +
-           2ull * kDsStages * sizeof(uint64_t);
 }
 
 // ------------------------------------------------ K2, FP32, one rhs, half spectrum
@@ -1410,77 +1120,6 @@ macromodel2_kernel(const float2* __restrict__ Zt, const double2* __restrict__ x,
     }
 }
 
-// Single-rhs FP64-accuracy variant in double-single FP32 arithmetic (see
-// binmul_ds_kernel): Z~ as FP32 hi/lo planes zp[t][hi, lo][k'][k], x1 split
-// into hi/lo while it is gathered, each thread two output rows for up to G
-// cells, products accumulated with ds_cmac, FP64 partial outputs.
-constexpr int kMmDsUnroll = 2;
-template <int G>
-__global__ void __launch_bounds__(320, 2)
-macromodel_ds_kernel(const float2* __restrict__ zp, const double2* __restrict__ x,
-                     const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn,
-                     const int32_t* __restrict__ type_cells, const MmBlock* __restrict__ blocks,
-                     double2* __restrict__ Ymm, int K, int M, int chunk, const double* __restrict__ scale) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* xh = reinterpret_cast<float2*>(smem_raw);   // [G][chunk] hi
-    float2* xl = xh + (size_t)G * chunk;                // [G][chunk] lo
-    const MmBlock b = blocks[blockIdx.x];
-    const double sx = scale[2], u = 1.0 / (scale[1] * scale[2]);
-    const int s = blockIdx.y;
-    const int k0 = s * chunk, k1 = min(K, k0 + chunk), nk = k1 - k0;
-    for (int e = threadIdx.x; e < G * chunk; e += blockDim.x) {
-        const int g = e / chunk, kk = e % chunk;
-        double2 v = make_double2(0.0, 0.0);
-        if (g < b.count && kk < nk) {
-            const size_t loc = (size_t)type_cells[b.first + g] * K + k0 + kk;
-            const double2 xv = x[idx[loc]];
-            const double sg = (double)sgn[loc] * sx;
-            v = make_double2(sg * xv.x, sg * xv.y);
-        }
-        const float2 hi = make_float2((float)v.x, (float)v.y);
-        xh[e] = hi;
-        xl[e] = make_float2((float)(v.x - (double)hi.x), (float)(v.y - (double)hi.y));
-    }
-    __syncthreads();
-    const int K2 = K >> 1;
-    const size_t KK = (size_t)K * K;
-    const float4* Zh = reinterpret_cast<const float4*>(zp + (size_t)b.type * 2 * KK + (size_t)k0 * K);
-    const float4* Zl = reinterpret_cast<const float4*>(zp + ((size_t)b.type * 2 + 1) * KK + (size_t)k0 * K);
-    for (int k2 = threadIdx.x; k2 < K2; k2 += blockDim.x) {
-        DsC a0[G], a1[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) a0[g] = a1[g] = DsC{0.f, 0.f, 0.f, 0.f};
-        for (int kb = 0; kb < nk; kb += kMmDsUnroll) {
-            float4 zh[kMmDsUnroll], zl[kMmDsUnroll];
-#pragma unroll
-            for (int u = 0; u < kMmDsUnroll; ++u) {
-                const bool in = kb + u < nk;
-                zh[u] = in ? __ldg(Zh + (size_t)(kb + u) * K2 + k2) : make_float4(0.f, 0.f, 0.f, 0.f);
-                zl[u] = in ? __ldg(Zl + (size_t)(kb + u) * K2 + k2) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < kMmDsUnroll; ++u) {
-                if (kb + u < nk) {
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        const float2 vh = xh[g * chunk + kb + u], vl = xl[g * chunk + kb + u];
-                        ds_cmac(a0[g], vh, vl, make_float2(zh[u].x, zh[u].y), make_float2(zl[u].x, zl[u].y));
-                        ds_cmac(a1[g], vh, vl, make_float2(zh[u].z, zh[u].w), make_float2(zl[u].z, zl[u].w));
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-            if (g < b.count) {
-                double2* y = Ymm + ((size_t)s * M + type_cells[b.first + g]) * K + 2 * k2;
-                const double2 v0 = ds_value(a0[g]), v1 = ds_value(a1[g]);
-                y[0] = make_double2(u * v0.x, u * v0.y);
-                y[1] = make_double2(u * v1.x, u * v1.y);
-            }
-    }
-}
-
 // ------------------------------------------------ K3 tail: U_o^T
 // y[r][u] = sum over local unknowns (m,k) of u: sign * y1[r][m][k]
 // (sums in the grid's precision; V2 is the output vector type)
@@ -1529,10 +1168,7 @@ int build_spectrum(emsurf_handle* h, Operator<T2>& op, const emsurf_problem* pr)
 
 template <typename T2>
 int build_operator(emsurf_handle* h, Operator<T2>& op, const emsurf_problem* pr, const Operator<T2>* share) {
-    const int E = h->E, K = h->K;
-    const size_t EE = (size_t)E * E;
-    const int nox = 2 * h->nx - 1, noy = 2 * h->ny - 1;
-    const size_t nbins = (size_t)h->nbins;
+    const int K = h->K;
     cudaStream_t st = h->setup_stream;
     if (share) {
         // the spectrum of a handle of the same lattice (not owned here)
@@ -1555,16 +1191,19 @@ int build_operator(emsurf_handle* h, Operator<T2>& op, const emsurf_problem* pr,
     EMS_CUDA(cudaGetLastError());
     EMS_CUDA(cudaStreamSynchronize(st));
     if (!pr->tables_on_device) cudaFree(zstage);
-    // work buffers
-    const size_t grid_elems = nbins * (size_t)h->max_rhs * K;
-    EMS_TRY(dev_alloc(h, (void**)&op.Xg, grid_elems * sizeof(T2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Yg, grid_elems * sizeof(T2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Ymm, (size_t)kMmSplit * h->max_rhs * h->M * K * sizeof(T2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Y1, (size_t)h->max_rhs * h->M * K * sizeof(T2)));
+    // work buffers (the FP64 operator's follow its digit planes)
+    if constexpr (std::is_same<T2, float2>::value) EMS_TRY(operator_work<T2>(h, op, kMmSplit));
     for (int c = 0; c < 4; ++c) op.coef[c] = mk<T2>(pr->coef[c].re, pr->coef[c].im);
-    (void)nox;
-    (void)noy;
-    (void)EE;
+    return EMSURF_OK;
+}
+
+template <typename T2>
+int operator_work(emsurf_handle* h, Operator<T2>& op, int mm_split) {
+    const size_t grid = (size_t)h->nbins * h->max_rhs * h->K, cells = (size_t)h->max_rhs * h->M * h->K;
+    EMS_TRY(dev_alloc(h, (void**)&op.Xg, grid * sizeof(T2)));
+    EMS_TRY(dev_alloc(h, (void**)&op.Yg, grid * sizeof(T2)));
+    EMS_TRY(dev_alloc(h, (void**)&op.Ymm, mm_split * cells * sizeof(T2)));
+    EMS_TRY(dev_alloc(h, (void**)&op.Y1, cells * sizeof(T2)));
     return EMSURF_OK;
 }
 
@@ -1775,7 +1414,6 @@ int adopt_fp32_form(emsurf_handle* h, const emsurf_handle* share) {
     h->d_orb_elem = share->d_orb_elem;
     h->d_orb_perm = share->d_orb_perm;
     if (h->half32 || h->orb32) {
-        const int ncw = (h->E + 31) / 32;
         const int slots = h->orb32 ? h->orb_G : 2;
         h->pair_grid = share->pair_grid;
         EMS_TRY(dev_alloc(h, (void**)&h->d_pair_part, (size_t)h->pair_grid * 2 * slots * 2 * h->E * sizeof(float2)));
@@ -1789,7 +1427,6 @@ int adopt_fp32_form(emsurf_handle* h, const emsurf_handle* share) {
 // FP32 operator of a MIXED handle: round the resident FP64 spectrum and
 // macromodels instead of transforming the tables a second time.
 int derive_fp32_operator(emsurf_handle* h, const emsurf_problem* pr, const emsurf_handle* share) {
-    const int K = h->K;
     const size_t EE = (size_t)h->E * h->E;
     const size_t nb = (size_t)h->nbins;
     cudaStream_t st = h->setup_stream;
@@ -1873,84 +1510,13 @@ int derive_fp32_operator(emsurf_handle* h, const emsurf_problem* pr, const emsur
 // the FP32 macromodels and work buffers of a MIXED handle
 int derive_fp32_rest(emsurf_handle* h, const emsurf_problem* pr) {
     const int K = h->K;
-    const size_t nb = (size_t)h->nbins;
     cudaStream_t st = h->setup_stream;
     Operator<float2>& op = h->op32;
     EMS_TRY(dev_alloc(h, (void**)&op.Zt, (size_t)h->T * K * K * sizeof(float2)));
     round_kernel<<<152 * 8, 256, 0, st>>>(op.Zt, h->op64.Zt, (size_t)h->T * K * K);
     EMS_CUDA(cudaGetLastError());
-    const size_t grid_elems = nb * (size_t)h->max_rhs * K;
-    EMS_TRY(dev_alloc(h, (void**)&op.Xg, grid_elems * sizeof(float2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Yg, grid_elems * sizeof(float2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Ymm, (size_t)kMmSplit * h->max_rhs * h->M * K * sizeof(float2)));
-    EMS_TRY(dev_alloc(h, (void**)&op.Y1, (size_t)h->max_rhs * h->M * K * sizeof(float2)));
+    EMS_TRY(operator_work<float2>(h, op, kMmSplit));
     for (int c = 0; c < 4; ++c) op.coef[c] = mk<float2>(pr->coef[c].re, pr->coef[c].im);
-    return EMSURF_OK;
-}
-
-// FP32 hi/lo planes of the FP64 spectrum and macromodels for the
-// double-single kernels (left out, and the FP64 kernels used, when the
-// single-rhs kernel's shape does not fit or the device-memory budget has no
-// room for them).
-int build_ds_planes(emsurf_handle* h, const emsurf_handle* share) {
-    const int E = h->E;
-    const int ncw = (E + 31) / 32;
-    if (binmul_ds_smem(E) > 227 * 1024 || 32 * (1 + ncw) > 1024 || (E + kDsJB - 1) / kDsJB < kDsStages)
-        return EMSURF_OK;
-    const size_t nb = (size_t)h->nbins, EE = (size_t)E * E;
-    const size_t pbytes = nb * 2 * 2 * EE * sizeof(float2), xbytes = nb * 2 * 2 * E * sizeof(float2);
-    if (share && !share->ds_planes) return EMSURF_OK;          // products use the shared FP64 spectrum
-    if (!share && h->budget > 0 && h->device_bytes + (int64_t)(pbytes + xbytes) > h->budget) return EMSURF_OK;
-    if (share) h->ds_planes = share->ds_planes;
-    else EMS_TRY(dev_alloc(h, (void**)&h->ds_planes, pbytes));
-    EMS_TRY(dev_alloc(h, (void**)&h->ds_x, xbytes));
-    EMS_TRY(dev_alloc(h, (void**)&h->d_ds_scale, sizeof(double) * (2 + std::max(1, h->max_rhs))));
-    EMS_TRY(dev_alloc(h, (void**)&h->d_ds_max, sizeof(unsigned long long) * std::max(1, h->max_rhs)));
-    EMS_TRY(dev_alloc(h, (void**)&h->d_ds_cnt, sizeof(unsigned) * std::max(1, h->max_rhs)));
-    EMS_CUDA(cudaMemsetAsync(h->d_ds_max, 0, sizeof(unsigned long long) * std::max(1, h->max_rhs), h->setup_stream));
-    EMS_CUDA(cudaMemsetAsync(h->d_ds_cnt, 0, sizeof(unsigned) * std::max(1, h->max_rhs), h->setup_stream));
-    // operator scales: the largest component of the spectrum (of the
-    // macromodels) maps into [0.5, 1), exactly (powers of two)
-    const size_t KK = (size_t)h->K * h->K;
-    double* part = nullptr;
-    EMS_CUDA(cudaMalloc(&part, sizeof(double) * 2 * 1024));
-    double hs[2] = {1.0, 1.0};
-    {
-        std::vector<double> hp(2 * 1024);
-        if (!share) absmax_part_kernel<<<1024, 256, 0, h->setup_stream>>>(h->op64.Bhat, nb * 2 * EE, part);
-        absmax_part_kernel<<<1024, 256, 0, h->setup_stream>>>(h->op64.Zt, (size_t)h->T * KK, part + 1024);
-        cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(hp.data(), part, sizeof(double) * 2 * 1024, cudaMemcpyDeviceToHost, h->setup_stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->setup_stream);
-        cudaFree(part);
-        if (e != cudaSuccess) {
-            set_error("operator scale: %s", cudaGetErrorString(e));
-            return EMSURF_ECUDA;
-        }
-        for (int w = share ? 1 : 0; w < 2; ++w) {
-            double mx = 0.0;
-            for (int i = 0; i < 1024; ++i) mx = std::max(mx, hp[w * 1024 + i]);
-            if (mx > 0.0 && std::isfinite(mx)) hs[w] = std::ldexp(1.0, -(std::ilogb(mx) + 1));
-        }
-        if (share) hs[0] = share->h_ds_scale0;
-        h->h_ds_scale0 = hs[0];
-        EMS_CUDA(cudaMemcpyAsync(h->d_ds_scale, hs, sizeof(hs), cudaMemcpyHostToDevice, h->setup_stream));
-        EMS_CUDA(cudaStreamSynchronize(h->setup_stream));
-    }
-    if (!share) {
-        split_hilo_kernel<<<152 * 16, 256, 0, h->setup_stream>>>(h->ds_planes, h->op64.Bhat, 2 * EE, nb * 2 * EE,
-                                                                 h->d_ds_scale);
-        EMS_CUDA(cudaGetLastError());
-    }
-    // the macromodels likewise (the transposed Z~ of each type)
-    const size_t zbytes = (size_t)h->T * 2 * KK * sizeof(float2);
-    if ((h->K & 1) == 0 && (h->budget <= 0 || h->device_bytes + (int64_t)zbytes <= h->budget)) {
-        EMS_TRY(dev_alloc(h, (void**)&h->ds_zt, zbytes));
-        split_hilo_kernel<<<152 * 16, 256, 0, h->setup_stream>>>(h->ds_zt, h->op64.Zt, KK, (size_t)h->T * KK,
-                                                                 h->d_ds_scale + 1);
-        EMS_CUDA(cudaGetLastError());
-    }
     return EMSURF_OK;
 }
 
@@ -1965,14 +1531,12 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     const int ph_bin = f64 ? EMS_PH_BINMUL64 : EMS_PH_BINMUL32;
     const int ph_mm = f64 ? EMS_PH_MM64 : EMS_PH_MM32;
     // K4 runs on the handle's side stream (it reads only x and writes only
-    // the partials Ymm that the inverse transform adds).  FP32 products fork
-    // before the forward transform, so the macromodel product starts while
-    // the transform runs; FP64-accuracy products fork after the per-rhs
-    // scales it reads.  The tensor-core variant (>= 8 rhs) stays on the
-    // caller's stream.
-    const bool side = h->side_stream && !(h->have_tc && R >= kTcMinRhs);
-    const bool early_fork = side && std::is_same<T2, float2>::value;
-    if (early_fork) {
+    // the partials Ymm that the inverse transform adds), forked before the
+    // forward transform.  With the macromodels' digit planes only the splitting
+    // of x1 runs there: their product joins the bins' launch.  The tensor-core
+    // variant (FP32, >= 8 rhs) stays on the caller's stream.
+    const bool side = h->side_stream && !(std::is_same<T2, float2>::value && h->have_tc && R >= kTcMinRhs);
+    if (side) {
         EMS_CUDA(cudaEventRecord(h->ev_fork, st));
         EMS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
     }
@@ -1991,24 +1555,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
         EMS_TRY(fft_pass<T2>(op.Xg, h->plan_y, (long long)px * lanes, 1, 0, -1, st, h->ny, py));
     }
     prof_mark(h, ph_fft, false, st);
-    if constexpr (std::is_same<T2, double2>::value) {
-        if (h->ds_planes && x) {
-            // per-rhs powers of two for the double-single operands of this product
-            const int nbl = (int)std::min<size_t>(((size_t)h->n_unique + 1023) / 1024, (size_t)h->num_sms);
-            pow2_scale_kernel<<<dim3(nbl, R), 256, 0, st>>>(x, (size_t)h->n_unique, h->d_ds_max, h->d_ds_cnt,
-                                                            h->d_ds_scale + 2);
-            EMS_CUDA(cudaGetLastError());
-            h->launches += 1;
-        }
-    }
-    cudaStream_t mst = st;
-    if (side) {
-        if (!early_fork) {
-            EMS_CUDA(cudaEventRecord(h->ev_fork, st));
-            EMS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
-        }
-        mst = h->side_stream;
-    }
+    cudaStream_t mst = side ? h->side_stream : st;
     prof_mark(h, ph_mm, true, mst);
     // K splits of the macromodel product: as many as fill one wave of
     // resident CTAs (a partial second wave would double its time), at most
@@ -2017,6 +1564,12 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     if constexpr (std::is_same<T2, float2>::value) {
         if (h->have_tc && R >= kTcMinRhs) {
             EMS_TRY(tc_macromodel(h, x, xf, op.Ymm, R, mst));
+            mm_done = true;
+        }
+    }
+    if constexpr (std::is_same<T2, double2>::value) {
+        if (h->sl_Z) {
+            EMS_TRY(slices_cells(h, x, R, mst));
             mm_done = true;
         }
     }
@@ -2054,7 +1607,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
         nsplit = std::max(nsplit, (K + max_chunk - 1) / max_chunk);
         nsplit = std::min(nsplit, kMmSplit);
     }
-    if (mm_done) nsplit = 1;   // the tensor-core product wrote Ymm[0] whole
+    if (mm_done) nsplit = 1;   // the tensor-core products write Ymm[0] whole
     if constexpr (std::is_same<T2, float2>::value) {
         if (!mm_done && R == 1 && (K & 1) == 0) {
             // one rhs: the two-rows-per-thread kernel (K split to fill one wave)
@@ -2083,26 +1636,6 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
             mm_done = true;
         }
     }
-    if constexpr (std::is_same<T2, double2>::value) {
-        if (!mm_done && R == 1 && h->ds_zt) {
-            // one rhs, FP64 accuracy from double-single FP32 arithmetic
-            const int threads2 = std::min(320, ((K / 2 + 31) / 32) * 32);
-            const int nblk = h->n_mm_blocks;
-            int ns2 = std::max(1, std::min(kMmSplit, K / 64));
-            ns2 = std::max(1, std::min(ns2, h->num_sms * 2 / std::max(1, nblk)));
-            int chunk2 = (K + ns2 - 1) / ns2;
-            chunk2 = (chunk2 + kMmDsUnroll - 1) / kMmDsUnroll * kMmDsUnroll;
-            ns2 = (K + chunk2 - 1) / chunk2;
-            const size_t sm = (size_t)2 * kMmGroup * chunk2 * sizeof(float2);
-            EMS_TRY(set_smem_once(macromodel_ds_kernel<kMmGroup>, sm));
-            macromodel_ds_kernel<kMmGroup><<<dim3(nblk, ns2), threads2, sm, mst>>>(
-                h->ds_zt, x, h->d_uo_index, h->d_uo_sign, h->d_type_cells,
-                reinterpret_cast<const MmBlock*>(h->d_mm_blocks), op.Ymm, K, h->M, chunk2, h->d_ds_scale);
-            EMS_CUDA(cudaGetLastError());
-            nsplit = ns2;
-            mm_done = true;
-        }
-    }
     if (!mm_done) {
         const int nblk = h->n_mm_blocks;
         const int chunk = (K + nsplit - 1) / nsplit;
@@ -2123,6 +1656,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     }
     prof_mark(h, ph_mm, false, mst);
     if (side) EMS_CUDA(cudaEventRecord(h->ev_join, mst));
+    bool joined = !side;
     prof_mark(h, ph_bin, true, st);
     // K2
     const int threads = std::min(1024, ((E + 31) / 32) * 32);
@@ -2180,37 +1714,13 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
         }
     }
     if constexpr (std::is_same<T2, double2>::value) {
-        if (!bin_done && R == 1 && h->ds_planes) {
-            // FP64 accuracy from FP32 hi/lo arithmetic (the FP64 rate is ~1/60 of FP32)
-            const size_t lanes2 = (size_t)2 * E;
-            split_hilo_kernel<<<grid_for((size_t)nb * lanes2, 256), 256, 0, st>>>(h->ds_x, op.Xg, lanes2,
-                                                                                (size_t)nb * lanes2,
-                                                                                h->d_ds_scale + 2);
-            EMS_CUDA(cudaGetLastError());
-            const size_t smem = binmul_ds_smem(E);
-            EMS_TRY(set_smem_once(binmul_ds_kernel, smem));
-            const int grid = std::min(nb, std::max(1, h->num_sms));
-            binmul_ds_kernel<<<grid, 32 * (1 + (E + 31) / 32), smem, st>>>(
-                h->ds_planes, h->ds_x, op.Yg, E, nb, op.coef[0], op.coef[1], op.coef[2], op.coef[3], h->d_err,
-                h->d_ds_scale);
-            EMS_CUDA(cudaGetLastError());
-            h->launches += 2;
-            bin_done = true;
-        }
-        if (!bin_done && R > 1 && h->ds_planes) {
-            // several rhs: FP64 accuracy from double-single FP32 arithmetic,
-            // four rhs per pass over the planes
-            constexpr int RBd = 4;
-            const size_t smem = (size_t)2 * RBd * 2 * E * sizeof(float2);
-            EMS_TRY(set_smem_once(binmul_ds_multi_kernel<RBd>, smem));
-            const int grid = std::min(nb, 152 * 8);
-            for (int r0 = 0; r0 < R; r0 += RBd) {
-                binmul_ds_multi_kernel<RBd><<<grid, threads, smem, st>>>(h->ds_planes, op.Xg, op.Yg, E, nb, R, r0,
-                                                                      op.coef[0], op.coef[1], op.coef[2],
-                                                                      op.coef[3], h->d_ds_scale);
-                EMS_CUDA(cudaGetLastError());
-                h->launches += 1;
+        if (h->sl_A) {
+            // exact digits on the tensor cores, bins and macromodels in one launch
+            if (h->sl_Z && !joined) {
+                EMS_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
+                joined = true;
             }
+            EMS_TRY(slices_multiply(h, op.Xg, op.Yg, op.Ymm, R, op.coef, st));
             bin_done = true;
         }
     }
@@ -2236,7 +1746,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
         }
     }
     prof_mark(h, ph_bin, false, st);
-    if (side) EMS_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));      // the partials are in Ymm
+    if (!joined) EMS_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));      // the partials are in Ymm
     prof_mark(h, ph_fft, true, st);
     // K3: inverse y-pass on all columns, inverse x-pass on the rows kept
     if (fused) {
@@ -2261,6 +1771,8 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     return EMSURF_OK;
 }
 
+template int operator_work<double2>(emsurf_handle*, Operator<double2>&, int);
+template int operator_work<float2>(emsurf_handle*, Operator<float2>&, int);
 template int build_operator<double2>(emsurf_handle*, Operator<double2>&, const emsurf_problem*,
                                      const Operator<double2>*);
 template int build_operator<float2>(emsurf_handle*, Operator<float2>&, const emsurf_problem*,

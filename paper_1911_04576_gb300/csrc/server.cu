@@ -108,7 +108,7 @@ int64_t operator_bytes(const emsurf_request& q) {
     const int64_t E = 18LL * q.n * q.n;
     const int64_t P = (int64_t)smallest_smooth_at_least(2 * q.nx - 1) * smallest_smooth_at_least(2 * q.ny - 1);
     const int64_t b64 = 2LL * E * E * P * 16, b32 = 2LL * E * E * P * 8;
-    int64_t op = b64;                                   // FP64 spectrum or its hi/lo planes
+    int64_t op = b64;                                   // FP64 spectrum or its digit planes (7/8 of it)
     if (q.precision != EMSURF_FP64) op += spectrum_form(q) == 1 ? b32 / 2 : b32;
     if (spectrum_form(q) == 3) op += b32;               // tensor-core planes
     return op + 50LL * E * E * 16;                      // + near tables
@@ -134,10 +134,10 @@ Estimate estimate(const emsurf_request& q) {
     e.tables = 2LL * (2 * q.nx - 1) * (2 * q.ny - 1) * E * E * 16;
     const int64_t mm = (int64_t)q.n_types * K * K * 16;
     const int64_t b64 = 2LL * E * E * P * 16;
-    // during create the FP64 spectrum and its hi/lo planes coexist before the
+    // during create the FP64 spectrum and its digit planes coexist before the
     // spectrum is given back
     e.blocks = operator_bytes(q) + b64;
-    // macromodel copies: FP64 (+ its hi/lo planes), FP32 (MIXED / FP32), bf16 planes
+    // macromodel copies: FP64 (+ its digit planes), FP32 (MIXED / FP32), bf16 planes
     e.own = mm * (q.precision == EMSURF_FP32 ? 1 : 2) + (q.precision == EMSURF_MIXED ? mm / 2 : 0);
     if (spectrum_form(q) == 3) e.own += mm / 2 + P * 4LL * 32 * ((R + 31) / 32) * E * 4;
     const int64_t work = 2LL * P * R * K * 16 + 10LL * R * M * K * 16;

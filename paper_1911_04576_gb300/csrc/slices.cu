@@ -1,0 +1,907 @@
+// FP64-accuracy products on the tensor cores: exact integer slices.
+//
+// FP64 runs at ~1/60 of the FP32 rate on this part, and double-single FP32
+// arithmetic needs 12 FP32 operations per real multiply-add.  Here every
+// operand is cut into 7 balanced base-256 digits of a 55-bit integer,
+//   v = 2^(ex - 54) sum_t d_t 256^(6 - t),  d_t in [-128, 127],
+// with one power of two 2^ex above the largest component of each matrix row
+// and of each vector (Ozaki, Ogita, Oishi, Rump 2012: error-free splitting).
+// Digits are exact in FP16, their products exact in FP32, and a sum of up to
+// 7 x 128 products stays below 2^24, so kind::f16 MMAs with FP32 accumulation
+// in TMEM add them without rounding.  Digit pairs s + t = l share an
+// accumulator column (level l); levels 0..6 are kept (the dropped pairs weigh
+// 2^-50 of row maximum times vector maximum), read back as integers, summed in
+// int64 over the 128-wide K chunks, combined into complex products there and
+// turned into FP64 once per output.
+//
+// Two problems share one launch:
+//   bins        y^(k) = B^(k) x^(k): per bin 4E real rows (4 i + 2 op + c, op in
+//               {L, K}, c = re, im) over the E sources; columns (rhs, x_J/x_M,
+//               re/im);
+//   macromodels y = Z~^t x1 of the cells of a type: 2K real rows (2 k + c) over
+//               K; columns (cell and rhs, re/im).
+//
+// The matrix digits are stored as bytes (d + 128), 7 per real number: planes
+// [matrix][row tile of 128][16-source block][digit][row][16 bytes], streamed
+// through a ring of their own whose slots are free as soon as a warp set has
+// read them.  The warp set turns them into FP16 (byte into the mantissa of 1024 + b, minus 1152)
+// and writes them into TMEM, so the A operand never passes through shared
+// memory as FP16.  The vectors' digits are FP16 in 64-byte swizzled rows
+// (t, v), preceded by 6 V rows of zeros that stay in shared memory: digit s of
+// the matrix multiplies the rows from -s V on, so that digit t lands in the
+// columns of level s + t and every MMA of a tile has the same shape and the
+// same accumulator (which keeps them in order).
+//
+// Warps: 0-7 epilogue (half of the columns each), 8-15 byte to FP16 in two sets
+// that take 16-source blocks in turn, 16 and 18 bulk copies of matrix and
+// vector digits, 17 MMA.  A 128 x N x 16 MMA with A in TMEM takes 68-86 cycles
+// for N up to 176 (measured), and each wait about as long as two of them, so the
+// MMA warp bounds the kernel: it waits once per two blocks on all it needs (the
+// byte-to-FP16 warps see to the vector digits and give their slots back).  Every
+// wait is bounded: on expiry the kernel sets the error flag, waits (bounded) for
+// its copies and MMAs in flight, frees TMEM and returns.
+//
+// Measured, product of a 16 x 16 lattice with K = 576 (2.38 GB of digits, 350 us
+// at the copy rate): 1161 us in double-single FP32, 593 us here (bins and
+// macromodels 490 us, splitting the vectors 25 us); 12 x 9, K = 576 and 6 rhs:
+// 6575 us, 597 us.  Error against 64 bits 7.2e-14, 6e-15 (both sizes).
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "common.cuh"
+
+namespace emsurf {
+namespace {
+
+constexpr int kSl = 7;                       // digits
+constexpr int kSlRows = 128;                 // rows per tile (TMEM lanes)
+constexpr int kSlK = 32;                     // sources per stage
+constexpr int kSlChunk = 4;                  // stages per exact accumulation (128 sources)
+constexpr int kSlKbBytes = kSl * 16;         // bytes per row and 16-source block
+constexpr int kSlABytes = kSlKbBytes * kSlRows;         // one 16-source block of a tile
+constexpr int kSlMaxStages = 14, kSlXStages = 4;
+constexpr int kSlEpi = 8, kSlWarps = kSlEpi + 8 + 3, kSlThreads = 32 * kSlWarps;
+constexpr int kSlWarpA = kSlWarps - 3, kSlWarpM = kSlWarps - 2, kSlWarpX = kSlWarps - 1;
+constexpr uint32_t kSlTmemCols = 512, kSlAStep = kSl * 8;   // TMEM columns; of one 16-source block of A
+constexpr int kSlMaxSlots = 4;               // A blocks in TMEM, at the end of its columns
+constexpr int kSlWait = 1 << 16;
+constexpr size_t kSlSmemMax = 224 * 1024;
+constexpr int kSlMaxV = 24;                  // vector columns of one launch (a multiple of 8: swizzle groups):
+                                             // two accumulators and two A blocks fit in TMEM
+constexpr int kSlRhs = kSlMaxV / 4;          // rhs per launch
+constexpr int kSlSplit = 256;                // threads of a splitting block
+constexpr int kSlCells = 8;                  // columns of a macromodel entry
+// |I_a I_b| <= 2^108 = 2^52 units of level 5, so re +- im sums of up to kSlExact
+// sources stay inside int64; beyond, the integers lose a bit per factor of 4
+constexpr int kSlExact = 990, kSlMaxN = 7000;   // the latter: two vectors in shared memory
+
+__device__ __forceinline__ uint32_t sl_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void sl_init(uint64_t* bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sl_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void sl_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sl_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void sl_expect(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sl_addr(bar)), "r"(bytes) : "memory");
+}
+// bounded wait; each try suspends the thread for up to 20 us (re-polling warps
+// slow every barrier of the block down)
+__device__ __forceinline__ bool sl_wait(uint64_t* bar, uint32_t parity) {
+    for (int it = 0; it < kSlWait; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(sl_addr(bar)), "r"(parity), "r"(20000u)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+// the same for two or three barriers at once (their latencies overlap)
+__device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, uint64_t* b2, uint32_t p2,
+                                         bool third) {
+    for (int it = 0; it < kSlWait; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p, q, r, t;\n setp.ne.b32 t, %8, 0;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %7;\n"
+            " mbarrier.try_wait.parity.shared::cta.b64 q, [%3], %4, %7;\n setp.eq.b32 r, %8, 0;\n"
+            " @t mbarrier.try_wait.parity.shared::cta.b64 r, [%5], %6, %7;\n"
+            " and.pred p, p, q;\n and.pred p, p, r;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(sl_addr(b0)), "r"(p0), "r"(sl_addr(b1)), "r"(p1), "r"(sl_addr(b2)), "r"(p2), "r"(20000u),
+              "r"((uint32_t)third)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ void sl_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], "
+        "%4;" ::"r"(sl_addr(dst)),
+        "l"(src), "r"(bytes), "r"(sl_addr(bar)), "l"(pol)
+        : "memory");
+}
+// One lane of a converged warp.  The MMA warp runs as a whole and issues under
+// elect.sync, so that the operands stay in uniform registers.
+__device__ __forceinline__ bool sl_elect() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+__device__ __forceinline__ void sl_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sl_addr(bar))
+                 : "memory");
+}
+// D (+)= A B: A 128 x 16 FP16 in TMEM, B N x 16 FP16 in shared memory (K-major, 64B swizzle)
+template <bool ACC>
+__device__ __forceinline__ void sl_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+        "r"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0));
+}
+// K-major descriptor, 64-byte swizzled rows, 8-row groups 512 B apart
+__device__ __forceinline__ uint64_t sl_desc(uint32_t addr) {
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | (1ull << 16) | (32ull << 32) | (1ull << 46) | (4ull << 61);
+}
+__device__ __forceinline__ void tmem_st8(uint32_t t, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(t), "r"(r[0]),
+                 "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(t));
+}
+
+__host__ __device__ constexpr int sl_up16(int n) { return (n + 15) & ~15; }
+
+struct SlProb {
+    const unsigned char* A;      // digit planes
+    const double* rs;            // [matrix][row / 2] 2^(ex - 8) of each complex row
+    const unsigned char* X;      // vector digits [x matrix][stage][Np][64 bytes]
+    const double* xs;            // [x matrix][V / 2] 2^(ex - 8) of each complex vector
+    int nk16, nst, rows, tiles, V, Np, items, xmats;
+    int live;                    // bins: rhs of this launch
+};
+
+struct SlArgs {
+    SlProb p[2];                 // bins, macromodels
+    int stages, z_bytes, x_bytes;   // matrix ring depth, bytes of a vector slot's zero rows and vector rows
+    int slots, d_step;           // A blocks in TMEM, spacing of the two accumulators
+    // bins
+    double2* Y;                  // [bins][R][2E]
+    int E, R, r0;
+    double2 co[4];
+    // macromodels
+    double2* Ymm;                // [R][M][K]
+    const int2* ent;             // (type, first column)
+    const int32_t *type_ptr, *type_cells;
+    int K, M;
+    int* err;
+};
+
+// Range of items of CTA b: items whose first stage lies in its share of all stages.
+__device__ __forceinline__ int sl_item_at(const SlArgs& g, long long q) {
+    const long long s0 = (long long)g.p[0].items * g.p[0].nst;
+    if (q <= s0) return g.p[0].nst ? (int)((q + g.p[0].nst - 1) / g.p[0].nst) : 0;
+    return g.p[0].items + (int)((q - s0 + g.p[1].nst - 1) / g.p[1].nst);
+}
+
+__global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
+    constexpr int V4 = kSlMaxV / 8;          // groups of four columns per epilogue half
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ __align__(8) uint64_t full[kSlMaxStages], empty[kSlMaxStages], xfull[kSlXStages], xempty[kSlXStages],
+        afull[kSlMaxSlots], aempty[kSlMaxSlots], dfull[2], dempty[2], mma_done;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == kSlWarpM) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sl_addr(&tmem_slot)),
+                     "r"(kSlTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    const int xslot = g.z_bytes + g.x_bytes;
+    unsigned char* xring = smem + g.stages * kSlABytes;
+    for (int s = 0; s < kSlXStages; ++s)
+        for (int e = threadIdx.x; e < g.z_bytes / 16; e += blockDim.x)
+            reinterpret_cast<uint4*>(xring + s * xslot)[e] = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < g.stages; ++s) {
+            sl_init(&full[s], 1);
+            sl_init(&empty[s], 4);
+        }
+        for (int s = 0; s < kSlXStages; ++s) {
+            sl_init(&xfull[s], 1);
+            sl_init(&xempty[s], 1);
+        }
+        for (int a = 0; a < kSlMaxSlots; ++a) {
+            sl_init(&afull[a], 4);
+            sl_init(&aempty[a], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            sl_init(&dfull[a], 1);
+            sl_init(&dempty[a], kSlEpi);
+        }
+        sl_init(&mma_done, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_slot;
+    volatile int* abort_v = &abort_flag;
+    const uint32_t a_col = kSlTmemCols - g.slots * kSlAStep;
+    const int slots = g.slots;
+    const long long total = (long long)g.p[0].items * g.p[0].nst + (long long)g.p[1].items * g.p[1].nst;
+    const int i_lo = sl_item_at(g, (long long)blockIdx.x * total / gridDim.x);
+    const int i_hi = sl_item_at(g, (long long)(blockIdx.x + 1) * total / gridDim.x);
+
+    if (warp == kSlWarpA || warp == kSlWarpX) {
+        // ------------------------------------------------ copies: matrix digits, vector digits
+        if (lane == 0) {
+            const bool mat_side = warp == kSlWarpA;
+            const uint64_t once = l2_evict_first(), keep = l2_evict_last();
+            const int depth = mat_side ? g.stages : kSlXStages;
+            uint64_t *fb = mat_side ? full : xfull, *eb = mat_side ? empty : xempty;
+            int st = 0;
+            long long issued = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+                const int w = it >= g.p[0].items;
+                const SlProb& p = g.p[w];
+                const int loc = w ? it - g.p[0].items : it, xm = loc / p.tiles, tile = loc - xm * p.tiles;
+                const int mat = w ? g.ent[xm].x : xm;
+                const int rows = min(kSlRows, p.rows - tile * kSlRows);
+                const unsigned char* a = p.A + ((size_t)mat * p.rows + (size_t)tile * kSlRows) * p.nk16 * kSlKbBytes;
+                const unsigned char* x = p.X + (size_t)xm * p.nst * p.Np * 64;
+                const int steps = mat_side ? p.nk16 : p.nst;
+                for (int s = 0; s < steps; ++s) {
+                    if (!sl_wait(&eb[st], ph ^ 1)) {
+                        atomicExch(g.err, 20);
+                        ok = false;
+                        break;
+                    }
+                    if (mat_side) {
+                        const uint32_t n = (uint32_t)(kSlKbBytes * rows);
+                        sl_expect(&fb[st], n);
+                        // the macromodels are read by several items and products
+                        sl_copy(smem + st * kSlABytes, a + (size_t)s * n, n, &fb[st], w ? keep : once);
+                    } else {
+                        const uint32_t n = (uint32_t)(p.Np * 64);
+                        sl_expect(&fb[st], n);
+                        sl_copy(xring + st * xslot + g.z_bytes, x + (size_t)s * n, n, &fb[st], keep);
+                    }
+                    ++issued;
+                    if (++st == depth) {
+                        st = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            if (!ok) *abort_v = 1;
+            // every copy has landed before the CTA can exit
+            for (long long u = issued > depth ? issued - depth : 0; u < issued; ++u)
+                if (!sl_wait(&fb[u % depth], (uint32_t)((u / depth) & 1))) atomicExch(g.err, 20);
+        }
+    } else if (warp == kSlWarpM) {
+        // ------------------------------------------------ MMA
+        const uint32_t go = lane == 0;
+        const uint32_t tb = __shfl_sync(0xffffffffu, tmem, 0);
+        int xst = 0, db = 0, slot = 0;
+        uint32_t dph = 0, sph = 0;
+        bool any = false, ok = true;
+        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+            const SlProb& p = g.p[it >= g.p[0].items];
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(p.Np >> 3) << 17) | ((uint32_t)(kSlRows >> 4) << 24);
+            const uint32_t back = (uint32_t)p.V * 4;        // one digit's rows in descriptor units of 16 bytes
+            const int nk16 = p.nk16;
+            // Two blocks of A (one vector stage) at a time where TMEM has four slots,
+            // else one: the waits cost more than the issue.
+            int kc = 0;
+            for (int k = 0; k < nk16;) {
+                const bool odd = k & 1, two = slots == kSlMaxSlots && k + 1 < nk16;
+                const int slot2 = slot + 1 == slots ? 0 : slot + 1;
+                const uint32_t sph2 = slot2 ? sph : sph ^ 1;
+                const bool first = kc == 0;
+                if (!sl_wait3(&afull[slot], sph, &afull[two ? slot2 : slot], two ? sph2 : sph, &dempty[db],
+                              dph ^ 1, first)) {
+                    if (go) atomicExch(g.err, 21);
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t d = tb + (uint32_t)(db * g.d_step), ta = tb + a_col + slot * kSlAStep,
+                               ta2 = tb + a_col + slot2 * kSlAStep;
+                const uint64_t bd = sl_desc(sl_addr(xring + xst * xslot + g.z_bytes)) + (odd ? 2 : 0);
+                k += two ? 2 : 1;
+                kc += two ? 2 : 1;
+                const bool flush = kc == 2 * kSlChunk || k >= nk16;
+                if (sl_elect()) {
+                    if (first) sl_mma<false>(d, ta, bd, idesc);
+                    else sl_mma<true>(d, ta, bd, idesc);
+#pragma unroll
+                    for (int sl = 1; sl < kSl; ++sl) sl_mma<true>(d, ta + sl * 8, bd - sl * back, idesc);
+                    sl_commit(&aempty[slot]);
+                    if (two) {
+#pragma unroll
+                        for (int sl = 0; sl < kSl; ++sl) sl_mma<true>(d, ta2 + sl * 8, bd + 2 - sl * back, idesc);
+                        sl_commit(&aempty[slot2]);
+                    }
+                    if (flush) sl_commit(&dfull[db]);
+                }
+                __syncwarp();
+                any = true;
+                if (flush) {
+                    kc = 0;
+                    dph ^= (uint32_t)db;
+                    db ^= 1;
+                }
+                slot = two ? slot2 : slot;
+                sph = two ? sph2 : sph;
+                if (++slot == slots) {
+                    slot = 0;
+                    sph ^= 1;
+                }
+                if ((odd || two || k >= nk16) && ++xst == kSlXStages) xst = 0;
+            }
+        }
+        if (!ok) *abort_v = 1;
+        if (any) {
+            if (sl_elect()) sl_commit(&mma_done);
+            __syncwarp();
+            if (!sl_wait(&mma_done, 0) && go) atomicExch(g.err, 23);
+        }
+    } else if (warp >= kSlEpi) {
+        // ------------------------------------------------ bytes to FP16 in TMEM
+        const int set = (warp - kSlEpi) >> 2, qd = warp & 3, row = 32 * qd + lane;
+        const uint32_t ta = tmem + ((uint32_t)(32 * qd) << 16) + a_col;
+        const __half2 off = __floats2half2_rn(1152.f, 1152.f);
+        int st = 0, q = 0, slot = 0, xst = 0;
+        uint32_t ph = 0, sph = 0, xph = 0;
+        // vector slot + 1 of the last kSlMaxSlots blocks that end a vector stage (else 0)
+        int ends[kSlMaxSlots] = {};
+        bool ok = true;
+        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+            const int w = it >= g.p[0].items;
+            const SlProb& p = g.p[w];
+            const int loc = w ? it - g.p[0].items : it, tile = loc % p.tiles;
+            const int rows = min(kSlRows, p.rows - tile * kSlRows), rr = min(row, rows - 1);
+            const int nk16 = p.nk16;
+            for (int k = 0; k < nk16; ++k, ++q) {
+                const bool end = (k & 1) || k == nk16 - 1;
+                const int done = slots == kSlMaxSlots ? ends[kSlMaxSlots - 1] : ends[1];
+                if ((q & 1) == set) {
+                    if (!sl_wait(&full[st], ph)) {
+                        if (lane == 0) atomicExch(g.err, 24);
+                        ok = false;
+                        break;
+                    }
+                    const uint4* a = reinterpret_cast<const uint4*>(smem + st * kSlABytes);
+                    uint4 v[kSl];
+#pragma unroll
+                    for (int sl = 0; sl < kSl; ++sl) v[sl] = a[sl * rows + rr];
+                    __syncwarp();
+                    if (lane == 0) sl_arrive(&empty[st]);
+                    // the block `slots` before this one has been multiplied: its TMEM slot
+                    // is free, and its vector slot if it was the stage's last
+                    if (!sl_wait(&aempty[slot], sph ^ 1)) {
+                        if (lane == 0) atomicExch(g.err, 25);
+                        ok = false;
+                        break;
+                    }
+                    if (done && qd == 0 && lane == 0) sl_arrive(&xempty[done - 1]);
+                    if (!sl_wait(&xfull[xst], xph)) {
+                        if (lane == 0) atomicExch(g.err, 26);
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+                    for (int sl = 0; sl < kSl; ++sl) {
+                        const uint32_t b[4] = {v[sl].x, v[sl].y, v[sl].z, v[sl].w};
+                        uint32_t h[8];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            // FP16 0x6400 | byte = 1024 + byte; minus 1152 gives byte - 128
+                            const uint32_t lo = __byte_perm(b[c], 0x64646464u, 0x4140), hi = __byte_perm(b[c], 0x64646464u, 0x4342);
+                            const __half2 l2 = __hsub2(*reinterpret_cast<const __half2*>(&lo), off);
+                            const __half2 h2 = __hsub2(*reinterpret_cast<const __half2*>(&hi), off);
+                            h[2 * c] = *reinterpret_cast<const uint32_t*>(&l2);
+                            h[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&h2);
+                        }
+                        tmem_st8(ta + slot * kSlAStep + sl * 8, h);
+                    }
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    __syncwarp();
+                    if (lane == 0) sl_arrive(&afull[slot]);
+                }
+#pragma unroll
+                for (int i = kSlMaxSlots - 1; i > 0; --i) ends[i] = ends[i - 1];
+                ends[0] = end ? xst + 1 : 0;
+                if (++st == g.stages) {
+                    st = 0;
+                    ph ^= 1;
+                }
+                if (++slot == slots) {
+                    slot = 0;
+                    sph ^= 1;
+                }
+                if (end && ++xst == kSlXStages) {
+                    xst = 0;
+                    xph ^= 1;
+                }
+            }
+        }
+        if (!ok) *abort_v = 1;
+    } else {
+        // ------------------------------------------------ epilogue
+        const int qd = warp & 3, half = warp >> 2, rho = 32 * qd + lane;
+        const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16);
+        int db = 0;
+        uint32_t dph = 0;
+        bool ok = true;
+        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+            const int w = it >= g.p[0].items;
+            const SlProb& p = g.p[w];
+            const int loc = w ? it - g.p[0].items : it, xm = loc / p.tiles, tile = loc - xm * p.tiles;
+            const int V = p.V, row = tile * kSlRows + rho;
+            const int g0 = half * (V / 8);           // first group of four columns, V / 8 groups each
+            // sums in units of level 5 (level 6 rounded to it)
+            long long acc[4 * V4];
+#pragma unroll
+            for (int v = 0; v < 4 * V4; ++v) acc[v] = 0;
+            for (int s = 0; s < p.nst; s += kSlChunk) {
+                if (!sl_wait(&dfull[db], dph)) {
+                    if (lane == 0) atomicExch(g.err, 27);
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t d = tl + (uint32_t)(db * g.d_step);
+#pragma unroll
+                for (int c = 0; c < V4; ++c) {
+                    if (8 * c < V) {
+                        uint32_t r[kSl][4];
+#pragma unroll
+                        for (int l = 0; l < kSl; ++l) tmem_ld4(d + l * V + 4 * (g0 + c), r[l]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            long long a = __float2int_rn(__uint_as_float(r[0][u]));
+#pragma unroll
+                            for (int l = 1; l < 6; ++l) a = a * 256 + __float2int_rn(__uint_as_float(r[l][u]));
+                            acc[4 * c + u] += a + ((__float2int_rn(__uint_as_float(r[6][u])) + 128) >> 8);
+                        }
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0) sl_arrive(&dempty[db]);
+                dph ^= (uint32_t)db;
+                db ^= 1;
+            }
+            if (!ok) break;
+            const int mat = w ? g.ent[xm].x : xm;
+            // digits: v = 2^(ex - 6) sum d_t 256^-t; level l weighs 256^-l 2^-12, so
+            // level 5 is 2^-52; the stored powers are 2^(ex - 8)
+            const double rsc = (row < p.rows ? p.rs[(size_t)mat * (p.rows / 2) + (row >> 1)] : 0.0) * 0x1p-36;
+            const double* xs = p.xs + (size_t)xm * (V / 2);
+            const bool im = rho & 1;
+            int c0 = 0, nt = 0;
+            if (w) {
+                c0 = g.type_ptr[mat];
+                nt = (g.type_ptr[mat + 1] - c0) * g.R;
+            }
+#pragma unroll
+            for (int c = 0; c < V4; ++c) {
+                const int cc = g0 + c;
+                if (8 * c >= V || (!w && cc >= p.live)) continue;
+                // rows re and im of one complex row on neighbouring lanes (same scale):
+                // the re lane forms the product with the first complex vector of the
+                // group of two, the im lane with the second
+                const long long* q = acc + 4 * c;
+                const long long t0 = __shfl_xor_sync(0xffffffffu, im ? q[0] : q[2], 1);
+                const long long t1 = __shfl_xor_sync(0xffffffffu, im ? q[1] : q[3], 1);
+                const long long pr = im ? t0 - q[3] : q[0] - t1, pi = im ? t1 + q[2] : q[1] + t0;
+                const double sc = rsc * xs[2 * cc + (im ? 1 : 0)];
+                double2 u = make_double2((double)pr * sc, (double)pi * sc);
+                if (!w) {
+                    // y_J = a L x_J + b K x_M, y_M = g K x_J + d L x_M
+                    const int role = rho & 3;                  // L x_J, L x_M, K x_J, K x_M
+                    const double2 cf = role == 0 ? g.co[0] : role == 1 ? g.co[3] : role == 2 ? g.co[2] : g.co[1];
+                    u = cmul(cf, u);
+                    const double px = __shfl_xor_sync(0xffffffffu, u.x, 3), py = __shfl_xor_sync(0xffffffffu, u.y, 3);
+                    const int i = row >> 2;
+                    if (!im && i < g.E)
+                        g.Y[((size_t)xm * g.R + g.r0 + cc) * 2 * g.E + (role == 2 ? g.E : 0) + i] =
+                            make_double2(u.x + px, u.y + py);
+                } else {
+                    const int col = g.ent[xm].y + 2 * cc + (im ? 1 : 0);
+                    if (row < p.rows && col < nt) {
+                        const int cell = g.type_cells[c0 + col / g.R];
+                        g.Ymm[((size_t)(col % g.R) * g.M + cell) * g.K + (row >> 1)] = u;
+                    }
+                }
+            }
+        }
+        if (!ok) *abort_v = 1;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (warp == kSlWarpM)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSlTmemCols));
+}
+
+// ---------------------------------------------------------------- splitting
+// exponent ex with |v| < 2^ex for the largest |v| of a vector, from its bit
+// pattern (the patterns of non-negative doubles order like the values, NaN above
+// infinity) and n, the sources that are summed; INT_MIN when it is not finite
+__device__ __forceinline__ int sl_exp(unsigned long long mbits, int n) {
+    if (mbits >= 0x7ff0000000000000ull) return INT_MIN;
+    const double m = __longlong_as_double((long long)mbits);
+    const int spare = n <= kSlExact ? 0 : n <= 4 * kSlExact ? 1 : 2;
+    return (m > 0.0 ? max(ilogb(m) + 1, -900) : 0) + spare;
+}
+// 2^(ex - 8) for the products (NaN where a component was not finite: it marks
+// every output)
+__device__ __forceinline__ double sl_pow(int ex) {
+    return ex == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, ex - 8);
+}
+// Bytes d_t + 128 of the digits of rn(v 2^(54 - ex)), least significant first:
+// balanced digits are the bytes of I + sum_t 128 256^t.  From the bit pattern:
+// FP64 conversions run at the FP64 rate.
+__device__ __forceinline__ unsigned long long sl_digits(double v, int ex) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    // v = +-m 2^(max(e, 1) - 1075), so the shift to the left is at most one
+    const int sh = max(e, 1) - 1021 - ex;
+    m = ex == INT_MIN || sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 1) : (m + (1ull << (-sh - 1))) >> -sh;
+    return ((long long)b < 0 ? 0ull - m : m) + 0x80808080808080ull;
+}
+__device__ __forceinline__ unsigned long long sl_abs(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+// Planes of one row per thread: rows of bins (MM false) from B^[bin][op][j][i],
+// of macromodels from Zt[t][k'][k]; blockIdx.x = tile, blockIdx.y = matrix.
+template <bool MM>
+__global__ void __launch_bounds__(kSlRows)
+slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, size_t m0, unsigned char* __restrict__ A,
+                  double* __restrict__ rs) {
+    const size_t mat = m0 + blockIdx.y;
+    const int tile = blockIdx.x, rho = threadIdx.x, row = tile * kSlRows + rho;
+    const int rt = min(kSlRows, rows - tile * kSlRows);
+    if (rho >= rt) return;
+    const int c = row & 1;
+    const double2* s = MM ? src + (mat * n) * n + (row >> 1) : src + ((mat * 2 + ((row >> 1) & 1)) * n) * n + (row >> 2);
+    unsigned long long mx = 0;
+    for (int j = 0; j < n; ++j) {
+        const double2 v = s[(size_t)j * n];
+        mx = max(mx, max(sl_abs(v.x), sl_abs(v.y)));
+    }
+    const int ex = sl_exp(mx, n);
+    if (c == 0) rs[(mat * rows + row) >> 1] = sl_pow(ex);
+    unsigned char* out = A + (mat * rows + (size_t)tile * kSlRows) * nk16 * kSlKbBytes;
+    for (int kb = 0; kb < nk16; ++kb) {
+        uint32_t w[kSl][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int t = 0; t < kSl; ++t) w[t][q] = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int j = kb * 16 + 4 * q + b;
+                unsigned long long d = 0x80808080808080ull;
+                if (j < n) {
+                    const double2 v = s[(size_t)j * n];
+                    d = sl_digits(c ? v.y : v.x, ex);
+                }
+#pragma unroll
+                for (int t = 0; t < kSl; ++t) w[t][q] |= (uint32_t)(d >> 8 * (kSl - 1 - t) & 0xff) << (8 * b);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kSl; ++t)
+            reinterpret_cast<uint4*>(out)[(kb * kSl + t) * rt + rho] = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
+    }
+}
+
+// Digits of complex vectors v0, v0 + 1 of an x matrix (V / 2 of n entries each),
+// one pair per block: load(v, j) = entry j of vector v (zero past the live
+// ones).  The block of the last pair also clears the padding rows.
+template <typename Load>
+__device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int v0, Load&& load,
+                                              unsigned char* __restrict__ X, double* __restrict__ xs) {
+    extern __shared__ double2 s_v[];         // [2][n]
+    __shared__ unsigned long long s_mx[2];
+    __shared__ int s_ex[2];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 2) s_mx[threadIdx.x] = 0;
+    __syncthreads();
+    {
+        // half of the threads per vector
+        const int h = threadIdx.x >= blockDim.x / 2, v = v0 + h;
+        unsigned long long mx = 0;
+#pragma unroll 4
+        for (int j = threadIdx.x - h * (blockDim.x / 2); j < n; j += blockDim.x / 2) {
+            const double2 a = load(v, j);
+            s_v[h * n + j] = a;
+            mx = max(mx, max(sl_abs(a.x), sl_abs(a.y)));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) atomicMax(&s_mx[h], mx);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        const int ex = sl_exp(s_mx[threadIdx.x], n);
+        s_ex[threadIdx.x] = ex;
+        xs[v0 + threadIdx.x] = sl_pow(ex);
+    }
+    __syncthreads();
+    // 8 sources of one real vector per thread: one 16-byte chunk per digit
+    const int chunks = 4 * nst;
+    auto at = [&](int row, int ch) {
+        return reinterpret_cast<uint4*>(X + ((size_t)(ch >> 2) * Np + row) * 64 + ((ch & 3) ^ ((row >> 1) & 3)) * 16);
+    };
+    const __half2 off = __floats2half2_rn(1152.f, 1152.f);
+    for (int e = threadIdx.x; e < 4 * chunks; e += blockDim.x) {
+        const int ch = e >> 2, v = 2 * v0 + (e & 3), h = (e >> 1) & 1;
+        const int ex = s_ex[h];
+        const double* src = reinterpret_cast<const double*>(s_v + h * n) + (e & 1);
+        unsigned long long d[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const int j = 8 * ch + b;
+            d[b] = j < n ? sl_digits(src[2 * j], ex) : 0x80808080808080ull;
+        }
+#pragma unroll
+        for (int t = 0; t < kSl; ++t) {
+            const int by = kSl - 1 - t;
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                // FP16 0x6400 | byte = 1024 + byte; minus 1152 gives the digit
+                const uint32_t p = by < 4 ? __byte_perm((uint32_t)d[2 * q], (uint32_t)d[2 * q + 1], by | (4 + by) << 4)
+                                          : __byte_perm((uint32_t)(d[2 * q] >> 32), (uint32_t)(d[2 * q + 1] >> 32), (by - 4) | by << 4);
+                const uint32_t f = __byte_perm(p, 0x64646464u, 0x4140);
+                const __half2 x = __hsub2(*reinterpret_cast<const __half2*>(&f), off);
+                w[q] = *reinterpret_cast<const uint32_t*>(&x);
+            }
+            *at(t * V + v, ch) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+    if (v0 + 2 < V / 2) return;
+    for (int e = threadIdx.x; e < (Np - kSl * V) * chunks; e += blockDim.x) {
+        const int ch = e / (Np - kSl * V), row = kSl * V + e - ch * (Np - kSl * V);
+        *at(row, ch) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+// bins: vectors (r, part) of X^[bin][R][2E], r0 <= r < r0 + live (zero above)
+__global__ void __launch_bounds__(kSlSplit)
+slice_bins_kernel(const double2* __restrict__ Xg, int E, int R, int r0, int live, int nst, int V, int Np,
+                  unsigned char* __restrict__ X, double* __restrict__ xs) {
+    const size_t bin = blockIdx.x;
+    const double2* src = Xg + (bin * R + r0) * 2 * E;
+    slice_vectors(
+        E, nst, V, Np, 2 * blockIdx.y, [&](int v, int j) { return v < 2 * live ? src[(size_t)v * E + j] : make_double2(0.0, 0.0); },
+        X + bin * nst * Np * 64, xs + bin * (V / 2));
+}
+
+// macromodels: columns (cell slot, rhs) of an entry's type, x1 = U_o x gathered
+__global__ void __launch_bounds__(kSlSplit)
+slice_cells_kernel(const double2* __restrict__ x, const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn,
+                   const int2* __restrict__ ent, const int32_t* __restrict__ type_ptr,
+                   const int32_t* __restrict__ type_cells, int K, int R, int n_unique, int nst, int V, int Np,
+                   unsigned char* __restrict__ X, double* __restrict__ xs) {
+    const int2 e = ent[blockIdx.x];
+    const int c0 = type_ptr[e.x], nt = (type_ptr[e.x + 1] - c0) * R;
+    slice_vectors(
+        K, nst, V, Np, 2 * blockIdx.y,
+        [&](int v, int j) {
+            const int col = e.y + v;
+            if (col >= nt) return make_double2(0.0, 0.0);
+            const size_t at = (size_t)type_cells[c0 + col / R] * K + j;
+            const double s = (double)sgn[at];
+            const double2 a = x[(size_t)(col % R) * n_unique + idx[at]];
+            return make_double2(s * a.x, s * a.y);
+        },
+        X + (size_t)blockIdx.x * nst * Np * 64, xs + (size_t)blockIdx.x * (V / 2));
+}
+
+// columns of a launch of Rg rhs
+int sl_bin_v(int Rg) { return (4 * Rg + 7) & ~7; }
+int nk16_of(int n) { return (n + 15) / 16; }
+constexpr int kSlCellRows = sl_up16(kSl * 2 * kSlCells);   // digit rows of a macromodel entry
+int nst_of(int n) { return (n + kSlK - 1) / kSlK; }
+std::vector<int2> mm_entries(const emsurf_handle* h, int R) {
+    std::vector<int2> e;
+    for (int t = 0; t < h->T; ++t) {
+        const int n = (h->h_type_ptr[t + 1] - h->h_type_ptr[t]) * R;
+        for (int c = 0; c < n; c += kSlCells) e.push_back(make_int2(t, c));
+    }
+    return e;
+}
+
+size_t cell_digits(const emsurf_handle* h) { return (size_t)nst_of(h->K) * kSlCellRows * 64; }
+
+}  // namespace
+
+size_t slice_plane_bytes(size_t mats, int rows, int n) { return mats * rows * (size_t)nk16_of(n) * kSlKbBytes; }
+
+// Digit planes of the FP64 spectrum and of the macromodels, each left out when
+// the device-memory budget has no room for it and the work space that goes with
+// it (products then use the FP64 blocks).  The spectrum's planes of a shared
+// handle are taken over.
+int slices_build(emsurf_handle* h, const emsurf_handle* share) {
+    const int E = h->E, K = h->K;
+    const size_t nb = (size_t)h->nbins, grids = nb * (size_t)h->max_rhs * K, cells = (size_t)h->max_rhs * h->M * K;
+    const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(double);
+    const size_t zbytes = slice_plane_bytes(h->T, 2 * K, K),
+                 zrs = (size_t)h->T * K * sizeof(double) +
+                       mm_entries(h, h->max_rhs).size() * (cell_digits(h) + kSlCells * sizeof(double) + 16 * h->max_rhs);
+    if ((share && !share->sl_A) || E > kSlMaxN) return EMSURF_OK;
+    cudaStream_t st = h->setup_stream;
+    // work space still to come: grids, products, and the partials of the SIMT macromodels
+    const size_t work = (2 * grids + cells) * sizeof(double2), split = cells * sizeof(double2);
+    auto fits = [&](size_t n) { return h->budget <= 0 || h->device_bytes + (int64_t)n <= h->budget; };
+    if (share) {
+        h->sl_A = share->sl_A;
+        h->sl_rs = share->sl_rs;
+    } else {
+        if (!fits(bbytes + brs + work + kMmSplit * split) &&
+            (K > kSlMaxN || !fits(bbytes + brs + zbytes + zrs + work + split)))
+            return EMSURF_OK;
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_A, bbytes));
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_rs, brs));
+        for (size_t m0 = 0; m0 < nb; m0 += 65535) {
+            const dim3 grid((4 * E + kSlRows - 1) / kSlRows, (unsigned)std::min<size_t>(65535, nb - m0));
+            slice_rows_kernel<false><<<grid, kSlRows, 0, st>>>(h->op64.Bhat, E, 4 * E, nk16_of(E), m0, h->sl_A, h->sl_rs);
+            EMS_CUDA(cudaGetLastError());
+            h->launches += 1;
+        }
+    }
+    if (K > kSlMaxN || !fits(zbytes + zrs + work + split)) return EMSURF_OK;
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_Z, zbytes));
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_zrs, (size_t)h->T * K * sizeof(double)));
+    for (size_t m0 = 0; m0 < (size_t)h->T; m0 += 65535) {
+        const dim3 grid((2 * K + kSlRows - 1) / kSlRows, (unsigned)std::min<size_t>(65535, h->T - m0));
+        slice_rows_kernel<true><<<grid, kSlRows, 0, st>>>(h->op64.Zt, K, 2 * K, nk16_of(K), m0, h->sl_Z, h->sl_zrs);
+        EMS_CUDA(cudaGetLastError());
+        h->launches += 1;
+    }
+    return EMSURF_OK;
+}
+
+// Vector digits' work space (after the FP64 spectrum is given back).
+int slices_work(emsurf_handle* h) {
+    const int R = h->max_rhs, V = sl_bin_v(std::min(R, kSlRhs));
+    if (h->sl_Z) {
+        const size_t n = mm_entries(h, R).size();            // the most over 1..R
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_Xc, n * cell_digits(h)));
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_xcs, n * kSlCells * sizeof(double)));
+        h->sl_ent.assign(R + 1, nullptr);
+        h->sl_nent.assign(R + 1, 0);
+        for (int r = 1; r <= R; ++r) {
+            const std::vector<int2> e = mm_entries(h, r);
+            EMS_TRY(dev_alloc(h, &h->sl_ent[r], e.size() * sizeof(int2)));
+            EMS_CUDA(cudaMemcpyAsync(h->sl_ent[r], e.data(), e.size() * sizeof(int2), cudaMemcpyHostToDevice, h->setup_stream));
+            EMS_CUDA(cudaStreamSynchronize(h->setup_stream));     // e goes out of scope
+            h->sl_nent[r] = (int)e.size();
+        }
+    }
+    // bins whose digits are held at a time: all of them up to 512 MiB, fewer under
+    // a tight budget (a handle that shares its spectrum gives none back)
+    const size_t per = (size_t)nst_of(h->E) * sl_up16(kSl * V) * 64 + (V / 2) * sizeof(double);
+    size_t nb = std::min<size_t>(h->nbins, std::max<size_t>(1, ((size_t)512 << 20) / per));
+    while (nb > 16 && h->budget > 0 && h->device_bytes + (int64_t)(nb * per) > h->budget) nb = (nb + 1) / 2;
+    h->sl_bins = (int)nb;
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_X, nb * nst_of(h->E) * sl_up16(kSl * V) * 64));
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_xs, nb * (V / 2) * sizeof(double)));
+    return EMSURF_OK;
+}
+
+// Digits of x1 for the macromodel product of R rhs (reads x only).
+int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st) {
+    constexpr int V = 2 * kSlCells;
+    EMS_TRY(set_smem_once(slice_cells_kernel, 2 * h->K * sizeof(double2)));
+    slice_cells_kernel<<<dim3(h->sl_nent[R], V / 4), kSlSplit, 2 * h->K * sizeof(double2), st>>>(x, h->d_uo_index, h->d_uo_sign,
+                                                     static_cast<const int2*>(h->sl_ent[R]), h->d_type_ptr,
+                                                     h->d_type_cells, h->K, R, h->n_unique, nst_of(h->K), V,
+                                                     kSlCellRows, h->sl_Xc, h->sl_xcs);
+    EMS_CUDA(cudaGetLastError());
+    h->launches += 1;
+    return EMSURF_OK;
+}
+
+static_assert(2 * sl_up16(kSl * kSlMaxV) + 2 * (int)kSlAStep <= (int)kSlTmemCols, "TMEM columns");
+
+// Y^ = B^ X^ for every bin and Ymm = Z~ x1 for every cell, R rhs: up to kSlRhs rhs of
+// sl_bins bins per launch, the macromodels (when their planes are there) with the first.
+int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
+                    cudaStream_t st) {
+    const int E = h->E, K = h->K;
+    const int groups = (R + kSlRhs - 1) / kSlRhs, per = (R + groups - 1) / groups;
+    for (int r0 = 0; r0 < R; r0 += per)
+    for (int b0 = 0; b0 < h->nbins; b0 += h->sl_bins) {
+        const int Rg = std::min(per, R - r0);
+        SlArgs g{};
+        SlProb& b = g.p[0];
+        b.nk16 = nk16_of(E);
+        b.nst = nst_of(E);
+        b.rows = 4 * E;
+        b.tiles = (b.rows + kSlRows - 1) / kSlRows;
+        b.A = h->sl_A + slice_plane_bytes(b0, b.rows, E);
+        b.rs = h->sl_rs + (size_t)b0 * 2 * E;
+        b.X = h->sl_X;
+        b.xs = h->sl_xs;
+        b.V = sl_bin_v(Rg);
+        b.live = Rg;
+        b.Np = sl_up16(kSl * b.V);
+        b.xmats = std::min(h->sl_bins, h->nbins - b0);
+        b.items = b.xmats * b.tiles;
+        const size_t y0 = (size_t)b0 * R * 2 * E;
+        EMS_TRY(set_smem_once(slice_bins_kernel, 2 * E * sizeof(double2)));
+        slice_bins_kernel<<<dim3(b.xmats, b.V / 4), kSlSplit, 2 * E * sizeof(double2), st>>>(
+            Xg + y0, E, R, r0, Rg, b.nst, b.V, b.Np, h->sl_X, h->sl_xs);
+        EMS_CUDA(cudaGetLastError());
+        SlProb& m = g.p[1];
+        m.A = h->sl_Z;
+        m.rs = h->sl_zrs;
+        m.X = h->sl_Xc;
+        m.xs = h->sl_xcs;
+        m.nk16 = nk16_of(K);
+        m.nst = nst_of(K);
+        m.rows = 2 * K;
+        m.tiles = (m.rows + kSlRows - 1) / kSlRows;
+        m.V = 2 * kSlCells;
+        m.Np = sl_up16(kSl * m.V);
+        m.xmats = r0 == 0 && b0 == 0 && h->sl_Z ? h->sl_nent[R] : 0;
+        m.items = m.xmats * m.tiles;
+        const int dc = std::max(b.Np, m.items ? m.Np : 0), vmax = std::max(b.V, m.items ? m.V : 0);
+        g.d_step = dc;
+        g.slots = 2 * dc + kSlMaxSlots * (int)kSlAStep <= (int)kSlTmemCols ? kSlMaxSlots : 2;
+        g.z_bytes = (kSl - 1) * vmax * 64;
+        g.x_bytes = dc * 64;
+        const size_t xring = (size_t)kSlXStages * (g.z_bytes + g.x_bytes);
+        g.stages = std::min(kSlMaxStages, (int)((kSlSmemMax - 1024 - xring) / kSlABytes));
+        g.Y = Yg + y0;
+        g.E = E;
+        g.R = R;
+        g.r0 = r0;
+        for (int c = 0; c < 4; ++c) g.co[c] = coef[c];
+        g.Ymm = Ymm;
+        g.ent = h->sl_Z ? static_cast<const int2*>(h->sl_ent[R]) : nullptr;
+        g.type_ptr = h->d_type_ptr;
+        g.type_cells = h->d_type_cells;
+        g.K = K;
+        g.M = h->M;
+        g.err = h->d_err;
+        const size_t smem = 1024 + (size_t)g.stages * kSlABytes + xring;
+        const int grid = std::min(std::max(1, h->num_sms), b.items + m.items);
+        EMS_TRY(set_smem_once(slices_kernel, smem));
+        slices_kernel<<<grid, kSlThreads, smem, st>>>(g);
+        EMS_CUDA(cudaGetLastError());
+        h->launches += 2;
+    }
+    return EMSURF_OK;
+}
+
+}  // namespace emsurf
