@@ -254,6 +254,7 @@ struct emsurf_handle {
     float tc_tune_ms[2] = {0.f, 0.f};      // the two shapes' times at create
     int mm_occ[4] = {0, 0, 0, 0};          // resident macromodel CTAs per SM (FP32, FP64; x 1 / 4 rhs)
     int mm_threads[4] = {0, 0, 0, 0};      // macromodel block size per variant
+    int bm_occ[9] = {};                    // resident CTAs per SM of the full-spectrum multiply of 1..8 rhs
     int mm2_occ = 0;                       // resident single-rhs FP32 macromodel CTAs per SM
     cudaStream_t setup_stream = nullptr;   // stream of the create-time work
     cudaStream_t side_stream = nullptr;    // the macromodel product beside the bin multiply

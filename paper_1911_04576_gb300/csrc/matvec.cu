@@ -196,7 +196,7 @@ __global__ void binmul_kernel(const T2* __restrict__ Bhat, const T2* __restrict_
     }
 }
 
-// ------------------------------------------------ K2, FP32, one rhs: TMA-fed
+// ------------------------------------------------ K2, FP32, full spectrum: TMA-fed
 // Persistent CTAs walk their bins as a sequence of stages; a stage is a block
 // of JB source columns j of L^T and K^T (two contiguous JB x E slabs, since j
 // is the outer index), brought into a ring of kBmStages shared-memory slots
@@ -205,8 +205,13 @@ __global__ void binmul_kernel(const T2* __restrict__ Bhat, const T2* __restrict_
 // copies; the other warps own one test row i each and release a slot with an
 // mbarrier arrive.  Every wait is bounded: on expiry the kernel sets *err,
 // the producer waits (bounded) for its copies in flight, and all return.
+// Up to 8 rhs share one pass over the spectrum (16 FMA per element and rhs: HBM
+// bounds up to 3 rhs, the FP32 rate more).  40 x 25 bins, K = 324, 3 rhs (420 MB):
+// 118 us, 229 us in two passes of binmul_kernel, which stays for other E.
 constexpr int kBmJB = 8;
 constexpr int kBmStages = 4;
+constexpr int kBmMaxRhs = 8;             // rhs whose accumulators a thread holds
+constexpr int kBmMaxThreads = 512;       // of a CTA with several rhs (128 registers each)
 constexpr long long kWaitLimit = 1LL << 22;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -266,14 +271,15 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
-__global__ void binmul_tma_kernel(const float2* __restrict__ Bhat, const float2* __restrict__ Xh,
-                                  float2* __restrict__ Yh, int E, int nbins, float2 ca, float2 cb,
-                                  float2 cg, float2 cd, int* __restrict__ err) {
+template <int RB>
+__global__ void __launch_bounds__(RB == 1 ? 1024 : kBmMaxThreads)
+binmul_tma_kernel(const float2* __restrict__ Bhat, const float2* __restrict__ Xh, float2* __restrict__ Yh, int E,
+                  int nbins, int R, int r0, float2 ca, float2 cb, float2 cg, float2 cd, int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int stage_elems = 2 * kBmJB * E;
+    const int stage_elems = 2 * kBmJB * E, K = 2 * E;
     float2* sbuf = reinterpret_cast<float2*>(smem_raw);
-    float2* xbuf = sbuf + (size_t)kBmStages * stage_elems;      // [2][2E]
-    uint64_t* full = reinterpret_cast<uint64_t*>(xbuf + 4 * E);
+    float2* xbuf = sbuf + (size_t)kBmStages * stage_elems;      // [2][RB][2E]
+    uint64_t* full = reinterpret_cast<uint64_t*>(xbuf + 2 * RB * K);
     uint64_t* empty = full + kBmStages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ncw = (E + 31) / 32;
@@ -288,65 +294,95 @@ __global__ void binmul_tma_kernel(const float2* __restrict__ Bhat, const float2*
     __syncthreads();
     const int nloc = (nbins - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const int nj = (E + kBmJB - 1) / kBmJB;
-    const long long total = (long long)nloc * nj;
+    const int total = nloc * nj;
+    const int live = min(RB, R - r0);
     if (warp == 0) {
         if (lane != 0) return;
         const uint64_t pol = l2_evict_first();
-        long long issued = 0;
+        int issued = 0;
         bool ok = true;
-        for (long long q = 0; q < total; ++q) {
-            const int s = (int)(q % kBmStages);
+        for (int q = 0, t = 0, jb = 0; q < total; ++q) {
+            const int s = q % kBmStages;
             if (q >= kBmStages && !mbar_wait(&empty[s], (uint32_t)((q / kBmStages - 1) & 1))) {
                 ok = false;
                 break;
             }
-            const int t = (int)(q / nj), jb = (int)(q % nj);
             const int bin = (int)blockIdx.x + t * (int)gridDim.x;
             const int j0 = jb * kBmJB, jn = min(kBmJB, E - j0);
             const uint32_t bytes_op = (uint32_t)(jn * E * sizeof(float2));
-            const uint32_t bytes_x = (uint32_t)(2 * E * sizeof(float2));
+            const uint32_t bytes_x = (uint32_t)(live * K * sizeof(float2));
             mbar_expect_tx(&full[s], 2 * bytes_op + (jb == 0 ? bytes_x : 0u));
             const float2* src = Bhat + (size_t)bin * 2 * E * E + (size_t)j0 * E;
             float2* dst = sbuf + (size_t)s * stage_elems;
             bulk_g2s_hint(dst, src, bytes_op, &full[s], pol);
             bulk_g2s_hint(dst + kBmJB * E, src + (size_t)E * E, bytes_op, &full[s], pol);
-            if (jb == 0) bulk_g2s(xbuf + (t & 1) * 2 * E, Xh + (size_t)bin * 2 * E, bytes_x, &full[s]);
+            if (jb == 0) bulk_g2s(xbuf + (t & 1) * RB * K, Xh + ((size_t)bin * R + r0) * K, bytes_x, &full[s]);
             issued = q + 1;
+            if (++jb == nj) {
+                jb = 0;
+                ++t;
+            }
         }
         if (!ok) {
             atomicExch(err, 1);
             // wait (bounded) for the copies still in flight before leaving
-            for (long long q = (issued > kBmStages ? issued - kBmStages : 0); q < issued; ++q)
+            for (int q = (issued > kBmStages ? issued - kBmStages : 0); q < issued; ++q)
                 mbar_wait(&full[q % kBmStages], (uint32_t)((q / kBmStages) & 1));
         }
         return;
     }
     const int i = (warp - 1) * 32 + lane;
-    float2 lj = make_float2(0.f, 0.f), lm = lj, kj = lj, km = lj;
-    for (long long q = 0; q < total; ++q) {
-        const int s = (int)(q % kBmStages);
-        const int t = (int)(q / nj), jb = (int)(q % nj);
+    float2 lj[RB], lm[RB], kj[RB], km[RB];
+    for (int q = 0, t = 0, jb = 0; q < total; ++q) {
+        const int s = q % kBmStages;
         if (!mbar_wait(&full[s], (uint32_t)((q / kBmStages) & 1))) {
             atomicExch(err, 1);
             return;
         }
-        if (jb == 0) lj = lm = kj = km = make_float2(0.f, 0.f);
+        if (jb == 0) {
+#pragma unroll
+            for (int r = 0; r < RB; ++r) lj[r] = lm[r] = kj[r] = km[r] = make_float2(0.f, 0.f);
+        }
         const float2* Ls = sbuf + (size_t)s * stage_elems;
         const float2* Ks = Ls + kBmJB * E;
-        const float2* xs = xbuf + (t & 1) * 2 * E;
+        const float2* xs = xbuf + (t & 1) * RB * K;
         const int j0 = jb * kBmJB, jn = min(kBmJB, E - j0);
         if (i < E) {
+            if constexpr (RB == 1) {
 #pragma unroll
-            for (int jj = 0; jj < kBmJB; ++jj) {
-                if (jj < jn) {
-                    const float2 l = Ls[jj * E + i];
-                    const float2 k = Ks[jj * E + i];
-                    const float2 xj = xs[j0 + jj];
-                    const float2 xm = xs[E + j0 + jj];
-                    cfma(lj, l, xj);
-                    cfma(lm, l, xm);
-                    cfma(kj, k, xj);
-                    cfma(km, k, xm);
+                for (int jj = 0; jj < kBmJB; ++jj) {
+                    if (jj < jn) {
+                        const float2 l = Ls[jj * E + i];
+                        const float2 k = Ks[jj * E + i];
+                        const float2 xj = xs[j0 + jj];
+                        const float2 xm = xs[E + j0 + jj];
+                        cfma(lj[0], l, xj);
+                        cfma(lm[0], l, xm);
+                        cfma(kj[0], k, xj);
+                        cfma(km[0], k, xm);
+                    }
+                }
+            } else {
+                // two sources at a time: their x in one 16-byte load (E is even)
+#pragma unroll
+                for (int jj = 0; jj < kBmJB; jj += 2) {
+                    if (jj < jn) {
+                        const float2 l0 = Ls[jj * E + i], l1 = Ls[jj * E + E + i];
+                        const float2 k0 = Ks[jj * E + i], k1 = Ks[jj * E + E + i];
+#pragma unroll
+                        for (int r = 0; r < RB; ++r) {
+                            const float4 xj = *reinterpret_cast<const float4*>(xs + r * K + j0 + jj);
+                            const float4 xm = *reinterpret_cast<const float4*>(xs + r * K + E + j0 + jj);
+                            cfma(lj[r], l0, make_float2(xj.x, xj.y));
+                            cfma(lm[r], l0, make_float2(xm.x, xm.y));
+                            cfma(kj[r], k0, make_float2(xj.x, xj.y));
+                            cfma(km[r], k0, make_float2(xm.x, xm.y));
+                            cfma(lj[r], l1, make_float2(xj.z, xj.w));
+                            cfma(lm[r], l1, make_float2(xm.z, xm.w));
+                            cfma(kj[r], k1, make_float2(xj.z, xj.w));
+                            cfma(km[r], k1, make_float2(xm.z, xm.w));
+                        }
+                    }
                 }
             }
         }
@@ -354,16 +390,36 @@ __global__ void binmul_tma_kernel(const float2* __restrict__ Bhat, const float2*
         if (lane == 0) mbar_arrive(&empty[s]);
         if (jb == nj - 1 && i < E) {
             const int bin = (int)blockIdx.x + t * (int)gridDim.x;
-            float2* Y = Yh + (size_t)bin * 2 * E;
-            Y[i] = cadd(cmul(ca, lj), cmul(cb, km));
-            Y[E + i] = cadd(cmul(cg, kj), cmul(cd, lm));
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                if (r < live) {
+                    float2* Y = Yh + ((size_t)bin * R + r0 + r) * K;
+                    Y[i] = cadd(cmul(ca, lj[r]), cmul(cb, km[r]));
+                    Y[E + i] = cadd(cmul(cg, kj[r]), cmul(cd, lm[r]));
+                }
+            }
+        }
+        if (++jb == nj) {
+            jb = 0;
+            ++t;
         }
     }
 }
 
-size_t binmul_tma_smem(int E) {
-    return (size_t)kBmStages * 2 * kBmJB * E * sizeof(float2) + 4ull * E * sizeof(float2) +
+size_t binmul_tma_smem(int E, int rb) {
+    return (size_t)kBmStages * 2 * kBmJB * E * sizeof(float2) + 4ull * rb * E * sizeof(float2) +
            2ull * kBmStages * sizeof(uint64_t);
+}
+// rhs per launch: all of up to kBmMaxRhs in one pass over the spectrum, more in equal groups
+int binmul_tma_rhs(int R) {
+    const int groups = (R + kBmMaxRhs - 1) / kBmMaxRhs;
+    return (R + groups - 1) / groups;
+}
+// the x double buffer needs at least kBmStages stages per bin; the copies'
+// sizes and the pairwise reads of x need an even E
+bool binmul_tma_ok(int E, int rb) {
+    return binmul_tma_smem(E, rb) <= 227 * 1024 && E + 32 <= (rb == 1 ? 1024 : kBmMaxThreads) &&
+           E % 2 == 0 && (E + kBmJB - 1) / kBmJB >= kBmStages;
 }
 
 // ------------------------------------------------ K2, FP32, one rhs, half spectrum
@@ -1701,15 +1757,37 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
             h->launches += 1;
             bin_done = true;
         }
-        const size_t smem = binmul_tma_smem(E);
-        // the x double buffer needs at least kBmStages stages per bin
-        if (!bin_done && R == 1 && smem <= 227 * 1024 && E + 32 <= 1024 && (E + kBmJB - 1) / kBmJB >= kBmStages) {
-            EMS_TRY(set_smem_once(binmul_tma_kernel, smem));
-            const int grid = std::min(nb, std::max(1, h->num_sms));
-            binmul_tma_kernel<<<grid, 32 * (1 + (E + 31) / 32), smem, st>>>(
-                op.Bhat, op.Xg, op.Yg, E, nb, op.coef[0], op.coef[1], op.coef[2], op.coef[3], h->d_err);
-            EMS_CUDA(cudaGetLastError());
-            h->launches += 1;
+        const int rb = binmul_tma_rhs(R);
+        if (!bin_done && binmul_tma_ok(E, rb)) {
+            const size_t smem = binmul_tma_smem(E, rb);
+            const int threads_tma = 32 * (1 + (E + 31) / 32);
+            auto go = [&](auto kern, int r0) -> int {
+                EMS_TRY(set_smem_once(kern, smem));
+                int& occ = h->bm_occ[rb];
+                if (!occ) {
+                    int b = 0;
+                    EMS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, threads_tma, smem));
+                    occ = std::max(b, 1);
+                }
+                const int grid = std::min(nb, std::max(1, h->num_sms) * (rb == 1 ? 1 : occ));
+                kern<<<grid, threads_tma, smem, st>>>(op.Bhat, op.Xg, op.Yg, E, nb, R, r0, op.coef[0], op.coef[1],
+                                                      op.coef[2], op.coef[3], h->d_err);
+                EMS_CUDA(cudaGetLastError());
+                h->launches += 1;
+                return EMSURF_OK;
+            };
+            for (int r0 = 0; r0 < R; r0 += rb) {
+                switch (rb) {
+                    case 1: EMS_TRY(go(binmul_tma_kernel<1>, r0)); break;
+                    case 2: EMS_TRY(go(binmul_tma_kernel<2>, r0)); break;
+                    case 3: EMS_TRY(go(binmul_tma_kernel<3>, r0)); break;
+                    case 4: EMS_TRY(go(binmul_tma_kernel<4>, r0)); break;
+                    case 5: EMS_TRY(go(binmul_tma_kernel<5>, r0)); break;
+                    case 6: EMS_TRY(go(binmul_tma_kernel<6>, r0)); break;
+                    case 7: EMS_TRY(go(binmul_tma_kernel<7>, r0)); break;
+                    default: EMS_TRY(go(binmul_tma_kernel<8>, r0)); break;
+                }
+            }
             bin_done = true;
         }
     }
