@@ -441,11 +441,7 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         EMS_TRY(slab_cell_plan(a, b, h, n, zlevels, sides[t], patch_n, ring_layers, plan[t]));
         E = plan[t].E;
         SlabType& T = ty[t];
-        for (int v = 0; v < 2; ++v) {
-            T.Ev[v] = plan[t].region[v].E;
-            T.offL[v] = nLK;
-            nLK += 2ll * T.Ev[v] * T.Ev[v];
-        }
+        for (int v = 0; v < 2; ++v) T.Ev[v] = plan[t].region[v].E;
         T.N = plan[t].N;
         T.nint = plan[t].n_int;
         T.offB = nB;
@@ -454,6 +450,12 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         nMap += 2ll * T.N;
         max_nint = std::max(max_nint, T.nint);
     }
+    // the tables of one region's types lie one after another
+    for (int v = 0; v < 2; ++v)
+        for (SlabType& T : ty) {
+            T.offL[v] = nLK;
+            nLK += 2ll * T.Ev[v] * T.Ev[v];
+        }
     const int K = 2 * E;
     // region wavenumbers: air k0, slab k0 sqrt(eps) (principal root, Im <= 0)
     const double er = eps_slab.re, ei = eps_slab.im, mod = std::sqrt(er * er + ei * ei);
@@ -480,17 +482,23 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
     alloc((void**)&dsgn, nMap);
     alloc((void**)&dty, sizeof(SlabType) * n_types);
     alloc((void**)&dstat, sizeof(int));
-    const double zero3[3] = {0.0, 0.0, 0.0};
-    const int8_t one = 1;
     std::vector<int32_t> hcpy(nMap);
     std::vector<int8_t> hsgn(nMap);
-    for (int t = 0; t < n_types && !status; ++t) {
-        for (int v = 0; v < 2 && !status; ++v) {
-            const SlabRegionMesh& rm = plan[t].region[v];
-            const MeshView mv{rm.verts.data(), rm.tris.data(), rm.slot_rwg.data(), rm.slot_sgn.data(), rm.T, rm.E};
-            double2* L = LK + ty[t].offL[v];
-            status = tabulate_blocks_cx(mv, mv, zero3, &one, 1, kv_re[v], kv_im[v], L,
-                                        L + (size_t)rm.E * rm.E, st);
+    auto view = [&](int t, int v) {
+        const SlabRegionMesh& rm = plan[t].region[v];
+        return MeshView{rm.verts.data(), rm.tris.data(), rm.slot_rwg.data(), rm.slot_sgn.data(), rm.T, rm.E};
+    };
+    for (int v = 0; v < 2 && !status; ++v) {
+        // runs of types with meshes of the same size in one go: one type's pairs
+        // fill the chip less than twice
+        for (int t = 0; t < n_types && !status;) {
+            std::vector<MeshView> cells;
+            const int t0 = t;
+            for (; t < n_types && plan[t].region[v].T == plan[t0].region[v].T && plan[t].region[v].E == plan[t0].region[v].E; ++t)
+                cells.push_back(view(t, v));
+            status = tabulate_cells_cx(cells, kv_re[v], kv_im[v], LK + ty[t0].offL[v], st);
+        }
+        for (int t = 0; t < n_types; ++t) {
             std::copy(plan[t].copy[v].begin(), plan[t].copy[v].end(), hcpy.begin() + ty[t].offMap + (size_t)v * ty[t].N);
             std::copy(plan[t].sgn[v].begin(), plan[t].sgn[v].end(), hsgn.begin() + ty[t].offMap + (size_t)v * ty[t].N);
         }

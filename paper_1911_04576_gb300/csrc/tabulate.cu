@@ -83,36 +83,33 @@ __device__ __forceinline__ void green_far(double R2, double k, double kpi, doubl
     gfac = make_double2(m * fma(-kR, G.y, G.x), m * fma(kR, G.x, G.y));
 }
 
-// remainder after removing 1/R (times 4 pi): power series for kR < 0.5 (no
-// cancellation), closed form otherwise
-__device__ __forceinline__ void green_smooth(double R, double k, double kpi, double2& Gs, double2& gfac) {
-    const double z = k * R;
+// 1/R (refined) and R of R2 = R^2 > 0
+__device__ __forceinline__ double inv_dist(double R2, double& R) {
+    const double ri = rsqrt(R2), R1 = R2 * ri;
+    R = fma(0.5 * ri, fma(-R1, R1, R2), R1);
+    return ri;
+}
+
+// Remainder after removing 1/R (times 4 pi), (e^{-jz} - 1) / R and
+// (1 - (1 + jz) e^{-jz}) / R^3 for z = kR.  With the sine s and cosine c of z / 2
+// no difference of near-equal terms is left (1 - cos z = 2 s^2,
+// 1 - cos z - z sin z = 2 s (s - z c)) but one: sin z - z cos z takes its power
+// series below 0.5.
+__device__ __forceinline__ void green_smooth(double R2, double k, double kpi, double2& Gs, double2& gfac) {
+    double R, s, c;
+    const double ri = inv_dist(R2, R), z = k * R;
+    sincospi(0.5 * kpi * R, &s, &c);
+    const double s2 = 2.0 * s, sn = s2 * c, ri3 = ri * ri * ri;
+    Gs = make_double2(-s2 * s * ri, -sn * ri);
+    gfac.x = s2 * fma(-z, c, s) * ri3;
     if (z < 0.5) {
-        // (e^{-jz} - 1) / R and (1 - (1 + jz) e^{-jz}) / R^3 with e^{-jz} = cos z - j sin z:
-        // real and imaginary parts are even/odd series in w = z^2
+        // (sin z - z cos z) / z^3 = sum (-1)^(m+1) 2m / (2m + 1)! w^(m-1), w = z^2
         const double w = z * z;
         constexpr double f3 = 1.0 / 6, f5 = f3 / 20, f7 = f5 / 42, f9 = f7 / 72, f11 = f9 / 110, f13 = f11 / 156, f15 = f13 / 210;
-        constexpr double f2 = 0.5, f4 = f2 / 12, f6 = f4 / 30, f8 = f6 / 56, f10 = f8 / 90, f12 = f10 / 132, f14 = f12 / 182, f16 = f14 / 240;
-        // (1 - cos z) / w, sin z / z
-        const double pc = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, f14, -f12), f10), -f8), f6), -f4), f2);
-        const double ps = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, f15, -f13), f11), -f9), f7), -f5), f3);
-        // sin z / z = 1 - w (f3 - w f5 + w^2 f7 - ...)
-        Gs = make_double2(-k * z * pc, -k * fma(-w, ps, 1.0));
-        // (1 - cos z - z sin z) / w = sum (-1)^m (2m - 1) / (2m)! w^(m-1)
-        const double qr = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, 15 * f16, -13 * f14), 11 * f12), -9 * f10), 7 * f8), -5 * f6), 3 * f4), -f2);
-        // (sin z - z cos z) / z^3 = sum (-1)^(m+1) 2m / (2m + 1)! w^(m-1)
-        const double qi = fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, 14 * f15, -12 * f13), 10 * f11), -8 * f9), 6 * f7), -4 * f5), 2 * f3);
-        const double ri = R > 0.0 ? 1.0 / R : 0.0;
-        const double k2 = k * k;
-        gfac = make_double2(k2 * ri * qr, R > 0.0 ? k2 * k * qi : 0.0);
-        return;
+        gfac.y = k * k * k * fma(w, fma(w, fma(w, fma(w, fma(w, fma(w, 14 * f15, -12 * f13), 10 * f11), -8 * f9), 6 * f7), -4 * f5), 2 * f3);
+    } else {
+        gfac.y = ri3 * fma(-z, fma(-s2, s, 1.0), sn);
     }
-    const double ri = 1.0 / R;
-    double s, c;
-    sincospi(kpi * R, &s, &c);
-    Gs = make_double2((c - 1.0) * ri, -s * ri);
-    const double ri3 = ri * ri * ri;
-    gfac = make_double2(ri3 * (1.0 - fma(z, s, c)), ri3 * fma(-z, c, s));
 }
 
 // Lossy region (Sec. II-B, k_v = w sqrt(mu0 eps_v) with complex eps_v): the
@@ -133,42 +130,56 @@ __device__ __forceinline__ void green_far_cx(double R2, double kr, double kpi, d
     gfac = make_double2(ae.x * d, ae.y * d);
 }
 
-__device__ __forceinline__ void green_smooth_cx(double R, double kr, double kpi, double ki, double2& Gs,
+// e^a - 1: Taylor polynomial (relative error below 2^-57) for |a| < 1/64 (low loss)
+__device__ __forceinline__ double expm1_small(double a) {
+    if (fabs(a) < 0x1p-6) {
+        constexpr double f2 = 1.0 / 2, f3 = f2 / 3, f4 = f3 / 4, f5 = f4 / 5, f6 = f5 / 6, f7 = f6 / 7;
+        return a * fma(a, fma(a, fma(a, fma(a, fma(a, fma(a, f7, f6), f5), f4), f3), f2), 1.0);
+    }
+    return expm1(a);
+}
+
+__device__ __forceinline__ void green_smooth_cx(double R2, double kr, double kpi, double ki, double2& Gs,
                                                 double2& gfac) {
+    double R, s, c;
+    const double ri = inv_dist(R2, R);
     const double2 z = make_double2(ki * R, -kr * R);                    // -jkR
-    const double2 jk = make_double2(ki, -kr);                           // -jk
-    if (z.x * z.x + z.y * z.y < 0.25) {
-        // (e^z - 1) / z = sum z^m / (m + 1)!, (1 - (1 - z) e^z) / z^2 = sum z^m (m + 1) / (m + 2)!
-        double2 g = make_double2(0.0, 0.0), h = make_double2(0.0, 0.0);
+    sincospi(0.5 * kpi * R, &s, &c);
+    const double em = expm1_small(z.x), s2 = 2.0 * s;
+    const double cs = fma(-s2, s, 1.0), sn = s2 * c, ez = 1.0 + em;
+    Gs = make_double2(fma(em, cs, -s2 * s) * ri, -ez * sn * ri);        // (e^z - 1) / R
+    const double r = 2.0 * z.x, q = fma(z.x, z.x, z.y * z.y);
+    if (q < 0.25) {
+        // (1 - (1 - z) e^z) / z^2 = sum z^m (m + 1) / (m + 2)!, the real polynomial at a
+        // complex point by the recurrence of z^2 = 2 Re z z - |z|^2 (Knuth 4.6.4)
+        double b1 = 0.0, b0 = 0.0;
 #pragma unroll
-        for (int m = 14; m >= 0; --m) {
+        for (int m = 14; m >= 1; --m) {
             double f = 1.0;
 #pragma unroll
-            for (int i = 2; i <= m + 1; ++i) f /= i;                    // 1 / (m + 1)!
-            g = cmul(g, z);
-            g.x += f;
-            h = cmul(h, z);
-            h.x += f * (m + 1) / (m + 2);
+            for (int i = 2; i <= m + 2; ++i) f /= i;                    // 1 / (m + 2)!
+            const double t = fma(r, b0, fma(-q, b1, f * (m + 1)));
+            b1 = b0;
+            b0 = t;
         }
-        Gs = cmul(jk, g);
-        const double ri = R > 0.0 ? 1.0 / R : 0.0;
-        const double2 k2 = cmul(jk, jk);
-        const double2 hh = cmul(k2, h);
+        // h = 1/2 - |z|^2 b1 + z b0
+        const double hx = fma(z.x, b0, fma(-q, b1, 0.5)), hy = z.y * b0;
+        const double2 jk = make_double2(ki, -kr), hh = cmul(cmul(jk, jk), make_double2(hx, hy));
         gfac = make_double2(hh.x * ri, hh.y * ri);
         return;
     }
-    const double ri = 1.0 / R;
-    const double2 e = exp_mjkR(R, kpi, ki);
-    Gs = make_double2((e.x - 1.0) * ri, e.y * ri);
-    const double2 ae = cmul(make_double2(1.0 - ki * R, kr * R), e);
+    const double2 ae = cmul(make_double2(1.0 - z.x, -z.y), make_double2(ez * cs, -ez * sn));
     const double ri3 = ri * ri * ri;
     gfac = make_double2((1.0 - ae.x) * ri3, -ae.y * ri3);
 }
 
 __device__ __forceinline__ double edge_log(double lp, double lm, double Rp, double Rm, double R02) {
-    if (lm >= 0.0) return log((Rp + lp) / (Rm + lm));
-    if (lp <= 0.0) return log((Rm - lm) / (Rp - lp));
-    return log((Rp + lp) * (Rm - lm) / R02);
+    // the operands are chosen first: one division and one logarithm for all lanes
+    const bool ahead = lm >= 0.0, behind = lp <= 0.0;
+    const double sp = Rp + lp, sm = Rm - lm;
+    const double num = ahead ? sp : behind ? sm : sp * sm;
+    const double den = ahead ? Rm + lm : behind ? Rp - lp : R02;
+    return log(num / den);
 }
 
 // closed-form int 1/R, int (rho'-rho)/R, int grad_r(1/R) over source triangle;
@@ -178,28 +189,49 @@ __device__ __forceinline__ void potentials(Vec3 r, const TriGeo& T, double& I0, 
     double d = dot(n, r - v0);
     if (fabs(d) <= 1e-9 * T.scale) d = 0.0;
     rho = r - d * n;
-    const double ad = fabs(d);
+    const double ad = fabs(d), d2 = d * d;
     I0 = 0.0;
     I1 = {0.0, 0.0, 0.0};
     Vec3 fu = {0.0, 0.0, 0.0};
-    double bsum = 0.0;
+    // distances to the vertices, each the end of two edges
+    Vec3 a[3];
+    double Rv[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const Vec3 a = v3(T.v + 3 * i), b = v3(T.v + 3 * ((i + 1) % 3));
+        a[i] = v3(T.v + 3 * i) - rho;
+        Rv[i] = sqrt(dot(a[i], a[i]) + d2);
+    }
+    // the edges' angles atan2(t l, R02 + |d| R), ends' difference, add up to the
+    // solid angle: one atan2 of the product of the three complex numbers
+    const double iu = 1.0 / fma(T.scale, T.scale, d2);
+    double px = 1.0, py = 0.0;
+    bool inside = true;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
         const Vec3 lh = v3(T.lh + 3 * i), u = v3(T.u + 3 * i);
-        const double lp = dot(b - rho, lh), lm = dot(a - rho, lh);
-        const double t = dot(a - rho, u);
-        const double R02 = t * t + d * d;
-        const double Rp = sqrt(R02 + lp * lp), Rm = sqrt(R02 + lm * lm);
+        const double lp = dot(a[(i + 1) % 3], lh), lm = dot(a[i], lh);
+        const double t = dot(a[i], u);
+        const double R02 = t * t + d2;
+        const double Rp = Rv[(i + 1) % 3], Rm = Rv[i];
         const double f = edge_log(lp, lm, Rp, Rm, R02);
         I0 += t * f;
         I1 = I1 + (0.5 * (R02 * f + lp * Rp - lm * Rm)) * u;
         fu = fu + f * u;
         if (ad > 0.0) {
-            // difference of the two angles atan2(t l, R02 + |d| R), both inside (-pi/2, pi/2)
-            const double xp = R02 + ad * Rp, xm = R02 + ad * Rm, yp = t * lp, ym = t * lm;
-            bsum += atan2(yp * xm - xp * ym, xp * xm + yp * ym);
+            // in units of the triangle's size, so that the products stay in range
+            const double xp = fma(ad, Rp, R02), xm = fma(ad, Rm, R02), yp = t * lp, ym = t * lm;
+            const double X = (xp * iu) * (xm * iu) + (yp * iu) * (ym * iu), Y = (yp * iu) * (xm * iu) - (xp * iu) * (ym * iu);
+            const double nx = px * X - py * Y;
+            py = px * Y + py * X;
+            px = nx;
+            inside = inside && t > 0.0;
         }
+    }
+    double bsum = 0.0;
+    if (ad > 0.0) {
+        // in [0, pi] unless the projection is inside the triangle: there up to 2 pi
+        bsum = atan2(py, px);
+        if (inside && bsum < 0.0) bsum += 6.283185307179586476925286766559;
     }
     I0 -= ad * bsum;
     const double sg = (d > 0.0) - (d < 0.0);
@@ -222,19 +254,24 @@ __device__ __forceinline__ void potentials(Vec3 r, const TriGeo& T, double& I0, 
 // distance, rsqrt, sincospi and 7 operations for the moments are left per
 // point pair, 0.135 ns on average over 25 blocks of 192 x 192 triangles
 // (6.1 ms), against 0.37 ns (16.6 ms) when each point pair updated the 9 + 9
-// slot integrals.
+// slot integrals.  With closed-form parts (32 cells of 256 + 192 triangles in
+// batches that fill the chip, 160 M point pairs): 59 ms, 100 ms with a full
+// series beside the closed form of the remainder, three branches with a
+// logarithm each per edge and three atan2 per point.
 template <bool CX, bool SING>
 __global__ void __launch_bounds__(128)
-tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict__ sg, int Ts,
+tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict__ sg, int Ts, int own,
                  const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out) {
     const int pair = blockIdx.x * blockDim.x + threadIdx.x;
     if (pair >= Tt * Ts) return;
     const int t = pair / Ts, s = pair - t * Ts;
     const int bl = blockIdx.y;
-    const TriGeo& A = tg[t];
-    const TriGeo& S = sg[s];
-    const Vec3 sh = v3(shifts + 3 * (b0 + bl));
+    // own: every block has its own mesh, test = source, not shifted
+    const TriGeo& A = tg[(own ? (b0 + bl) * Tt : 0) + t];
+    const TriGeo& S = sg[(own ? (b0 + bl) * Ts : 0) + s];
+    const Vec3 sh = own ? Vec3{0.0, 0.0, 0.0} : v3(shifts + 3 * (b0 + bl));
     const double kpi = k * 0.31830988618379067154;
+    const double tiny2 = (1e-9 * S.scale) * (1e-9 * S.scale);
     // [G.x, G.y, g.x, g.y] of the moments
     double M[3][3][4];
 #pragma unroll
@@ -267,10 +304,14 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
             if constexpr (SING) {
                 // coincident points (up to rounding) take the R -> 0 limit of the
                 // remainder: -jk/(4 pi) and no gradient term
-                double R = sqrt(R2);
-                if (R <= 1e-9 * S.scale) R = 0.0;
-                if constexpr (CX) green_smooth_cx(R, k, kpi, ki, G, g);
-                else green_smooth(R, k, kpi, G, g);
+                const bool same = R2 <= tiny2;
+                const double Rs = same ? tiny2 : R2;
+                if constexpr (CX) green_smooth_cx(Rs, k, kpi, ki, G, g);
+                else green_smooth(Rs, k, kpi, G, g);
+                if (same) {
+                    G = make_double2(CX ? ki : 0.0, -k);
+                    g = make_double2(0.0, 0.0);
+                }
             } else {
                 if constexpr (CX) green_far_cx(R2, k, kpi, ki, G, g);
                 else green_far(R2, k, kpi, G, g);
@@ -385,10 +426,10 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
 }
 
 // L[o][m][n], K[o][m][n], o = slot[b] (b without a slot list), from the slot
-// integrals of one chunk
+// integrals of one chunk; own: every block's own RWGs, its K after its L
 __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots* __restrict__ tr,
                                   int Et, const RwgSlots* __restrict__ sr, int Es, int Tt, int Ts,
-                                  int b0, int nb, const int32_t* __restrict__ slot, double2* __restrict__ L,
+                                  int b0, int nb, int own, const int32_t* __restrict__ slot, double2* __restrict__ L,
                                   double2* __restrict__ K) {
     const size_t total = (size_t)nb * Et * Es;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
@@ -397,7 +438,7 @@ __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots*
         const size_t t2 = e / Es;
         const int m = (int)(t2 % Et);
         const int bl = (int)(t2 / Et);
-        const RwgSlots A = tr[m], B = sr[n];
+        const RwgSlots A = tr[(own ? (b0 + bl) * Et : 0) + m], B = sr[(own ? (b0 + bl) * Es : 0) + n];
         double2 l = make_double2(0.0, 0.0), kk = make_double2(0.0, 0.0);
 #pragma unroll
         for (int x = 0; x < 2; ++x)
@@ -411,7 +452,7 @@ __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots*
                 kk.x += c * p[9 + ij].x;
                 kk.y += c * p[9 + ij].y;
             }
-        const size_t o = ((size_t)(slot ? slot[b0 + bl] : b0 + bl) * Et + m) * Es + n;
+        const size_t o = ((size_t)(slot ? slot[b0 + bl] : own ? 2 * (b0 + bl) : b0 + bl) * Et + m) * Es + n;
         L[o] = l;
         K[o] = kk;
     }
@@ -501,21 +542,21 @@ void rule_moments(double wl[21]) {
 
 // slot integrals of blocks b0 .. b0 + nc - 1 (singular: host flags), one
 // launch per run of equal flags
-cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, const double* shifts,
+cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, bool own, const double* shifts,
                          const int8_t* singular, int b0, int nc, double k, double ki, double2* out, cudaStream_t st) {
     const unsigned gx = (unsigned)(((long long)Tt * Ts + 127) / 128);
     for (int c = 0; c < nc;) {
         int e = c + 1;
-        while (e < nc && (singular[b0 + e] != 0) == (singular[b0 + c] != 0) && e - c < 65535) ++e;
+        while (e < nc && (own || (singular[b0 + e] != 0) == (singular[b0 + c] != 0)) && e - c < 65535) ++e;
         const dim3 g(gx, (unsigned)(e - c));
         double2* o = out + (size_t)c * Tt * Ts * 18;
-        const bool s = singular[b0 + c] != 0;
+        const bool s = own || singular[b0 + c] != 0;
         if (ki != 0.0) {
-            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, ki, o);
-            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, ki, o);
+            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o);
+            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o);
         } else {
-            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, 0.0, o);
-            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, shifts, b0 + c, k, 0.0, o);
+            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o);
+            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o);
         }
         const cudaError_t err = cudaGetLastError();
         if (err != cudaSuccess) return err;
@@ -526,18 +567,28 @@ cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, con
 }  // namespace
 
 // L, K: device [nb][Et][Es] (block b at slot[b] when slot is not NULL);
-// wavenumber k + j ki (ki = 0: lossless)
-int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* shifts,
-                       const int8_t* singular, int nb, double k, double ki, double2* L, double2* K,
-                       cudaStream_t st, const int32_t* slot) {
+// wavenumber k + j ki (ki = 0: lossless).  cells: nb meshes instead, each tested
+// on itself (test = src = cells[b], singular), L = [nb][L, K][E][E].
+static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshView& src, const double* shifts,
+                        const int8_t* singular, int nb, double k, double ki, double2* L, double2* K, cudaStream_t st,
+                        const int32_t* slot) {
     if (!(k > 0.0) || !(ki <= 0.0) || nb < 1) {
         set_error("tabulate needs Re k > 0, Im k <= 0 and >= 1 block");
         return EMSURF_EINVAL;
     }
+    const bool own = cells != nullptr;
     std::vector<TriGeo> tg, sgeo;
     std::vector<RwgSlots> tr, sr;
-    EMS_TRY(prepare_mesh(test.verts, test.tris, test.slot_rwg, test.slot_sgn, test.T, test.E, tg, tr));
-    EMS_TRY(prepare_mesh(src.verts, src.tris, src.slot_rwg, src.slot_sgn, src.T, src.E, sgeo, sr));
+    for (int b = 0; b < (own ? nb : 0); ++b) {
+        const MeshView& m = cells[b];
+        EMS_TRY(prepare_mesh(m.verts, m.tris, m.slot_rwg, m.slot_sgn, m.T, m.E, sgeo, sr));
+        tg.insert(tg.end(), sgeo.begin(), sgeo.end());
+        tr.insert(tr.end(), sr.begin(), sr.end());
+    }
+    if (!own) {
+        EMS_TRY(prepare_mesh(test.verts, test.tris, test.slot_rwg, test.slot_sgn, test.T, test.E, tg, tr));
+        EMS_TRY(prepare_mesh(src.verts, src.tris, src.slot_rwg, src.slot_sgn, src.T, src.E, sgeo, sr));
+    }
     double wl[21];
     rule_moments(wl);
     EMS_CUDA(cudaMemcpyToSymbolAsync(c_wl, wl, sizeof(wl), 0, cudaMemcpyHostToDevice, st));
@@ -555,27 +606,31 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
     };
     cudaError_t e;
     if ((e = cudaMalloc(&dtg, sizeof(TriGeo) * tg.size())) != cudaSuccess) fail(e, "alloc");
-    if (!status && (e = cudaMalloc(&dsg, sizeof(TriGeo) * sgeo.size())) != cudaSuccess) fail(e, "alloc");
+    if (!status && !own && (e = cudaMalloc(&dsg, sizeof(TriGeo) * sgeo.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&dtr, sizeof(RwgSlots) * tr.size())) != cudaSuccess) fail(e, "alloc");
-    if (!status && (e = cudaMalloc(&dsr, sizeof(RwgSlots) * sr.size())) != cudaSuccess) fail(e, "alloc");
-    if (!status && (e = cudaMalloc(&dsh, sizeof(double) * 3 * nb)) != cudaSuccess) fail(e, "alloc");
+    if (!status && !own && (e = cudaMalloc(&dsr, sizeof(RwgSlots) * sr.size())) != cudaSuccess) fail(e, "alloc");
+    if (!status && !own && (e = cudaMalloc(&dsh, sizeof(double) * 3 * nb)) != cudaSuccess) fail(e, "alloc");
     if (!status && slot && (e = cudaMalloc(&dslot, sizeof(int32_t) * nb)) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&scratch, per_block * chunk)) != cudaSuccess) fail(e, "scratch alloc");
     if (!status) {
         cudaMemcpyAsync(dtg, tg.data(), sizeof(TriGeo) * tg.size(), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(dsg, sgeo.data(), sizeof(TriGeo) * sgeo.size(), cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(dtr, tr.data(), sizeof(RwgSlots) * tr.size(), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(dsr, sr.data(), sizeof(RwgSlots) * sr.size(), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(dsh, shifts, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, st);
+        if (!own) {
+            cudaMemcpyAsync(dsg, sgeo.data(), sizeof(TriGeo) * sgeo.size(), cudaMemcpyHostToDevice, st);
+            cudaMemcpyAsync(dsr, sr.data(), sizeof(RwgSlots) * sr.size(), cudaMemcpyHostToDevice, st);
+            cudaMemcpyAsync(dsh, shifts, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, st);
+        }
         if (slot) cudaMemcpyAsync(dslot, slot, sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st);
+        const TriGeo* ds = own ? dtg : dsg;
+        const RwgSlots* drs = own ? dtr : dsr;
         for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
             const int nc = std::min(chunk, nb - b0);
-            e = launch_pairs(dtg, test.T, dsg, src.T, dsh, singular, b0, nc, k, ki, scratch, st);
+            e = launch_pairs(dtg, test.T, ds, src.T, own, dsh, singular, b0, nc, k, ki, scratch, st);
             if (e != cudaSuccess) { fail(e, "tri_pairs_kernel"); break; }
             const size_t tot = (size_t)nc * test.E * src.E;
             const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
-            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, dsr, src.E, test.T, src.T, b0,
-                                                  nc, dslot, L, K);
+            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, drs, src.E, test.T, src.T, b0, nc, own, dslot, L,
+                                                  own ? L + (size_t)test.E * src.E : K);
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "rwg_gather_kernel"); break; }
         }
         if (!status && (e = cudaStreamSynchronize(st)) != cudaSuccess) fail(e, "synchronize");
@@ -588,6 +643,18 @@ int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* 
     cudaFree(dslot);
     cudaFree(scratch);
     return status;
+}
+
+int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* shifts,
+                       const int8_t* singular, int nb, double k, double ki, double2* L, double2* K,
+                       cudaStream_t st, const int32_t* slot) {
+    return tabulate_any(nullptr, test, src, shifts, singular, nb, k, ki, L, K, st, slot);
+}
+
+// LK[b] = L, K of cell b on itself; all meshes have the same number of triangles and RWGs
+int tabulate_cells_cx(const std::vector<MeshView>& cells, double k, double ki, double2* LK, cudaStream_t st) {
+    return tabulate_any(cells.data(), cells[0], cells[0], nullptr, nullptr, (int)cells.size(), k, ki, LK, nullptr, st,
+                        nullptr);
 }
 
 int tabulate_blocks(const MeshView& test, const MeshView& src, const double* shifts,
@@ -714,11 +781,11 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
     // every pair integral is written before it is read, so nothing needs clearing
     for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
         const int nc = std::min(chunk, nb - b0);
-        step(launch_pairs(dtg, test.T, dsg, src.T, dsh, singular, b0, nc, k, 0.0, pairs, st), "tri_pairs_kernel");
+        step(launch_pairs(dtg, test.T, dsg, src.T, false, dsh, singular, b0, nc, k, 0.0, pairs, st), "tri_pairs_kernel");
         if (status) break;
         const size_t tot = (size_t)nc * test.E * src.E;
         const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
-        rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc,
+        rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc, 0,
                                               nullptr, L, K);
         step(cudaGetLastError(), "rwg_gather_kernel");
     }
