@@ -17,7 +17,7 @@
 #include <cmath>
 #include <vector>
 
-#include "common.cuh"
+#include "slab_lu.cuh"
 
 namespace emsurf {
 
@@ -305,19 +305,10 @@ EMSURF_API int emsurf_macromodel_pec_patch(double a, double b, double h, int32_t
 //      Z_v = [[j k0 L_v, K_v], [-K_v, j k0 eps_v L_v]];
 //   3. the Schur complement of Eq. Zmacromodel by Gaussian elimination of
 //      the interior unknowns (ordered first), partial pivoting among the
-//      interior rows only: after n_int steps the trailing 2E x 2E block is
-//      Z~ = Z_ee - Z_ei Z_ii^{-1} Z_ie.  Each step reads one buffer and writes
-//      the other, so the CTAs of a type need no synchronisation.
+//      interior rows only (slab_lu.cu): the trailing 2E x 2E block becomes
+//      Z~ = Z_ee - Z_ei Z_ii^{-1} Z_ie.
 namespace emsurf {
 namespace {
-
-struct SlabType {
-    long long offL[2];   // region v's L in the table buffer; its K follows at + E_v^2
-    int Ev[2];
-    int N, nint;
-    long long offB;      // this type's N x N matrix in the elimination buffers
-    long long offMap;    // this type's copy/sign arrays ([2][N])
-};
 
 __global__ void slab_assemble_kernel(const SlabType* __restrict__ ty, const double2* __restrict__ LK,
                                      const int32_t* __restrict__ cpy, const int8_t* __restrict__ sgn,
@@ -352,69 +343,12 @@ __global__ void slab_assemble_kernel(const SlabType* __restrict__ ty, const doub
     }
 }
 
-// one elimination step c for every type: Bout = trailing block of Bin after
-// moving the pivot row of column 0 to the top and eliminating column 0
-__global__ void __launch_bounds__(256)
-slab_eliminate_kernel(const SlabType* __restrict__ ty, int c, const double2* __restrict__ Bin,
-                      double2* __restrict__ Bout, int* __restrict__ status) {
-    const SlabType T = ty[blockIdx.y];
-    const double2* bi = Bin + T.offB;
-    double2* bo = Bout + T.offB;
-    const int N = T.N;
-    if (c >= T.nint) {                 // this type is done: carry its Z~ over
-        const int n = N - T.nint;
-        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x)
-            bo[(size_t)(e / n) * N + e % n] = bi[(size_t)(e / n) * N + e % n];
-        return;
-    }
-    __shared__ double s_m[256];
-    __shared__ int s_i[256];
-    double best = -1.0;
-    int bi_row = 0;
-    for (int r = threadIdx.x; r < T.nint - c; r += blockDim.x) {
-        const double2 v = bi[(size_t)r * N];
-        const double m = v.x * v.x + v.y * v.y;
-        if (m > best) { best = m; bi_row = r; }
-    }
-    s_m[threadIdx.x] = best;
-    s_i[threadIdx.x] = bi_row;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            const double m2 = s_m[threadIdx.x + w];
-            const int i2 = s_i[threadIdx.x + w];
-            if (m2 > s_m[threadIdx.x] || (m2 == s_m[threadIdx.x] && i2 < s_i[threadIdx.x])) {
-                s_m[threadIdx.x] = m2;
-                s_i[threadIdx.x] = i2;
-            }
-        }
-        __syncthreads();
-    }
-    const int p = s_i[0];
-    if (!(s_m[0] > 0.0)) {
-        if (threadIdx.x == 0 && blockIdx.x == 0) atomicExch(status, 1);
-        return;
-    }
-    const double2 piv = bi[(size_t)p * N];
-    const double dd = 1.0 / (piv.x * piv.x + piv.y * piv.y);
-    const double2 inv = make_double2(piv.x * dd, -piv.y * dd);
-    const int no = N - c - 1;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < no * no; e += gridDim.x * blockDim.x) {
-        const int i = e / no, j = e % no;
-        const int ro = (i + 1 == p) ? 0 : i + 1;
-        const double2 l = cmul(bi[(size_t)ro * N], inv);
-        const double2 u = bi[(size_t)p * N + j + 1];
-        const double2 a = bi[(size_t)ro * N + j + 1];
-        bo[(size_t)i * N + j] = make_double2(a.x - (l.x * u.x - l.y * u.y), a.y - (l.x * u.y + l.y * u.x));
-    }
-}
-
 __global__ void slab_copy_out_kernel(const SlabType* __restrict__ ty, const double2* __restrict__ B,
                                      int K, double2* __restrict__ Z) {
     const SlabType T = ty[blockIdx.y];
     double2* z = Z + (size_t)blockIdx.y * K * K;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < K * K; e += gridDim.x * blockDim.x)
-        z[e] = B[T.offB + (size_t)(e / K) * T.N + e % K];
+        z[e] = B[T.offB + (size_t)(T.nint + e / K) * T.N + T.nint + e % K];
 }
 
 }  // namespace
@@ -436,7 +370,7 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
     std::vector<SlabPlan> plan(n_types);
     std::vector<SlabType> ty(n_types);
     long long nLK = 0, nB = 0, nMap = 0;
-    int E = 0, max_nint = 0;
+    int E = 0, max_nint = 0, max_n = 0;
     for (int t = 0; t < n_types; ++t) {
         EMS_TRY(slab_cell_plan(a, b, h, n, zlevels, sides[t], patch_n, ring_layers, plan[t]));
         E = plan[t].E;
@@ -449,6 +383,7 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         T.offMap = nMap;
         nMap += 2ll * T.N;
         max_nint = std::max(max_nint, T.nint);
+        max_n = std::max(max_n, T.N);
     }
     // the tables of one region's types lie one after another
     for (int v = 0; v < 2; ++v)
@@ -461,7 +396,8 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
     const double er = eps_slab.re, ei = eps_slab.im, mod = std::sqrt(er * er + ei * ei);
     const double sr = std::sqrt(0.5 * (mod + er)), si = -std::sqrt(std::max(0.0, 0.5 * (mod - er)));
     const double kv_re[2] = {k0, k0 * sr}, kv_im[2] = {0.0, k0 * si};
-    double2 *LK = nullptr, *B0 = nullptr, *B1 = nullptr;
+    double2 *LK = nullptr, *B = nullptr;
+    void* work = nullptr;
     int32_t* dcpy = nullptr;
     int8_t* dsgn = nullptr;
     SlabType* dty = nullptr;
@@ -476,8 +412,8 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         }
     };
     alloc((void**)&LK, sizeof(double2) * nLK);
-    alloc((void**)&B0, sizeof(double2) * nB);
-    alloc((void**)&B1, sizeof(double2) * nB);
+    alloc((void**)&B, sizeof(double2) * nB);
+    alloc(&work, slab_lu_bytes(n_types, max_n, max_nint));
     alloc((void**)&dcpy, sizeof(int32_t) * nMap);
     alloc((void**)&dsgn, nMap);
     alloc((void**)&dty, sizeof(SlabType) * n_types);
@@ -511,17 +447,12 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         const int gx = std::max(1, 152 * 8 / n_types);
         if (e == cudaSuccess) {
             slab_assemble_kernel<<<dim3(gx, n_types), 256, 0, st>>>(dty, LK, dcpy, dsgn, k0,
-                                                                    make_double2(er, ei), B0);
+                                                                    make_double2(er, ei), B);
             e = cudaGetLastError();
         }
-        double2 *bin = B0, *bout = B1;
-        for (int c = 0; c < max_nint && e == cudaSuccess; ++c) {
-            slab_eliminate_kernel<<<dim3(gx, n_types), 256, 0, st>>>(dty, c, bin, bout, dstat);
-            e = cudaGetLastError();
-            std::swap(bin, bout);
-        }
+        if (e == cudaSuccess) e = slab_lu(dty, n_types, max_n, max_nint, B, work, dstat, st);
         if (e == cudaSuccess) {
-            slab_copy_out_kernel<<<dim3(gx, n_types), 256, 0, st>>>(dty, bin, K, reinterpret_cast<double2*>(Z));
+            slab_copy_out_kernel<<<dim3(gx, n_types), 256, 0, st>>>(dty, B, K, reinterpret_cast<double2*>(Z));
             e = cudaGetLastError();
         }
         const cudaError_t es = cudaStreamSynchronize(st);
@@ -533,12 +464,13 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
             int hs = 0;
             cudaMemcpy(&hs, dstat, sizeof(int), cudaMemcpyDeviceToHost);
             if (hs) {
-                set_error("emsurf_macromodel_slab_patch: singular interior block");
-                status = EMSURF_EINVAL;
+                set_error(hs == 1 ? "emsurf_macromodel_slab_patch: singular interior block"
+                                  : "emsurf_macromodel_slab_patch: a device wait expired");
+                status = hs == 1 ? EMSURF_EINVAL : EMSURF_ETIMEDOUT;
             }
         }
     }
-    for (void* p : {(void*)LK, (void*)B0, (void*)B1, (void*)dcpy, (void*)dsgn, (void*)dty, (void*)dstat})
+    for (void* p : {(void*)LK, (void*)B, work, (void*)dcpy, (void*)dsgn, (void*)dty, (void*)dstat})
         cudaFree(p);
     return status;
 }

@@ -45,17 +45,14 @@
 // at the copy rate): 1161 us in double-single FP32, 593 us here (bins and
 // macromodels 490 us, splitting the vectors 25 us); 12 x 9, K = 576 and 6 rhs:
 // 6575 us, 597 us.  Error against 64 bits 7.2e-14, 6e-15 (both sizes).
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <vector>
 
-#include "common.cuh"
+#include "digits.cuh"
 
 namespace emsurf {
 namespace {
 
-constexpr int kSl = 7;                       // digits
 constexpr int kSlRows = 128;                 // rows per tile (TMEM lanes)
 constexpr int kSlK = 32;                     // sources per stage
 constexpr int kSlChunk = 4;                  // stages per exact accumulation (128 sources)
@@ -66,42 +63,12 @@ constexpr int kSlEpi = 8, kSlWarps = kSlEpi + 8 + 3, kSlThreads = 32 * kSlWarps;
 constexpr int kSlWarpA = kSlWarps - 3, kSlWarpM = kSlWarps - 2, kSlWarpX = kSlWarps - 1;
 constexpr uint32_t kSlTmemCols = 512, kSlAStep = kSl * 8;   // TMEM columns; of one 16-source block of A
 constexpr int kSlMaxSlots = 4;               // A blocks in TMEM, at the end of its columns
-constexpr int kSlWait = 1 << 16;
 constexpr size_t kSlSmemMax = 224 * 1024;
 constexpr int kSlMaxV = 24;                  // vector columns of one launch (a multiple of 8: swizzle groups):
                                              // two accumulators and two A blocks fit in TMEM
 constexpr int kSlRhs = kSlMaxV / 4;          // rhs per launch
 constexpr int kSlSplit = 256;                // threads of a splitting block
 constexpr int kSlCells = 8;                  // columns of a macromodel entry
-// |I_a I_b| <= 2^108 = 2^52 units of level 5, so re +- im sums of up to kSlExact
-// sources stay inside int64; beyond, the integers lose a bit per factor of 4
-constexpr int kSlExact = 990, kSlMaxN = 7000;   // the latter: two vectors in shared memory
-
-__device__ __forceinline__ uint32_t sl_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void sl_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sl_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void sl_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sl_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void sl_expect(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sl_addr(bar)), "r"(bytes) : "memory");
-}
-// bounded wait; each try suspends the thread for up to 20 us (re-polling warps
-// slow every barrier of the block down)
-__device__ __forceinline__ bool sl_wait(uint64_t* bar, uint32_t parity) {
-    for (int it = 0; it < kSlWait; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(sl_addr(bar)), "r"(parity), "r"(20000u)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
 // the same for two or three barriers at once (their latencies overlap)
 __device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, uint64_t* b2, uint32_t p2,
                                          bool third) {
@@ -120,32 +87,6 @@ __device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1
     }
     return false;
 }
-__device__ __forceinline__ void sl_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], "
-        "%4;" ::"r"(sl_addr(dst)),
-        "l"(src), "r"(bytes), "r"(sl_addr(bar)), "l"(pol)
-        : "memory");
-}
-// One lane of a converged warp.  The MMA warp runs as a whole and issues under
-// elect.sync, so that the operands stay in uniform registers.
-__device__ __forceinline__ bool sl_elect() {
-    uint32_t r;
-    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
-    return r != 0;
-}
-__device__ __forceinline__ void sl_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sl_addr(bar))
-                 : "memory");
-}
-// D (+)= A B: A 128 x 16 FP16 in TMEM, B N x 16 FP16 in shared memory (K-major, 64B swizzle)
-template <bool ACC>
-__device__ __forceinline__ void sl_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-        "r"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0));
-}
 // K-major descriptor, 64-byte swizzled rows, 8-row groups 512 B apart
 __device__ __forceinline__ uint64_t sl_desc(uint32_t addr) {
     return (uint64_t)((addr & 0x3FFFF) >> 4) | (1ull << 16) | (32ull << 32) | (1ull << 46) | (4ull << 61);
@@ -155,12 +96,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t t, const uint32_t (&r)[8]) {
                  "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                  : "memory");
 }
-__device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t (&r)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(t));
-}
-
 __host__ __device__ constexpr int sl_up16(int n) { return (n + 15) & ~15; }
 
 struct SlProb {
@@ -548,36 +483,6 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
 }
 
 // ---------------------------------------------------------------- splitting
-// exponent ex with |v| < 2^ex for the largest |v| of a vector, from its bit
-// pattern (the patterns of non-negative doubles order like the values, NaN above
-// infinity) and n, the sources that are summed; INT_MIN when it is not finite
-__device__ __forceinline__ int sl_exp(unsigned long long mbits, int n) {
-    if (mbits >= 0x7ff0000000000000ull) return INT_MIN;
-    const double m = __longlong_as_double((long long)mbits);
-    const int spare = n <= kSlExact ? 0 : n <= 4 * kSlExact ? 1 : 2;
-    return (m > 0.0 ? max(ilogb(m) + 1, -900) : 0) + spare;
-}
-// 2^(ex - 8) for the products (NaN where a component was not finite: it marks
-// every output)
-__device__ __forceinline__ double sl_pow(int ex) {
-    return ex == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, ex - 8);
-}
-// Bytes d_t + 128 of the digits of rn(v 2^(54 - ex)), least significant first:
-// balanced digits are the bytes of I + sum_t 128 256^t.  From the bit pattern:
-// FP64 conversions run at the FP64 rate.
-__device__ __forceinline__ unsigned long long sl_digits(double v, int ex) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int e = (int)(b >> 52) & 0x7ff;
-    unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-    // v = +-m 2^(max(e, 1) - 1075), so the shift to the left is at most one
-    const int sh = max(e, 1) - 1021 - ex;
-    m = ex == INT_MIN || sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 1) : (m + (1ull << (-sh - 1))) >> -sh;
-    return ((long long)b < 0 ? 0ull - m : m) + 0x80808080808080ull;
-}
-__device__ __forceinline__ unsigned long long sl_abs(double v) {
-    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-}
-
 // Planes of one row per thread: rows of bins (MM false) from B^[bin][op][j][i],
 // of macromodels from Zt[t][k'][k]; blockIdx.x = tile, blockIdx.y = matrix.
 template <bool MM>
@@ -660,7 +565,6 @@ __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int
     auto at = [&](int row, int ch) {
         return reinterpret_cast<uint4*>(X + ((size_t)(ch >> 2) * Np + row) * 64 + ((ch & 3) ^ ((row >> 1) & 3)) * 16);
     };
-    const __half2 off = __floats2half2_rn(1152.f, 1152.f);
     for (int e = threadIdx.x; e < 4 * chunks; e += blockDim.x) {
         const int ch = e >> 2, v = 2 * v0 + (e & 3), h = (e >> 1) & 1;
         const int ex = s_ex[h];
@@ -672,20 +576,7 @@ __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int
             d[b] = j < n ? sl_digits(src[2 * j], ex) : 0x80808080808080ull;
         }
 #pragma unroll
-        for (int t = 0; t < kSl; ++t) {
-            const int by = kSl - 1 - t;
-            uint32_t w[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                // FP16 0x6400 | byte = 1024 + byte; minus 1152 gives the digit
-                const uint32_t p = by < 4 ? __byte_perm((uint32_t)d[2 * q], (uint32_t)d[2 * q + 1], by | (4 + by) << 4)
-                                          : __byte_perm((uint32_t)(d[2 * q] >> 32), (uint32_t)(d[2 * q + 1] >> 32), (by - 4) | by << 4);
-                const uint32_t f = __byte_perm(p, 0x64646464u, 0x4140);
-                const __half2 x = __hsub2(*reinterpret_cast<const __half2*>(&f), off);
-                w[q] = *reinterpret_cast<const uint32_t*>(&x);
-            }
-            *at(t * V + v, ch) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        for (int t = 0; t < kSl; ++t) *at(t * V + v, ch) = sl_halves(d, t);
     }
     if (v0 + 2 < V / 2) return;
     for (int e = threadIdx.x; e < (Np - kSl * V) * chunks; e += blockDim.x) {

@@ -35,3 +35,23 @@ def test_library_equals_single_cells(emsurf_lib, n, patch_n, layers, sides, eps)
     for t in sorted({0, 1 % len(sides), len(sides) // 2, len(sides) - 1}):
         one = models(sides[t:t + 1])[0]
         assert float((Z[t] - one).norm()) <= 1e-12 * float(one.norm()), t
+
+
+@pytest.mark.parametrize("n,patch_n,layers,side", [(2, 1, 1, 0.3), (2, 5, 4, 0.2), (2, 6, 5, 0.4)])
+def test_elimination_of_few_and_many_interior_unknowns(emsurf_lib, n, patch_n, layers, side):
+    """Panels of less than 32 columns, remainders, and interior blocks too
+    large for shared memory, against the oracle (same quadrature: the slab
+    tests' 1e-10 in norm); the second type is an empty cell."""
+    import torch
+    from oracle import macromodel
+    from oracle.mesh import box_mesh, slab_zlevels
+    from paper_1911_04576_gb300 import binding as B
+    K = 36 * n * n
+    sides = np.array([side * W.LAMBDA, 0.0])
+    Z = torch.full((2, K, K), float("nan"), dtype=torch.complex128, device="cuda")
+    B.emsurf_macromodel_slab_patch(A, A, H, n, B.emsurf_setup_slab_zlevels(H, n, W.SLAB_T), sides, patch_n, layers,
+                                   W.EPS_SLAB, K0, Z)
+    box = box_mesh(A, A, H, n, slab_zlevels(H, n, W.SLAB_T))
+    for t, s in enumerate(sides):
+        ref = macromodel.slab_patch(box, n, s, patch_n, W.EPS_SLAB, K0, W.SLAB_T, ring_layers=layers)
+        assert np.linalg.norm(Z[t].cpu().numpy() - ref) <= 1e-10 * np.linalg.norm(ref), t
