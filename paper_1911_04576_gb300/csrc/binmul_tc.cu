@@ -139,6 +139,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 struct TcArgs {
     float2* Y;            // [bins][R][2E]
     int E, nbins, R, groups, chunks, nk, items;
+    int a_rows;           // rows of a copy of the X^ planes: those of a group's rhs, 32, 64 or all 128
     float2 ca, cb, cg, cd;
     int* err;
 };
@@ -193,7 +194,7 @@ binmul_tc_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant_
                         break;
                     }
                     unsigned char* st = smem + stage * BmShape<KC>::StageBytes;
-                    bar_expect(&full[stage], BmShape<KC>::StageBytes);
+                    bar_expect(&full[stage], 2 * g.a_rows * KC * 2 + 4 * BmShape<KC>::BBytes);
                     const int j0 = ks * KC;
                     tma3d(st, &mAh, j0, kTcM * grp, bin, &full[stage]);
                     tma3d(st + BmShape<KC>::ABytes, &mAl, j0, kTcM * grp, bin, &full[stage]);
@@ -366,24 +367,45 @@ __global__ void tc_split_spectrum_kernel(const float2* __restrict__ Bhat, __nv_b
     }
 }
 
+// hi/lo planes of 8 complex numbers: rows (Re, Im) at out and out + ld
+__device__ __forceinline__ void split8(const float2 (&v)[8], __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                       size_t at, size_t ld) {
+    uint4 w[4];      // hi Re, hi Im, lo Re, lo Im
+    uint32_t* h = reinterpret_cast<uint32_t*>(w);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const float2 x = v[2 * p], y = v[2 * p + 1];
+        const __nv_bfloat162 hr = __floats2bfloat162_rn(x.x, y.x), hm = __floats2bfloat162_rn(x.y, y.y);
+        const float2 fr = __bfloat1622float2(hr), fm = __bfloat1622float2(hm);
+        const __nv_bfloat162 lr = __floats2bfloat162_rn(x.x - fr.x, y.x - fr.y), lm = __floats2bfloat162_rn(x.y - fm.x, y.y - fm.y);
+        h[p] = *reinterpret_cast<const uint32_t*>(&hr);
+        h[4 + p] = *reinterpret_cast<const uint32_t*>(&hm);
+        h[8 + p] = *reinterpret_cast<const uint32_t*>(&lr);
+        h[12 + p] = *reinterpret_cast<const uint32_t*>(&lm);
+    }
+    *reinterpret_cast<uint4*>(hi + at) = w[0];
+    *reinterpret_cast<uint4*>(hi + at + ld) = w[1];
+    *reinterpret_cast<uint4*>(lo + at) = w[2];
+    *reinterpret_cast<uint4*>(lo + at + ld) = w[3];
+}
+
 // Split planes of X^: out[bin][4r+q][j], q = (Re x_J, Im x_J, Re x_M, Im x_M),
-// zero for r >= R and j >= E.
-__global__ void tc_split_x_kernel(const float2* __restrict__ X, __nv_bfloat16* __restrict__ hi,
-                                  __nv_bfloat16* __restrict__ lo, int E, int ej, int R, int rows, size_t total) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e % ej);
-        const size_t br = e / ej;
-        const int rho = (int)(br % rows);
-        const size_t bin = br / rows;
-        const int r = rho >> 2, q = rho & 3;
-        float v = 0.f;
-        if (r < R && j < E) {
-            const float2 x = X[(bin * R + r) * (size_t)(2 * E) + (q >> 1) * E + j];
-            v = (q & 1) ? x.y : x.x;
+// zero for j >= E; rows past 4R are not written (they reach no output).  Eight
+// sources per thread, 16-byte stores: HBM-bound (48 x 48 bins, K = 576, 32 rhs:
+// 680 MB, 112 us; 306 us with one 2-byte element per thread).
+__global__ void __launch_bounds__(256)
+tc_split_x_kernel(const float2* __restrict__ X, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int E,
+                  int ej, int R, int rows, int nbins) {
+    const int nc = ej / 8, per = 2 * R * nc;
+    for (int bin = blockIdx.x; bin < nbins; bin += gridDim.x) {
+        const float2* src = X + (size_t)bin * R * 2 * E;
+        for (int e = threadIdx.x; e < per; e += blockDim.x) {
+            const int rp = e / nc, j = 8 * (e - rp * nc);             // rp = 2 r + part
+            float2 v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v[b] = j + b < E ? src[(size_t)rp * E + j + b] : make_float2(0.f, 0.f);
+            split8(v, hi, lo, ((size_t)bin * rows + 2 * rp) * ej + j, ej);
         }
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[e] = h;
-        lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
 }
 
@@ -585,34 +607,36 @@ mm_tc_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CU
 
 // x1 planes of the macromodel tiles: out[tile][2c+q][k'] = hi/lo of
 // (q ? Im : Re)(sign * x[r][U_o index]) for column c = (cell slot, rhs) of
-// the tile's type; zero past the type's columns and for k' >= K.
-__global__ void tc_mm_gather_kernel(const double2* __restrict__ x, const float2* __restrict__ xf,
-                                    const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn,
-                                    const int2* __restrict__ tiles, const int32_t* __restrict__ type_ptr,
-                                    const int32_t* __restrict__ type_cells, __nv_bfloat16* __restrict__ hi,
-                                    __nv_bfloat16* __restrict__ lo, int K, int kp, int R, int n_unique,
-                                    size_t total) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int kk = (int)(e % kp);
-        const size_t tr = e / kp;
-        const int rho = (int)(tr % kTcM);
-        const int tile = (int)(tr / kTcM);
+// the tile's type; zero for k' >= K, not written past the type's columns (such
+// rows reach no output).  Eight k' per thread.
+__global__ void __launch_bounds__(256)
+tc_mm_gather_kernel(const double2* __restrict__ x, const float2* __restrict__ xf, const int32_t* __restrict__ idx,
+                    const int8_t* __restrict__ sgn, const int2* __restrict__ tiles, const int32_t* __restrict__ type_ptr,
+                    const int32_t* __restrict__ type_cells, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                    int K, int kp, int R, int n_unique, int ntiles) {
+    const int nc = kp / 8, per = (kTcM / 2) * nc;
+    for (int u = blockIdx.x; u < 4 * ntiles; u += gridDim.x) {        // a quarter of a tile per block
+        const int tile = u >> 2;
         const int2 tl = tiles[tile];
-        const int col = tl.y + (rho >> 1), q = rho & 1;
-        const int n_t = type_ptr[tl.x + 1] - type_ptr[tl.x];
-        float v = 0.f;
-        if (col < n_t * R && kk < K) {
-            const int slot = col / R, r = col % R;
-            const int cell = type_cells[type_ptr[tl.x] + slot];
-            const size_t loc = (size_t)cell * K + kk;
-            const size_t at = (size_t)r * n_unique + idx[loc];
-            const float s = (float)sgn[loc];
-            if (xf) v = s * (q ? xf[at].y : xf[at].x);
-            else v = s * (float)(q ? x[at].y : x[at].x);
+        const int c0 = type_ptr[tl.x], n_t = (type_ptr[tl.x + 1] - c0) * R;
+        for (int e = (u & 3) * (per / 4) + threadIdx.x; e < ((u & 3) + 1) * (per / 4); e += blockDim.x) {
+            const int c = e / nc, k = 8 * (e - c * nc), col = tl.y + c;
+            if (col >= n_t) continue;
+            const int slot = col / R, r = col - slot * R;
+            const size_t loc = (size_t)type_cells[c0 + slot] * K + k, xr = (size_t)r * n_unique;
+            float2 v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                v[b] = make_float2(0.f, 0.f);
+                if (k + b < K) {
+                    const size_t at = xr + idx[loc + b];
+                    const float s = (float)sgn[loc + b];
+                    if (xf) v[b] = make_float2(s * xf[at].x, s * xf[at].y);
+                    else v[b] = make_float2(s * (float)x[at].x, s * (float)x[at].y);
+                }
+            }
+            split8(v, hi, lo, ((size_t)tile * kTcM + 2 * c) * kp + k, kp);
         }
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[e] = h;
-        lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
 }
 
@@ -632,6 +656,7 @@ struct PcArgs {
     const int32_t* sub_ptr;
     const int32_t* sub_ids;
     int R, n_unique, nitems;
+    int a_rows;                    // rows of a copy of the r planes: 32, 64 or 128, at least 2R
     int* err;
 };
 
@@ -684,7 +709,7 @@ pc_tc_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CU
                         break;
                     }
                     unsigned char* st = smem + stage * kMmStageBytes;
-                    bar_expect(&full[stage], kMmStageBytes);
+                    bar_expect(&full[stage], 2 * g.a_rows * kTcKc * 2 + 2 * kTcBBytes);
                     const int j0 = ks * kTcKc;
                     tma3d(st, &mAh, j0, 0, it.x, &full[stage]);
                     tma3d(st + kTcABytes, &mAl, j0, 0, it.x, &full[stage]);
@@ -829,26 +854,28 @@ __global__ void pc_tc_split_rows_kernel(const float2* __restrict__ X, const int6
 }
 
 // gathered r planes per cell: out[m][2c+q][j] = hi/lo of (q ? Im : Re)
-// r[c][sub_m[j]] for rhs c < R and j < n_m, zero otherwise
+// r[c][sub_m[j]] for rhs c < R and j < n_m, zero for j >= n_m; rows past 2R are
+// not written (they reach no output).  Eight j per thread.
 template <typename VT>
-__global__ void pc_tc_gather_kernel(const VT* __restrict__ r, const int32_t* __restrict__ sub_ptr,
-                                    const int32_t* __restrict__ sub_ids, const int32_t* __restrict__ nsz,
-                                    int R, int n_unique, int np, __nv_bfloat16* __restrict__ hi,
-                                    __nv_bfloat16* __restrict__ lo, size_t total) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e % np);
-        const size_t mr = e / np;
-        const int rho = (int)(mr % kTcM);
-        const int m = (int)(mr / kTcM);
-        const int cc = rho >> 1, q = rho & 1;
-        float v = 0.f;
-        if (cc < R && j < nsz[m]) {
-            const VT x = r[(size_t)cc * n_unique + sub_ids[sub_ptr[m] + j]];
-            v = (float)(q ? x.y : x.x);
+__global__ void __launch_bounds__(256)
+pc_tc_gather_kernel(const VT* __restrict__ r, const int32_t* __restrict__ sub_ptr, const int32_t* __restrict__ sub_ids,
+                    const int32_t* __restrict__ nsz, int R, int n_unique, int np, __nv_bfloat16* __restrict__ hi,
+                    __nv_bfloat16* __restrict__ lo, int total) {
+    const int nc = np / 8, per = R * nc;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int m = e / per, o = e - m * per, c = o / nc, j = 8 * (o - c * nc);
+        const int n = nsz[m];
+        const int32_t* ids = sub_ids + sub_ptr[m];
+        float2 v[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            v[b] = make_float2(0.f, 0.f);
+            if (j + b < n) {
+                const VT x = r[(size_t)c * n_unique + ids[j + b]];
+                v[b] = make_float2((float)x.x, (float)x.y);
+            }
         }
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[e] = h;
-        lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
+        split8(v, hi, lo, ((size_t)m * kTcM + 2 * c) * np + j, np);
     }
 }
 
@@ -927,6 +954,13 @@ int tc_build(emsurf_handle* h, const emsurf_handle* share) {
     EMS_TRY(encode3d(&m[3], h->tc_Bl, ej, 2 * E, 2 * nb, 32, kTcN, CU_TENSOR_MAP_SWIZZLE_64B));
     EMS_TRY(encode3d(&m[8], h->tc_Xh, ej, rows, nb, 64, kTcM));
     EMS_TRY(encode3d(&m[9], h->tc_Xl, ej, rows, nb, 64, kTcM));
+    // boxes of 32 and 64 rows of X^ (up to 8 and 16 rhs)
+    for (int b = 0; b < 2; ++b) {
+        EMS_TRY(encode3d(&m[12 + 4 * b], h->tc_Xh, ej, rows, nb, 32, 32 << b, CU_TENSOR_MAP_SWIZZLE_64B));
+        EMS_TRY(encode3d(&m[13 + 4 * b], h->tc_Xl, ej, rows, nb, 32, 32 << b, CU_TENSOR_MAP_SWIZZLE_64B));
+        EMS_TRY(encode3d(&m[14 + 4 * b], h->tc_Xh, ej, rows, nb, 64, 32 << b));
+        EMS_TRY(encode3d(&m[15 + 4 * b], h->tc_Xl, ej, rows, nb, 64, 32 << b));
+    }
     EMS_TRY(encode3d(&m[10], h->tc_Bh, ej, 2 * E, 2 * nb, 64, kTcN));
     EMS_TRY(encode3d(&m[11], h->tc_Bl, ej, 2 * E, 2 * nb, 64, kTcN));
     h->tc_ej = ej;
@@ -987,11 +1021,10 @@ int tc_macromodel(emsurf_handle* h, const double2* x, const float2* xf, float2* 
     }
     const int ntiles = h->tc_mm_ntiles[R];
     const int2* tiles = static_cast<const int2*>(h->tc_mm_tiles[R]);
-    const size_t total = (size_t)ntiles * kTcM * kp;
-    tc_mm_gather_kernel<<<(int)std::min<size_t>((total + 255) / 256, (size_t)h->num_sms * 16), 256, 0, st>>>(
+    tc_mm_gather_kernel<<<std::min(4 * ntiles, h->num_sms * 16), 256, 0, st>>>(
         x, xf, h->d_uo_index, h->d_uo_sign, tiles, h->d_type_ptr, h->d_type_cells,
         reinterpret_cast<__nv_bfloat16*>(h->tc_Mh), reinterpret_cast<__nv_bfloat16*>(h->tc_Ml), K, kp, R,
-        h->n_unique, total);
+        h->n_unique, ntiles);
     EMS_CUDA(cudaGetLastError());
     MmArgs a;
     a.Y = Ymm;
@@ -1035,14 +1068,17 @@ int tc_binmul_launch(emsurf_handle* h, float2* Y, int R, const float2* coef, int
     a.err = h->d_err;
     const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(h->tc_maps);
     const int grid = std::min(a.items, h->num_sms);
+    a.a_rows = R <= 8 ? 32 : R <= 16 ? 64 : kTcM;
+    const int mx = R <= 8 ? 12 : R <= 16 ? 16 : 0;      // maps of the X^ planes, both ring shapes
+    const int m32 = mx, m64 = mx ? mx + 2 : 8;
     if (variant == 0) {
         constexpr int sm = bm_smem<32, 5>();
         EMS_TRY(set_smem_once(binmul_tc_kernel<32, 5>, (size_t)sm));
-        binmul_tc_kernel<32, 5><<<grid, kTcThreads, sm, st>>>(m[0], m[1], m[2], m[3], a);
+        binmul_tc_kernel<32, 5><<<grid, kTcThreads, sm, st>>>(m[m32], m[m32 + 1], m[2], m[3], a);
     } else {
         constexpr int sm = bm_smem<64, 2>();
         EMS_TRY(set_smem_once(binmul_tc_kernel<64, 2>, (size_t)sm));
-        binmul_tc_kernel<64, 2><<<grid, kTcThreads, sm, st>>>(m[8], m[9], m[10], m[11], a);
+        binmul_tc_kernel<64, 2><<<grid, kTcThreads, sm, st>>>(m[m64], m[m64 + 1], m[10], m[11], a);
     }
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
@@ -1053,9 +1089,8 @@ int tc_binmul_launch(emsurf_handle* h, float2* Y, int R, const float2* coef, int
 int tc_binmul(emsurf_handle* h, const float2* X, float2* Y, int R, const float2* coef, cudaStream_t st) {
     const int E = h->E, ej = h->tc_ej, rows = h->tc_rows;
     const size_t nb = (size_t)h->nbins;
-    const size_t xs = nb * rows * ej;
-    tc_split_x_kernel<<<(int)std::min<size_t>((xs + 255) / 256, (size_t)h->num_sms * 16), 256, 0, st>>>(
-        X, reinterpret_cast<__nv_bfloat16*>(h->tc_Xh), reinterpret_cast<__nv_bfloat16*>(h->tc_Xl), E, ej, R, rows, xs);
+    tc_split_x_kernel<<<(int)std::min<size_t>(nb, (size_t)h->num_sms * 8), 256, 0, st>>>(
+        X, reinterpret_cast<__nv_bfloat16*>(h->tc_Xh), reinterpret_cast<__nv_bfloat16*>(h->tc_Xl), E, ej, R, rows, (int)nb);
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
     return tc_binmul_launch(h, Y, R, coef, h->tc_variant, st);
@@ -1130,6 +1165,11 @@ int pc_tc_build(emsurf_handle* h, const std::vector<int32_t>& optr) {
     CUtensorMap* m = reinterpret_cast<CUtensorMap*>(h->pc_tc_maps);
     EMS_TRY(encode3d(&m[0], h->pc_tc_Rh, np, kTcM, h->M, kTcKc, kTcM));
     EMS_TRY(encode3d(&m[1], h->pc_tc_Rl, np, kTcM, h->M, kTcKc, kTcM));
+    // boxes of 32 and 64 rows (up to 16 and 32 rhs)
+    for (int b = 0; b < 2; ++b) {
+        EMS_TRY(encode3d(&m[4 + 2 * b], h->pc_tc_Rh, np, kTcM, h->M, kTcKc, 32 << b));
+        EMS_TRY(encode3d(&m[5 + 2 * b], h->pc_tc_Rl, np, kTcM, h->M, kTcKc, 32 << b));
+    }
     EMS_TRY(encode3d(&m[2], h->pc_tc_Xh, np, rows, 1, kTcKc, kTcN));
     EMS_TRY(encode3d(&m[3], h->pc_tc_Xl, np, rows, 1, kTcKc, kTcN));
     h->have_pc_tc = true;
@@ -1139,8 +1179,8 @@ int pc_tc_build(emsurf_handle* h, const std::vector<int32_t>& optr) {
 template <typename VT>
 int pc_tc_apply(emsurf_handle* h, const VT* r, VT* y, int R, cudaStream_t st) {
     const int np = h->pc_tc_np;
-    const size_t gs = (size_t)h->M * kTcM * np;
-    pc_tc_gather_kernel<VT><<<(int)std::min<size_t>((gs + 255) / 256, (size_t)h->num_sms * 16), 256, 0, st>>>(
+    const int gs = h->M * R * (np / 8);
+    pc_tc_gather_kernel<VT><<<std::min((gs + 255) / 256, h->num_sms * 16), 256, 0, st>>>(
         r, h->pc_sub_ptr, h->pc_sub_ids, h->pc_n, R, h->n_unique, np,
         reinterpret_cast<__nv_bfloat16*>(h->pc_tc_Rh), reinterpret_cast<__nv_bfloat16*>(h->pc_tc_Rl), gs);
     EMS_CUDA(cudaGetLastError());
@@ -1158,7 +1198,9 @@ int pc_tc_apply(emsurf_handle* h, const VT* r, VT* y, int R, cudaStream_t st) {
     a.err = h->d_err;
     EMS_TRY(set_smem_once(pc_tc_kernel, (size_t)kMmSmem));
     const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(h->pc_tc_maps);
-    pc_tc_kernel<<<std::min(a.nitems, h->num_sms), kTcThreads, kMmSmem, st>>>(m[0], m[1], m[2], m[3], a);
+    a.a_rows = R <= 16 ? 32 : R <= 32 ? 64 : kTcM;
+    const int ma = R <= 16 ? 4 : R <= 32 ? 6 : 0;
+    pc_tc_kernel<<<std::min(a.nitems, h->num_sms), kTcThreads, kMmSmem, st>>>(m[ma], m[ma + 1], m[2], m[3], a);
     EMS_CUDA(cudaGetLastError());
     h->launches += 2;
     return EMSURF_OK;

@@ -249,7 +249,7 @@ struct emsurf_handle {
     std::vector<void*> tc_mm_tiles;   // per rhs count: device (type, first column) tile list
     std::vector<int> tc_mm_ntiles;
     // tensor maps: X hi, X lo, B hi, B lo (bin multiply); x1 hi, x1 lo, Z hi, Z lo (macromodels)
-    alignas(64) unsigned char tc_maps[12][128];
+    alignas(64) unsigned char tc_maps[20][128];
     int tc_variant = 0;                    // bin multiply ring shape picked by the autotuner
     float tc_tune_ms[2] = {0.f, 0.f};      // the two shapes' times at create
     int mm_occ[4] = {0, 0, 0, 0};          // resident macromodel CTAs per SM (FP32, FP64; x 1 / 4 rhs)
@@ -284,7 +284,7 @@ struct emsurf_handle {
     void* pc_tc_Rl = nullptr;
     void* pc_tc_items = nullptr;    // (cell, first owned row) per item
     int pc_tc_nitems = 0, pc_tc_np = 0;
-    alignas(64) unsigned char pc_tc_maps[4][128];
+    alignas(64) unsigned char pc_tc_maps[8][128];
     const double2* near_L = nullptr;  // near offset tables [5][5][E][E] (|dx|, |dy| <= 2)
     const double2* near_K = nullptr;
     int32_t* pc_n = nullptr;        // [M] subdomain sizes
