@@ -345,7 +345,7 @@ int slab_top(double a, double b, double z, int n, double side, int patch_n, int 
 // complex wavenumber k = kr + j ki (Im k < 0 in a lossy region, e^{jwt})
 int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* shifts,
                        const int8_t* singular, int nb, double kr, double ki, double2* L,
-                       double2* K, cudaStream_t st, const int32_t* slot = nullptr);
+                       double2* K, cudaStream_t st);
 // L, K [cell][L, K][E][E] of each mesh tested on itself; equal T and E in all meshes
 int tabulate_cells_cx(const std::vector<MeshView>& cells, double kr, double ki, double2* LK, cudaStream_t st);
 // Galerkin L, K [nb][test E][src E] on the device for nb test-mesh shifts

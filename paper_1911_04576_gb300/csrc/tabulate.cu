@@ -238,6 +238,22 @@ __device__ __forceinline__ void potentials(Vec3 r, const TriGeo& T, double& I0, 
     Ig = (-sg * bsum) * n - fu;
 }
 
+// Pairs of triangles that a lattice of boxes repeats: key of (block, test, source)
+// = both shapes (triangles equal up to a shift along the box's grid) and the grid
+// displacement between them.  tab[key] = row of the class in the table of slot
+// integrals.
+struct PairClasses {
+    int* tab;                    // [shapes][shapes][nx][ny]
+    const int* shape;            // [T]
+    const int2* at;              // [T] grid position of each triangle
+    const int2* off;             // [block] grid displacement of the test box
+    int shapes, nx, ny, x0, y0;
+    __device__ __forceinline__ size_t key(int b, int t, int s) const {
+        const int2 d = off[b], p = at[t], q = at[s];
+        return (((size_t)shape[t] * shapes + shape[s]) * nx + (p.x + d.x - q.x - x0)) * ny + (p.y + d.y - q.y - y0);
+    }
+};
+
 // out[((b*Tt + t)*Ts + s)*18 + {0..8: L(i,j), 9..17: K(i,j)}]; CX: complex
 // wavenumber k + j ki (lossy region), else ki is ignored; SING: closed-form
 // 1/R parts.
@@ -261,11 +277,21 @@ __device__ __forceinline__ void potentials(Vec3 r, const TriGeo& T, double& I0, 
 template <bool CX, bool SING>
 __global__ void __launch_bounds__(128)
 tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict__ sg, int Ts, int own,
-                 const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out) {
-    const int pair = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pair >= Tt * Ts) return;
+                 const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out,
+                 const int* __restrict__ reps, int n_reps) {
+    int pair = blockIdx.x * blockDim.x + threadIdx.x, bl = blockIdx.y;
+    size_t row = (size_t)bl * Tt * Ts + pair;
+    if (reps) {
+        // one member (b Tt + t) Ts + s of each class of pairs
+        if (pair >= n_reps) return;
+        row = pair;
+        const int r = reps[pair];
+        bl = r / (Tt * Ts);
+        pair = r - bl * (Tt * Ts);
+    } else if (pair >= Tt * Ts) {
+        return;
+    }
     const int t = pair / Ts, s = pair - t * Ts;
-    const int bl = blockIdx.y;
     // own: every block has its own mesh, test = source, not shifted
     const TriGeo& A = tg[(own ? (b0 + bl) * Tt : 0) + t];
     const TriGeo& S = sg[(own ? (b0 + bl) * Ts : 0) + s];
@@ -384,7 +410,7 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
     if constexpr (SING) div.x += fs * (PB[0] + PB[1] + PB[2]);
     if constexpr (CX) div = cmul(ik2, div);
     else div = make_double2(ik2.x * div.x, ik2.x * div.y);
-    double2* o = out + ((size_t)bl * Tt * Ts + pair) * 18;
+    double2* o = out + row * 18;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -425,11 +451,11 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
         }
 }
 
-// L[o][m][n], K[o][m][n], o = slot[b] (b without a slot list), from the slot
-// integrals of one chunk; own: every block's own RWGs, its K after its L
+// L[b][m][n], K[b][m][n] from the slot integrals of one chunk; own: every
+// block's own RWGs, its K after its L
 __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots* __restrict__ tr,
                                   int Et, const RwgSlots* __restrict__ sr, int Es, int Tt, int Ts,
-                                  int b0, int nb, int own, const int32_t* __restrict__ slot, double2* __restrict__ L,
+                                  int b0, int nb, int own, double2* __restrict__ L,
                                   double2* __restrict__ K) {
     const size_t total = (size_t)nb * Et * Es;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
@@ -452,7 +478,61 @@ __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots*
                 kk.x += c * p[9 + ij].x;
                 kk.y += c * p[9 + ij].y;
             }
-        const size_t o = ((size_t)(slot ? slot[b0 + bl] : own ? 2 * (b0 + bl) : b0 + bl) * Et + m) * Es + n;
+        const size_t o = ((size_t)(own ? 2 * (b0 + bl) : b0 + bl) * Et + m) * Es + n;
+        L[o] = l;
+        K[o] = kk;
+    }
+}
+
+constexpr int kNoMember = 0x7f7f7f7f;        // memset pattern
+// the lowest member (b T + t) T + s, b from b0, of every class of the blocks b0 ..
+__global__ void mark_classes_kernel(PairClasses c, int T, int b0, int total) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int b = e / (T * T), p = e - b * (T * T);
+        atomicMin(c.tab + c.key(b0 + b, p / T, p % T), e);
+    }
+}
+// rows for the marked classes (tab: member -> row) and their members; rows past
+// cap are only counted
+__global__ void number_classes_kernel(int* __restrict__ tab, size_t n, int* __restrict__ reps, int cap,
+                                      int* __restrict__ count) {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        const int m = tab[e];
+        const bool live = m != kNoMember;
+        const unsigned who = __ballot_sync(__activemask(), live);
+        if (!live) continue;
+        const int lane = threadIdx.x & 31, first = __ffs(who) - 1;
+        int base = 0;
+        if (lane == first) base = atomicAdd(count, __popc(who));
+        base = __shfl_sync(who, base, first) + __popc(who & ((1u << lane) - 1));
+        tab[e] = base;
+        if (base < cap) reps[base] = m;
+    }
+}
+// L[slot][m][n], K[slot][m][n] from the classes' slot integrals, blocks b0 ..
+__global__ void class_gather_kernel(const double2* __restrict__ S, PairClasses c, const RwgSlots* __restrict__ rw, int E,
+                                    int b0, int nb, const int32_t* __restrict__ slot, double2* __restrict__ L,
+                                    double2* __restrict__ K) {
+    const size_t total = (size_t)nb * E * E;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const int n = (int)(e % E);
+        const size_t t2 = e / E;
+        const int m = (int)(t2 % E), b = b0 + (int)(t2 / E);
+        const RwgSlots A = rw[m], B = rw[n];
+        double2 l = make_double2(0.0, 0.0), kk = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const double f = A.c[x] * B.c[y];
+                const double2* p = S + (size_t)c.tab[c.key(b, A.t[x], B.t[y])] * 18 + 3 * A.s[x] + B.s[y];
+                const double2 pl = p[0], pk = p[9];
+                l.x += f * pl.x;
+                l.y += f * pl.y;
+                kk.x += f * pk.x;
+                kk.y += f * pk.y;
+            }
+        const size_t o = ((size_t)slot[b] * E + m) * E + n;
         L[o] = l;
         K[o] = kk;
     }
@@ -552,11 +632,11 @@ cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, boo
         double2* o = out + (size_t)c * Tt * Ts * 18;
         const bool s = own || singular[b0 + c] != 0;
         if (ki != 0.0) {
-            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o);
-            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o);
+            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o, nullptr, 0);
+            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o, nullptr, 0);
         } else {
-            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o);
-            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o);
+            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o, nullptr, 0);
+            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o, nullptr, 0);
         }
         const cudaError_t err = cudaGetLastError();
         if (err != cudaSuccess) return err;
@@ -566,12 +646,10 @@ cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, boo
 }
 }  // namespace
 
-// L, K: device [nb][Et][Es] (block b at slot[b] when slot is not NULL);
-// wavenumber k + j ki (ki = 0: lossless).  cells: nb meshes instead, each tested
+// L, K: device [nb][Et][Es]; wavenumber k + j ki (ki = 0: lossless).  cells: nb meshes instead, each tested
 // on itself (test = src = cells[b], singular), L = [nb][L, K][E][E].
 static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshView& src, const double* shifts,
-                        const int8_t* singular, int nb, double k, double ki, double2* L, double2* K, cudaStream_t st,
-                        const int32_t* slot) {
+                        const int8_t* singular, int nb, double k, double ki, double2* L, double2* K, cudaStream_t st) {
     if (!(k > 0.0) || !(ki <= 0.0) || nb < 1) {
         set_error("tabulate needs Re k > 0, Im k <= 0 and >= 1 block");
         return EMSURF_EINVAL;
@@ -597,7 +675,6 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     TriGeo *dtg = nullptr, *dsg = nullptr;
     RwgSlots *dtr = nullptr, *dsr = nullptr;
     double* dsh = nullptr;
-    int32_t* dslot = nullptr;
     double2* scratch = nullptr;
     int status = EMSURF_OK;
     auto fail = [&](cudaError_t e, const char* what) {
@@ -610,7 +687,6 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     if (!status && (e = cudaMalloc(&dtr, sizeof(RwgSlots) * tr.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && !own && (e = cudaMalloc(&dsr, sizeof(RwgSlots) * sr.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && !own && (e = cudaMalloc(&dsh, sizeof(double) * 3 * nb)) != cudaSuccess) fail(e, "alloc");
-    if (!status && slot && (e = cudaMalloc(&dslot, sizeof(int32_t) * nb)) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&scratch, per_block * chunk)) != cudaSuccess) fail(e, "scratch alloc");
     if (!status) {
         cudaMemcpyAsync(dtg, tg.data(), sizeof(TriGeo) * tg.size(), cudaMemcpyHostToDevice, st);
@@ -620,7 +696,6 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
             cudaMemcpyAsync(dsr, sr.data(), sizeof(RwgSlots) * sr.size(), cudaMemcpyHostToDevice, st);
             cudaMemcpyAsync(dsh, shifts, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, st);
         }
-        if (slot) cudaMemcpyAsync(dslot, slot, sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st);
         const TriGeo* ds = own ? dtg : dsg;
         const RwgSlots* drs = own ? dtr : dsr;
         for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
@@ -629,7 +704,7 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
             if (e != cudaSuccess) { fail(e, "tri_pairs_kernel"); break; }
             const size_t tot = (size_t)nc * test.E * src.E;
             const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
-            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, drs, src.E, test.T, src.T, b0, nc, own, dslot, L,
+            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, drs, src.E, test.T, src.T, b0, nc, own, L,
                                                   own ? L + (size_t)test.E * src.E : K);
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "rwg_gather_kernel"); break; }
         }
@@ -640,21 +715,179 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     cudaFree(dtr);
     cudaFree(dsr);
     cudaFree(dsh);
-    cudaFree(dslot);
     cudaFree(scratch);
     return status;
 }
 
 int tabulate_blocks_cx(const MeshView& test, const MeshView& src, const double* shifts,
                        const int8_t* singular, int nb, double k, double ki, double2* L, double2* K,
-                       cudaStream_t st, const int32_t* slot) {
-    return tabulate_any(nullptr, test, src, shifts, singular, nb, k, ki, L, K, st, slot);
+                       cudaStream_t st) {
+    return tabulate_any(nullptr, test, src, shifts, singular, nb, k, ki, L, K, st);
 }
 
 // LK[b] = L, K of cell b on itself; all meshes have the same number of triangles and RWGs
 int tabulate_cells_cx(const std::vector<MeshView>& cells, double k, double ki, double2* LK, cudaStream_t st) {
-    return tabulate_any(cells.data(), cells[0], cells[0], nullptr, nullptr, (int)cells.size(), k, ki, LK, nullptr, st,
-                        nullptr);
+    return tabulate_any(cells.data(), cells[0], cells[0], nullptr, nullptr, (int)cells.size(), k, ki, LK, nullptr, st);
+}
+
+// L, K of one box against its copies at the grid displacements off (box sides of
+// nq grid steps; the first n_touch blocks touch), block b at slot[b].  The mesh
+// repeats itself along its faces and from box to box, so most pairs of triangles
+// are shifted copies of others: one of each class is integrated (16 x 16 boxes
+// of 192 triangles: 1.6 of 4.9 million pairs), and the blocks are gathered from
+// the classes' table.  Chunks of blocks keep the table below kScratchBytes.
+static int tabulate_lattice(const MeshView& m, const std::vector<int2>& off, int nq, double a, double b_, int n_touch,
+                            double k, double2* L, double2* K, const std::vector<int32_t>& slot, cudaStream_t st) {
+    if (!(k > 0.0)) {
+        set_error("tabulate needs k > 0");
+        return EMSURF_EINVAL;
+    }
+    std::vector<TriGeo> geo;
+    std::vector<RwgSlots> rw;
+    EMS_TRY(prepare_mesh(m.verts, m.tris, m.slot_rwg, m.slot_sgn, m.T, m.E, geo, rw));
+    const int nb = (int)off.size(), T = m.T;
+    const double hx = a / nq, hy = b_ / nq;
+    // grid position of each triangle's lowest corner and its shape: equal vertices
+    // relative to it, in any order of triangles; one off the grid is a shape of its own
+    std::vector<int> shape(T, -1);
+    std::vector<int2> at(T);
+    std::vector<int> first;                       // a triangle of each shape
+    double mx = geo[0].v[0], my = geo[0].v[1];
+    for (const TriGeo& g : geo)
+        for (int v = 0; v < 3; ++v) {
+            mx = std::min(mx, g.v[3 * v]);
+            my = std::min(my, g.v[3 * v + 1]);
+        }
+    auto corner = [&](const TriGeo& g, int x) { return std::min(g.v[x], std::min(g.v[3 + x], g.v[6 + x])); };
+    for (int t = 0; t < T; ++t) {
+        const double px = (corner(geo[t], 0) - mx) / hx, py = (corner(geo[t], 1) - my) / hy;
+        at[t] = make_int2((int)std::lround(px), (int)std::lround(py));
+        const bool on = std::fabs(px - at[t].x) <= 1e-9 && std::fabs(py - at[t].y) <= 1e-9;
+        for (int f = 0; on && f < (int)first.size() && shape[t] < 0; ++f) {
+            bool same = true;
+            for (int v = 0; v < 9 && same; ++v) {
+                const int x = v % 3;
+                const double u = geo[t].v[v] - (x < 2 ? corner(geo[t], x) : 0.0);
+                const double w = geo[first[f]].v[v] - (x < 2 ? corner(geo[first[f]], x) : 0.0);
+                same = std::fabs(u - w) <= 1e-9 * std::min(hx, hy);
+            }
+            if (same) shape[t] = f;
+        }
+        if (shape[t] < 0) {
+            shape[t] = (int)first.size();
+            first.push_back(t);
+        }
+    }
+    const int S = (int)first.size();
+    std::vector<double> shifts(3 * (size_t)nb);
+    for (int b = 0; b < nb; ++b) {
+        shifts[3 * b] = off[b].x / nq * a;
+        shifts[3 * b + 1] = off[b].y / nq * b_;
+        shifts[3 * b + 2] = 0.0;
+    }
+    // classes of blocks b0 .. b0 + nc: extent of the displacements
+    auto extent = [&](int b0, int nc, PairClasses& c) {
+        int lx = off[b0].x, hx_ = lx, ly = off[b0].y, hy_ = ly;
+        for (int b = b0; b < b0 + nc; ++b) {
+            lx = std::min(lx, off[b].x);
+            hx_ = std::max(hx_, off[b].x);
+            ly = std::min(ly, off[b].y);
+            hy_ = std::max(hy_, off[b].y);
+        }
+        c.x0 = lx - nq;
+        c.y0 = ly - nq;
+        c.nx = hx_ - lx + 2 * nq + 1;
+        c.ny = hy_ - ly + 2 * nq + 1;
+        return (size_t)S * S * c.nx * c.ny;
+    };
+    constexpr size_t kTabBytes = 64ull << 20;
+    const int cap = (int)std::max<size_t>(kScratchBytes / (18 * sizeof(double2)), (size_t)T * T);
+    // the most blocks a chunk may have, then less until its classes fit
+    auto chunk_of = [&](int b0, int end) {
+        PairClasses c;
+        int nc = (int)std::min<long long>(end - b0, kNoMember / ((long long)T * T));
+        while (nc > 1 && extent(b0, nc, c) * sizeof(int) > kTabBytes) nc = (nc + 1) / 2;
+        return std::max(nc, 1);
+    };
+    // a chunk's extent is that of one block, below the limit, or that of all blocks
+    PairClasses whole;
+    const size_t one = (size_t)S * S * (2 * nq + 1) * (2 * nq + 1);
+    const size_t tab_n = std::min(std::max(kTabBytes / sizeof(int), one), extent(0, nb, whole));
+    double wl[21];
+    rule_moments(wl);
+    EMS_CUDA(cudaMemcpyToSymbolAsync(c_wl, wl, sizeof(wl), 0, cudaMemcpyHostToDevice, st));
+    // one buffer: class table, members, slot integrals, then the mesh and the blocks
+    size_t bytes = 0;
+    auto part = [&](size_t n) {
+        const size_t o = bytes;
+        bytes += (n + 255) & ~(size_t)255;
+        return o;
+    };
+    const long long all = (long long)nb * T * T;
+    const int rows = (int)std::min<long long>(cap, all);
+    const size_t o_tab = part(tab_n * sizeof(int)), o_rep = part((size_t)rows * sizeof(int)), o_cnt = part(sizeof(int)),
+                 o_S = part((size_t)rows * 18 * sizeof(double2)), o_geo = part(T * sizeof(TriGeo)),
+                 o_rw = part(m.E * sizeof(RwgSlots)), o_sh = part(T * sizeof(int)), o_at = part(T * sizeof(int2)),
+                 o_off = part(nb * sizeof(int2)), o_slot = part(nb * sizeof(int32_t)), o_shift = part(3 * nb * sizeof(double));
+    unsigned char* w = nullptr;
+    cudaError_t e = cudaMalloc(&w, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        set_error("tabulate: device allocation of %zu bytes: %s", bytes, cudaGetErrorString(e));
+        return EMSURF_ECUDA;
+    }
+    auto put = [&](size_t o, const void* src, size_t n) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(w + o, src, n, cudaMemcpyHostToDevice, st);
+    };
+    put(o_geo, geo.data(), T * sizeof(TriGeo));
+    put(o_rw, rw.data(), m.E * sizeof(RwgSlots));
+    put(o_sh, shape.data(), T * sizeof(int));
+    put(o_at, at.data(), T * sizeof(int2));
+    put(o_off, off.data(), nb * sizeof(int2));
+    put(o_slot, slot.data(), nb * sizeof(int32_t));
+    put(o_shift, shifts.data(), 3 * nb * sizeof(double));
+    int *tab = reinterpret_cast<int*>(w + o_tab), *reps = reinterpret_cast<int*>(w + o_rep), *cnt = reinterpret_cast<int*>(w + o_cnt);
+    double2* U = reinterpret_cast<double2*>(w + o_S);
+    const TriGeo* dg = reinterpret_cast<const TriGeo*>(w + o_geo);
+    const RwgSlots* dr = reinterpret_cast<const RwgSlots*>(w + o_rw);
+    const double* dsh = reinterpret_cast<const double*>(w + o_shift);
+    for (int b0 = 0; b0 < nb && e == cudaSuccess;) {
+        const bool touch = b0 < n_touch;
+        int nc = chunk_of(b0, touch ? n_touch : nb), n_cls = 0;
+        PairClasses c{tab, reinterpret_cast<const int*>(w + o_sh), reinterpret_cast<const int2*>(w + o_at),
+                      reinterpret_cast<const int2*>(w + o_off), S, 0, 0, 0, 0};
+        for (;;) {
+            const size_t n = extent(b0, nc, c);
+            const int total = nc * T * T;
+            e = cudaMemsetAsync(tab, 0x7f, n * sizeof(int), st);          // 0x7f7f7f7f: no member
+            if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(int), st);
+            if (e != cudaSuccess) break;
+            mark_classes_kernel<<<std::min((total + 255) / 256, 152 * 32), 256, 0, st>>>(c, T, b0, total);
+            number_classes_kernel<<<(int)std::min<size_t>((n + 255) / 256, 152 * 16), 256, 0, st>>>(tab, n, reps, rows, cnt);
+            e = cudaGetLastError();
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&n_cls, cnt, sizeof(int), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess || n_cls <= rows) break;
+            nc = std::max(1, std::min(nc - 1, (int)((double)nc * rows / n_cls * 0.95)));
+        }
+        if (e != cudaSuccess) break;
+        const dim3 g((unsigned)((n_cls + 127) / 128));
+        if (touch) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(dg, T, dg, T, 0, dsh, b0, k, 0.0, U, reps, n_cls);
+        else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(dg, T, dg, T, 0, dsh, b0, k, 0.0, U, reps, n_cls);
+        const size_t tot = (size_t)nc * m.E * m.E;
+        class_gather_kernel<<<(int)std::min<size_t>((tot + 255) / 256, 152 * 64), 256, 0, st>>>(
+            U, c, dr, m.E, b0, nc, reinterpret_cast<const int32_t*>(w + o_slot), L, K);
+        e = cudaGetLastError();
+        b0 += nc;
+    }
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
+    cudaFree(w);
+    if (e != cudaSuccess) {
+        set_error("tabulate: %s", cudaGetErrorString(e));
+        return EMSURF_ECUDA;
+    }
+    return EMSURF_OK;
 }
 
 int tabulate_blocks(const MeshView& test, const MeshView& src, const double* shifts,
@@ -786,7 +1019,7 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
         const size_t tot = (size_t)nc * test.E * src.E;
         const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
         rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc, 0,
-                                              nullptr, L, K);
+                                              L, K);
         step(cudaGetLastError(), "rwg_gather_kernel");
     }
     step(cudaStreamSynchronize(st), "synchronize");
@@ -913,8 +1146,9 @@ extern "C" {
 // each orbit is integrated (136 of 961 on a 16 x 16 lattice of square cells
 // with even n), touching ones together with their -d; the others are signed
 // permutations of it.  Tabulation is bound by the FP64 rate, so its time
-// follows the integrated offsets: 38 ms for 16 x 16 boxes of 288 RWGs, 650 ms
-// with every offset integrated point pair by point pair.
+// follows the integrated pairs: 15.4 ms for 16 x 16 boxes of 288 RWGs, 38 ms
+// without the classes of shifted pairs, 650 ms with every offset integrated
+// point pair by point pair.
 EMSURF_API int emsurf_tabulate_offsets(double a, double b, double h, int32_t n,
                                        const double* zlevels, int32_t nx, int32_t ny, double k,
                                        emsurf_c128* L, emsurf_c128* K, void* stream) {
@@ -987,19 +1221,14 @@ EMSURF_API int emsurf_tabulate_offsets(double a, double b, double h, int32_t n,
     }
     const int n_touch = (int)slot.size();
     slot.insert(slot.end(), far.begin(), far.end());
-    std::vector<double> shifts(3 * slot.size());
-    std::vector<int8_t> sing(slot.size());
-    for (size_t i = 0; i < slot.size(); ++i) {
-        shifts[3 * i] = (slot[i] % nox - (nx - 1)) * a;
-        shifts[3 * i + 1] = (slot[i] / nox - (ny - 1)) * b;
-        shifts[3 * i + 2] = 0.0;
-        sing[i] = (int)i < n_touch ? 1 : 0;
-    }
+    std::vector<int2> off(slot.size());
+    for (size_t i = 0; i < slot.size(); ++i)
+        off[i] = make_int2((slot[i] % nox - (nx - 1)) * n, (slot[i] / nox - (ny - 1)) * n);
     MeshView mv{verts.data(), tris.data(), srw.data(), ssg.data(), T, E};
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     double2* Ld = reinterpret_cast<double2*>(L);
     double2* Kd = reinterpret_cast<double2*>(K);
-    EMS_TRY(tabulate_blocks_cx(mv, mv, shifts.data(), sing.data(), (int)slot.size(), k, 0.0, Ld, Kd, st, slot.data()));
+    EMS_TRY(tabulate_lattice(mv, off, n, a, b, n_touch, k, Ld, Kd, slot, st));
     // reciprocal part of the touching blocks, then the images
     unsigned char* dbuf = nullptr;
     const size_t b_touch = touch.size() * sizeof(int2), b_inv = inv.size() * sizeof(uint32_t);
