@@ -41,6 +41,26 @@ int set_smem_once(F* kernel, size_t bytes) {
     return set_smem_attr(reinterpret_cast<const void*>(kernel), bytes);
 }
 
+// A kernel launched with launch_after may start while the one before it in the
+// stream drains (once all of that one's blocks have called dep_trigger or
+// ended): what it does before dep_wait must not depend on earlier kernels.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------- complex
 __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);

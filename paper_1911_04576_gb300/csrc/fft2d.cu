@@ -60,6 +60,7 @@ fft2d_fwd_kernel(T2* __restrict__ Xg, long long lanes, F2Plan f, int K, int n_un
                  const float2* __restrict__ xf, const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_k[kF2MaxW], s_r[kF2MaxW];
+    dep_trigger();
     T2* cur = reinterpret_cast<T2*>(smem_raw);
     T2* nxt = cur + f.buf0;
     T2* tx = nxt + f.buf1;
@@ -139,6 +140,7 @@ fft2d_inv_kernel(const T2* __restrict__ Yg, long long lanes, F2Plan f, int K, in
                  T2* __restrict__ y1) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_k[kF2MaxW], s_r[kF2MaxW];
+    dep_trigger();
     T2* cur = reinterpret_cast<T2*>(smem_raw);
     T2* nxt = cur + f.buf0;
     T2* tx = nxt + f.buf1;

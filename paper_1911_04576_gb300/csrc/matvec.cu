@@ -205,6 +205,10 @@ __global__ void binmul_kernel(const T2* __restrict__ Bhat, const T2* __restrict_
 // copies; the other warps own one test row i each and release a slot with an
 // mbarrier arrive.  Every wait is bounded: on expiry the kernel sets *err,
 // the producer waits (bounded) for its copies in flight, and all return.
+// Launched after the forward transform with programmatic serialisation (as is
+// the pair kernel): the first slabs, which do not depend on X^, stream while that
+// one's last blocks drain (8 x 8 boxes, K = 324, one rhs: product 48.2 -> 44.6 us).
+// The orbit kernel, whose blocks leave no room for the macromodel's, is not.
 // Up to 8 rhs share one pass over the spectrum (16 FMA per element and rhs: HBM
 // bounds up to 3 rhs, the FP32 rate more).  40 x 25 bins, K = 324, 3 rhs (420 MB):
 // 118 us, 229 us in two passes of binmul_kernel, which stays for other E.
@@ -224,6 +228,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
                  "r"(bytes)
                  : "memory");
+}
+// adds to the bytes of the phase without arriving
+__device__ __forceinline__ void mbar_add_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -301,6 +309,21 @@ binmul_tma_kernel(const float2* __restrict__ Bhat, const float2* __restrict__ Xh
         const uint64_t pol = l2_evict_first();
         int issued = 0;
         bool ok = true;
+        auto copy_slab = [&](int q, int bin, int jb) {
+            const int j0 = jb * kBmJB;
+            const uint32_t bytes_op = (uint32_t)(min(kBmJB, E - j0) * E * sizeof(float2));
+            const float2* src = Bhat + (size_t)bin * 2 * E * E + (size_t)j0 * E;
+            float2* dst = sbuf + (size_t)(q % kBmStages) * stage_elems;
+            bulk_g2s_hint(dst, src, bytes_op, &full[q % kBmStages], pol);
+            bulk_g2s_hint(dst + kBmJB * E, src + (size_t)E * E, bytes_op, &full[q % kBmStages], pol);
+        };
+        // the first slabs do not wait for X^ (a bin has at least kBmStages of them)
+        const int pre = min(kBmStages, total);
+        for (int q = 0; q < pre; ++q) {
+            mbar_add_tx(&full[q], 2 * (uint32_t)(min(kBmJB, E - q * kBmJB) * E * sizeof(float2)));
+            copy_slab(q, (int)blockIdx.x, q);
+        }
+        dep_wait();
         for (int q = 0, t = 0, jb = 0; q < total; ++q) {
             const int s = q % kBmStages;
             if (q >= kBmStages && !mbar_wait(&empty[s], (uint32_t)((q / kBmStages - 1) & 1))) {
@@ -311,11 +334,8 @@ binmul_tma_kernel(const float2* __restrict__ Bhat, const float2* __restrict__ Xh
             const int j0 = jb * kBmJB, jn = min(kBmJB, E - j0);
             const uint32_t bytes_op = (uint32_t)(jn * E * sizeof(float2));
             const uint32_t bytes_x = (uint32_t)(live * K * sizeof(float2));
-            mbar_expect_tx(&full[s], 2 * bytes_op + (jb == 0 ? bytes_x : 0u));
-            const float2* src = Bhat + (size_t)bin * 2 * E * E + (size_t)j0 * E;
-            float2* dst = sbuf + (size_t)s * stage_elems;
-            bulk_g2s_hint(dst, src, bytes_op, &full[s], pol);
-            bulk_g2s_hint(dst + kBmJB * E, src + (size_t)E * E, bytes_op, &full[s], pol);
+            mbar_expect_tx(&full[s], (q < pre ? 0u : 2 * bytes_op) + (jb == 0 ? bytes_x : 0u));
+            if (q >= pre) copy_slab(q, bin, jb);
             if (jb == 0) bulk_g2s(xbuf + (t & 1) * RB * K, Xh + ((size_t)bin * R + r0) * K, bytes_x, &full[s]);
             issued = q + 1;
             if (++jb == nj) {
@@ -495,6 +515,21 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) binmul_tma_pair_kernel(con
         uint32_t ph = 0;
         long long issued = 0;
         bool ok = true;
+        // the first slabs do not wait for X^
+        const int pre = (int)min((long long)kPairStages, q1 - q0);
+        for (int u = 0, b = sb0, j = jb0; u < pre; ++u) {
+            const uint32_t n = (uint32_t)(min(kPairJB, E - j * kPairJB) * E * sizeof(float2));
+            const float2* src = Bhat + (size_t)b * 2 * E * E + (size_t)j * kPairJB * E;
+            float2* dst = sbuf + (size_t)u * stage_elems;
+            mbar_add_tx(&full[u], 2 * n);
+            bulk_g2s_hint(dst, src, n, &full[u], pol);
+            bulk_g2s_hint(dst + kPairJB * E, src + (size_t)E * E, n, &full[u], pol);
+            if (++j == nj) {
+                j = 0;
+                ++b;
+            }
+        }
+        dep_wait();
         for (long long q = q0; q < q1; ++q) {
             if (q - q0 >= kPairStages && !mbar_wait(&empty[s], ph ^ 1u)) {
                 ok = false;
@@ -509,11 +544,13 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) binmul_tma_pair_kernel(con
                 prt = st_part[sb];
             }
             const uint32_t xb = newbin ? (prt != bin ? 2 * bytes_x : bytes_x) : 0u;
-            mbar_expect_tx(&full[s], 2 * bytes_op + xb);
-            const float2* src = Bhat + (size_t)sb * 2 * E * E + (size_t)j0 * E;
-            float2* dst = sbuf + (size_t)s * stage_elems;
-            bulk_g2s_hint(dst, src, bytes_op, &full[s], pol);
-            bulk_g2s_hint(dst + kPairJB * E, src + (size_t)E * E, bytes_op, &full[s], pol);
+            mbar_expect_tx(&full[s], (q - q0 >= pre ? 2 * bytes_op : 0u) + xb);
+            if (q - q0 >= pre) {
+                const float2* src = Bhat + (size_t)sb * 2 * E * E + (size_t)j0 * E;
+                float2* dst = sbuf + (size_t)s * stage_elems;
+                bulk_g2s_hint(dst, src, bytes_op, &full[s], pol);
+                bulk_g2s_hint(dst + kPairJB * E, src + (size_t)E * E, bytes_op, &full[s], pol);
+            }
             if (newbin) {
                 float2* xd = xbuf + (t & 1) * 4 * E;
                 bulk_g2s(xd, Xh + (size_t)bin * 2 * E, bytes_x, &full[s]);
@@ -1185,6 +1222,7 @@ __global__ void scatter_kernel(V2* __restrict__ y, const T2* __restrict__ y1,
                                const int8_t* __restrict__ esg, int MK, int R, int n_unique) {
     using S = decltype(y1[0].x);
     const size_t total = (size_t)R * n_unique;
+    dep_wait();
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
          e += (size_t)gridDim.x * blockDim.x) {
         const int u = (int)(e % n_unique);
@@ -1750,10 +1788,9 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
             // half spectrum (single rhs): one read of each stored bin serves k and -k
             const size_t smem = binmul_tma_pair_smem(E);
             EMS_TRY(set_smem_once(binmul_tma_pair_kernel, smem));
-            binmul_tma_pair_kernel<<<h->pair_grid, 32 * (1 + (E + 31) / 32 + kPairColWarps), smem, st>>>(
+            EMS_CUDA(launch_after(binmul_tma_pair_kernel, dim3(h->pair_grid), 32 * (1 + (E + 31) / 32 + kPairColWarps), smem, st,
                 op.Bhat, op.Xg, op.Yg, h->d_st_bin, h->d_st_part, E, h->nst, op.coef[0], op.coef[1], op.coef[2],
-                op.coef[3], h->d_pair_part, h->d_pair_cnt, h->d_err);
-            EMS_CUDA(cudaGetLastError());
+                op.coef[3], h->d_pair_part, h->d_pair_cnt, h->d_err));
             h->launches += 1;
             bin_done = true;
         }
@@ -1770,9 +1807,8 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
                     occ = std::max(b, 1);
                 }
                 const int grid = std::min(nb, std::max(1, h->num_sms) * (rb == 1 ? 1 : occ));
-                kern<<<grid, threads_tma, smem, st>>>(op.Bhat, op.Xg, op.Yg, E, nb, R, r0, op.coef[0], op.coef[1],
-                                                      op.coef[2], op.coef[3], h->d_err);
-                EMS_CUDA(cudaGetLastError());
+                EMS_CUDA(launch_after(kern, dim3(grid), threads_tma, smem, st, op.Bhat, op.Xg, op.Yg, E, nb, R, r0, op.coef[0],
+                                      op.coef[1], op.coef[2], op.coef[3], h->d_err));
                 h->launches += 1;
                 return EMSURF_OK;
             };
@@ -1838,11 +1874,11 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
     prof_mark(h, ph_fft, false, st);
     prof_mark(h, EMS_PH_SCATTER, true, st);
     if (yf)
-        scatter_kernel<T2, float2><<<grid_for((size_t)R * h->n_unique, 256), 256, 0, st>>>(
-            yf, op.Y1, h->d_inv_ptr, h->d_inv_ent, h->d_inv_sgn, h->M * K, R, h->n_unique);
+        EMS_CUDA(launch_after(scatter_kernel<T2, float2>, dim3(grid_for((size_t)R * h->n_unique, 256)), 256, 0, st, 
+            yf, op.Y1, h->d_inv_ptr, h->d_inv_ent, h->d_inv_sgn, h->M * K, R, h->n_unique));
     else
-        scatter_kernel<T2, double2><<<grid_for((size_t)R * h->n_unique, 256), 256, 0, st>>>(
-            y, op.Y1, h->d_inv_ptr, h->d_inv_ent, h->d_inv_sgn, h->M * K, R, h->n_unique);
+        EMS_CUDA(launch_after(scatter_kernel<T2, double2>, dim3(grid_for((size_t)R * h->n_unique, 256)), 256, 0, st, 
+            y, op.Y1, h->d_inv_ptr, h->d_inv_ent, h->d_inv_sgn, h->M * K, R, h->n_unique));
     EMS_CUDA(cudaGetLastError());
     prof_mark(h, EMS_PH_SCATTER, false, st);
     h->launches += fused ? 4 : 6;   // FFTs (2 fused or 4 passes), macromodel, scatter

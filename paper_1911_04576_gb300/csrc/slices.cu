@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
             long long issued = 0;
             uint32_t ph = 0;
             bool ok = true;
+            if (!mat_side) dep_wait();           // the matrix digits do not depend on the splitting kernel
             for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
                 const int w = it >= g.p[0].items;
                 const SlProb& p = g.p[w];
@@ -384,6 +385,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
         if (!ok) *abort_v = 1;
     } else {
         // ------------------------------------------------ epilogue
+        dep_wait();
         const int qd = warp & 3, half = warp >> 2, rho = 32 * qd + lane;
         const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16);
         int db = 0;
@@ -533,6 +535,7 @@ slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, si
 template <typename Load>
 __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int v0, Load&& load,
                                               unsigned char* __restrict__ X, double* __restrict__ xs) {
+    dep_trigger();
     extern __shared__ double2 s_v[];         // [2][n]
     __shared__ unsigned long long s_mx[2];
     __shared__ int s_ex[2];
@@ -788,8 +791,7 @@ int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Y
         const size_t smem = 1024 + (size_t)g.stages * kSlABytes + xring;
         const int grid = std::min(std::max(1, h->num_sms), b.items + m.items);
         EMS_TRY(set_smem_once(slices_kernel, smem));
-        slices_kernel<<<grid, kSlThreads, smem, st>>>(g);
-        EMS_CUDA(cudaGetLastError());
+        EMS_CUDA(launch_after(slices_kernel, dim3(grid), kSlThreads, smem, st, g));
         h->launches += 2;
     }
     return EMSURF_OK;
