@@ -21,6 +21,7 @@
 // Blocks are processed in chunks so the scratch stays below 256 MB.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -271,13 +272,14 @@ struct PairClasses {
 // point pair, 0.135 ns on average over 25 blocks of 192 x 192 triangles
 // (6.1 ms), against 0.37 ns (16.6 ms) when each point pair updated the 9 + 9
 // slot integrals.  With closed-form parts (32 cells of 256 + 192 triangles in
-// batches that fill the chip, 160 M point pairs): 59 ms, 100 ms with a full
+// batches that fill the chip, pairs of the boxes' triangles once for all cells,
+// 160 M point pairs if they were not): 48 ms, 59 ms without that, 100 ms with a full
 // series beside the closed form of the remainder, three branches with a
 // logarithm each per edge and three atan2 per point.
 template <bool CX, bool SING>
 __global__ void __launch_bounds__(128)
 tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict__ sg, int Ts, int own,
-                 const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out,
+                 int common, const double* __restrict__ shifts, int b0, double k, double ki, double2* __restrict__ out,
                  const int* __restrict__ reps, int n_reps) {
     int pair = blockIdx.x * blockDim.x + threadIdx.x, bl = blockIdx.y;
     size_t row = (size_t)bl * Tt * Ts + pair;
@@ -288,11 +290,17 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
         const int r = reps[pair];
         bl = r / (Tt * Ts);
         pair = r - bl * (Tt * Ts);
-    } else if (pair >= Tt * Ts) {
+    } else if (pair >= Tt * Ts - common * common) {
         return;
+    } else if (common) {
+        // pairs of the first `common` triangles are left out: rows t < common start there
+        const int w = Ts - common, first = common * w;
+        pair = pair < first ? pair / w * Ts + common + pair % w : pair - first + common * Ts;
+        row = (size_t)bl * Tt * Ts + pair;
     }
     const int t = pair / Ts, s = pair - t * Ts;
-    // own: every block has its own mesh, test = source, not shifted
+    // own: every block has its own mesh, test = source, not shifted; its first
+    // `common` triangles are those of all blocks
     const TriGeo& A = tg[(own ? (b0 + bl) * Tt : 0) + t];
     const TriGeo& S = sg[(own ? (b0 + bl) * Ts : 0) + s];
     const Vec3 sh = own ? Vec3{0.0, 0.0, 0.0} : v3(shifts + 3 * (b0 + bl));
@@ -452,10 +460,11 @@ tri_pairs_kernel(const TriGeo* __restrict__ tg, int Tt, const TriGeo* __restrict
 }
 
 // L[b][m][n], K[b][m][n] from the slot integrals of one chunk; own: every
-// block's own RWGs, its K after its L
+// block's own RWGs, its K after its L, pairs of common triangles from Sc
 __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots* __restrict__ tr,
                                   int Et, const RwgSlots* __restrict__ sr, int Es, int Tt, int Ts,
-                                  int b0, int nb, int own, double2* __restrict__ L,
+                                  int b0, int nb, int own, int common,
+                                  const double2* __restrict__ Sc, double2* __restrict__ L,
                                   double2* __restrict__ K) {
     const size_t total = (size_t)nb * Et * Es;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
@@ -471,7 +480,9 @@ __global__ void rwg_gather_kernel(const double2* __restrict__ S, const RwgSlots*
 #pragma unroll
             for (int y = 0; y < 2; ++y) {
                 const double c = A.c[x] * B.c[y];
-                const double2* p = S + (((size_t)bl * Tt + A.t[x]) * Ts + B.t[y]) * 18;
+                const double2* p = A.t[x] < common && B.t[y] < common
+                                       ? Sc + ((size_t)A.t[x] * common + B.t[y]) * 18
+                                       : S + (((size_t)bl * Tt + A.t[x]) * Ts + B.t[y]) * 18;
                 const int ij = 3 * A.s[x] + B.s[y];
                 l.x += c * p[ij].x;
                 l.y += c * p[ij].y;
@@ -622,9 +633,10 @@ void rule_moments(double wl[21]) {
 
 // slot integrals of blocks b0 .. b0 + nc - 1 (singular: host flags), one
 // launch per run of equal flags
-cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, bool own, const double* shifts,
-                         const int8_t* singular, int b0, int nc, double k, double ki, double2* out, cudaStream_t st) {
-    const unsigned gx = (unsigned)(((long long)Tt * Ts + 127) / 128);
+cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, bool own, int common,
+                         const double* shifts, const int8_t* singular, int b0, int nc, double k, double ki, double2* out, cudaStream_t st) {
+    const unsigned gx = (unsigned)(((long long)Tt * Ts - (long long)common * common + 127) / 128);
+    if (gx == 0) return cudaSuccess;
     for (int c = 0; c < nc;) {
         int e = c + 1;
         while (e < nc && (own || (singular[b0 + e] != 0) == (singular[b0 + c] != 0)) && e - c < 65535) ++e;
@@ -632,11 +644,11 @@ cudaError_t launch_pairs(const TriGeo* tg, int Tt, const TriGeo* sg, int Ts, boo
         double2* o = out + (size_t)c * Tt * Ts * 18;
         const bool s = own || singular[b0 + c] != 0;
         if (ki != 0.0) {
-            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o, nullptr, 0);
-            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, ki, o, nullptr, 0);
+            if (s) tri_pairs_kernel<true, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, common, shifts, b0 + c, k, ki, o, nullptr, 0);
+            else tri_pairs_kernel<true, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, common, shifts, b0 + c, k, ki, o, nullptr, 0);
         } else {
-            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o, nullptr, 0);
-            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, shifts, b0 + c, k, 0.0, o, nullptr, 0);
+            if (s) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, common, shifts, b0 + c, k, 0.0, o, nullptr, 0);
+            else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(tg, Tt, sg, Ts, own, common, shifts, b0 + c, k, 0.0, o, nullptr, 0);
         }
         const cudaError_t err = cudaGetLastError();
         if (err != cudaSuccess) return err;
@@ -672,10 +684,18 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     EMS_CUDA(cudaMemcpyToSymbolAsync(c_wl, wl, sizeof(wl), 0, cudaMemcpyHostToDevice, st));
     const size_t per_block = (size_t)test.T * src.T * 18 * sizeof(double2);
     const int chunk = (int)std::max<size_t>(1, std::min<size_t>(nb, kScratchBytes / per_block));
+    // leading triangles that all cells share (a library's boxes), bit for bit: their
+    // pairs are integrated once
+    int common = own && nb > 1 ? test.T : 0;
+    for (int b = 1; b < (own ? nb : 0); ++b) {
+        int c = 0;
+        while (c < common && !std::memcmp(&tg[c], &tg[(size_t)b * test.T + c], sizeof(TriGeo))) ++c;
+        common = c;
+    }
     TriGeo *dtg = nullptr, *dsg = nullptr;
     RwgSlots *dtr = nullptr, *dsr = nullptr;
     double* dsh = nullptr;
-    double2* scratch = nullptr;
+    double2 *scratch = nullptr, *shared = nullptr;
     int status = EMSURF_OK;
     auto fail = [&](cudaError_t e, const char* what) {
         set_error("tabulate: %s: %s", what, cudaGetErrorString(e));
@@ -688,6 +708,8 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     if (!status && !own && (e = cudaMalloc(&dsr, sizeof(RwgSlots) * sr.size())) != cudaSuccess) fail(e, "alloc");
     if (!status && !own && (e = cudaMalloc(&dsh, sizeof(double) * 3 * nb)) != cudaSuccess) fail(e, "alloc");
     if (!status && (e = cudaMalloc(&scratch, per_block * chunk)) != cudaSuccess) fail(e, "scratch alloc");
+    if (!status && common && (e = cudaMalloc(&shared, (size_t)common * common * 18 * sizeof(double2))) != cudaSuccess)
+        fail(e, "scratch alloc");
     if (!status) {
         cudaMemcpyAsync(dtg, tg.data(), sizeof(TriGeo) * tg.size(), cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(dtr, tr.data(), sizeof(RwgSlots) * tr.size(), cudaMemcpyHostToDevice, st);
@@ -698,13 +720,15 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
         }
         const TriGeo* ds = own ? dtg : dsg;
         const RwgSlots* drs = own ? dtr : dsr;
+        if (common && (e = launch_pairs(dtg, common, dtg, common, true, 0, dsh, singular, 0, 1, k, ki, shared, st)) != cudaSuccess)
+            fail(e, "tri_pairs_kernel");
         for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
             const int nc = std::min(chunk, nb - b0);
-            e = launch_pairs(dtg, test.T, ds, src.T, own, dsh, singular, b0, nc, k, ki, scratch, st);
+            e = launch_pairs(dtg, test.T, ds, src.T, own, common, dsh, singular, b0, nc, k, ki, scratch, st);
             if (e != cudaSuccess) { fail(e, "tri_pairs_kernel"); break; }
             const size_t tot = (size_t)nc * test.E * src.E;
             const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
-            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, drs, src.E, test.T, src.T, b0, nc, own, L,
+            rwg_gather_kernel<<<g2, 256, 0, st>>>(scratch, dtr, test.E, drs, src.E, test.T, src.T, b0, nc, own, common, shared, L,
                                                   own ? L + (size_t)test.E * src.E : K);
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "rwg_gather_kernel"); break; }
         }
@@ -716,6 +740,7 @@ static int tabulate_any(const MeshView* cells, const MeshView& test, const MeshV
     cudaFree(dsr);
     cudaFree(dsh);
     cudaFree(scratch);
+    cudaFree(shared);
     return status;
 }
 
@@ -872,8 +897,8 @@ static int tabulate_lattice(const MeshView& m, const std::vector<int2>& off, int
         }
         if (e != cudaSuccess) break;
         const dim3 g((unsigned)((n_cls + 127) / 128));
-        if (touch) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(dg, T, dg, T, 0, dsh, b0, k, 0.0, U, reps, n_cls);
-        else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(dg, T, dg, T, 0, dsh, b0, k, 0.0, U, reps, n_cls);
+        if (touch) tri_pairs_kernel<false, true><<<g, 128, 0, st>>>(dg, T, dg, T, 0, 0, dsh, b0, k, 0.0, U, reps, n_cls);
+        else tri_pairs_kernel<false, false><<<g, 128, 0, st>>>(dg, T, dg, T, 0, 0, dsh, b0, k, 0.0, U, reps, n_cls);
         const size_t tot = (size_t)nc * m.E * m.E;
         class_gather_kernel<<<(int)std::min<size_t>((tot + 255) / 256, 152 * 64), 256, 0, st>>>(
             U, c, dr, m.E, b0, nc, reinterpret_cast<const int32_t*>(w + o_slot), L, K);
@@ -1014,12 +1039,12 @@ int tabulate_blocks_noalloc(const MeshView& test, const MeshView& src, const dou
     // every pair integral is written before it is read, so nothing needs clearing
     for (int b0 = 0; b0 < nb && !status; b0 += chunk) {
         const int nc = std::min(chunk, nb - b0);
-        step(launch_pairs(dtg, test.T, dsg, src.T, false, dsh, singular, b0, nc, k, 0.0, pairs, st), "tri_pairs_kernel");
+        step(launch_pairs(dtg, test.T, dsg, src.T, false, 0, dsh, singular, b0, nc, k, 0.0, pairs, st), "tri_pairs_kernel");
         if (status) break;
         const size_t tot = (size_t)nc * test.E * src.E;
         const int g2 = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
-        rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc, 0,
-                                              L, K);
+        rwg_gather_kernel<<<g2, 256, 0, st>>>(pairs, dtr, test.E, dsr, src.E, test.T, src.T, b0, nc, 0, 0,
+                                              nullptr, L, K);
         step(cudaGetLastError(), "rwg_gather_kernel");
     }
     step(cudaStreamSynchronize(st), "synchronize");
