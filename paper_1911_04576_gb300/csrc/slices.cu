@@ -44,7 +44,8 @@
 // Measured, product of a 16 x 16 lattice with K = 576 (2.38 GB of digits, 350 us
 // at the copy rate): 1161 us in double-single FP32, 593 us here (bins and
 // macromodels 490 us, splitting the vectors 25 us); 12 x 9, K = 576 and 6 rhs:
-// 6575 us, 597 us.  Error against 64 bits 7.2e-14, 6e-15 (both sizes).
+// 6575 us, 567 us (594 us with 8 instead of 12 macromodel columns per entry).
+// Error against 64 bits 7.2e-14, 7e-15 (both sizes).
 #include <algorithm>
 #include <vector>
 
@@ -68,7 +69,6 @@ constexpr int kSlMaxV = 24;                  // vector columns of one launch (a 
                                              // two accumulators and two A blocks fit in TMEM
 constexpr int kSlRhs = kSlMaxV / 4;          // rhs per launch
 constexpr int kSlSplit = 256;                // threads of a splitting block
-constexpr int kSlCells = 8;                  // columns of a macromodel entry
 // the same for two or three barriers at once (their latencies overlap)
 __device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, uint64_t* b2, uint32_t p2,
                                          bool third) {
@@ -623,18 +623,36 @@ slice_cells_kernel(const double2* __restrict__ x, const int32_t* __restrict__ id
 // columns of a launch of Rg rhs
 int sl_bin_v(int Rg) { return (4 * Rg + 7) & ~7; }
 int nk16_of(int n) { return (n + 15) / 16; }
-constexpr int kSlCellRows = sl_up16(kSl * 2 * kSlCells);   // digit rows of a macromodel entry
+// rhs of a launch
+int rhs_per(int R) {
+    const int groups = (R + kSlRhs - 1) / kSlRhs;
+    return (R + groups - 1) / groups;
+}
+// columns of a macromodel entry: as many as the bins' accumulators have room for
+// anyway (an MMA costs the same up to N = 176), at least 8
+int cells_of(int R) { return sl_bin_v(rhs_per(R)) == kSlMaxV ? kSlMaxV / 2 : 8; }
+int cell_rows(int R) { return sl_up16(kSl * 2 * cells_of(R)); }   // digit rows of an entry
 int nst_of(int n) { return (n + kSlK - 1) / kSlK; }
 std::vector<int2> mm_entries(const emsurf_handle* h, int R) {
     std::vector<int2> e;
     for (int t = 0; t < h->T; ++t) {
         const int n = (h->h_type_ptr[t + 1] - h->h_type_ptr[t]) * R;
-        for (int c = 0; c < n; c += kSlCells) e.push_back(make_int2(t, c));
+        for (int c = 0; c < n; c += cells_of(R)) e.push_back(make_int2(t, c));
     }
     return e;
 }
 
-size_t cell_digits(const emsurf_handle* h) { return (size_t)nst_of(h->K) * kSlCellRows * 64; }
+// bytes of the macromodel columns' digits and scales, the most over 1..max_rhs
+size_t cell_digits(const emsurf_handle* h) {
+    size_t n = 0;
+    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * nst_of(h->K) * cell_rows(r) * 64);
+    return n;
+}
+size_t cell_scales(const emsurf_handle* h) {
+    size_t n = 0;
+    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * cells_of(r) * sizeof(double));
+    return n;
+}
 
 }  // namespace
 
@@ -650,7 +668,7 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(double);
     const size_t zbytes = slice_plane_bytes(h->T, 2 * K, K),
                  zrs = (size_t)h->T * K * sizeof(double) +
-                       mm_entries(h, h->max_rhs).size() * (cell_digits(h) + kSlCells * sizeof(double) + 16 * h->max_rhs);
+                       cell_digits(h) + cell_scales(h) + mm_entries(h, h->max_rhs).size() * 16 * h->max_rhs;
     if ((share && !share->sl_A) || E > kSlMaxN) return EMSURF_OK;
     cudaStream_t st = h->setup_stream;
     // work space still to come: grids, products, and the partials of the SIMT macromodels
@@ -688,9 +706,8 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
 int slices_work(emsurf_handle* h) {
     const int R = h->max_rhs, V = sl_bin_v(std::min(R, kSlRhs));
     if (h->sl_Z) {
-        const size_t n = mm_entries(h, R).size();            // the most over 1..R
-        EMS_TRY(dev_alloc(h, (void**)&h->sl_Xc, n * cell_digits(h)));
-        EMS_TRY(dev_alloc(h, (void**)&h->sl_xcs, n * kSlCells * sizeof(double)));
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_Xc, cell_digits(h)));
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_xcs, cell_scales(h)));
         h->sl_ent.assign(R + 1, nullptr);
         h->sl_nent.assign(R + 1, 0);
         for (int r = 1; r <= R; ++r) {
@@ -714,12 +731,12 @@ int slices_work(emsurf_handle* h) {
 
 // Digits of x1 for the macromodel product of R rhs (reads x only).
 int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st) {
-    constexpr int V = 2 * kSlCells;
+    const int V = 2 * cells_of(R);
     EMS_TRY(set_smem_once(slice_cells_kernel, 2 * h->K * sizeof(double2)));
     slice_cells_kernel<<<dim3(h->sl_nent[R], V / 4), kSlSplit, 2 * h->K * sizeof(double2), st>>>(x, h->d_uo_index, h->d_uo_sign,
                                                      static_cast<const int2*>(h->sl_ent[R]), h->d_type_ptr,
                                                      h->d_type_cells, h->K, R, h->n_unique, nst_of(h->K), V,
-                                                     kSlCellRows, h->sl_Xc, h->sl_xcs);
+                                                     cell_rows(R), h->sl_Xc, h->sl_xcs);
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
     return EMSURF_OK;
@@ -732,7 +749,7 @@ static_assert(2 * sl_up16(kSl * kSlMaxV) + 2 * (int)kSlAStep <= (int)kSlTmemCols
 int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
                     cudaStream_t st) {
     const int E = h->E, K = h->K;
-    const int groups = (R + kSlRhs - 1) / kSlRhs, per = (R + groups - 1) / groups;
+    const int per = rhs_per(R);
     for (int r0 = 0; r0 < R; r0 += per)
     for (int b0 = 0; b0 < h->nbins; b0 += h->sl_bins) {
         const int Rg = std::min(per, R - r0);
@@ -765,7 +782,7 @@ int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Y
         m.nst = nst_of(K);
         m.rows = 2 * K;
         m.tiles = (m.rows + kSlRows - 1) / kSlRows;
-        m.V = 2 * kSlCells;
+        m.V = 2 * cells_of(R);
         m.Np = sl_up16(kSl * m.V);
         m.xmats = r0 == 0 && b0 == 0 && h->sl_Z ? h->sl_nent[R] : 0;
         m.items = m.xmats * m.tiles;
