@@ -285,10 +285,13 @@ EMSURF_API int emsurf_check(emsurf_handle* h);
 /* Self-test of the bounded-wait paths (no counterpart in the paper): one
  * kernel waits on an mbarrier that nothing arrives on, another at a grid
  * barrier for a block that is never launched, each at most `limit` polls
- * (1..2^22); on expiry they set the handle's error flag exactly as the bin
- * multiply's and the cooperative Arnoldi step's waits do.  The next
- * emsurf_check returns ETIMEDOUT and clears the flag and the barrier
- * state.  Nothing faults or hangs.                                        */
+ * (1..2^22); the macromodels' trailing update and, on a handle with digit
+ * planes, the FP64-accuracy product run with operands that never arrive (at
+ * most min(limit, 4096) tries per wait; they write no output).  Where every
+ * one of them has given up, the handle's error flag is set exactly as the
+ * bin multiply's and the cooperative Arnoldi step's waits set it: the next
+ * emsurf_check returns ETIMEDOUT and clears the flag and the barrier state.
+ * Nothing faults or hangs.  Synchronises `stream`.                        */
 EMSURF_API int emsurf_selftest_wait(emsurf_handle* h, int64_t limit, void* stream);
 
 /* Number of CUDA kernels this handle has launched since creation.        */

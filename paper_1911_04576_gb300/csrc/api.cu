@@ -152,6 +152,17 @@ int upload(emsurf_handle* h, T** d, const T* src, size_t n) {
     return EMSURF_OK;
 }
 
+constexpr int kSelfTests = 4;
+// the handle's error flag is set if each of n self-tests has set its own
+__global__ void selftest_result_kernel(int* err, int n) {
+    bool all = true;
+    for (int i = 1; i <= n; ++i) {
+        all = all && err[i];
+        err[i] = 0;
+    }
+    if (all) atomicExch(err, 1);
+}
+
 int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* share) {
     h->device = p->device;
     h->setup_stream = reinterpret_cast<cudaStream_t>(p->stream);
@@ -172,8 +183,8 @@ int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* 
     EMS_CUDA(cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking));
     EMS_CUDA(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     EMS_CUDA(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
-    EMS_TRY(dev_alloc(h, (void**)&h->d_err, sizeof(int)));
-    EMS_CUDA(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->setup_stream));
+    EMS_TRY(dev_alloc(h, (void**)&h->d_err, (1 + kSelfTests) * sizeof(int)));
+    EMS_CUDA(cudaMemsetAsync(h->d_err, 0, (1 + kSelfTests) * sizeof(int), h->setup_stream));
     EMS_TRY(dev_alloc(h, (void**)&h->d_grid_bar, 2 * sizeof(unsigned)));
     EMS_CUDA(cudaMemsetAsync(h->d_grid_bar, 0, 2 * sizeof(unsigned), h->setup_stream));
     EMS_TRY(fft_plan_create(h->plan_x, h->px));
@@ -562,8 +573,18 @@ EMSURF_API int emsurf_selftest_wait(emsurf_handle* h, int64_t limit, void* strea
         return EMSURF_EINVAL;
     }
     DeviceGuard dg(h->device);
-    EMS_TRY(wait_selftest(h, (long long)limit, reinterpret_cast<cudaStream_t>(stream)));
-    return grid_barrier_selftest(h, (long long)limit, reinterpret_cast<cudaStream_t>(stream));
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    // the digit kernels' tries suspend a thread for up to 20 us each
+    const int tries = (int)std::min<int64_t>(limit, 1 << 12);
+    int n = 0;
+    EMS_TRY(wait_selftest(h, (long long)limit, h->d_err + ++n, st));
+    EMS_TRY(grid_barrier_selftest(h, (long long)limit, h->d_err + ++n, st));
+    EMS_TRY(slab_lu_selftest(tries, h->d_err + ++n, st));
+    if (h->sl_A) EMS_TRY(slices_selftest(h, tries, h->d_err + ++n, st));
+    selftest_result_kernel<<<1, 1, 0, st>>>(h->d_err, n);
+    EMS_CUDA(cudaGetLastError());
+    h->launches += 2;
+    return EMSURF_OK;
 }
 
 EMSURF_API int emsurf_launch_count(const emsurf_handle* h, int64_t* launches) {

@@ -311,7 +311,7 @@ struct emsurf_handle {
     int32_t* pc_own = nullptr;      // [M] owned unknowns (first in each subdomain)
     int32_t* pc_sub_ptr = nullptr;  // [M+1]
     int32_t* pc_sub_ids = nullptr;  // unique ids of each subdomain
-    int* d_err = nullptr;             // device error flag of bounded waits (0 = ok)
+    int* d_err = nullptr;             // device error flag of bounded waits (0 = ok), then those of the self-tests
     unsigned* d_grid_bar = nullptr;   // [2] count and generation of the cooperative Arnoldi step's grid barrier
     bool coop_ok = true;              // the cooperative Arnoldi step may be used (no overlapping solves)
     // GMRES workspace (FP64), allocated lazily by emsurf_solve
@@ -399,7 +399,10 @@ int slices_work(emsurf_handle* h);
 int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st);
 int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
                     cudaStream_t st);
-int grid_barrier_selftest(emsurf_handle* h, long long limit, cudaStream_t st);
+// self-tests of the bounded waits: each sets its own flag when every wait expired
+int slices_selftest(emsurf_handle* h, int tries, int* err, cudaStream_t st);
+int slab_lu_selftest(int tries, int* err, cudaStream_t st);
+int grid_barrier_selftest(emsurf_handle* h, long long limit, int* err, cudaStream_t st);
 template <typename T2>
 int apply_operator(emsurf_handle* h, Operator<T2>& op, const double2* x, double2* y, int nrhs,
                    cudaStream_t st);
@@ -407,7 +410,7 @@ int apply_operator(emsurf_handle* h, Operator<T2>& op, const double2* x, double2
 int apply_operator_f32(emsurf_handle* h, const float2* x, float2* y, int R, cudaStream_t st);
 int pc_build(emsurf_handle* h, const emsurf_problem* p);
 int stage_near_tables(emsurf_handle* h, const emsurf_problem* p);
-int wait_selftest(emsurf_handle* h, long long limit, cudaStream_t st);
+int wait_selftest(emsurf_handle* h, long long limit, int* err, cudaStream_t st);
 // tensor-core bin multiply (BF16x3) for nrhs >= kTcMinRhs
 constexpr int kTcMinRhs = 8;
 int tc_build(emsurf_handle* h, const emsurf_handle* share = nullptr);

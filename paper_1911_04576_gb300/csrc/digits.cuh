@@ -14,7 +14,7 @@ namespace emsurf {
 namespace {
 
 constexpr int kSl = 7;                       // digits
-constexpr int kSlWait = 1 << 16;             // tries of a bounded wait
+constexpr int kSlWait = 1 << 16;             // tries of a bounded wait (1.3 s)
 // |I_a I_b| <= 2^108 = 2^52 units of level 5, so re +- im sums of up to kSlExact
 // sources stay inside int64; beyond, the integers lose a bit per factor of 4
 constexpr int kSlExact = 990, kSlMaxN = 7000;   // the latter: two vectors in shared memory
@@ -29,21 +29,34 @@ __device__ __forceinline__ void sl_arrive(uint64_t* bar) {
 __device__ __forceinline__ void sl_expect(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sl_addr(bar)), "r"(bytes) : "memory");
 }
-// bounded wait; each try suspends the thread for up to 20 us (re-polling warps
-// slow every barrier of the block down)
-__device__ __forceinline__ bool sl_wait(uint64_t* bar, uint32_t parity) {
-    for (int it = 0; it < kSlWait; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(sl_addr(bar)), "r"(parity), "r"(20000u)
-            : "memory");
-        if (ok) return true;
-    }
+// one try of a wait; suspends the thread for up to 20 us (re-polling warps slow
+// every barrier of the block down)
+__device__ __forceinline__ uint32_t sl_try(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(sl_addr(bar)), "r"(parity), "r"(20000u)
+        : "memory");
+    return ok;
+}
+// bounded wait of a single thread
+__device__ __forceinline__ bool sl_wait(uint64_t* bar, uint32_t parity, int tries) {
+    for (int it = 0; it < tries; ++it)
+        if (sl_try(bar, parity)) return true;
     return false;
 }
+// Bounded wait of a whole warp: every try is voted on, so that the lanes leave
+// together with the same result also when the barrier completes around the last
+// try (warp-wide instructions follow on both ways).
+__device__ __forceinline__ bool sl_wait_warp(uint64_t* bar, uint32_t parity, int tries) {
+    for (int it = 0; it < tries; ++it)
+        if (__all_sync(0xffffffffu, sl_try(bar, parity))) return true;
+    return false;
+}
+// the block's abort flag, the same answer for a whole warp
+__device__ __forceinline__ bool sl_abort(volatile int* flag) { return __any_sync(0xffffffffu, *flag); }
 __device__ __forceinline__ void sl_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], "

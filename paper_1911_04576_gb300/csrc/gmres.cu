@@ -1050,8 +1050,8 @@ int true_residual(emsurf_handle* h, Gm* g, Apply<double2>& A, const double2* b, 
 
 }  // namespace
 
-int grid_barrier_selftest(emsurf_handle* h, long long limit, cudaStream_t st) {
-    grid_barrier_selftest_kernel<<<1, 32, 0, st>>>(h->d_grid_bar, h->d_err, limit);
+int grid_barrier_selftest(emsurf_handle* h, long long limit, int* err, cudaStream_t st) {
+    grid_barrier_selftest_kernel<<<1, 32, 0, st>>>(h->d_grid_bar, err, limit);
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
     return EMSURF_OK;

@@ -1909,8 +1909,8 @@ template int apply_operator<float2>(emsurf_handle*, Operator<float2>&, const dou
 }  // namespace emsurf
 
 namespace emsurf {
-int wait_selftest(emsurf_handle* h, long long limit, cudaStream_t st) {
-    wait_selftest_kernel<<<1, 32, 0, st>>>(limit, h->d_err);
+int wait_selftest(emsurf_handle* h, long long limit, int* err, cudaStream_t st) {
+    wait_selftest_kernel<<<1, 32, 0, st>>>(limit, err);
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
     return EMSURF_OK;

@@ -296,7 +296,7 @@ __device__ __forceinline__ double lu_double(long long x) {
 __global__ void __launch_bounds__(kLuGemmThreads, 1)
 lu_gemm_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, const unsigned char* __restrict__ A,
                const double* __restrict__ rs, int tiles_a, const unsigned char* __restrict__ D,
-               const double* __restrict__ cs, int tiles_b, int max_n, int* __restrict__ status) {
+               const double* __restrict__ cs, int tiles_b, int max_n, int* __restrict__ status, int tries, int starve) {
     const SlabType T = ty[blockIdx.z];
     if (T.nint <= c) return;
     const int kb = min(kLuNb, T.nint - c), N = T.N, rem = N - c - kb;
@@ -338,13 +338,13 @@ lu_gemm_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, 
         for (int t = 0; t < nct; ++t) {
             if (lane == 0) {
                 sl_expect(&full, kLuBTile + (t == 0 ? kLuATile : 0));
-                if (t == 0) sl_copy(sa, ga, kLuATile, &full, keep);
-                sl_copy(sb, gb + (size_t)t * kLuBTile, kLuBTile, &full, keep);
+                if (t == 0 && !starve) sl_copy(sa, ga, kLuATile, &full, keep);
+                if (!starve) sl_copy(sb, gb + (size_t)t * kLuBTile, kLuBTile, &full, keep);
             }
             __syncwarp();
             copying = true;
             // the operands are there and the last tile's sums have been read
-            if (!sl_wait(&full, fph) || (t > 0 && !sl_wait(&tfree, (uint32_t)(t - 1) & 1))) {
+            if (!sl_wait_warp(&full, fph, tries) || (t > 0 && !sl_wait_warp(&tfree, (uint32_t)(t - 1) & 1, tries))) {
                 ok = false;
                 break;
             }
@@ -365,7 +365,7 @@ lu_gemm_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, 
             }
             __syncwarp();
             multiplying = true;
-            if (!sl_wait(&done, dph)) {
+            if (!sl_wait_warp(&done, dph, tries)) {
                 ok = false;
                 break;
             }
@@ -376,8 +376,8 @@ lu_gemm_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, 
             if (lane == 0) atomicExch(status, 2);
             *abort_v = 1;
             // copies and MMAs in flight end before the CTA does
-            if (copying) sl_wait(&full, fph);
-            if (multiplying) sl_wait(&done, dph);
+            if (copying) sl_wait_warp(&full, fph, tries);
+            if (multiplying) sl_wait_warp(&done, dph, tries);
         }
     } else {
         const int qd = warp & 3, half = warp >> 2, rho = 32 * qd + lane;
@@ -388,7 +388,7 @@ lu_gemm_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, 
         const double rsc = live ? -rs[(size_t)blockIdx.z * max_n + i] * 0x1p-52 : 0.0;
         double2* row = B + T.offB + (size_t)(c + kb + (live ? i : 0)) * N + c + kb;
         for (int t = 0; t < nct; ++t) {
-            if (*abort_v || !sl_wait(&done, (uint32_t)t & 1)) {
+            if (sl_abort(abort_v) || !sl_wait_warp(&done, (uint32_t)t & 1, tries)) {
                 if (lane == 0) atomicExch(status, 2);
                 break;
             }
@@ -484,10 +484,33 @@ cudaError_t slab_lu(const SlabType* ty, int types, int max_n, int max_nint, doub
         lu_cols_kernel<<<dim3((rem + kLuN - 1) / kLuN, types), kLuN, 0, st>>>(ty, c, B, src, mv, D, cs, z.tiles_b, max_n);
         const int ta = (2 * rem + kLuM - 1) / kLuM, tc = (rem + kLuN - 1) / kLuN;
         lu_gemm_kernel<<<dim3(ta, (tc + kLuGroup - 1) / kLuGroup, types), kLuGemmThreads, kLuGemmSmem, st>>>(
-            ty, c, B, A, rs, z.tiles_a, D, cs, z.tiles_b, max_n, status);
+            ty, c, B, A, rs, z.tiles_a, D, cs, z.tiles_b, max_n, status, kSlWait, 0);
         e = cudaGetLastError();
     }
     return e;
+}
+
+// One trailing update whose operands never arrive: every wait expires (no entry is
+// touched).  Synchronises the stream.
+int slab_lu_selftest(int tries, int* err, cudaStream_t st) {
+    unsigned char* w = nullptr;
+    EMS_CUDA(cudaMalloc(&w, 256 + 4 * sizeof(double2) + 4 * sizeof(double)));
+    const SlabType ty{{0, 0}, {0, 0}, 2, 1, 0, 0};
+    double2* B = reinterpret_cast<double2*>(w + 256);
+    double* sc = reinterpret_cast<double*>(B + 4);
+    cudaError_t e = cudaFuncSetAttribute(lu_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLuGemmSmem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, 256 + 4 * sizeof(double2) + 4 * sizeof(double), st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(w, &ty, sizeof(ty), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        lu_gemm_kernel<<<dim3(1, 1, 1), kLuGemmThreads, kLuGemmSmem, st>>>(reinterpret_cast<const SlabType*>(w), 0, B, w, sc, 1,
+                                                                           w, sc + 2, 1, 2, err, tries, 1);
+        e = cudaGetLastError();
+    }
+    const cudaError_t es = cudaStreamSynchronize(st);
+    cudaFree(w);
+    EMS_CUDA(e);
+    EMS_CUDA(es);
+    return EMSURF_OK;
 }
 
 }  // namespace emsurf

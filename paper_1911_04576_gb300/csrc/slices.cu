@@ -69,10 +69,10 @@ constexpr int kSlMaxV = 24;                  // vector columns of one launch (a 
                                              // two accumulators and two A blocks fit in TMEM
 constexpr int kSlRhs = kSlMaxV / 4;          // rhs per launch
 constexpr int kSlSplit = 256;                // threads of a splitting block
-// the same for two or three barriers at once (their latencies overlap)
+// sl_wait_warp for two or three barriers at once (their latencies overlap)
 __device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, uint64_t* b2, uint32_t p2,
-                                         bool third) {
-    for (int it = 0; it < kSlWait; ++it) {
+                                         bool third, int tries) {
+    for (int it = 0; it < tries; ++it) {
         uint32_t ok;
         asm volatile(
             "{\n .reg .pred p, q, r, t;\n setp.ne.b32 t, %8, 0;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %7;\n"
@@ -83,7 +83,7 @@ __device__ __forceinline__ bool sl_wait3(uint64_t* b0, uint32_t p0, uint64_t* b1
             : "r"(sl_addr(b0)), "r"(p0), "r"(sl_addr(b1)), "r"(p1), "r"(sl_addr(b2)), "r"(p2), "r"(20000u),
               "r"((uint32_t)third)
             : "memory");
-        if (ok) return true;
+        if (__all_sync(0xffffffffu, ok)) return true;
     }
     return false;
 }
@@ -121,6 +121,8 @@ struct SlArgs {
     const int32_t *type_ptr, *type_cells;
     int K, M;
     int* err;
+    int tries;                   // of a wait
+    int starve;                  // self-test: the vectors' digits never arrive
 };
 
 // Range of items of CTA b: items whose first stage lies in its share of all stages.
@@ -195,7 +197,8 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
             uint32_t ph = 0;
             bool ok = true;
             if (!mat_side) dep_wait();           // the matrix digits do not depend on the splitting kernel
-            for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+            const int i_end = g.starve && !mat_side ? i_lo : i_hi;
+            for (int it = i_lo; it < i_end && ok && !*abort_v; ++it) {
                 const int w = it >= g.p[0].items;
                 const SlProb& p = g.p[w];
                 const int loc = w ? it - g.p[0].items : it, xm = loc / p.tiles, tile = loc - xm * p.tiles;
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                 const unsigned char* x = p.X + (size_t)xm * p.nst * p.Np * 64;
                 const int steps = mat_side ? p.nk16 : p.nst;
                 for (int s = 0; s < steps; ++s) {
-                    if (!sl_wait(&eb[st], ph ^ 1)) {
+                    if (!sl_wait(&eb[st], ph ^ 1, g.tries)) {
                         atomicExch(g.err, 20);
                         ok = false;
                         break;
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
             if (!ok) *abort_v = 1;
             // every copy has landed before the CTA can exit
             for (long long u = issued > depth ? issued - depth : 0; u < issued; ++u)
-                if (!sl_wait(&fb[u % depth], (uint32_t)((u / depth) & 1))) atomicExch(g.err, 20);
+                if (!sl_wait(&fb[u % depth], (uint32_t)((u / depth) & 1), kSlWait)) atomicExch(g.err, 20);
         }
     } else if (warp == kSlWarpM) {
         // ------------------------------------------------ MMA
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
         int xst = 0, db = 0, slot = 0;
         uint32_t dph = 0, sph = 0;
         bool any = false, ok = true;
-        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+        for (int it = i_lo; it < i_hi && ok && !sl_abort(abort_v); ++it) {
             const SlProb& p = g.p[it >= g.p[0].items];
             const uint32_t idesc = (1u << 4) | ((uint32_t)(p.Np >> 3) << 17) | ((uint32_t)(kSlRows >> 4) << 24);
             const uint32_t back = (uint32_t)p.V * 4;        // one digit's rows in descriptor units of 16 bytes
@@ -253,7 +256,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                 const uint32_t sph2 = slot2 ? sph : sph ^ 1;
                 const bool first = kc == 0;
                 if (!sl_wait3(&afull[slot], sph, &afull[two ? slot2 : slot], two ? sph2 : sph, &dempty[db],
-                              dph ^ 1, first)) {
+                              dph ^ 1, first, g.tries)) {
                     if (go) atomicExch(g.err, 21);
                     ok = false;
                     break;
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
         if (any) {
             if (sl_elect()) sl_commit(&mma_done);
             __syncwarp();
-            if (!sl_wait(&mma_done, 0) && go) atomicExch(g.err, 23);
+            if (!sl_wait_warp(&mma_done, 0, kSlWait) && go) atomicExch(g.err, 23);
         }
     } else if (warp >= kSlEpi) {
         // ------------------------------------------------ bytes to FP16 in TMEM
@@ -310,7 +313,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
         // vector slot + 1 of the last kSlMaxSlots blocks that end a vector stage (else 0)
         int ends[kSlMaxSlots] = {};
         bool ok = true;
-        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+        for (int it = i_lo; it < i_hi && ok && !sl_abort(abort_v); ++it) {
             const int w = it >= g.p[0].items;
             const SlProb& p = g.p[w];
             const int loc = w ? it - g.p[0].items : it, tile = loc % p.tiles;
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                 const bool end = (k & 1) || k == nk16 - 1;
                 const int done = slots == kSlMaxSlots ? ends[kSlMaxSlots - 1] : ends[1];
                 if ((q & 1) == set) {
-                    if (!sl_wait(&full[st], ph)) {
+                    if (!sl_wait_warp(&full[st], ph, g.tries)) {
                         if (lane == 0) atomicExch(g.err, 24);
                         ok = false;
                         break;
@@ -333,13 +336,13 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                     if (lane == 0) sl_arrive(&empty[st]);
                     // the block `slots` before this one has been multiplied: its TMEM slot
                     // is free, and its vector slot if it was the stage's last
-                    if (!sl_wait(&aempty[slot], sph ^ 1)) {
+                    if (!sl_wait_warp(&aempty[slot], sph ^ 1, g.tries)) {
                         if (lane == 0) atomicExch(g.err, 25);
                         ok = false;
                         break;
                     }
                     if (done && qd == 0 && lane == 0) sl_arrive(&xempty[done - 1]);
-                    if (!sl_wait(&xfull[xst], xph)) {
+                    if (!sl_wait_warp(&xfull[xst], xph, g.tries)) {
                         if (lane == 0) atomicExch(g.err, 26);
                         ok = false;
                         break;
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
         int db = 0;
         uint32_t dph = 0;
         bool ok = true;
-        for (int it = i_lo; it < i_hi && ok && !*abort_v; ++it) {
+        for (int it = i_lo; it < i_hi && ok && !sl_abort(abort_v); ++it) {
             const int w = it >= g.p[0].items;
             const SlProb& p = g.p[w];
             const int loc = w ? it - g.p[0].items : it, xm = loc / p.tiles, tile = loc - xm * p.tiles;
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
 #pragma unroll
             for (int v = 0; v < 4 * V4; ++v) acc[v] = 0;
             for (int s = 0; s < p.nst; s += kSlChunk) {
-                if (!sl_wait(&dfull[db], dph)) {
+                if (!sl_wait_warp(&dfull[db], dph, g.tries)) {
                     if (lane == 0) atomicExch(g.err, 27);
                     ok = false;
                     break;
@@ -744,73 +747,99 @@ int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st) {
 
 static_assert(2 * sl_up16(kSl * kSlMaxV) + 2 * (int)kSlAStep <= (int)kSlTmemCols, "TMEM columns");
 
+namespace {
+// Launch of rhs r0 .. r0 + Rg - 1 of R and the bins from b0: arguments, blocks, shared memory.
+struct SlLaunch {
+    SlArgs g;
+    int grid;
+    size_t smem;
+};
+SlLaunch sl_launch(const emsurf_handle* h, double2* Yg, double2* Ymm, int R, int r0, int Rg, int b0, const double2* coef) {
+    const int E = h->E, K = h->K;
+    SlArgs g{};
+    SlProb& b = g.p[0];
+    b.nk16 = nk16_of(E);
+    b.nst = nst_of(E);
+    b.rows = 4 * E;
+    b.tiles = (b.rows + kSlRows - 1) / kSlRows;
+    b.A = h->sl_A + slice_plane_bytes(b0, b.rows, E);
+    b.rs = h->sl_rs + (size_t)b0 * 2 * E;
+    b.X = h->sl_X;
+    b.xs = h->sl_xs;
+    b.V = sl_bin_v(Rg);
+    b.live = Rg;
+    b.Np = sl_up16(kSl * b.V);
+    b.xmats = std::min(h->sl_bins, h->nbins - b0);
+    b.items = b.xmats * b.tiles;
+    SlProb& m = g.p[1];
+    m.A = h->sl_Z;
+    m.rs = h->sl_zrs;
+    m.X = h->sl_Xc;
+    m.xs = h->sl_xcs;
+    m.nk16 = nk16_of(K);
+    m.nst = nst_of(K);
+    m.rows = 2 * K;
+    m.tiles = (m.rows + kSlRows - 1) / kSlRows;
+    m.V = 2 * cells_of(R);
+    m.Np = sl_up16(kSl * m.V);
+    m.xmats = r0 == 0 && b0 == 0 && h->sl_Z ? h->sl_nent[R] : 0;
+    m.items = m.xmats * m.tiles;
+    const int dc = std::max(b.Np, m.items ? m.Np : 0), vmax = std::max(b.V, m.items ? m.V : 0);
+    g.d_step = dc;
+    g.slots = 2 * dc + kSlMaxSlots * (int)kSlAStep <= (int)kSlTmemCols ? kSlMaxSlots : 2;
+    g.z_bytes = (kSl - 1) * vmax * 64;
+    g.x_bytes = dc * 64;
+    const size_t xring = (size_t)kSlXStages * (g.z_bytes + g.x_bytes);
+    g.stages = std::min(kSlMaxStages, (int)((kSlSmemMax - 1024 - xring) / kSlABytes));
+    g.Y = Yg + (size_t)b0 * R * 2 * E;
+    g.E = E;
+    g.R = R;
+    g.r0 = r0;
+    for (int c = 0; c < 4; ++c) g.co[c] = coef[c];
+    g.Ymm = Ymm;
+    g.ent = h->sl_Z ? static_cast<const int2*>(h->sl_ent[R]) : nullptr;
+    g.type_ptr = h->d_type_ptr;
+    g.type_cells = h->d_type_cells;
+    g.K = K;
+    g.M = h->M;
+    g.err = h->d_err;
+    g.tries = kSlWait;
+    return {g, std::min(std::max(1, h->num_sms), b.items + m.items), 1024 + (size_t)g.stages * kSlABytes + xring};
+}
+}  // namespace
+
 // Y^ = B^ X^ for every bin and Ymm = Z~ x1 for every cell, R rhs: up to kSlRhs rhs of
 // sl_bins bins per launch, the macromodels (when their planes are there) with the first.
 int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
                     cudaStream_t st) {
-    const int E = h->E, K = h->K;
-    const int per = rhs_per(R);
+    const int E = h->E, per = rhs_per(R);
     for (int r0 = 0; r0 < R; r0 += per)
-    for (int b0 = 0; b0 < h->nbins; b0 += h->sl_bins) {
-        const int Rg = std::min(per, R - r0);
-        SlArgs g{};
-        SlProb& b = g.p[0];
-        b.nk16 = nk16_of(E);
-        b.nst = nst_of(E);
-        b.rows = 4 * E;
-        b.tiles = (b.rows + kSlRows - 1) / kSlRows;
-        b.A = h->sl_A + slice_plane_bytes(b0, b.rows, E);
-        b.rs = h->sl_rs + (size_t)b0 * 2 * E;
-        b.X = h->sl_X;
-        b.xs = h->sl_xs;
-        b.V = sl_bin_v(Rg);
-        b.live = Rg;
-        b.Np = sl_up16(kSl * b.V);
-        b.xmats = std::min(h->sl_bins, h->nbins - b0);
-        b.items = b.xmats * b.tiles;
-        const size_t y0 = (size_t)b0 * R * 2 * E;
-        EMS_TRY(set_smem_once(slice_bins_kernel, 2 * E * sizeof(double2)));
-        slice_bins_kernel<<<dim3(b.xmats, b.V / 4), kSlSplit, 2 * E * sizeof(double2), st>>>(
-            Xg + y0, E, R, r0, Rg, b.nst, b.V, b.Np, h->sl_X, h->sl_xs);
-        EMS_CUDA(cudaGetLastError());
-        SlProb& m = g.p[1];
-        m.A = h->sl_Z;
-        m.rs = h->sl_zrs;
-        m.X = h->sl_Xc;
-        m.xs = h->sl_xcs;
-        m.nk16 = nk16_of(K);
-        m.nst = nst_of(K);
-        m.rows = 2 * K;
-        m.tiles = (m.rows + kSlRows - 1) / kSlRows;
-        m.V = 2 * cells_of(R);
-        m.Np = sl_up16(kSl * m.V);
-        m.xmats = r0 == 0 && b0 == 0 && h->sl_Z ? h->sl_nent[R] : 0;
-        m.items = m.xmats * m.tiles;
-        const int dc = std::max(b.Np, m.items ? m.Np : 0), vmax = std::max(b.V, m.items ? m.V : 0);
-        g.d_step = dc;
-        g.slots = 2 * dc + kSlMaxSlots * (int)kSlAStep <= (int)kSlTmemCols ? kSlMaxSlots : 2;
-        g.z_bytes = (kSl - 1) * vmax * 64;
-        g.x_bytes = dc * 64;
-        const size_t xring = (size_t)kSlXStages * (g.z_bytes + g.x_bytes);
-        g.stages = std::min(kSlMaxStages, (int)((kSlSmemMax - 1024 - xring) / kSlABytes));
-        g.Y = Yg + y0;
-        g.E = E;
-        g.R = R;
-        g.r0 = r0;
-        for (int c = 0; c < 4; ++c) g.co[c] = coef[c];
-        g.Ymm = Ymm;
-        g.ent = h->sl_Z ? static_cast<const int2*>(h->sl_ent[R]) : nullptr;
-        g.type_ptr = h->d_type_ptr;
-        g.type_cells = h->d_type_cells;
-        g.K = K;
-        g.M = h->M;
-        g.err = h->d_err;
-        const size_t smem = 1024 + (size_t)g.stages * kSlABytes + xring;
-        const int grid = std::min(std::max(1, h->num_sms), b.items + m.items);
-        EMS_TRY(set_smem_once(slices_kernel, smem));
-        EMS_CUDA(launch_after(slices_kernel, dim3(grid), kSlThreads, smem, st, g));
-        h->launches += 2;
-    }
+        for (int b0 = 0; b0 < h->nbins; b0 += h->sl_bins) {
+            const int Rg = std::min(per, R - r0);
+            const SlLaunch l = sl_launch(h, Yg, Ymm, R, r0, Rg, b0, coef);
+            const SlProb& b = l.g.p[0];
+            EMS_TRY(set_smem_once(slice_bins_kernel, 2 * E * sizeof(double2)));
+            slice_bins_kernel<<<dim3(b.xmats, b.V / 4), kSlSplit, 2 * E * sizeof(double2), st>>>(
+                Xg + (size_t)b0 * R * 2 * E, E, R, r0, Rg, b.nst, b.V, b.Np, h->sl_X, h->sl_xs);
+            EMS_CUDA(cudaGetLastError());
+            EMS_TRY(set_smem_once(slices_kernel, l.smem));
+            EMS_CUDA(launch_after(slices_kernel, dim3(l.grid), kSlThreads, l.smem, st, l.g));
+            h->launches += 2;
+        }
+    return EMSURF_OK;
+}
+
+// Products whose vector digits never arrive: every role's wait expires (no output
+// is written).
+int slices_selftest(emsurf_handle* h, int tries, int* err, cudaStream_t st) {
+    SlLaunch l = sl_launch(h, h->op64.Yg, h->op64.Ymm, 1, 0, 1, 0, h->op64.coef);
+    l.g.err = err;
+    l.g.tries = tries;
+    l.g.starve = 1;
+    EMS_TRY(set_smem_once(slices_kernel, l.smem));
+    slices_kernel<<<l.grid, kSlThreads, l.smem, st>>>(l.g);
+    EMS_CUDA(cudaGetLastError());
+    h->launches += 1;
     return EMSURF_OK;
 }
 
