@@ -450,8 +450,8 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
                                                                     make_double2(er, ei), B);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = slab_lu(dty, n_types, max_n, max_nint, B, work, dstat, st);
-        if (e == cudaSuccess) {
+        if (e == cudaSuccess) status = slab_lu(dty, n_types, max_n, max_nint, B, work, dstat, st);
+        if (e == cudaSuccess && !status) {
             slab_copy_out_kernel<<<dim3(gx, n_types), 256, 0, st>>>(dty, B, K, reinterpret_cast<double2*>(Z));
             e = cudaGetLastError();
         }
@@ -460,7 +460,7 @@ EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_
         if (e != cudaSuccess) {
             set_error("emsurf_macromodel_slab_patch: %s", cudaGetErrorString(e));
             status = EMSURF_ECUDA;
-        } else {
+        } else if (!status) {
             int hs = 0;
             cudaMemcpy(&hs, dstat, sizeof(int), cudaMemcpyDeviceToHost);
             if (hs) {

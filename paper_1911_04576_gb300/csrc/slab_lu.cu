@@ -457,9 +457,8 @@ LuSizes lu_sizes(int types, int max_n, int max_nint) {
 
 size_t slab_lu_bytes(int types, int max_n, int max_nint) { return lu_sizes(types, max_n, max_nint).total(); }
 
-// status: 1 a singular interior block, 2 an expired wait
-cudaError_t slab_lu(const SlabType* ty, int types, int max_n, int max_nint, double2* B, void* work, int* status,
-                    cudaStream_t st) {
+// *status: 1 a singular interior block, 2 an expired wait
+int slab_lu(const SlabType* ty, int types, int max_n, int max_nint, double2* B, void* work, int* status, cudaStream_t st) {
     const LuSizes z = lu_sizes(types, max_n, max_nint);
     unsigned char* w = static_cast<unsigned char*>(work);
     auto carve = [&](size_t b) {
@@ -473,10 +472,10 @@ cudaError_t slab_lu(const SlabType* ty, int types, int max_n, int max_nint, doub
     int2* mv = reinterpret_cast<int2*>(carve(z.mv));
     const size_t panel = (size_t)max_nint * kLuLd * sizeof(double2);
     const bool sm = panel <= 220 * 1024;         // the panel of the largest type fits in shared memory
-    cudaError_t e = cudaFuncSetAttribute(lu_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLuGemmSmem);
-    if (e == cudaSuccess && sm)
-        e = cudaFuncSetAttribute(lu_panel_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel);
-    for (int c = 0; c < max_nint && e == cudaSuccess; c += kLuNb) {
+    // the limits only grow: another thread may be launching larger panels
+    EMS_TRY(set_smem_once(lu_gemm_kernel, kLuGemmSmem));
+    if (sm) EMS_TRY(set_smem_once(lu_panel_kernel<true>, panel));
+    for (int c = 0; c < max_nint; c += kLuNb) {
         const int rem = max_n - c - 1;           // at most
         if (sm) lu_panel_kernel<true><<<types, kLuPanelThreads, panel, st>>>(ty, c, B, src, mv, perm, max_nint, status);
         else lu_panel_kernel<false><<<types, kLuPanelThreads, 0, st>>>(ty, c, B, src, mv, perm, max_nint, status);
@@ -485,21 +484,21 @@ cudaError_t slab_lu(const SlabType* ty, int types, int max_n, int max_nint, doub
         const int ta = (2 * rem + kLuM - 1) / kLuM, tc = (rem + kLuN - 1) / kLuN;
         lu_gemm_kernel<<<dim3(ta, (tc + kLuGroup - 1) / kLuGroup, types), kLuGemmThreads, kLuGemmSmem, st>>>(
             ty, c, B, A, rs, z.tiles_a, D, cs, z.tiles_b, max_n, status, kSlWait, 0);
-        e = cudaGetLastError();
+        EMS_CUDA(cudaGetLastError());
     }
-    return e;
+    return EMSURF_OK;
 }
 
 // One trailing update whose operands never arrive: every wait expires (no entry is
 // touched).  Synchronises the stream.
 int slab_lu_selftest(int tries, int* err, cudaStream_t st) {
+    EMS_TRY(set_smem_once(lu_gemm_kernel, kLuGemmSmem));
     unsigned char* w = nullptr;
     EMS_CUDA(cudaMalloc(&w, 256 + 4 * sizeof(double2) + 4 * sizeof(double)));
     const SlabType ty{{0, 0}, {0, 0}, 2, 1, 0, 0};
     double2* B = reinterpret_cast<double2*>(w + 256);
     double* sc = reinterpret_cast<double*>(B + 4);
-    cudaError_t e = cudaFuncSetAttribute(lu_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLuGemmSmem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, 256 + 4 * sizeof(double2) + 4 * sizeof(double), st);
+    cudaError_t e = cudaMemsetAsync(w, 0, 256 + 4 * sizeof(double2) + 4 * sizeof(double), st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(w, &ty, sizeof(ty), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         lu_gemm_kernel<<<dim3(1, 1, 1), kLuGemmThreads, kLuGemmSmem, st>>>(reinterpret_cast<const SlabType*>(w), 0, B, w, sc, 1,

@@ -16,7 +16,6 @@ struct SlabType {
 // in place: its trailing (N - nint) block becomes the Schur complement.  work:
 // slab_lu_bytes of device memory; *status: 1 singular interior block, 2 expired wait.
 size_t slab_lu_bytes(int types, int max_n, int max_nint);
-cudaError_t slab_lu(const SlabType* ty, int types, int max_n, int max_nint, double2* B, void* work, int* status,
-                    cudaStream_t st);
+int slab_lu(const SlabType* ty, int types, int max_n, int max_nint, double2* B, void* work, int* status, cudaStream_t st);
 
 }  // namespace emsurf
