@@ -240,14 +240,14 @@ struct emsurf_handle {
     int32_t* d_orb_elem = nullptr;    // [nst][orb_G] its group element
     uint32_t* d_orb_perm = nullptr;   // [orb_G][2E] signed index of T_e
     // FP64-accuracy products from exact integer digits (slices.cu): digit planes
-    // and row scales of the spectrum and the macromodels, work space of the
+    // and row exponents of the spectrum and the macromodels, work space of the
     // vectors' digits, macromodel entries (type, first column) per rhs count
     unsigned char* sl_A = nullptr;
-    double* sl_rs = nullptr;
+    int* sl_rs = nullptr;
     unsigned char* sl_Z = nullptr;
-    double* sl_zrs = nullptr;
+    int* sl_zrs = nullptr;
     unsigned char *sl_X = nullptr, *sl_Xc = nullptr;
-    double *sl_xs = nullptr, *sl_xcs = nullptr;
+    int *sl_xs = nullptr, *sl_xcs = nullptr;
     int sl_bins = 0;                  // bins whose vectors' digits are held at a time
     std::vector<void*> sl_ent;
     std::vector<int> sl_nent;

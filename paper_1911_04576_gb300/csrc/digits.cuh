@@ -91,17 +91,17 @@ __device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t (&r)[4]) {
 
 // exponent ex with |v| < 2^ex for the largest |v| of a vector, from its bit
 // pattern (the patterns of non-negative doubles order like the values, NaN above
-// infinity) and n, the sources that are summed; INT_MIN when it is not finite
+// infinity) and n, the sources that are summed; INT_MIN when it is not finite.
+// From -1073 (the smallest subnormal) to 1026.
 __device__ __forceinline__ int sl_exp(unsigned long long mbits, int n) {
     if (mbits >= 0x7ff0000000000000ull) return INT_MIN;
     const double m = __longlong_as_double((long long)mbits);
     const int spare = n <= kSlExact ? 0 : n <= 4 * kSlExact ? 1 : 2;
-    return (m > 0.0 ? max(ilogb(m) + 1, -900) : 0) + spare;
+    return (m > 0.0 ? ilogb(m) + 1 : 0) + spare;
 }
-// 2^(ex - 8) for the products (NaN where a component was not finite: it marks
-// every output)
-__device__ __forceinline__ double sl_pow(int ex) {
-    return ex == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, ex - 8);
+// 2^e for -1022 <= e <= 1023, NaN for a row or vector that is not finite
+__device__ __forceinline__ double sl_pow2(int e, bool finite = true) {
+    return __longlong_as_double(finite ? (long long)(e + 1023) << 52 : 0x7ff8000000000000ll);
 }
 // Bytes d_t + 128 of the digits of rn(v 2^(54 - ex)), least significant first:
 // balanced digits are the bytes of I + sum_t 128 256^t.  From the bit pattern:
@@ -110,9 +110,10 @@ __device__ __forceinline__ unsigned long long sl_digits(double v, int ex) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const int e = (int)(b >> 52) & 0x7ff;
     unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-    // v = +-m 2^(max(e, 1) - 1075), so the shift to the left is at most one
-    const int sh = max(e, 1) - 1021 - ex;
-    m = ex == INT_MIN || sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 1) : (m + (1ull << (-sh - 1))) >> -sh;
+    // v = +-m 2^(max(e, 1) - 1075) below 2^ex: a shift to the left (by at most one,
+    // more only for subnormal v) stays below 2^54
+    const int sh = max(e, 1) - 1021 - max(ex, -1073);
+    m = ex == INT_MIN || sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 63) : (m + (1ull << (-sh - 1))) >> -sh;
     return ((long long)b < 0 ? 0ull - m : m) + 0x80808080808080ull;
 }
 __device__ __forceinline__ unsigned long long sl_abs(double v) {

@@ -141,6 +141,14 @@ lu_panel_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B,
     }
 }
 
+// exponent of a row of L or a column of U (64 real sources) and 2^(ex - 8) (NaN
+// where an entry was not finite): contributions below 2^-1000 may lose digits
+__device__ __forceinline__ int lu_exp(unsigned long long mbits) {
+    const int ex = sl_exp(mbits, 2 * kLuNb);
+    return ex == INT_MIN ? ex : max(ex, -1000);
+}
+__device__ __forceinline__ double lu_pow(int ex) { return sl_pow2(ex == INT_MIN ? 0 : ex - 8, ex != INT_MIN); }
+
 // L of the rows below the panel, one row per thread, and their digits: real rows
 // 2 i = [Re, -Im] and 2 i + 1 = [Im, Re] of the 32 columns, 128-byte swizzled.
 __global__ void __launch_bounds__(128)
@@ -181,8 +189,8 @@ lu_rows_kernel(const SlabType* __restrict__ ty, int c, const double2* __restrict
     unsigned long long mx = 0;
 #pragma unroll
     for (int j = 0; j < kLuNb; ++j) mx = max(mx, max(sl_abs(v[j].x), sl_abs(v[j].y)));
-    const int ex = sl_exp(mx, 2 * kLuNb);
-    rs[(size_t)blockIdx.y * max_n + i] = sl_pow(ex);
+    const int ex = lu_exp(mx);
+    rs[(size_t)blockIdx.y * max_n + i] = lu_pow(ex);
     unsigned char* out = A + ((size_t)blockIdx.y * tiles + i / (kLuM / 2)) * kLuATile;
     const int r0 = 2 * (i % (kLuM / 2));
 #pragma unroll
@@ -254,8 +262,8 @@ lu_cols_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B, 
     unsigned long long mx = 0;
 #pragma unroll
     for (int j = 0; j < kLuNb; ++j) mx = max(mx, max(sl_abs(v[j].x), sl_abs(v[j].y)));
-    const int ex = sl_exp(mx, 2 * kLuNb);
-    cs[(size_t)blockIdx.y * max_n + i] = sl_pow(ex);
+    const int ex = lu_exp(mx);
+    cs[(size_t)blockIdx.y * max_n + i] = lu_pow(ex);
     unsigned char* out = D + ((size_t)blockIdx.y * tiles + blockIdx.x) * kLuBTile;
     const int r = threadIdx.x;
 #pragma unroll

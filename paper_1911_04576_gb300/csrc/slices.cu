@@ -100,9 +100,9 @@ __host__ __device__ constexpr int sl_up16(int n) { return (n + 15) & ~15; }
 
 struct SlProb {
     const unsigned char* A;      // digit planes
-    const double* rs;            // [matrix][row / 2] 2^(ex - 8) of each complex row
+    const int* rs;               // [matrix][row / 2] exponent of each complex row (sl_exp)
     const unsigned char* X;      // vector digits [x matrix][stage][Np][64 bytes]
-    const double* xs;            // [x matrix][V / 2] 2^(ex - 8) of each complex vector
+    const int* xs;               // [x matrix][V / 2] exponent of each complex vector
     int nk16, nst, rows, tiles, V, Np, items, xmats;
     int live;                    // bins: rhs of this launch
 };
@@ -437,9 +437,9 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
             if (!ok) break;
             const int mat = w ? g.ent[xm].x : xm;
             // digits: v = 2^(ex - 6) sum d_t 256^-t; level l weighs 256^-l 2^-12, so
-            // level 5 is 2^-52; the stored powers are 2^(ex - 8)
-            const double rsc = (row < p.rows ? p.rs[(size_t)mat * (p.rows / 2) + (row >> 1)] : 0.0) * 0x1p-36;
-            const double* xs = p.xs + (size_t)xm * (V / 2);
+            // level 5 is 2^-52
+            const int rex = row < p.rows ? p.rs[(size_t)mat * (p.rows / 2) + (row >> 1)] : 0;
+            const int* xs = p.xs + (size_t)xm * (V / 2);
             const bool im = rho & 1;
             int c0 = 0, nt = 0;
             if (w) {
@@ -457,8 +457,17 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                 const long long t0 = __shfl_xor_sync(0xffffffffu, im ? q[0] : q[2], 1);
                 const long long t1 = __shfl_xor_sync(0xffffffffu, im ? q[1] : q[3], 1);
                 const long long pr = im ? t0 - q[3] : q[0] - t1, pi = im ? t1 + q[2] : q[1] + t0;
-                const double sc = rsc * xs[2 * cc + (im ? 1 : 0)];
+                // the sums scaled by 2^e, in two steps where that power or a product with it
+                // (below 2^63) could leave FP64's range; a component that was not finite
+                // marks every output
+                const int xex = xs[2 * cc + (im ? 1 : 0)], e = max(max(rex, -2000) + max(xex, -2000) - 52, -2000);
+                const int e0 = e >= -1000 && e <= 900 ? e : e / 2;
+                const double sc = sl_pow2(e0, min(rex, xex) != INT_MIN);
                 double2 u = make_double2((double)pr * sc, (double)pi * sc);
+                if (e0 != e) {
+                    const double s2 = sl_pow2(e - e0);
+                    u = make_double2(u.x * s2, u.y * s2);
+                }
                 if (!w) {
                     // y_J = a L x_J + b K x_M, y_M = g K x_J + d L x_M
                     const int role = rho & 3;                  // L x_J, L x_M, K x_J, K x_M
@@ -493,7 +502,7 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
 template <bool MM>
 __global__ void __launch_bounds__(kSlRows)
 slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, size_t m0, unsigned char* __restrict__ A,
-                  double* __restrict__ rs) {
+                  int* __restrict__ rs) {
     const size_t mat = m0 + blockIdx.y;
     const int tile = blockIdx.x, rho = threadIdx.x, row = tile * kSlRows + rho;
     const int rt = min(kSlRows, rows - tile * kSlRows);
@@ -506,7 +515,7 @@ slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, si
         mx = max(mx, max(sl_abs(v.x), sl_abs(v.y)));
     }
     const int ex = sl_exp(mx, n);
-    if (c == 0) rs[(mat * rows + row) >> 1] = sl_pow(ex);
+    if (c == 0) rs[(mat * rows + row) >> 1] = ex;
     unsigned char* out = A + (mat * rows + (size_t)tile * kSlRows) * nk16 * kSlKbBytes;
     for (int kb = 0; kb < nk16; ++kb) {
         uint32_t w[kSl][4];
@@ -537,7 +546,7 @@ slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, si
 // ones).  The block of the last pair also clears the padding rows.
 template <typename Load>
 __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int v0, Load&& load,
-                                              unsigned char* __restrict__ X, double* __restrict__ xs) {
+                                              unsigned char* __restrict__ X, int* __restrict__ xs) {
     dep_trigger();
     extern __shared__ double2 s_v[];         // [2][n]
     __shared__ unsigned long long s_mx[2];
@@ -563,7 +572,7 @@ __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int
     if (threadIdx.x < 2) {
         const int ex = sl_exp(s_mx[threadIdx.x], n);
         s_ex[threadIdx.x] = ex;
-        xs[v0 + threadIdx.x] = sl_pow(ex);
+        xs[v0 + threadIdx.x] = ex;
     }
     __syncthreads();
     // 8 sources of one real vector per thread: one 16-byte chunk per digit
@@ -594,7 +603,7 @@ __device__ __forceinline__ void slice_vectors(int n, int nst, int V, int Np, int
 // bins: vectors (r, part) of X^[bin][R][2E], r0 <= r < r0 + live (zero above)
 __global__ void __launch_bounds__(kSlSplit)
 slice_bins_kernel(const double2* __restrict__ Xg, int E, int R, int r0, int live, int nst, int V, int Np,
-                  unsigned char* __restrict__ X, double* __restrict__ xs) {
+                  unsigned char* __restrict__ X, int* __restrict__ xs) {
     const size_t bin = blockIdx.x;
     const double2* src = Xg + (bin * R + r0) * 2 * E;
     slice_vectors(
@@ -607,7 +616,7 @@ __global__ void __launch_bounds__(kSlSplit)
 slice_cells_kernel(const double2* __restrict__ x, const int32_t* __restrict__ idx, const int8_t* __restrict__ sgn,
                    const int2* __restrict__ ent, const int32_t* __restrict__ type_ptr,
                    const int32_t* __restrict__ type_cells, int K, int R, int n_unique, int nst, int V, int Np,
-                   unsigned char* __restrict__ X, double* __restrict__ xs) {
+                   unsigned char* __restrict__ X, int* __restrict__ xs) {
     const int2 e = ent[blockIdx.x];
     const int c0 = type_ptr[e.x], nt = (type_ptr[e.x + 1] - c0) * R;
     slice_vectors(
@@ -653,7 +662,7 @@ size_t cell_digits(const emsurf_handle* h) {
 }
 size_t cell_scales(const emsurf_handle* h) {
     size_t n = 0;
-    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * cells_of(r) * sizeof(double));
+    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * cells_of(r) * sizeof(int));
     return n;
 }
 
@@ -668,9 +677,9 @@ size_t slice_plane_bytes(size_t mats, int rows, int n) { return mats * rows * (s
 int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     const int E = h->E, K = h->K;
     const size_t nb = (size_t)h->nbins, grids = nb * (size_t)h->max_rhs * K, cells = (size_t)h->max_rhs * h->M * K;
-    const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(double);
+    const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(int);
     const size_t zbytes = slice_plane_bytes(h->T, 2 * K, K),
-                 zrs = (size_t)h->T * K * sizeof(double) +
+                 zrs = (size_t)h->T * K * sizeof(int) +
                        cell_digits(h) + cell_scales(h) + mm_entries(h, h->max_rhs).size() * 16 * h->max_rhs;
     if ((share && !share->sl_A) || E > kSlMaxN) return EMSURF_OK;
     cudaStream_t st = h->setup_stream;
@@ -695,7 +704,7 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     }
     if (K > kSlMaxN || !fits(zbytes + zrs + work + split)) return EMSURF_OK;
     EMS_TRY(dev_alloc(h, (void**)&h->sl_Z, zbytes));
-    EMS_TRY(dev_alloc(h, (void**)&h->sl_zrs, (size_t)h->T * K * sizeof(double)));
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_zrs, (size_t)h->T * K * sizeof(int)));
     for (size_t m0 = 0; m0 < (size_t)h->T; m0 += 65535) {
         const dim3 grid((2 * K + kSlRows - 1) / kSlRows, (unsigned)std::min<size_t>(65535, h->T - m0));
         slice_rows_kernel<true><<<grid, kSlRows, 0, st>>>(h->op64.Zt, K, 2 * K, nk16_of(K), m0, h->sl_Z, h->sl_zrs);
@@ -723,12 +732,12 @@ int slices_work(emsurf_handle* h) {
     }
     // bins whose digits are held at a time: all of them up to 512 MiB, fewer under
     // a tight budget (a handle that shares its spectrum gives none back)
-    const size_t per = (size_t)nst_of(h->E) * sl_up16(kSl * V) * 64 + (V / 2) * sizeof(double);
+    const size_t per = (size_t)nst_of(h->E) * sl_up16(kSl * V) * 64 + (V / 2) * sizeof(int);
     size_t nb = std::min<size_t>(h->nbins, std::max<size_t>(1, ((size_t)512 << 20) / per));
     while (nb > 16 && h->budget > 0 && h->device_bytes + (int64_t)(nb * per) > h->budget) nb = (nb + 1) / 2;
     h->sl_bins = (int)nb;
     EMS_TRY(dev_alloc(h, (void**)&h->sl_X, nb * nst_of(h->E) * sl_up16(kSl * V) * 64));
-    EMS_TRY(dev_alloc(h, (void**)&h->sl_xs, nb * (V / 2) * sizeof(double)));
+    EMS_TRY(dev_alloc(h, (void**)&h->sl_xs, nb * (V / 2) * sizeof(int)));
     return EMSURF_OK;
 }
 
