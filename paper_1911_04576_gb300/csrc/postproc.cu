@@ -613,9 +613,12 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
         return EMSURF_EINVAL;
     }
     // directions in chunks whose column sums stay in L2 between the two kernels
-    // (at least enough directions to fill the device)
+    // (at least enough directions to fill the device), sums and phase tables below
+    // 512 MB
+    const size_t per_dir = (size_t)(N + h->nx + h->ny) * sizeof(C);
     const int chunk = (int)std::min<size_t>(
-        ndir, std::max<size_t>(4096, (48ull << 20) / ((size_t)N * sizeof(C))));
+        ndir, std::max<size_t>(1, std::min<size_t>(std::max<size_t>(4096, (48ull << 20) / ((size_t)N * sizeof(C))),
+                                                   (512ull << 20) / per_dir)));
     // one device buffer: currents, column sums, directions and the box tables
     size_t bytes = 0;
     auto part = [&](size_t n) {
