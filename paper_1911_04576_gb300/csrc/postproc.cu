@@ -116,12 +116,11 @@ __global__ void gather_cells_kernel(const double2* __restrict__ Y, const int32_t
 
 // The array factor of every column: S[d][n] = sum_m e^{jk rhat_d . c_m}
 // X1[m][n], c_m = (ix a, iy b, 0).  A block computes 32 directions x 96
-// columns, 16 cells at a time: X1 and the cells' phases are staged in shared
-// memory, the phases as products of the direction's e^{jk rx a ix} and
-// e^{jk ry b iy} (from phase_table_kernel; TAB false: one sincos per direction
-// and cell, for lattices whose tables do not fit).  A warp holds 4
-// directions, each lane 3 columns, so a phase is one broadcast read for the
-// warp.  T: arithmetic type (double for FP64 handles; float, with float
+// columns, 16 cells at a time (8 where the tables leave no room for more): X1
+// and the cells' phases are staged in shared memory, the phases as products of
+// the direction's e^{jk rx a ix} and e^{jk ry b iy} (from phase_table_kernel).
+// A warp holds 4 directions, each lane 3 columns, so a phase is one broadcast
+// read for the warp.  T: arithmetic type (double for FP64 handles; float, with float
 // accumulation over the cells, for FP32 / MIXED handles).  Bound by the FMA
 // rate.  16 x 16 cells, 576 columns, 65,160 directions (1.1 ms at the FP32 FMA
 // rate): 1.9 ms and 0.14 ms for the tables; 3.5 ms with 2 x 4 sums per thread, the tables formed by
@@ -129,7 +128,6 @@ __global__ void gather_cells_kernel(const double2* __restrict__ Y, const int32_t
 // every thread.  64 directions per block (8 per warp) left one block per SM
 // and took a quarter longer.
 constexpr int kLsM = 16, kLsThreads = 256, kLsCpt = 3, kLsDpt = 4;
-
 
 // tab[d][i] = e^{jk rx a i} for i < nx, e^{jk ry b (i - nx)} for the ny above
 template <typename T, typename C>
@@ -146,28 +144,32 @@ __global__ void phase_table_kernel(const double* __restrict__ rhat, int nd, int 
     }
 }
 
-template <typename T, typename C, bool TAB>
+// shared bytes of a block with ms cells per stage
+template <typename C>
+size_t lattice_sum_smem(int ms, int nx, int ny) {
+    return ((size_t)ms * (32 * kLsCpt + 8 * kLsDpt) + (size_t)8 * kLsDpt * (nx + ny)) * sizeof(C);
+}
+
+template <typename T, typename C, int MS>
 __global__ void __launch_bounds__(kLsThreads)
-lattice_sum_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, double a, double b,
-                   const double* __restrict__ rhat, const C* __restrict__ tab, int nd, double k, C* __restrict__ S) {
+lattice_sum_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, const C* __restrict__ tab, int nd,
+                   C* __restrict__ S) {
     constexpr int DPT = kLsDpt, ND = 8 * DPT, NC = 32 * kLsCpt;
-    constexpr int kXPer = kLsM * NC / kLsThreads;
+    constexpr int kXPer = MS * NC / kLsThreads;        // X1 entries of a thread and stage
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* xs = reinterpret_cast<C*>(smem_raw);            // [kLsM][NC]
-    C* ps = xs + kLsM * NC;                            // [kLsM][ND]
-    C* px = ps + kLsM * ND;                            // [nx][ND]
-    C* py = px + (TAB ? nx * ND : 0);                  // [ny][ND]
+    C* xs = reinterpret_cast<C*>(smem_raw);            // [MS][NC]
+    C* ps = xs + MS * NC;                              // [MS][ND]
+    C* px = ps + MS * ND;                              // [nx][ND]
+    C* py = px + nx * ND;                              // [ny][ND]
     const int d0 = blockIdx.y * ND, n0 = blockIdx.x * NC;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if constexpr (TAB) {
-        for (int e = threadIdx.x; e < ND * (nx + ny); e += blockDim.x) {
-            const int i = e / ND, dd = e - i * ND, d = d0 + dd;
-            C v;
-            v.x = (T)1;
-            v.y = (T)0;
-            if (d < nd) v = tab[(size_t)d * (nx + ny) + i];
-            px[e] = v;
-        }
+    for (int e = threadIdx.x; e < ND * (nx + ny); e += blockDim.x) {
+        const int i = e / ND, dd = e - i * ND, d = d0 + dd;
+        C v;
+        v.x = (T)1;
+        v.y = (T)0;
+        if (d < nd) v = tab[(size_t)d * (nx + ny) + i];
+        px[e] = v;
     }
     C acc[DPT][kLsCpt];
 #pragma unroll
@@ -187,27 +189,19 @@ lattice_sum_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, doubl
         }
     };
     load(0);
-    for (int m0 = 0; m0 < M; m0 += kLsM) {
+    for (int m0 = 0; m0 < M; m0 += MS) {
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kXPer; ++q) xs[threadIdx.x + q * kLsThreads] = xr[q];
-        for (int e = threadIdx.x; e < kLsM * ND; e += kLsThreads) {
+        for (int e = threadIdx.x; e < MS * ND; e += kLsThreads) {
             const int mm = e / ND, dd = e - mm * ND, m = min(m0 + mm, M - 1), iy = m / nx, ix = m - iy * nx;
+            const C u = px[ix * ND + dd], w = py[iy * ND + dd];
             C v;
-            if constexpr (TAB) {
-                const C u = px[ix * ND + dd], w = py[iy * ND + dd];
-                v.x = u.x * w.x - u.y * w.y;
-                v.y = u.x * w.y + u.y * w.x;
-            } else {
-                const int d = min(d0 + dd, nd - 1);
-                double sn, cs;
-                sincos(k * (a * rhat[3 * d] * ix + b * rhat[3 * d + 1] * iy), &sn, &cs);
-                v.x = (T)cs;
-                v.y = (T)sn;
-            }
+            v.x = u.x * w.x - u.y * w.y;
+            v.y = u.x * w.y + u.y * w.x;
             ps[e] = v;
         }
-        if (m0 + kLsM < M) load(m0 + kLsM);
+        if (m0 + MS < M) load(m0 + MS);
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < DPT; ++i)
@@ -215,7 +209,7 @@ lattice_sum_kernel(const C* __restrict__ X1, int M, int N, int nx, int ny, doubl
             for (int c = 0; c < kLsCpt; ++c) part[i][c].x = part[i][c].y = (T)0;
         // cells past M: X1 is zero there
 #pragma unroll 4
-        for (int mm = 0; mm < kLsM; ++mm) {
+        for (int mm = 0; mm < MS; ++mm) {
             C x[kLsCpt];
 #pragma unroll
             for (int c = 0; c < kLsCpt; ++c) x[c] = xs[mm * NC + lane + 32 * c];
@@ -298,21 +292,21 @@ struct BoxDev {
 // F[r][d] = -(jk/4pi) [N_perp - rhat x L_M] of the column sums S[d][r K + e]
 // (S_J in e < E, S_M in e >= E), one warp per direction; lanes share the
 // coordinate phases, the shapes' points and the (shape, slot) sums through the
-// warp's shared memory.  PH: the triangles' phases are kept there too (else
-// they are formed per member, for meshes whose phases do not fit).  All FP64,
-// and bound by its rate.  16 x 16 boxes of 288 RWGs, 65,160 directions: 2.9 ms;
+// warp's shared memory.  tri_ph: the triangles' phases are kept there too (else
+// they are formed per member).  All FP64, and bound by its rate.
+// 16 x 16 boxes of 288 RWGs, 65,160 directions: 2.9 ms;
 // with the radiation vectors of every (direction, RWG) written out first this
 // and the kernel before it took 20.6 ms.
 constexpr int kFfWarps = 4;     // directions per block (fewer where their shared memory does not fit)
 
-template <typename C, bool PH>
+template <typename C>
 __global__ void __launch_bounds__(32 * kFfWarps)
 far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ rhat, int nd, int E, int R, double k,
-                 double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
+                 bool tri_ph, double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncoord = g.nx + g.ny + g.nz;
-    const int per = ncoord + 7 * g.nshape + 3 * g.nslot + (PH ? g.ntri : 0);
+    const int per = ncoord + 7 * g.nshape + 3 * g.nslot + (tri_ph ? g.ntri : 0);
     double2* cp = reinterpret_cast<double2*>(smem_raw) + (size_t)warp * per;   // coordinate phases
     double2* eq = cp + ncoord;                                                 // point phases [shape][7]
     double2* U = eq + 7 * g.nshape;                                            // [slot][3]
@@ -334,7 +328,7 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
         auto tri_phase = [&](const BoxTri t) {
             return cmul(cmul(cp[t.ix], cp[g.nx + t.iy]), cp[g.nx + g.ny + t.iz]);
         };
-        if constexpr (PH)
+        if (tri_ph)
             for (int t = lane; t < g.ntri; t += 32) tp[t] = tri_phase(g.tri[t]);
         for (int s = lane; s < g.nslot; s += 32) {
             const int c = g.slot[s] / 3, i = g.slot[s] - 3 * c;
@@ -370,9 +364,7 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
                         sm.x = -sm.x;
                         sm.y = -sm.y;
                     }
-                    double2 ph;
-                    if constexpr (PH) ph = tp[b.tri];
-                    else ph = tri_phase(g.tri[b.tri]);
+                    const double2 ph = tri_ph ? tp[b.tri] : tri_phase(g.tri[b.tri]);
                     cfma(aj, ph, make_double2((double)sj.x, (double)sj.y));
                     cfma(am, ph, make_double2((double)sm.x, (double)sm.y));
                 }
@@ -588,17 +580,16 @@ struct Scoped {
     }
 };
 
-template <typename T, typename C, bool TAB>
-int launch_lattice_sum(emsurf_handle* h, const C* X1, int N, double a, double b, const double* dr, const C* tab, int nd,
-                       double k, C* S, size_t smem, cudaStream_t st) {
+template <typename T, typename C, int MS>
+int launch_lattice_sum(emsurf_handle* h, const C* X1, int N, const C* tab, int nd, C* S, cudaStream_t st) {
     constexpr int ND = 8 * kLsDpt, kMaxDirs = 65535 * ND;      // directions in grid rows
-    EMS_TRY(set_smem_once(lattice_sum_kernel<T, C, TAB>, smem));
+    const size_t smem = lattice_sum_smem<C>(MS, h->nx, h->ny);
+    EMS_TRY(set_smem_once(lattice_sum_kernel<T, C, MS>, smem));
     for (int d0 = 0; d0 < nd; d0 += kMaxDirs) {
         const int n = std::min(nd - d0, kMaxDirs);
         const dim3 g((unsigned)((N + 32 * kLsCpt - 1) / (32 * kLsCpt)), (unsigned)((n + ND - 1) / ND));
-        lattice_sum_kernel<T, C, TAB><<<g, kLsThreads, smem, st>>>(
-            X1, h->M, N, h->nx, h->ny, a, b, dr + 3 * (size_t)d0, TAB ? tab + (size_t)d0 * (h->nx + h->ny) : nullptr, n, k,
-            S + (size_t)d0 * N);
+        lattice_sum_kernel<T, C, MS><<<g, kLsThreads, smem, st>>>(X1, h->M, N, h->nx, h->ny,
+                                                                   tab + (size_t)d0 * (h->nx + h->ny), n, S + (size_t)d0 * N);
         EMS_CUDA(cudaGetLastError());
     }
     return EMSURF_OK;
@@ -608,7 +599,10 @@ template <typename T, typename C>
 int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, double k, const emsurf_c128* Y,
                   int nrhs, int ndir, const double* rhat, emsurf_c128* F, double* rcs, cudaStream_t st) {
     const int E = h->E, K = h->K, M = h->M, N = nrhs * K;
-    if ((32 * (size_t)(h->nx + h->ny) + 16 * 64) * sizeof(C) > 227 * 1024) {
+    // cells per stage of the lattice sum: the phase tables take what room they need
+    constexpr size_t kMaxSmem = 227 * 1024;
+    const int ms = lattice_sum_smem<C>(kLsM, h->nx, h->ny) <= kMaxSmem ? kLsM : kLsM / 2;
+    if (lattice_sum_smem<C>(ms, h->nx, h->ny) > kMaxSmem) {
         set_error("emsurf_far_field: lattice %d x %d too large for the phase tables", h->nx, h->ny);
         return EMSURF_EINVAL;
     }
@@ -627,11 +621,7 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
         return at;
     };
     const size_t o_x = part(sizeof(C) * (size_t)M * N), o_s = part(sizeof(C) * (size_t)chunk * N);
-    // phase tables, while a block's part fits in shared memory
-    const size_t lsm0 = ((size_t)kLsM * 32 * kLsCpt + (size_t)kLsM * 8 * kLsDpt) * sizeof(C);
-    const size_t lsm = lsm0 + (size_t)8 * kLsDpt * (h->nx + h->ny) * sizeof(C);
-    const bool tabs = lsm <= 227 * 1024;
-    const size_t o_p = part(tabs ? sizeof(C) * (size_t)chunk * (h->nx + h->ny) : 0);
+    const size_t o_p = part(sizeof(C) * (size_t)chunk * (h->nx + h->ny));
     const size_t o_r = part(sizeof(double) * 3 * (size_t)ndir);
     const size_t o_tab = bytes;
     const size_t o_shape = part(box.shape.size() * sizeof(BoxShape)), o_tri = part(box.tri.size() * sizeof(BoxTri));
@@ -641,6 +631,7 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     unsigned char* buf = nullptr;
     EMS_CUDA(cudaMalloc(&buf, bytes));
     sc.p.push_back(buf);
+    auto dev = [&](size_t o) { return buf + o; };
     std::vector<unsigned char> tab(bytes - o_tab);
     auto fill = [&](size_t at, const auto& v) { std::memcpy(tab.data() + at - o_tab, v.data(), v.size() * sizeof(v[0])); };
     fill(o_shape, box.shape);
@@ -649,47 +640,41 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     fill(o_slot, box.slot);
     fill(o_ptr, box.ptr);
     fill(o_mem, box.mem);
-    EMS_CUDA(cudaMemcpyAsync(buf + o_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
-    EMS_CUDA(cudaMemcpyAsync(buf + o_r, rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
-    C *X1 = reinterpret_cast<C*>(buf + o_x), *S = reinterpret_cast<C*>(buf + o_s);
-    const double* dr = reinterpret_cast<const double*>(buf + o_r);
-    const BoxDev g{reinterpret_cast<const BoxShape*>(buf + o_shape), reinterpret_cast<const BoxTri*>(buf + o_tri),
-                   reinterpret_cast<const double*>(buf + o_coord), reinterpret_cast<const int32_t*>(buf + o_slot),
-                   reinterpret_cast<const int32_t*>(buf + o_ptr), reinterpret_cast<const BoxMember*>(buf + o_mem),
+    EMS_CUDA(cudaMemcpyAsync(dev(o_tab), tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
+    EMS_CUDA(cudaMemcpyAsync(dev(o_r), rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
+    C *X1 = reinterpret_cast<C*>(dev(o_x)), *S = reinterpret_cast<C*>(dev(o_s));
+    const double* dr = reinterpret_cast<const double*>(dev(o_r));
+    const BoxDev g{reinterpret_cast<const BoxShape*>(dev(o_shape)), reinterpret_cast<const BoxTri*>(dev(o_tri)),
+                   reinterpret_cast<const double*>(dev(o_coord)), reinterpret_cast<const int32_t*>(dev(o_slot)),
+                   reinterpret_cast<const int32_t*>(dev(o_ptr)), reinterpret_cast<const BoxMember*>(dev(o_mem)),
                    (int)box.shape.size(), (int)box.tri.size(), box.nc[0], box.nc[1], box.nc[2], (int)box.slot.size()};
     gather_cells_kernel<C><<<(int)std::min<size_t>(((size_t)M * N + 255) / 256, 152 * 32), 256, 0, st>>>(
         reinterpret_cast<const double2*>(Y), h->d_uo_index, h->d_uo_sign, M, K, nrhs, h->n_unique, X1);
     EMS_CUDA(cudaGetLastError());
-    // far field: triangle phases in shared memory while one warp's fit
+    // far field: triangle phases in shared memory while those of four warps fit an SM
+    // (20,000 directions, 16 x 16 per face: 13.4 ms, formed per member 14.2; 18 x 18,
+    // where two warps would fit: 30.3 and 17.9)
     const size_t per = (box.coord.size() + 7 * box.shape.size() + 3 * box.slot.size()) * sizeof(double2);
     const size_t per_ph = per + box.tri.size() * sizeof(double2);
-    const bool ph = per_ph <= 200 * 1024;
+    const bool ph = 4 * per_ph <= 224 * 1024;
     int warps = kFfWarps;
     while (warps > 1 && (ph ? per_ph : per) * warps > 200 * 1024) warps /= 2;
     const size_t fsm = (ph ? per_ph : per) * warps;
-    if (ph) EMS_TRY(set_smem_once(far_field_kernel<C, true>, fsm));
-    else EMS_TRY(set_smem_once(far_field_kernel<C, false>, fsm));
+    EMS_TRY(set_smem_once(far_field_kernel<C>, fsm));
     double2* Fo = reinterpret_cast<double2*>(F);
     for (int d0 = 0; d0 < ndir; d0 += chunk) {
         const int nd = std::min(chunk, ndir - d0);
         const double* drc = dr + 3 * (size_t)d0;
-        if (tabs) {
-            C* tab = reinterpret_cast<C*>(buf + o_p);
-            const size_t tn = (size_t)nd * (h->nx + h->ny);
-            phase_table_kernel<T, C><<<(int)std::min<size_t>((tn + 127) / 128, 152 * 32), 128, 0, st>>>(
-                drc, nd, h->nx, h->ny, a, b, k, tab);
-            EMS_CUDA(cudaGetLastError());
-            EMS_TRY((launch_lattice_sum<T, C, true>(h, X1, N, a, b, drc, tab, nd, k, S, lsm, st)));
-        } else {
-            EMS_TRY((launch_lattice_sum<T, C, false>(h, X1, N, a, b, drc, nullptr, nd, k, S, lsm0, st)));
-        }
+        C* tab = reinterpret_cast<C*>(dev(o_p));
+        const size_t tn = (size_t)nd * (h->nx + h->ny);
+        phase_table_kernel<T, C><<<(int)std::min<size_t>((tn + 127) / 128, 152 * 32), 128, 0, st>>>(drc, nd, h->nx, h->ny, a,
+                                                                                               b, k, tab);
+        EMS_CUDA(cudaGetLastError());
+        if (ms == kLsM) EMS_TRY((launch_lattice_sum<T, C, kLsM>(h, X1, N, tab, nd, S, st)));
+        else EMS_TRY((launch_lattice_sum<T, C, kLsM / 2>(h, X1, N, tab, nd, S, st)));
         const int blocks = std::min((nd + warps - 1) / warps, h->num_sms * 32);
-        if (ph)
-            far_field_kernel<C, true><<<blocks, 32 * warps, fsm, st>>>(S, g, drc, nd, E, nrhs, k, Fo + (size_t)d0 * 3,
-                                                                           rcs ? rcs + d0 : nullptr, ndir);
-        else
-            far_field_kernel<C, false><<<blocks, 32 * warps, fsm, st>>>(S, g, drc, nd, E, nrhs, k, Fo + (size_t)d0 * 3,
-                                                                         rcs ? rcs + d0 : nullptr, ndir);
+        far_field_kernel<C><<<blocks, 32 * warps, fsm, st>>>(
+            S, g, drc, nd, E, nrhs, k, ph, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
         EMS_CUDA(cudaGetLastError());
     }
     EMS_CUDA(cudaStreamSynchronize(st));
