@@ -292,8 +292,10 @@ struct BoxDev {
 // F[r][d] = -(jk/4pi) [N_perp - rhat x L_M] of the column sums S[d][r K + e]
 // (S_J in e < E, S_M in e >= E), one warp per direction; lanes share the
 // coordinate phases, the shapes' points and the (shape, slot) sums through the
-// warp's shared memory.  tri_ph: the triangles' phases are kept there too (else
-// they are formed per member).  All FP64, and bound by its rate.
+// warp's shared memory; the last step, from the six sums to F, is done for up to 32
+// rhs at once.  tri_ph: the triangles' phases are kept there too (else
+// they are formed per member).  blockIdx.y takes rp of the R rhs: few directions
+// with many rhs would leave SMs without a warp.  All FP64, and bound by its rate.
 // 16 x 16 boxes of 288 RWGs, 65,160 directions: 2.9 ms;
 // with the radiation vectors of every (direction, RWG) written out first this
 // and the kernel before it took 20.6 ms.
@@ -301,7 +303,7 @@ constexpr int kFfWarps = 4;     // directions per block (fewer where their share
 
 template <typename C>
 __global__ void __launch_bounds__(32 * kFfWarps)
-far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ rhat, int nd, int E, int R, double k,
+far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ rhat, int nd, int E, int R, int rp, double k,
                  bool tri_ph, double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -312,7 +314,7 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
     double2* U = eq + 7 * g.nshape;                                            // [slot][3]
     double2* tp = U + 3 * g.nslot;                                             // triangle phases
     const int K = 2 * E;
-    const int nw = blockDim.x >> 5;
+    const int nw = blockDim.x >> 5, r_lo = blockIdx.y * rp, r_hi = min(R, r_lo + rp);
     const double kpi = k * 0.31830988618379067154, k4 = k / kFourPi;
     for (int d = blockIdx.x * nw + warp; d < nd; d += gridDim.x * nw) {
         const double rh[3] = {rhat[3 * d], rhat[3 * d + 1], rhat[3 * d + 2]};
@@ -347,11 +349,13 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
             for (int x = 0; x < 3; ++x) U[3 * s + x] = u[x];
         }
         __syncwarp();
-        for (int r = 0; r < R; ++r) {
+        // the sums of up to 32 rhs, one rhs per lane
+        double2 NL[6];
+        for (int r = r_lo; r < r_hi; ++r) {
             const C* sr = S + (size_t)d * R * K + (size_t)r * K;
-            double2 NL[6];
+            double2 part[6];
 #pragma unroll
-            for (int x = 0; x < 6; ++x) NL[x] = make_double2(0, 0);
+            for (int x = 0; x < 6; ++x) part[x] = make_double2(0, 0);
             for (int s = lane; s < g.nslot; s += 32) {
                 double2 aj = make_double2(0, 0), am = make_double2(0, 0);
                 for (int q = g.ptr[s]; q < g.ptr[s + 1]; ++q) {
@@ -371,17 +375,17 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
 #pragma unroll
                 for (int x = 0; x < 3; ++x) {
                     const double2 u = U[3 * s + x];
-                    cfma(NL[x], aj, u);
-                    cfma(NL[3 + x], am, u);
+                    cfma(part[x], aj, u);
+                    cfma(part[3 + x], am, u);
                 }
             }
             // reduce-scatter of the 12 sums (padded to 16) over the warp: lanes 2 v
-            // and 2 v + 1 end with value v, which is then shared out
+            // and 2 v + 1 end with value v, which the lane of this rhs takes
             double v[16];
 #pragma unroll
             for (int x = 0; x < 6; ++x) {
-                v[2 * x] = NL[x].x;
-                v[2 * x + 1] = NL[x].y;
+                v[2 * x] = part[x].x;
+                v[2 * x + 1] = part[x].y;
             }
             v[12] = v[13] = v[14] = v[15] = 0.0;
 #pragma unroll
@@ -397,9 +401,12 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
             v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 #pragma unroll
             for (int x = 0; x < 6; ++x) {
-                NL[x].x = __shfl_sync(0xffffffffu, v[0], 4 * x);
-                NL[x].y = __shfl_sync(0xffffffffu, v[0], 4 * x + 2);
+                const double re = __shfl_sync(0xffffffffu, v[0], 4 * x), im = __shfl_sync(0xffffffffu, v[0], 4 * x + 2);
+                if (lane == ((r - r_lo) & 31)) NL[x] = make_double2(re, im);
             }
+            if (((r - r_lo) & 31) != 31 && r + 1 < r_hi) continue;
+            const int rl = r - ((r - r_lo) & 31) + lane;            // this lane's rhs
+            if (rl > r) continue;
             const double2 *N = NL, *L = NL + 3;
             double2 rn = make_double2(0, 0);
 #pragma unroll
@@ -408,7 +415,7 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
                 rn.y += rh[c] * N[c].y;
             }
             double mag = 0.0;
-            double2* f = F + ((size_t)r * ndir_all + d) * 3;
+            double2* f = F + ((size_t)rl * ndir_all + d) * 3;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
@@ -417,10 +424,10 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
                                                  rh[c1] * L[c2].y - rh[c2] * L[c1].y);
                 const double2 w = make_double2(N[c].x - rn.x * rh[c] - rxl.x, N[c].y - rn.y * rh[c] - rxl.y);
                 const double2 fc = make_double2(k4 * w.y, -k4 * w.x);
-                if (lane == c) f[c] = fc;
+                f[c] = fc;
                 mag += fc.x * fc.x + fc.y * fc.y;
             }
-            if (rcs && lane == 0) rcs[(size_t)r * ndir_all + d] = kFourPi * mag;
+            if (rcs) rcs[(size_t)rl * ndir_all + d] = kFourPi * mag;
         }
     }
 }
@@ -627,11 +634,26 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     const size_t o_shape = part(box.shape.size() * sizeof(BoxShape)), o_tri = part(box.tri.size() * sizeof(BoxTri));
     const size_t o_coord = part(box.coord.size() * sizeof(double)), o_slot = part(box.slot.size() * sizeof(int32_t));
     const size_t o_ptr = part(box.ptr.size() * sizeof(int32_t)), o_mem = part(box.mem.size() * sizeof(BoxMember));
+    // one allocation, or below CUDA's 2 MB blocks (shared by small allocations, where
+    // a smaller piece is more likely to find room) currents, sums and the rest apart
     Scoped sc;
-    unsigned char* buf = nullptr;
-    EMS_CUDA(cudaMalloc(&buf, bytes));
-    sc.p.push_back(buf);
-    auto dev = [&](size_t o) { return buf + o; };
+    unsigned char *buf = nullptr, *bx = nullptr, *bs = nullptr;
+    size_t lo = 0;                       // offset at which buf starts
+    if (bytes > (2u << 20)) {
+        EMS_CUDA(cudaMalloc(&buf, bytes));
+        sc.p.push_back(buf);
+        bx = buf + o_x;
+        bs = buf + o_s;
+    } else {
+        EMS_CUDA(cudaMalloc(&bx, o_s - o_x));
+        sc.p.push_back(bx);
+        EMS_CUDA(cudaMalloc(&bs, o_p - o_s));
+        sc.p.push_back(bs);
+        EMS_CUDA(cudaMalloc(&buf, bytes - o_p));
+        sc.p.push_back(buf);
+        lo = o_p;
+    }
+    auto dev = [&](size_t o) { return buf + (o - lo); };
     std::vector<unsigned char> tab(bytes - o_tab);
     auto fill = [&](size_t at, const auto& v) { std::memcpy(tab.data() + at - o_tab, v.data(), v.size() * sizeof(v[0])); };
     fill(o_shape, box.shape);
@@ -642,7 +664,7 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     fill(o_mem, box.mem);
     EMS_CUDA(cudaMemcpyAsync(dev(o_tab), tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
     EMS_CUDA(cudaMemcpyAsync(dev(o_r), rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
-    C *X1 = reinterpret_cast<C*>(dev(o_x)), *S = reinterpret_cast<C*>(dev(o_s));
+    C *X1 = reinterpret_cast<C*>(bx), *S = reinterpret_cast<C*>(bs);
     const double* dr = reinterpret_cast<const double*>(dev(o_r));
     const BoxDev g{reinterpret_cast<const BoxShape*>(dev(o_shape)), reinterpret_cast<const BoxTri*>(dev(o_tri)),
                    reinterpret_cast<const double*>(dev(o_coord)), reinterpret_cast<const int32_t*>(dev(o_slot)),
@@ -672,9 +694,11 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
         EMS_CUDA(cudaGetLastError());
         if (ms == kLsM) EMS_TRY((launch_lattice_sum<T, C, kLsM>(h, X1, N, tab, nd, S, st)));
         else EMS_TRY((launch_lattice_sum<T, C, kLsM / 2>(h, X1, N, tab, nd, S, st)));
+        // rhs in groups while that fills the device: each forms its directions' phases again
         const int blocks = std::min((nd + warps - 1) / warps, h->num_sms * 32);
-        far_field_kernel<C><<<blocks, 32 * warps, fsm, st>>>(
-            S, g, drc, nd, E, nrhs, k, ph, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
+        const int rn = std::min(nrhs, (int)std::max<long long>((long long)nrhs * blocks / (4 * h->num_sms), (nrhs + 65534) / 65535));
+        far_field_kernel<C><<<dim3(blocks, (nrhs + rn - 1) / rn), 32 * warps, fsm, st>>>(
+            S, g, drc, nd, E, nrhs, rn, k, ph, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
         EMS_CUDA(cudaGetLastError());
     }
     EMS_CUDA(cudaStreamSynchronize(st));

@@ -1,7 +1,8 @@
 """Far fields at the limits of their launch rules, against the sum over the
-cells of one box's radiation integrals times e^{jk rhat . c_m}: a lattice whose
-phase tables leave room for 8 cells per stage only (nx + ny from 391 to 422 in
-FP64), a box whose triangle phases are formed per member, and a nearly full device.
+cells of one box's radiation integrals times e^{jk rhat . c_m}: few directions
+with more right-hand sides than a warp has lanes, a lattice whose phase tables
+leave room for 8 cells per stage only (nx + ny from 391 to 422 in FP64), a box
+whose triangle phases are formed per member, and a nearly full device.
 
 FP64 handles: 1e-11 of the largest |F| (the setup rows' tolerance).  MIXED and
 FP32 handles sum M cells in FP32: (M + 8) 2^-24 sqrt(M) of the largest |F| as in
@@ -56,9 +57,10 @@ def reference(box, nx, ny, Y, idx, sgn, rhat):
 
 
 @pytest.mark.parametrize("prec,n,nx,ny,R,nd", [
+    ("FP64", 1, 3, 2, 33, 3), ("MIXED", 2, 2, 2, 70, 1), ("MIXED", 1, 4, 3, 32, 130), ("FP64", 2, 1, 1, 31, 2),
     ("FP64", 1, 390, 1, 1, 40), ("FP64", 1, 391, 1, 2, 33), ("FP64", 1, 400, 1, 1, 1),
 ])
-def test_long_lattices(emsurf_lib, prec, n, nx, ny, R, nd):
+def test_many_rhs_and_long_lattices(emsurf_lib, prec, n, nx, ny, R, nd):
     import torch
     from paper_1911_04576_gb300 import binding as B
     h, idx, sgn, nu = handle(B, n, nx, ny, getattr(B, prec))
