@@ -30,7 +30,7 @@ namespace {
 using namespace fftc;
 
 constexpr int kF2MaxRad = 10;
-constexpr int kF2MaxW = 8;
+constexpr int kF2MaxLw = 5, kF2MaxW = 1 << kF2MaxLw;
 constexpr int kF2MaxSplit = 8;   // macromodel partials (kMmSplit of the product)
 constexpr size_t kF2MaxSmem = 220 * 1024;
 
@@ -252,17 +252,23 @@ size_t f2_layout(F2Plan& f, int px, int py, bool inverse) {
 #define EMS_F2_SIZES(X) X(5) X(8) X(15) X(16) X(24) X(32) X(40) X(48) X(64)
 
 
-// lanes per CTA: 32 bytes of them (a whole sector per bin), halved while that
-// leaves SMs without a CTA
-int f2_pick_lanes(int max_lw, long long lanes) {
+// lanes per CTA: 32 bytes of them (a whole sector per bin), doubled while the grids
+// of all stay below 8 KB (a stage of fewer lanes would leave most of a CTA's
+// threads without a butterfly), halved while that leaves more than a tenth of the
+// SMs without a CTA (16 x 16 boxes, one rhs: 144 CTAs of 4 lanes on 152 SMs, 10.2 us).
+// One box with 33 rhs (K = 576): 47.6 -> 7.9 us per transform, 11 x 1 boxes with
+// 33 (K = 324) 51.8 -> 14.9.
+template <typename T2>
+constexpr int f2_full_lw() { return sizeof(T2) == sizeof(float2) ? 2 : 1; }
+template <typename T2>
+int f2_pick_lanes(int points, long long lanes) {
     const int sms = sm_count();
-    for (int lw = max_lw; lw > 0; --lw)
+    int lw = f2_full_lw<T2>();
+    while (lw < kF2MaxLw && ((size_t)points << lw) * sizeof(T2) < 8192) ++lw;
+    for (; lw > 0; --lw)
         if (((lanes - 1) >> lw) + 1 >= (long long)sms * 9 / 10) return lw;
     return 0;
 }
-
-template <typename T2>
-constexpr int f2_full_lw() { return sizeof(T2) == sizeof(float2) ? 2 : 1; }
 
 template <typename T2>
 int f2_plan(F2Plan& f, int px, int py, int nx, int ny, long long lanes, bool inverse, size_t& smem, int& threads) {
@@ -272,7 +278,7 @@ int f2_plan(F2Plan& f, int px, int py, int nx, int ny, long long lanes, bool inv
     }
     f.nx = nx;
     f.ny = ny;
-    f.lw = f2_pick_lanes(f2_full_lw<T2>(), lanes);
+    f.lw = f2_pick_lanes<T2>(px * py, lanes);
     smem = f2_layout<T2>(f, px, py, inverse);
     // measured (forward and inverse, average): float, 16 x 16 boxes, one rhs (144
     // CTAs of 4 lanes): 512 threads 10.2 us, 384 11.6, 256 12.4; 24 x 24 boxes, 32
@@ -283,6 +289,11 @@ int f2_plan(F2Plan& f, int px, int py, int nx, int ny, long long lanes, bool inv
     const int sms = sm_count();
     if (sizeof(T2) == sizeof(float2)) threads = ctas <= sms ? 512 : 384;
     else threads = ctas <= 2 * sms ? 256 : 128;
+    // no more than the largest stage has butterflies
+    int work = 1 << f.lw;
+    for (int s = 0; s < f.x.n; ++s) work = std::max(work, px / f.x.rad[s] * ny << f.lw);
+    for (int s = 0; s < f.y.n; ++s) work = std::max(work, py / f.y.rad[s] * px << f.lw);
+    threads = std::min(threads, (std::max(work, 64) + 31) / 32 * 32);
     return EMSURF_OK;
 }
 
