@@ -392,14 +392,17 @@ __device__ __forceinline__ void split8(const float2 (&v)[8], __nv_bfloat16* __re
 // Split planes of X^: out[bin][4r+q][j], q = (Re x_J, Im x_J, Re x_M, Im x_M),
 // zero for j >= E; rows past 4R are not written (they reach no output).  Eight
 // sources per thread, 16-byte stores: HBM-bound (48 x 48 bins, K = 576, 32 rhs:
-// 680 MB, 112 us; 306 us with one 2-byte element per thread).
+// 680 MB, 112 us; 306 us with one 2-byte element per thread).  A bin's work goes to
+// `parts` blocks: a lattice of a few bins would leave most SMs without one (one box,
+// 33 rhs: product 63.7 -> 51.4 us with this and tc_mm_gather_kernel's parts).
 __global__ void __launch_bounds__(256)
 tc_split_x_kernel(const float2* __restrict__ X, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int E,
-                  int ej, int R, int rows, int nbins) {
+                  int ej, int R, int rows, int nbins, int parts) {
     const int nc = ej / 8, per = 2 * R * nc;
-    for (int bin = blockIdx.x; bin < nbins; bin += gridDim.x) {
+    for (long long u = blockIdx.x; u < (long long)nbins * parts; u += gridDim.x) {
+        const int bin = (int)(u / parts), part = (int)(u - (long long)bin * parts);
         const float2* src = X + (size_t)bin * R * 2 * E;
-        for (int e = threadIdx.x; e < per; e += blockDim.x) {
+        for (int e = part * blockDim.x + threadIdx.x; e < per; e += parts * blockDim.x) {
             const int rp = e / nc, j = 8 * (e - rp * nc);             // rp = 2 r + part
             float2 v[8];
 #pragma unroll
@@ -613,13 +616,13 @@ __global__ void __launch_bounds__(256)
 tc_mm_gather_kernel(const double2* __restrict__ x, const float2* __restrict__ xf, const int32_t* __restrict__ idx,
                     const int8_t* __restrict__ sgn, const int2* __restrict__ tiles, const int32_t* __restrict__ type_ptr,
                     const int32_t* __restrict__ type_cells, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                    int K, int kp, int R, int n_unique, int ntiles) {
+                    int K, int kp, int R, int n_unique, int ntiles, int parts) {
     const int nc = kp / 8, per = (kTcM / 2) * nc;
-    for (int u = blockIdx.x; u < 4 * ntiles; u += gridDim.x) {        // a quarter of a tile per block
-        const int tile = u >> 2;
+    for (int u = blockIdx.x; u < parts * ntiles; u += gridDim.x) {    // a part of a tile per block
+        const int tile = u / parts;
         const int2 tl = tiles[tile];
         const int c0 = type_ptr[tl.x], n_t = (type_ptr[tl.x + 1] - c0) * R;
-        for (int e = (u & 3) * (per / 4) + threadIdx.x; e < ((u & 3) + 1) * (per / 4); e += blockDim.x) {
+        for (int e = (u - tile * parts) * blockDim.x + threadIdx.x; e < per; e += parts * blockDim.x) {
             const int c = e / nc, k = 8 * (e - c * nc), col = tl.y + c;
             if (col >= n_t) continue;
             const int slot = col / R, r = col - slot * R;
@@ -1021,10 +1024,12 @@ int tc_macromodel(emsurf_handle* h, const double2* x, const float2* xf, float2* 
     }
     const int ntiles = h->tc_mm_ntiles[R];
     const int2* tiles = static_cast<const int2*>(h->tc_mm_tiles[R]);
-    tc_mm_gather_kernel<<<std::min(4 * ntiles, h->num_sms * 16), 256, 0, st>>>(
+    // parts of a tile: a quarter, smaller while that fills the device
+    const int parts = std::max(4, std::min((kTcM / 2 * (kp / 8) + 255) / 256, h->num_sms * 8 / std::max(1, ntiles)));
+    tc_mm_gather_kernel<<<(int)std::min<long long>((long long)parts * ntiles, h->num_sms * 16), 256, 0, st>>>(
         x, xf, h->d_uo_index, h->d_uo_sign, tiles, h->d_type_ptr, h->d_type_cells,
         reinterpret_cast<__nv_bfloat16*>(h->tc_Mh), reinterpret_cast<__nv_bfloat16*>(h->tc_Ml), K, kp, R,
-        h->n_unique, ntiles);
+        h->n_unique, ntiles, parts);
     EMS_CUDA(cudaGetLastError());
     MmArgs a;
     a.Y = Ymm;
@@ -1089,8 +1094,10 @@ int tc_binmul_launch(emsurf_handle* h, float2* Y, int R, const float2* coef, int
 int tc_binmul(emsurf_handle* h, const float2* X, float2* Y, int R, const float2* coef, cudaStream_t st) {
     const int E = h->E, ej = h->tc_ej, rows = h->tc_rows;
     const size_t nb = (size_t)h->nbins;
-    tc_split_x_kernel<<<(int)std::min<size_t>(nb, (size_t)h->num_sms * 8), 256, 0, st>>>(
-        X, reinterpret_cast<__nv_bfloat16*>(h->tc_Xh), reinterpret_cast<__nv_bfloat16*>(h->tc_Xl), E, ej, R, rows, (int)nb);
+    const int parts = std::max(1, std::min((2 * R * (ej / 8) + 255) / 256, h->num_sms * 8 / (int)nb));
+    tc_split_x_kernel<<<(int)std::min<size_t>(nb * parts, (size_t)h->num_sms * 8), 256, 0, st>>>(
+        X, reinterpret_cast<__nv_bfloat16*>(h->tc_Xh), reinterpret_cast<__nv_bfloat16*>(h->tc_Xl), E, ej, R, rows, (int)nb,
+        parts);
     EMS_CUDA(cudaGetLastError());
     h->launches += 1;
     return tc_binmul_launch(h, Y, R, coef, h->tc_variant, st);
