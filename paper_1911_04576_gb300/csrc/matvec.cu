@@ -210,7 +210,9 @@ __global__ void binmul_kernel(const T2* __restrict__ Bhat, const T2* __restrict_
 // one's last blocks drain (8 x 8 boxes, K = 324, one rhs: product 48.2 -> 44.6 us).
 // The orbit kernel, whose blocks leave no room for the macromodel's, is not.
 // Up to 8 rhs share one pass over the spectrum (16 FMA per element and rhs: HBM
-// bounds up to 3 rhs, the FP32 rate more).  40 x 25 bins, K = 324, 3 rhs (420 MB):
+// bounds up to 3 rhs, the FP32 rate more), with as many CTAs as fit: few sources
+// give a CTA few warps (one rhs, 24 x 24 boxes, K = 144: product 139 us with one
+// CTA per SM, 59 with all; 20 x 13 boxes, K = 324: 149 and 111).  40 x 25 bins, K = 324, 3 rhs (420 MB):
 // 118 us, 229 us in two passes of binmul_kernel, which stays for other E.
 constexpr int kBmJB = 8;
 constexpr int kBmStages = 4;
@@ -1806,7 +1808,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
                     EMS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, threads_tma, smem));
                     occ = std::max(b, 1);
                 }
-                const int grid = std::min(nb, std::max(1, h->num_sms) * (rb == 1 ? 1 : occ));
+                const int grid = std::min(nb, std::max(1, h->num_sms) * occ);
                 EMS_CUDA(launch_after(kern, dim3(grid), threads_tma, smem, st, op.Bhat, op.Xg, op.Yg, E, nb, R, r0, op.coef[0],
                                       op.coef[1], op.coef[2], op.coef[3], h->d_err));
                 h->launches += 1;
