@@ -497,27 +497,36 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
 }
 
 // ---------------------------------------------------------------- splitting
-// Planes of one row per thread: rows of bins (MM false) from B^[bin][op][j][i],
-// of macromodels from Zt[t][k'][k]; blockIdx.x = tile, blockIdx.y = matrix.
+// Planes of one row per threadIdx.x, its sources shared by the kSlRowParts values of
+// threadIdx.y: rows of bins (MM false) from B^[bin][op][j][i], of macromodels from
+// Zt[t][k'][k]; blockIdx.x = tile, blockIdx.y = matrix.  With one thread per row a
+// few matrices left the threads waiting for one load after another (create of one
+// box with K = 576: 1.24 ms, 1.00 with the parts and one upload of the entries).
+constexpr int kSlRowParts = 4;
 template <bool MM>
-__global__ void __launch_bounds__(kSlRows)
+__global__ void __launch_bounds__(kSlRows * kSlRowParts)
 slice_rows_kernel(const double2* __restrict__ src, int n, int rows, int nk16, size_t m0, unsigned char* __restrict__ A,
                   int* __restrict__ rs) {
     const size_t mat = m0 + blockIdx.y;
     const int tile = blockIdx.x, rho = threadIdx.x, row = tile * kSlRows + rho;
-    const int rt = min(kSlRows, rows - tile * kSlRows);
-    if (rho >= rt) return;
+    const int rt = min(kSlRows, rows - tile * kSlRows), part = threadIdx.y;
+    __shared__ unsigned long long s_mx[kSlRowParts][kSlRows];
     const int c = row & 1;
     const double2* s = MM ? src + (mat * n) * n + (row >> 1) : src + ((mat * 2 + ((row >> 1) & 1)) * n) * n + (row >> 2);
     unsigned long long mx = 0;
-    for (int j = 0; j < n; ++j) {
+    for (int j = part; j < n && rho < rt; j += kSlRowParts) {
         const double2 v = s[(size_t)j * n];
         mx = max(mx, max(sl_abs(v.x), sl_abs(v.y)));
     }
+    s_mx[part][rho] = mx;
+    __syncthreads();
+    if (rho >= rt) return;
+#pragma unroll
+    for (int q = 0; q < kSlRowParts; ++q) mx = max(mx, s_mx[q][rho]);
     const int ex = sl_exp(mx, n);
-    if (c == 0) rs[(mat * rows + row) >> 1] = ex;
+    if (c == 0 && part == 0) rs[(mat * rows + row) >> 1] = ex;
     unsigned char* out = A + (mat * rows + (size_t)tile * kSlRows) * nk16 * kSlKbBytes;
-    for (int kb = 0; kb < nk16; ++kb) {
+    for (int kb = part; kb < nk16; kb += kSlRowParts) {
         uint32_t w[kSl][4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -645,25 +654,28 @@ int rhs_per(int R) {
 int cells_of(int R) { return sl_bin_v(rhs_per(R)) == kSlMaxV ? kSlMaxV / 2 : 8; }
 int cell_rows(int R) { return sl_up16(kSl * 2 * cells_of(R)); }   // digit rows of an entry
 int nst_of(int n) { return (n + kSlK - 1) / kSlK; }
-std::vector<int2> mm_entries(const emsurf_handle* h, int R) {
-    std::vector<int2> e;
-    for (int t = 0; t < h->T; ++t) {
-        const int n = (h->h_type_ptr[t + 1] - h->h_type_ptr[t]) * R;
-        for (int c = 0; c < n; c += cells_of(R)) e.push_back(make_int2(t, c));
-    }
-    return e;
+// macromodel entries of R rhs
+size_t mm_entries(const emsurf_handle* h, int R) {
+    const int per = cells_of(R);
+    size_t n = 0;
+    for (int t = 0; t < h->T; ++t) n += ((h->h_type_ptr[t + 1] - h->h_type_ptr[t]) * (size_t)R + per - 1) / per;
+    return n;
 }
 
-// bytes of the macromodel columns' digits and scales, the most over 1..max_rhs
-size_t cell_digits(const emsurf_handle* h) {
-    size_t n = 0;
-    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * nst_of(h->K) * cell_rows(r) * 64);
-    return n;
-}
-size_t cell_scales(const emsurf_handle* h) {
-    size_t n = 0;
-    for (int r = 1; r <= h->max_rhs; ++r) n = std::max(n, mm_entries(h, r).size() * cells_of(r) * sizeof(int));
-    return n;
+// what the macromodel columns of 1..max_rhs rhs take: the most digits and exponents,
+// the entries of all
+struct CellSizes {
+    size_t digits = 0, exps = 0, entries = 0;
+};
+CellSizes cell_sizes(const emsurf_handle* h) {
+    CellSizes z;
+    for (int r = 1; r <= h->max_rhs; ++r) {
+        const size_t n = mm_entries(h, r);
+        z.digits = std::max(z.digits, n * nst_of(h->K) * cell_rows(r) * 64);
+        z.exps = std::max(z.exps, n * cells_of(r) * sizeof(int));
+        z.entries += n;
+    }
+    return z;
 }
 
 }  // namespace
@@ -678,9 +690,9 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     const int E = h->E, K = h->K;
     const size_t nb = (size_t)h->nbins, grids = nb * (size_t)h->max_rhs * K, cells = (size_t)h->max_rhs * h->M * K;
     const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(int);
+    const CellSizes cs = cell_sizes(h);
     const size_t zbytes = slice_plane_bytes(h->T, 2 * K, K),
-                 zrs = (size_t)h->T * K * sizeof(int) +
-                       cell_digits(h) + cell_scales(h) + mm_entries(h, h->max_rhs).size() * 16 * h->max_rhs;
+                 zrs = (size_t)h->T * K * sizeof(int) + cs.digits + cs.exps + cs.entries * sizeof(int2);
     if ((share && !share->sl_A) || E > kSlMaxN) return EMSURF_OK;
     cudaStream_t st = h->setup_stream;
     // work space still to come: grids, products, and the partials of the SIMT macromodels
@@ -697,7 +709,7 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
         EMS_TRY(dev_alloc(h, (void**)&h->sl_rs, brs));
         for (size_t m0 = 0; m0 < nb; m0 += 65535) {
             const dim3 grid((4 * E + kSlRows - 1) / kSlRows, (unsigned)std::min<size_t>(65535, nb - m0));
-            slice_rows_kernel<false><<<grid, kSlRows, 0, st>>>(h->op64.Bhat, E, 4 * E, nk16_of(E), m0, h->sl_A, h->sl_rs);
+            slice_rows_kernel<false><<<grid, dim3(kSlRows, kSlRowParts), 0, st>>>(h->op64.Bhat, E, 4 * E, nk16_of(E), m0, h->sl_A, h->sl_rs);
             EMS_CUDA(cudaGetLastError());
             h->launches += 1;
         }
@@ -707,7 +719,7 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     EMS_TRY(dev_alloc(h, (void**)&h->sl_zrs, (size_t)h->T * K * sizeof(int)));
     for (size_t m0 = 0; m0 < (size_t)h->T; m0 += 65535) {
         const dim3 grid((2 * K + kSlRows - 1) / kSlRows, (unsigned)std::min<size_t>(65535, h->T - m0));
-        slice_rows_kernel<true><<<grid, kSlRows, 0, st>>>(h->op64.Zt, K, 2 * K, nk16_of(K), m0, h->sl_Z, h->sl_zrs);
+        slice_rows_kernel<true><<<grid, dim3(kSlRows, kSlRowParts), 0, st>>>(h->op64.Zt, K, 2 * K, nk16_of(K), m0, h->sl_Z, h->sl_zrs);
         EMS_CUDA(cudaGetLastError());
         h->launches += 1;
     }
@@ -718,17 +730,23 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
 int slices_work(emsurf_handle* h) {
     const int R = h->max_rhs, V = sl_bin_v(std::min(R, kSlRhs));
     if (h->sl_Z) {
-        EMS_TRY(dev_alloc(h, (void**)&h->sl_Xc, cell_digits(h)));
-        EMS_TRY(dev_alloc(h, (void**)&h->sl_xcs, cell_scales(h)));
+        const CellSizes cs = cell_sizes(h);
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_Xc, cs.digits));
+        EMS_TRY(dev_alloc(h, (void**)&h->sl_xcs, cs.exps));
         h->sl_ent.assign(R + 1, nullptr);
         h->sl_nent.assign(R + 1, 0);
+        std::vector<int2> e;
+        e.reserve(cs.entries);
+        int2* dev = nullptr;
+        EMS_TRY(dev_alloc(h, (void**)&dev, cs.entries * sizeof(int2)));
         for (int r = 1; r <= R; ++r) {
-            const std::vector<int2> e = mm_entries(h, r);
-            EMS_TRY(dev_alloc(h, &h->sl_ent[r], e.size() * sizeof(int2)));
-            EMS_CUDA(cudaMemcpyAsync(h->sl_ent[r], e.data(), e.size() * sizeof(int2), cudaMemcpyHostToDevice, h->setup_stream));
-            EMS_CUDA(cudaStreamSynchronize(h->setup_stream));     // e goes out of scope
-            h->sl_nent[r] = (int)e.size();
+            h->sl_ent[r] = dev + e.size();
+            for (int t = 0; t < h->T; ++t)
+                for (int c = 0; c < (h->h_type_ptr[t + 1] - h->h_type_ptr[t]) * r; c += cells_of(r)) e.push_back(make_int2(t, c));
+            h->sl_nent[r] = (int)(dev + e.size() - static_cast<int2*>(h->sl_ent[r]));
         }
+        EMS_CUDA(cudaMemcpyAsync(dev, e.data(), e.size() * sizeof(int2), cudaMemcpyHostToDevice, h->setup_stream));
+        EMS_CUDA(cudaStreamSynchronize(h->setup_stream));     // e goes out of scope
     }
     // bins whose digits are held at a time: all of them up to 512 MiB, fewer under
     // a tight budget (a handle that shares its spectrum gives none back)
