@@ -261,8 +261,10 @@ EMSURF_API void emsurf_destroy(emsurf_handle* h);
 /* Tracing (no counterpart in the paper, which reports wall-clock phases
  * only): CUDA-event timers around each phase of emsurf_matvec, recorded on
  * the caller's stream while enabled.  enable != 0 clears and starts
- * recording; 0 stops.  Phases: 0 bin multiply FP32, 1 bin multiply FP64,
- * 2 macromodel multiply FP32, 3 macromodel FP64, 4 FFT passes + gather FP32,
+ * recording; 0 stops.  Phases: 0 bin multiply FP32, 1 bin multiply FP64 (on
+ * digit planes with the splitting of X^ and the macromodel multiply, which
+ * share its launches), 2 macromodel multiply FP32, 3 macromodel FP64 (on digit
+ * planes the splitting of x1 only), 4 FFT passes + gather FP32,
  * 5 the same FP64, 6 Arnoldi orthogonalisation/norm/Givens kernels of
  * emsurf_solve, 7 crop + U_o^T scatter of emsurf_matvec, 8 near-field
  * preconditioner applications of emsurf_solve.  emsurf_profile_read synchronises on the recorded events

@@ -1728,6 +1728,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
                 op.Zt, x, h->d_uo_index, h->d_uo_sign, h->d_type_cells,
                 reinterpret_cast<const MmBlock*>(h->d_mm_blocks), op.Ymm, K, h->M, h->n_unique, chunk2, xf);
             EMS_CUDA(cudaGetLastError());
+            h->launches += 1;
             nsplit = ns2;
             mm_done = true;
         }
@@ -1749,6 +1750,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
                 h->n_unique, chunk, xf);
         }
         EMS_CUDA(cudaGetLastError());
+        h->launches += 1;
     }
     prof_mark(h, ph_mm, false, mst);
     if (side) EMS_CUDA(cudaEventRecord(h->ev_join, mst));
@@ -1883,7 +1885,7 @@ int apply_operator_io(emsurf_handle* h, Operator<T2>& op, const double2* x, cons
             y, op.Y1, h->d_inv_ptr, h->d_inv_ent, h->d_inv_sgn, h->M * K, R, h->n_unique));
     EMS_CUDA(cudaGetLastError());
     prof_mark(h, EMS_PH_SCATTER, false, st);
-    h->launches += fused ? 4 : 6;   // FFTs (2 fused or 4 passes), macromodel, scatter
+    h->launches += fused ? 3 : 5;   // FFTs (2 fused or 4 passes), scatter; the products count their own
     return EMSURF_OK;
 }
 
