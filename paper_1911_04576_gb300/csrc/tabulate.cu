@@ -507,15 +507,17 @@ __global__ void mark_classes_kernel(PairClasses c, int T, int b0, int total) {
 // cap are only counted
 __global__ void number_classes_kernel(int* __restrict__ tab, size_t n, int* __restrict__ reps, int cap,
                                       int* __restrict__ count) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int m = tab[e];
-        const bool live = m != kNoMember;
-        const unsigned who = __ballot_sync(__activemask(), live);
-        if (!live) continue;
+    // whole warps: the vote and the shuffle are taken by all lanes
+    for (size_t e0 = blockIdx.x * (size_t)blockDim.x; e0 < n; e0 += (size_t)gridDim.x * blockDim.x) {
+        const size_t e = e0 + threadIdx.x;
+        const int m = e < n ? tab[e] : kNoMember;
+        const unsigned who = __ballot_sync(0xffffffffu, m != kNoMember);
+        if (!who) continue;
         const int lane = threadIdx.x & 31, first = __ffs(who) - 1;
         int base = 0;
         if (lane == first) base = atomicAdd(count, __popc(who));
-        base = __shfl_sync(who, base, first) + __popc(who & ((1u << lane) - 1));
+        base = __shfl_sync(0xffffffffu, base, first) + __popc(who & ((1u << lane) - 1));
+        if (m == kNoMember) continue;
         tab[e] = base;
         if (base < cap) reps[base] = m;
     }
