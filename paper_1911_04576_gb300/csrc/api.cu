@@ -163,7 +163,9 @@ __global__ void selftest_result_kernel(int* err, int n) {
     if (all) atomicExch(err, 1);
 }
 
-int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* share) {
+// digits: build the digit planes that there is room for (a sharer reads its share's
+// spectrum planes in any case)
+int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* share, bool digits) {
     h->device = p->device;
     h->setup_stream = reinterpret_cast<cudaStream_t>(p->stream);
     h->nx = p->nx;
@@ -250,7 +252,7 @@ int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* 
         h->have32 = true;
     }
     if (h->have64) {
-        EMS_TRY(slices_build(h, share));
+        EMS_TRY(slices_build(h, share, digits));
         EMS_TRY(operator_work<double2>(h, h->op64, h->sl_Z ? 1 : kMmSplit));
     }
     if (p->tensor_cores && h->have32 && h->E >= 64) EMS_TRY(tc_build(h, share));
@@ -274,7 +276,7 @@ int create_impl(const emsurf_problem* p, emsurf_handle* h, const emsurf_handle* 
         if (h->op64.Bhat && !share)
             dev_free(h, h->op64.Bhat, (size_t)h->nbins * 2 * (size_t)h->E * h->E * sizeof(double2));
         h->op64.Bhat = nullptr;
-        EMS_TRY(slices_work(h));
+        EMS_TRY(slices_work(h, digits));
     }
     return EMSURF_OK;
 }
@@ -330,6 +332,29 @@ int clear_wait_error(emsurf_handle* h) {
 
 }  // namespace emsurf
 
+namespace emsurf {
+namespace {
+// Builds a handle; one that does not fit with digit planes of its own and the work
+// space that goes with them is built with as little of both as it can.
+int create_handle(const emsurf_problem* p, const emsurf_handle* share, emsurf_handle** out) {
+    for (bool digits = true;; digits = false) {
+        emsurf_handle* h = new (std::nothrow) emsurf_handle();
+        if (!h) { set_error("host allocation failed"); return EMSURF_ENOMEM; }
+        const int s = create_impl(p, h, share, digits);
+        if (s == EMSURF_OK) {
+            *out = h;
+            return s;
+        }
+        const bool again = digits && s == EMSURF_ENOMEM && h->sl_A;
+        cudaStreamSynchronize(h->setup_stream);
+        gmres_release(h);
+        free_handle(h);
+        if (!again) return s;
+    }
+}
+}  // namespace
+}  // namespace emsurf
+
 using namespace emsurf;
 
 extern "C" {
@@ -342,17 +367,7 @@ EMSURF_API int emsurf_create(const emsurf_problem* problem, emsurf_handle** out)
     EMS_TRY(validate(problem));
     DeviceGuard dg(problem->device);
     if (!dg.ok()) { set_error("cannot select device %d", problem->device); return EMSURF_EINVAL; }
-    emsurf_handle* h = new (std::nothrow) emsurf_handle();
-    if (!h) { set_error("host allocation failed"); return EMSURF_ENOMEM; }
-    const int s = create_impl(problem, h, nullptr);
-    if (s != EMSURF_OK) {
-        cudaStreamSynchronize(h->setup_stream);
-        gmres_release(h);
-        free_handle(h);
-        return s;
-    }
-    *out = h;
-    return EMSURF_OK;
+    return create_handle(problem, nullptr, out);
 }
 
 EMSURF_API int emsurf_create_like(const emsurf_problem* problem, const emsurf_handle* share,
@@ -392,17 +407,7 @@ EMSURF_API int emsurf_create_like(const emsurf_problem* problem, const emsurf_ha
     }
     DeviceGuard dg(p.device);
     if (!dg.ok()) { set_error("cannot select device %d", p.device); return EMSURF_EINVAL; }
-    emsurf_handle* h = new (std::nothrow) emsurf_handle();
-    if (!h) { set_error("host allocation failed"); return EMSURF_ENOMEM; }
-    const int s = create_impl(&p, h, share);
-    if (s != EMSURF_OK) {
-        cudaStreamSynchronize(h->setup_stream);
-        gmres_release(h);
-        free_handle(h);
-        return s;
-    }
-    *out = h;
-    return EMSURF_OK;
+    return create_handle(&p, share, out);
 }
 
 EMSURF_API int emsurf_matvec(emsurf_handle* h, const emsurf_c128* x, emsurf_c128* y, int32_t nrhs,

@@ -394,8 +394,8 @@ int adopt_fp32_form(emsurf_handle* h, const emsurf_handle* share);
 int clear_wait_error(emsurf_handle* h);
 // exact-digit products (slices.cu)
 size_t slice_plane_bytes(size_t mats, int rows, int n);
-int slices_build(emsurf_handle* h, const emsurf_handle* share = nullptr);
-int slices_work(emsurf_handle* h);
+int slices_build(emsurf_handle* h, const emsurf_handle* share, bool digits);
+int slices_work(emsurf_handle* h, bool digits);
 int slices_cells(emsurf_handle* h, const double2* x, int R, cudaStream_t st);
 int slices_multiply(emsurf_handle* h, const double2* Xg, double2* Yg, double2* Ymm, int R, const double2* coef,
                     cudaStream_t st);

@@ -108,7 +108,8 @@ int64_t operator_bytes(const emsurf_request& q) {
     const int64_t E = 18LL * q.n * q.n;
     const int64_t P = (int64_t)smallest_smooth_at_least(2 * q.nx - 1) * smallest_smooth_at_least(2 * q.ny - 1);
     const int64_t b64 = 2LL * E * E * P * 16, b32 = 2LL * E * E * P * 8;
-    int64_t op = b64;                                   // FP64 spectrum or its digit planes (7/8 of it)
+    // FP64 spectrum or its digit planes (7/8 of it, more where E is not near a multiple of 16)
+    int64_t op = std::max<int64_t>(b64, (int64_t)slice_plane_bytes(P, 4 * (int)E, (int)E));
     if (q.precision != EMSURF_FP64) op += spectrum_form(q) == 1 ? b32 / 2 : b32;
     if (spectrum_form(q) == 3) op += b32;               // tensor-core planes
     return op + 50LL * E * E * 16;                      // + near tables

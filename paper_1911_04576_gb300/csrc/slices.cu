@@ -685,15 +685,15 @@ size_t slice_plane_bytes(size_t mats, int rows, int n) { return mats * rows * (s
 // Digit planes of the FP64 spectrum and of the macromodels, each left out when
 // the device-memory budget has no room for it and the work space that goes with
 // it (products then use the FP64 blocks).  The spectrum's planes of a shared
-// handle are taken over.
-int slices_build(emsurf_handle* h, const emsurf_handle* share) {
+// handle are taken over; digits false: nothing else.
+int slices_build(emsurf_handle* h, const emsurf_handle* share, bool digits) {
     const int E = h->E, K = h->K;
     const size_t nb = (size_t)h->nbins, grids = nb * (size_t)h->max_rhs * K, cells = (size_t)h->max_rhs * h->M * K;
     const size_t bbytes = slice_plane_bytes(nb, 4 * E, E), brs = nb * 2 * E * sizeof(int);
     const CellSizes cs = cell_sizes(h);
     const size_t zbytes = slice_plane_bytes(h->T, 2 * K, K),
                  zrs = (size_t)h->T * K * sizeof(int) + cs.digits + cs.exps + cs.entries * sizeof(int2);
-    if ((share && !share->sl_A) || E > kSlMaxN) return EMSURF_OK;
+    if (share ? !share->sl_A : !digits || E > kSlMaxN) return EMSURF_OK;
     cudaStream_t st = h->setup_stream;
     // work space still to come: grids, products, and the partials of the SIMT macromodels
     const size_t work = (2 * grids + cells) * sizeof(double2), split = cells * sizeof(double2);
@@ -714,7 +714,7 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
             h->launches += 1;
         }
     }
-    if (K > kSlMaxN || !fits(zbytes + zrs + work + split)) return EMSURF_OK;
+    if (!digits || K > kSlMaxN || !fits(zbytes + zrs + work + split)) return EMSURF_OK;
     EMS_TRY(dev_alloc(h, (void**)&h->sl_Z, zbytes));
     EMS_TRY(dev_alloc(h, (void**)&h->sl_zrs, (size_t)h->T * K * sizeof(int)));
     for (size_t m0 = 0; m0 < (size_t)h->T; m0 += 65535) {
@@ -726,8 +726,9 @@ int slices_build(emsurf_handle* h, const emsurf_handle* share) {
     return EMSURF_OK;
 }
 
-// Vector digits' work space (after the FP64 spectrum is given back).
-int slices_work(emsurf_handle* h) {
+// Vector digits' work space (after the FP64 spectrum is given back); digits as for
+// slices_build.
+int slices_work(emsurf_handle* h, bool digits) {
     const int R = h->max_rhs, V = sl_bin_v(std::min(R, kSlRhs));
     if (h->sl_Z) {
         const CellSizes cs = cell_sizes(h);
@@ -749,10 +750,11 @@ int slices_work(emsurf_handle* h) {
         EMS_CUDA(cudaStreamSynchronize(h->setup_stream));     // e goes out of scope
     }
     // bins whose digits are held at a time: all of them up to 512 MiB, fewer under
-    // a tight budget (a handle that shares its spectrum gives none back)
+    // a tight budget (a handle that shares its spectrum gives none back), one at
+    // worst where the handle is built without planes of its own
     const size_t per = (size_t)nst_of(h->E) * sl_up16(kSl * V) * 64 + (V / 2) * sizeof(int);
     size_t nb = std::min<size_t>(h->nbins, std::max<size_t>(1, ((size_t)512 << 20) / per));
-    while (nb > 16 && h->budget > 0 && h->device_bytes + (int64_t)(nb * per) > h->budget) nb = (nb + 1) / 2;
+    while (nb > (digits ? 16u : 1u) && h->budget > 0 && h->device_bytes + (int64_t)(nb * per) > h->budget) nb = (nb + 1) / 2;
     h->sl_bins = (int)nb;
     EMS_TRY(dev_alloc(h, (void**)&h->sl_X, nb * nst_of(h->E) * sl_up16(kSl * V) * 64));
     EMS_TRY(dev_alloc(h, (void**)&h->sl_xs, nb * (V / 2) * sizeof(int)));
