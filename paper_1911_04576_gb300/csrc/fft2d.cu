@@ -289,7 +289,9 @@ int f2_plan(F2Plan& f, int px, int py, int nx, int ny, long long lanes, bool inv
     const int sms = sm_count();
     if (sizeof(T2) == sizeof(float2)) threads = ctas <= sms ? 512 : 384;
     else threads = ctas <= 2 * sms ? 256 : 128;
-    // no more than the largest stage has butterflies
+    // no more than the largest stage has butterflies (idle threads cost nothing in a
+    // launch of one wave: there the same count as for larger grids)
+    if (ctas <= sms) return EMSURF_OK;
     int work = 1 << f.lw;
     for (int s = 0; s < f.x.n; ++s) work = std::max(work, px / f.x.rad[s] * ny << f.lw);
     for (int s = 0; s < f.y.n; ++s) work = std::max(work, py / f.y.rad[s] * px << f.lw);
