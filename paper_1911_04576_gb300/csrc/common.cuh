@@ -314,6 +314,9 @@ struct emsurf_handle {
     int* d_err = nullptr;             // device error flag of bounded waits (0 = ok), then those of the self-tests
     unsigned* d_grid_bar = nullptr;   // [2] count and generation of the cooperative Arnoldi step's grid barrier
     bool coop_ok = true;              // the cooperative Arnoldi step may be used (no overlapping solves)
+    // small far fields' work space, allocated by emsurf_far_field
+    void* ff_buf = nullptr;
+    size_t ff_bytes = 0;
     // GMRES workspace (FP64), allocated lazily by emsurf_solve
     void* gm = nullptr;
     // tracing: kernel launches issued by this handle, optional phase timers

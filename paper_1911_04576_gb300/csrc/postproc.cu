@@ -293,7 +293,8 @@ struct BoxDev {
 // (S_J in e < E, S_M in e >= E), one warp per direction; lanes share the
 // coordinate phases, the shapes' points and the (shape, slot) sums through the
 // warp's shared memory; the last step, from the six sums to F, is done for up to 32
-// rhs at once.  tri_ph: the triangles' phases are kept there too (else
+// rhs at once.  by_rhs: 32 rhs at a time, one per lane, each lane all members (boxes
+// with few of them leave lanes idle otherwise).  tri_ph: the triangles' phases are kept there too (else
 // they are formed per member).  blockIdx.y takes rp of the R rhs: few directions
 // with many rhs would leave SMs without a warp.  All FP64, and bound by its rate.
 // 16 x 16 boxes of 288 RWGs, 65,160 directions: 2.9 ms;
@@ -304,7 +305,7 @@ constexpr int kFfWarps = 4;     // directions per block (fewer where their share
 template <typename C>
 __global__ void __launch_bounds__(32 * kFfWarps)
 far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ rhat, int nd, int E, int R, int rp, double k,
-                 bool tri_ph, double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
+                 bool tri_ph, bool by_rhs, double2* __restrict__ F, double* __restrict__ rcs, int ndir_all) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncoord = g.nx + g.ny + g.nz;
@@ -349,14 +350,35 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
             for (int x = 0; x < 3; ++x) U[3 * s + x] = u[x];
         }
         __syncwarp();
-        // the sums of up to 32 rhs, one rhs per lane
-        double2 NL[6];
-        for (int r = r_lo; r < r_hi; ++r) {
-            const C* sr = S + (size_t)d * R * K + (size_t)r * K;
-            double2 part[6];
+        // F and RCS of one rhs from its sums N, L (NL)
+        auto finish = [&](const double2 (&NL)[6], int rl) {
+            const double2 *N = NL, *L = NL + 3;
+            double2 rn = make_double2(0, 0);
 #pragma unroll
-            for (int x = 0; x < 6; ++x) part[x] = make_double2(0, 0);
-            for (int s = lane; s < g.nslot; s += 32) {
+            for (int c = 0; c < 3; ++c) {
+                rn.x += rh[c] * N[c].x;
+                rn.y += rh[c] * N[c].y;
+            }
+            double mag = 0.0;
+            double2* f = F + ((size_t)rl * ndir_all + d) * 3;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+                // N_perp - rhat x L, times -(jk / 4pi)
+                const double2 rxl = make_double2(rh[c1] * L[c2].x - rh[c2] * L[c1].x,
+                                                 rh[c1] * L[c2].y - rh[c2] * L[c1].y);
+                const double2 w = make_double2(N[c].x - rn.x * rh[c] - rxl.x, N[c].y - rn.y * rh[c] - rxl.y);
+                const double2 fc = make_double2(k4 * w.y, -k4 * w.x);
+                f[c] = fc;
+                mag += fc.x * fc.x + fc.y * fc.y;
+            }
+            if (rcs) rcs[(size_t)rl * ndir_all + d] = kFourPi * mag;
+        };
+        // sums of a rhs from its column sums sr over slots s0, s0 + step, ..
+        auto slots = [&](const C* sr, int s0, int step, double2 (&NL)[6]) {
+#pragma unroll
+            for (int x = 0; x < 6; ++x) NL[x] = make_double2(0, 0);
+            for (int s = s0; s < g.nslot; s += step) {
                 double2 aj = make_double2(0, 0), am = make_double2(0, 0);
                 for (int q = g.ptr[s]; q < g.ptr[s + 1]; ++q) {
                     const BoxMember b = g.mem[q];
@@ -375,10 +397,22 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
 #pragma unroll
                 for (int x = 0; x < 3; ++x) {
                     const double2 u = U[3 * s + x];
-                    cfma(part[x], aj, u);
-                    cfma(part[3 + x], am, u);
+                    cfma(NL[x], aj, u);
+                    cfma(NL[3 + x], am, u);
                 }
             }
+        };
+        const C* sd = S + (size_t)d * R * K;
+        double2 NL[6];
+        int r_at = r_lo;
+        for (; by_rhs && r_hi - r_at >= 32; r_at += 32) {
+            slots(sd + (size_t)(r_at + lane) * K, 0, 1, NL);
+            finish(NL, r_at + lane);
+        }
+        // the sums of up to 32 rhs, one rhs per lane
+        for (int r = r_at; r < r_hi; ++r) {
+            double2 part[6];
+            slots(sd + (size_t)r * K, lane, 32, part);
             // reduce-scatter of the 12 sums (padded to 16) over the warp: lanes 2 v
             // and 2 v + 1 end with value v, which the lane of this rhs takes
             double v[16];
@@ -402,32 +436,12 @@ far_field_kernel(const C* __restrict__ S, BoxDev g, const double* __restrict__ r
 #pragma unroll
             for (int x = 0; x < 6; ++x) {
                 const double re = __shfl_sync(0xffffffffu, v[0], 4 * x), im = __shfl_sync(0xffffffffu, v[0], 4 * x + 2);
-                if (lane == ((r - r_lo) & 31)) NL[x] = make_double2(re, im);
+                if (lane == ((r - r_at) & 31)) NL[x] = make_double2(re, im);
             }
-            if (((r - r_lo) & 31) != 31 && r + 1 < r_hi) continue;
-            const int rl = r - ((r - r_lo) & 31) + lane;            // this lane's rhs
+            if (((r - r_at) & 31) != 31 && r + 1 < r_hi) continue;
+            const int rl = r - ((r - r_at) & 31) + lane;            // this lane's rhs
             if (rl > r) continue;
-            const double2 *N = NL, *L = NL + 3;
-            double2 rn = make_double2(0, 0);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                rn.x += rh[c] * N[c].x;
-                rn.y += rh[c] * N[c].y;
-            }
-            double mag = 0.0;
-            double2* f = F + ((size_t)rl * ndir_all + d) * 3;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-                // N_perp - rhat x L, times -(jk / 4pi)
-                const double2 rxl = make_double2(rh[c1] * L[c2].x - rh[c2] * L[c1].x,
-                                                 rh[c1] * L[c2].y - rh[c2] * L[c1].y);
-                const double2 w = make_double2(N[c].x - rn.x * rh[c] - rxl.x, N[c].y - rn.y * rh[c] - rxl.y);
-                const double2 fc = make_double2(k4 * w.y, -k4 * w.x);
-                f[c] = fc;
-                mag += fc.x * fc.x + fc.y * fc.y;
-            }
-            if (rcs) rcs[(size_t)rl * ndir_all + d] = kFourPi * mag;
+            finish(NL, rl);
         }
     }
 }
@@ -582,10 +596,14 @@ int to_device(T** d, const T* h, size_t n, cudaStream_t st) {
 
 struct Scoped {
     std::vector<void*> p;
+    cudaStream_t st = nullptr;
+    bool wait = false;
     ~Scoped() {
+        if (wait) cudaStreamSynchronize(st);
         for (void* x : p) cudaFree(x);
     }
 };
+constexpr size_t kFfKeep = 8 << 20;
 
 template <typename T, typename C, int MS>
 int launch_lattice_sum(emsurf_handle* h, const C* X1, int N, const C* tab, int nd, C* S, cudaStream_t st) {
@@ -634,26 +652,26 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     const size_t o_shape = part(box.shape.size() * sizeof(BoxShape)), o_tri = part(box.tri.size() * sizeof(BoxTri));
     const size_t o_coord = part(box.coord.size() * sizeof(double)), o_slot = part(box.slot.size() * sizeof(int32_t));
     const size_t o_ptr = part(box.ptr.size() * sizeof(int32_t)), o_mem = part(box.mem.size() * sizeof(BoxMember));
-    // one allocation, or below CUDA's 2 MB blocks (shared by small allocations, where
-    // a smaller piece is more likely to find room) currents, sums and the rest apart
+    // up to kFfKeep bytes stay with the handle (an allocation that CUDA has to map
+    // costs as much as a small far field), more are allocated for the call
     Scoped sc;
-    unsigned char *buf = nullptr, *bx = nullptr, *bs = nullptr;
-    size_t lo = 0;                       // offset at which buf starts
-    if (bytes > (2u << 20)) {
+    unsigned char* buf = nullptr;
+    if (bytes <= kFfKeep && h->ff_bytes < bytes) {
+        dev_free(h, h->ff_buf, h->ff_bytes);
+        h->ff_buf = nullptr;
+        h->ff_bytes = 0;
+        size_t keep = 256 << 10;
+        while (keep < bytes) keep *= 2;
+        if (dev_alloc(h, &h->ff_buf, keep) == EMSURF_OK) h->ff_bytes = keep;
+    }
+    if (bytes <= h->ff_bytes) {
+        buf = static_cast<unsigned char*>(h->ff_buf);
+        sc.st = st;                      // nothing of this call is in flight after it
+        sc.wait = true;
+    } else {
         EMS_CUDA(cudaMalloc(&buf, bytes));
         sc.p.push_back(buf);
-        bx = buf + o_x;
-        bs = buf + o_s;
-    } else {
-        EMS_CUDA(cudaMalloc(&bx, o_s - o_x));
-        sc.p.push_back(bx);
-        EMS_CUDA(cudaMalloc(&bs, o_p - o_s));
-        sc.p.push_back(bs);
-        EMS_CUDA(cudaMalloc(&buf, bytes - o_p));
-        sc.p.push_back(buf);
-        lo = o_p;
     }
-    auto dev = [&](size_t o) { return buf + (o - lo); };
     std::vector<unsigned char> tab(bytes - o_tab);
     auto fill = [&](size_t at, const auto& v) { std::memcpy(tab.data() + at - o_tab, v.data(), v.size() * sizeof(v[0])); };
     fill(o_shape, box.shape);
@@ -662,13 +680,13 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     fill(o_slot, box.slot);
     fill(o_ptr, box.ptr);
     fill(o_mem, box.mem);
-    EMS_CUDA(cudaMemcpyAsync(dev(o_tab), tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
-    EMS_CUDA(cudaMemcpyAsync(dev(o_r), rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
-    C *X1 = reinterpret_cast<C*>(bx), *S = reinterpret_cast<C*>(bs);
-    const double* dr = reinterpret_cast<const double*>(dev(o_r));
-    const BoxDev g{reinterpret_cast<const BoxShape*>(dev(o_shape)), reinterpret_cast<const BoxTri*>(dev(o_tri)),
-                   reinterpret_cast<const double*>(dev(o_coord)), reinterpret_cast<const int32_t*>(dev(o_slot)),
-                   reinterpret_cast<const int32_t*>(dev(o_ptr)), reinterpret_cast<const BoxMember*>(dev(o_mem)),
+    EMS_CUDA(cudaMemcpyAsync(buf + o_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
+    EMS_CUDA(cudaMemcpyAsync(buf + o_r, rhat, sizeof(double) * 3 * (size_t)ndir, cudaMemcpyHostToDevice, st));
+    C *X1 = reinterpret_cast<C*>(buf + o_x), *S = reinterpret_cast<C*>(buf + o_s);
+    const double* dr = reinterpret_cast<const double*>(buf + o_r);
+    const BoxDev g{reinterpret_cast<const BoxShape*>(buf + o_shape), reinterpret_cast<const BoxTri*>(buf + o_tri),
+                   reinterpret_cast<const double*>(buf + o_coord), reinterpret_cast<const int32_t*>(buf + o_slot),
+                   reinterpret_cast<const int32_t*>(buf + o_ptr), reinterpret_cast<const BoxMember*>(buf + o_mem),
                    (int)box.shape.size(), (int)box.tri.size(), box.nc[0], box.nc[1], box.nc[2], (int)box.slot.size()};
     gather_cells_kernel<C><<<(int)std::min<size_t>(((size_t)M * N + 255) / 256, 152 * 32), 256, 0, st>>>(
         reinterpret_cast<const double2*>(Y), h->d_uo_index, h->d_uo_sign, M, K, nrhs, h->n_unique, X1);
@@ -683,11 +701,16 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
     while (warps > 1 && (ph ? per_ph : per) * warps > 200 * 1024) warps /= 2;
     const size_t fsm = (ph ? per_ph : per) * warps;
     EMS_TRY(set_smem_once(far_field_kernel<C>, fsm));
+    // 32 rhs at a time by lanes: FP64 operations of a warp for them against 32 times
+    // those of a rhs by slots
+    long long by_lane = 8 * (long long)box.mem.size() + 24 * (long long)box.slot.size() + 42, by_slot = 17;
+    for (size_t s = 0; s < box.slot.size(); s += 32) by_slot += 8 * (box.ptr[s + 1] - box.ptr[s]) + 24;
+    const bool by_rhs = by_lane < 32 * by_slot;
     double2* Fo = reinterpret_cast<double2*>(F);
     for (int d0 = 0; d0 < ndir; d0 += chunk) {
         const int nd = std::min(chunk, ndir - d0);
         const double* drc = dr + 3 * (size_t)d0;
-        C* tab = reinterpret_cast<C*>(dev(o_p));
+        C* tab = reinterpret_cast<C*>(buf + o_p);
         const size_t tn = (size_t)nd * (h->nx + h->ny);
         phase_table_kernel<T, C><<<(int)std::min<size_t>((tn + 127) / 128, 152 * 32), 128, 0, st>>>(drc, nd, h->nx, h->ny, a,
                                                                                                b, k, tab);
@@ -696,11 +719,13 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
         else EMS_TRY((launch_lattice_sum<T, C, kLsM / 2>(h, X1, N, tab, nd, S, st)));
         // rhs in groups while that fills the device: each forms its directions' phases again
         const int blocks = std::min((nd + warps - 1) / warps, h->num_sms * 32);
-        const int rn = std::min(nrhs, (int)std::max<long long>((long long)nrhs * blocks / (4 * h->num_sms), (nrhs + 65534) / 65535));
+        int rn = std::min(nrhs, (int)std::max<long long>((long long)nrhs * blocks / (2 * h->num_sms), (nrhs + 65534) / 65535));
+        if (by_rhs && rn < 32 && (long long)blocks * (nrhs / 32) >= h->num_sms) rn = 32;
         far_field_kernel<C><<<dim3(blocks, (nrhs + rn - 1) / rn), 32 * warps, fsm, st>>>(
-            S, g, drc, nd, E, nrhs, rn, k, ph, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
+            S, g, drc, nd, E, nrhs, rn, k, ph, by_rhs, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
         EMS_CUDA(cudaGetLastError());
     }
+    sc.wait = false;
     EMS_CUDA(cudaStreamSynchronize(st));
     return EMSURF_OK;
 }

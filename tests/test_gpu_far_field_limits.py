@@ -1,6 +1,7 @@
 """Far fields at the limits of their launch rules, against the sum over the
 cells of one box's radiation integrals times e^{jk rhat . c_m}: few directions
-with more right-hand sides than a warp has lanes, a lattice whose phase tables
+with more right-hand sides than a warp has lanes, many of both (32 rhs at a time,
+one per lane), a lattice whose phase tables
 leave room for 8 cells per stage only (nx + ny from 391 to 422 in FP64), a box
 whose triangle phases are formed per member, and a nearly full device.
 
@@ -58,6 +59,7 @@ def reference(box, nx, ny, Y, idx, sgn, rhat):
 
 @pytest.mark.parametrize("prec,n,nx,ny,R,nd", [
     ("FP64", 1, 3, 2, 33, 3), ("MIXED", 2, 2, 2, 70, 1), ("MIXED", 1, 4, 3, 32, 130), ("FP64", 2, 1, 1, 31, 2),
+    ("MIXED", 1, 2, 2, 70, 1300), ("FP64", 2, 2, 1, 33, 2600), ("MIXED", 3, 1, 1, 64, 1300),
     ("FP64", 1, 390, 1, 1, 40), ("FP64", 1, 391, 1, 2, 33), ("FP64", 1, 400, 1, 1, 1),
 ])
 def test_many_rhs_and_long_lattices(emsurf_lib, prec, n, nx, ny, R, nd):
