@@ -76,9 +76,11 @@ typedef struct emsurf_handle emsurf_handle;
  *               number) for the FP64-accuracy kernels, when
  *               device_mem_budget leaves room.  The digits hold 55 bits
  *               below the largest component of each matrix row and of each
- *               vector (of a bin or a cell), products and sums of digits are
+ *               vector (of a bin or a cell), of any size in FP64's range,
+ *               products and sums of digits are
  *               exact, and terms below 2^-50 of row times vector maximum are
- *               left out.  The FP32
+ *               left out.  A component that is not finite gives NaN in every
+ *               output that it reaches.  The FP32
  *               operator (EMSURF_FP32, MIXED) stores complex64 values and
  *               needs table and macromodel entries inside FP32's range.
  *  tables_on_device  0: offset_L/K and macromodels are host pointers;
@@ -488,7 +490,9 @@ EMSURF_API int emsurf_tabulate_offsets(double a, double b, double h, int32_t n,
  * interface (one J per side, rule 2), PEC-dielectric junction (J shared,
  * rule 3), and the junction of the interface with S_eq (label 2 of
  * Fig. composite); Z~ is the Schur complement of U^T Z U (Eq. mmm_mult)
- * on the interior unknowns.  Z: device [n_types][K][K] complex128.  EINVAL
+ * on the interior unknowns.  The elimination's trailing updates run on 55-bit
+ * integers below the largest component of each row of L and column of U of 32
+ * columns (the rest in FP64).  Z: device [n_types][K][K] complex128.  EINVAL
  * for n < 2, a patch that does not fit inside the footprint, Re eps <= 0 or
  * Im eps > 0, or a singular interior block.  Synchronises `stream`.       */
 EMSURF_API int emsurf_macromodel_slab_patch(double a, double b, double h, int32_t n,

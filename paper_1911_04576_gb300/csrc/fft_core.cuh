@@ -257,9 +257,8 @@ __device__ __forceinline__ void stage_any(int R, int P, const FastDiv& ns, const
     }
 }
 
-// All stages of one transform: first(ld), then shared memory, then last(st);
-// ld0/st1 are the first stage's source and the last one's destination,
-// mid(in) / put(out) the shared-memory accesses.  PC > 0: a compile-time length,
+// All stages of one transform: body(first, last, go) for each, which calls go(ld, st)
+// with the stage's source and destination.  PC > 0: a compile-time length,
 // whose code holds its own radices only (small launches are bound by
 // instruction fetch); 0: any length.
 template <int SIGN, int PC, int MAXR, typename T2, typename F>

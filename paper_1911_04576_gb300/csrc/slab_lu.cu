@@ -10,7 +10,12 @@
 // runs on the tensor cores instead, on base-256 digits (digits.cuh) with levels
 // 0 to 7 kept: the dropped products weigh 2^-57 of row maximum times column
 // maximum, below FP64's own rounding.  352 rank-1 steps over the whole trailing
-// block (one launch each): 122 ms; this: 12 ms.
+// block (one launch each): 122 ms; this: 12 ms.  Entries of L and U keep 55 bits
+// below the maximum of their row (of L) or column (of U) of a panel instead of 53
+// of their own.  Against a 113-bit Schur complement of the same tables (n = 2, 3; 56
+// to 336 interior unknowns) the error in norm is 3.2e-16 to 7.4e-16 (in FP64
+// arithmetic 4.8e-16 to 1.2e-15), that of the worst row 2.0e-15 (2.1e-15), that of
+// the worst entry above 1e-6 of its row 4.0e-11 (4.5e-11).
 #include <algorithm>
 
 #include "digits.cuh"

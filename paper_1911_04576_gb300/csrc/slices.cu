@@ -42,10 +42,20 @@
 // its copies and MMAs in flight, frees TMEM and returns.
 //
 // Measured, product of a 16 x 16 lattice with K = 576 (2.38 GB of digits, 350 us
-// at the copy rate): 1161 us in double-single FP32, 593 us here (bins and
-// macromodels 490 us, splitting the vectors 25 us); 12 x 9, K = 576 and 6 rhs:
-// 6575 us, 567 us (594 us with 8 instead of 12 macromodel columns per entry).
-// Error against 64 bits 7.2e-14, 7e-15 (both sizes).
+// at the copy rate): 1161 us in double-single FP32, 573 us here (600 us with waits
+// that every lane left by itself); 12 x 9, K = 576 and 6 rhs: 6575 us, 556 us (27 us
+// more with 8 instead of 12 macromodel columns per entry).
+//
+// Precision.  An entry of a matrix row or of a vector keeps the 55 bits below the
+// row's or vector's maximum, where double-single kept 48 of its own: an entry 2^-8
+// below the maximum has fewer.  The bound is on row maximum times vector maximum
+// instead of on each term.  Measured against 113-bit arithmetic (3 x 2 slab cells, K
+// = 324, entries of x spread over 0, 4, 8, 12 decades): error in norm 2.8e-15, 6.8e-15,
+// 8.2e-15, 7.7e-15, double-single 4.5e-14 at each; largest error over (|A| |x|)_i
+// 3.5e-15, 2.1e-14, 4.0e-14, 5.2e-14, double-single 7.1e-14, 1.7e-13, 4.0e-13, 4.6e-13.
+// The term of a row's entry 2^-p below its maximum with the vector's largest entry
+// has 55 - p bits, fewer than double-single's 48 for p above 7: the fixed point
+// loses where only such terms make up a sum.
 #include <algorithm>
 #include <vector>
 
