@@ -20,7 +20,8 @@
  *   - every call returns an emsurf_status; on EMSURF_EINVAL no output is
  *     written; emsurf_last_error() gives a thread-local message;
  *   - a handle keeps per-handle device workspaces (FFT grids, split
- *     operands, Krylov basis, preconditioner buffers), so it serves one call
+ *     operands, Krylov basis, preconditioner buffers, up to 8 MB for far
+ *     fields), so it serves one call
  *     at a time: calls on one handle from different host threads or streams
  *     must be serialised by the caller (different handles are independent).
  */
