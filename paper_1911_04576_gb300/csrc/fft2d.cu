@@ -253,7 +253,7 @@ size_t f2_layout(F2Plan& f, int px, int py, bool inverse) {
 
 
 // lanes per CTA: 32 bytes of them (a whole sector per bin), doubled while the grids
-// of all stay below 8 KB (a stage of fewer lanes would leave most of a CTA's
+// of all stay below 4 KB (a stage of fewer lanes would leave most of a CTA's
 // threads without a butterfly), halved while that leaves more than a tenth of the
 // SMs without a CTA (16 x 16 boxes, one rhs: 144 CTAs of 4 lanes on 152 SMs, 10.2 us).
 // One box with 33 rhs (K = 576): 47.6 -> 7.9 us per transform, 11 x 1 boxes with
@@ -264,7 +264,7 @@ template <typename T2>
 int f2_pick_lanes(int points, long long lanes) {
     const int sms = sm_count();
     int lw = f2_full_lw<T2>();
-    while (lw < kF2MaxLw && ((size_t)points << lw) * sizeof(T2) < 8192) ++lw;
+    while (lw < kF2MaxLw && ((size_t)points << lw) * sizeof(T2) < 4096) ++lw;
     for (; lw > 0; --lw)
         if (((lanes - 1) >> lw) + 1 >= (long long)sms * 9 / 10) return lw;
     return 0;
