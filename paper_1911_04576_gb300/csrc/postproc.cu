@@ -717,9 +717,11 @@ int far_field_run(emsurf_handle* h, const BoxShapes& box, double a, double b, do
         EMS_CUDA(cudaGetLastError());
         if (ms == kLsM) EMS_TRY((launch_lattice_sum<T, C, kLsM>(h, X1, N, tab, nd, S, st)));
         else EMS_TRY((launch_lattice_sum<T, C, kLsM / 2>(h, X1, N, tab, nd, S, st)));
-        // rhs in groups while that fills the device: each forms its directions' phases again
+        // rhs in groups while the device has room for all of them at once (8 warps per SM
+        // keep its FP64 unit busy): each forms its directions' phases again
         const int blocks = std::min((nd + warps - 1) / warps, h->num_sms * 32);
-        int rn = std::min(nrhs, (int)std::max<long long>((long long)nrhs * blocks / (2 * h->num_sms), (nrhs + 65534) / 65535));
+        const int groups = std::max(1, std::min(std::min(nrhs, 65535), 8 * h->num_sms / (blocks * warps)));
+        int rn = (nrhs + groups - 1) / groups;
         if (by_rhs && rn < 32 && (long long)blocks * (nrhs / 32) >= h->num_sms) rn = 32;
         far_field_kernel<C><<<dim3(blocks, (nrhs + rn - 1) / rn), 32 * warps, fsm, st>>>(
             S, g, drc, nd, E, nrhs, rn, k, ph, by_rhs, Fo + (size_t)d0 * 3, rcs ? rcs + d0 : nullptr, ndir);
