@@ -91,18 +91,18 @@ __device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t (&r)[4]) {
 
 // exponent ex with |v| < 2^ex for the largest |v| of a vector, from its bit
 // pattern (the patterns of non-negative doubles order like the values, NaN above
-// infinity) and n, the sources that are summed; INT_MIN when it is not finite.
-// From -1073 (the smallest subnormal) to 1026.
+// infinity) and n, the sources that are summed: from -1073 (the smallest
+// subnormal) to 1026, kSlNan when it is not finite
+constexpr int kSlNan = 1 << 16;
 __device__ __forceinline__ int sl_exp(unsigned long long mbits, int n) {
-    if (mbits >= 0x7ff0000000000000ull) return INT_MIN;
+    if (mbits >= 0x7ff0000000000000ull) return kSlNan;
     const double m = __longlong_as_double((long long)mbits);
     const int spare = n <= kSlExact ? 0 : n <= 4 * kSlExact ? 1 : 2;
     return (m > 0.0 ? ilogb(m) + 1 : 0) + spare;
 }
-// 2^e for -1022 <= e <= 1023, NaN for a row or vector that is not finite
-__device__ __forceinline__ double sl_pow2(int e, bool finite = true) {
-    return __longlong_as_double(finite ? (long long)(e + 1023) << 52 : 0x7ff8000000000000ll);
-}
+// 2^e for -1022 <= e <= 1023
+__device__ __forceinline__ double sl_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+__device__ __forceinline__ double sl_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 // Bytes d_t + 128 of the digits of rn(v 2^(54 - ex)), least significant first:
 // balanced digits are the bytes of I + sum_t 128 256^t.  From the bit pattern:
 // FP64 conversions run at the FP64 rate.
@@ -112,8 +112,8 @@ __device__ __forceinline__ unsigned long long sl_digits(double v, int ex) {
     unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
     // v = +-m 2^(max(e, 1) - 1075) below 2^ex: a shift to the left (by at most one,
     // more only for subnormal v) stays below 2^54
-    const int sh = max(e, 1) - 1021 - max(ex, -1073);
-    m = ex == INT_MIN || sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 63) : (m + (1ull << (-sh - 1))) >> -sh;
+    const int sh = max(e, 1) - 1021 - ex;
+    m = sh < -54 ? 0ull : sh >= 0 ? m << min(sh, 63) : (m + (1ull << (-sh - 1))) >> -sh;
     return ((long long)b < 0 ? 0ull - m : m) + 0x80808080808080ull;
 }
 __device__ __forceinline__ unsigned long long sl_abs(double v) {

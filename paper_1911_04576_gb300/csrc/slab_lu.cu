@@ -149,10 +149,9 @@ lu_panel_kernel(const SlabType* __restrict__ ty, int c, double2* __restrict__ B,
 // exponent of a row of L or a column of U (64 real sources) and 2^(ex - 8) (NaN
 // where an entry was not finite): contributions below 2^-1000 may lose digits
 __device__ __forceinline__ int lu_exp(unsigned long long mbits) {
-    const int ex = sl_exp(mbits, 2 * kLuNb);
-    return ex == INT_MIN ? ex : max(ex, -1000);
+    return max(sl_exp(mbits, 2 * kLuNb), -1000);
 }
-__device__ __forceinline__ double lu_pow(int ex) { return sl_pow2(ex == INT_MIN ? 0 : ex - 8, ex != INT_MIN); }
+__device__ __forceinline__ double lu_pow(int ex) { return ex == kSlNan ? sl_nan() : sl_pow2(ex - 8); }
 
 // L of the rows below the panel, one row per thread, and their digits: real rows
 // 2 i = [Re, -Im] and 2 i + 1 = [Im, Re] of the 32 columns, 128-byte swizzled.

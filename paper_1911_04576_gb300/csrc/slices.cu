@@ -42,7 +42,7 @@
 // its copies and MMAs in flight, frees TMEM and returns.
 //
 // Measured, product of a 16 x 16 lattice with K = 576 (2.38 GB of digits, 350 us
-// at the copy rate): 1161 us in double-single FP32, 573 us here (600 us with waits
+// at the copy rate): 1161 us in double-single FP32, 568 us here (600 us with waits
 // that every lane left by itself); 12 x 9, K = 576 and 6 rhs: 6575 us, 556 us (27 us
 // more with 8 instead of 12 macromodel columns per entry).
 //
@@ -469,14 +469,16 @@ __global__ void __launch_bounds__(kSlThreads, 1) slices_kernel(SlArgs g) {
                 const long long pr = im ? t0 - q[3] : q[0] - t1, pi = im ? t1 + q[2] : q[1] + t0;
                 // the sums scaled by 2^e, in two steps where that power or a product with it
                 // (below 2^63) could leave FP64's range; a component that was not finite
-                // marks every output
-                const int xex = xs[2 * cc + (im ? 1 : 0)], e = max(max(rex, -2000) + max(xex, -2000) - 52, -2000);
-                const int e0 = e >= -1000 && e <= 900 ? e : e / 2;
-                const double sc = sl_pow2(e0, min(rex, xex) != INT_MIN);
-                double2 u = make_double2((double)pr * sc, (double)pi * sc);
-                if (e0 != e) {
-                    const double s2 = sl_pow2(e - e0);
-                    u = make_double2(u.x * s2, u.y * s2);
+                // (kSlNan) marks every output
+                const int e = rex + xs[2 * cc + (im ? 1 : 0)] - 52;
+                double2 u = make_double2((double)pr, (double)pi);
+                if (e >= -1000 && e <= 900) {
+                    const double sc = sl_pow2(e);
+                    u = make_double2(u.x * sc, u.y * sc);
+                } else {
+                    const int e1 = max(min(e, 2000), -2000), e0 = e1 / 2;
+                    const double sc = sl_pow2(e0), s2 = e > 4000 ? sl_nan() : sl_pow2(e1 - e0);
+                    u = make_double2(u.x * sc * s2, u.y * sc * s2);
                 }
                 if (!w) {
                     // y_J = a L x_J + b K x_M, y_M = g K x_J + d L x_M
